@@ -112,12 +112,16 @@ int compact_indices(const uint8_t* flags, int64_t n, int32_t* out, uint32_t* cou
 }  // namespace urchin
 
 // ---- the BVH object --------------------------------------------------------
-// Internal node layout (64 bytes, 4 float4), both children in one node:
-//   n[0] = (left.lo.xyz, left.ref)    n[1] = (left.hi.xyz, left.count)
-//   n[2] = (right.lo.xyz, right.ref)  n[3] = (right.hi.xyz, right.count)
-// ref/count are int bit patterns: count == 0 -> ref is an internal node
-// index; count > 0 -> leaf holding particles [ref, ref + count) in Morton
-// order.  An empty child has lo > hi.  Node 0 is the root.
+// Leaves are the subtrees of at most kLeafMax particles of the binary radix
+// tree, listed in the order of a depth-first walk that takes a node's leaf
+// children before its inner ones (the order in which a ray sums its hits).
+// Above them stands an implicit 32-ary tree over that list: entry g of level
+// l + 1 bounds entries [32 g, 32 g + 32) of level l.  An entry is two float4:
+//   boxes[2e] = (lo.xyz, first particle)   boxes[2e + 1] = (hi.xyz, particles)
+// (particle range in Morton order, as int bit patterns; levels above 0 hold
+// boxes only).  Level l starts at entry lev_off[l] and has lev_cnt[l]
+// entries; the top level (at least 1) has one.
+constexpr int kMaxLevels = 8;     // 32^6 = 2^30 particles, one per leaf, plus level 0 and a spare
 struct urchin_bvh {
     int64_t n = 0;
     int periodic = 0;
@@ -128,8 +132,10 @@ struct urchin_bvh {
     float root_lo[3] = {0, 0, 0};
     float root_hi[3] = {0, 0, 0};
     int device = 0;
-    int n_nodes = 0;
-    float4* nodes = nullptr;      // [4 * n_nodes]
+    int n_lev = 0;                // index of the top level
+    int lev_off[kMaxLevels] = {};
+    int lev_cnt[kMaxLevels] = {};
+    float4* boxes = nullptr;      // [2 * entries]
     float4* xyzh = nullptr;       // [n] Morton order
     float* A32 = nullptr;         // [n] sigma_th (m/m_p) (8/pi) / (h unit_cm)^2
     double* A64 = nullptr;        // [n]
@@ -141,12 +147,10 @@ struct urchin_bvh {
 namespace urchin {
 
 // Bits of the device status word shared by the kernels of one call.
-constexpr unsigned kStStack = 1u;       // traversal stack overflow
 constexpr unsigned kStOrigin = 2u;      // origin index out of range
 constexpr unsigned kStNonfinite = 4u;   // non-finite or non-positive x
 constexpr unsigned kStInput = 8u;       // n_H or T not finite and > 0
 constexpr unsigned kStWarm = 16u;       // warm-start x outside (0, 1]
-constexpr unsigned kStVisit = 32u;      // traversal visit limit (malformed tree)
 constexpr unsigned kStSegment = 64u;    // stored-segment fill disagrees with its count
 
 constexpr int kLeafMax = 32;      // subtrees with <= kLeafMax particles become leaves
@@ -158,7 +162,6 @@ constexpr int kKTab = 2048;       // intervals of the full-chord M4 table in t =
 // tabulated at t_i = i / kKTab as (K(t_i), dK/dt(t_i) / kKTab), host side.
 void m4_full_table(float2* out /* [kKTab + 1] */);
 constexpr int kChunkEntries = 32;   // MODE_CHUNK: segment entries per chunk
-constexpr int kStackMax = 64;     // traversal stack (tree depth <= 62 for 30-bit codes)
 
 // Column tracing shared by urchin_trace_columns and urchin_solve.
 struct TraceJob {

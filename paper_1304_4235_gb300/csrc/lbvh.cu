@@ -4,9 +4,10 @@
 // LBVH: 30-bit Morton codes of the sphere centres, stable radix sort, the
 // binary radix tree of Karras (2012, "Maximizing parallelism in the
 // construction of BVHs, octrees and k-d trees"), bottom-up refit of sphere
-// bounds, then a packed two-children-per-node layout in which subtrees of
-// at most kLeafMax particles become leaves.  The particle data are copied
-// into Morton order so that a leaf is a contiguous range.
+// bounds.  Subtrees of at most kLeafMax particles become leaves, listed in a
+// fixed depth-first order, and an implicit 32-ary tree of boxes over that list
+// is what the traversal reads (one lane tests one child).  The particle data
+// are copied into Morton order so that a leaf is a contiguous range.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -250,55 +251,127 @@ __global__ void k_refit(const float4* __restrict__ xyzh, int n, const int32_t* c
     }
 }
 
-__device__ __forceinline__ void pack_child(int32_t c, const float4* __restrict__ xyzh, const float* boxes,
-                                           const int32_t* first, const int32_t* last, float4* out0,
-                                           float4* out1)
+// Particles of child c of an inner node (c < 0: the single particle ~c).
+__device__ __forceinline__ int child_size(int32_t c, const int32_t* __restrict__ first,
+                                          const int32_t* __restrict__ last)
 {
-    float lo[3], hi[3];
-    child_box(c, xyzh, boxes, lo, hi);
-    int ref, cnt;
-    if (c < 0) {
-        ref = ~c;
-        cnt = 1;
-    } else {
-        int size = last[c] - first[c] + 1;
-        if (size <= kLeafMax) { ref = first[c]; cnt = size; }
-        else { ref = c; cnt = 0; }
+    return c < 0 ? 1 : last[c] - first[c] + 1;
+}
+
+__device__ __forceinline__ int child_first(int32_t c, const int32_t* __restrict__ first)
+{
+    return c < 0 ? ~c : first[c];
+}
+
+// flags[p] = 1 where a leaf starts at particle p: the children of at most
+// kLeafMax particles of the root and of every larger inner node
+__global__ void k_leaf_flags(int n, const int32_t* __restrict__ child_l, const int32_t* __restrict__ child_r,
+                             const int32_t* __restrict__ first, const int32_t* __restrict__ last, uint32_t* flags)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n - 1 || (i > 0 && last[i] - first[i] + 1 <= kLeafMax)) return;
+    const int32_t l = child_l[i], r = child_r[i];
+    if (child_size(l, first, last) <= kLeafMax) flags[child_first(l, first)] = 1u;
+    if (child_size(r, first, last) <= kLeafMax) flags[child_first(r, first)] = 1u;
+}
+
+// Leaves in subtree c, from the exclusive scan of the flags (start[n] = all)
+__device__ __forceinline__ int leaves_in(int32_t c, const int32_t* __restrict__ first,
+                                         const int32_t* __restrict__ last, const uint32_t* __restrict__ start)
+{
+    const int lo = child_first(c, first);
+    return (int)(start[lo + child_size(c, first, last)] - start[lo]);
+}
+
+// Every leaf to its place in the depth-first list (leaf children before
+// inner ones, left before right): the leaves that precede it below each of
+// its ancestors, summed on the way up.
+__global__ void k_leaf_place(const float4* __restrict__ xyzh, int n, const int32_t* __restrict__ child_l,
+                             const int32_t* __restrict__ child_r, const int32_t* __restrict__ first,
+                             const int32_t* __restrict__ last, const int32_t* __restrict__ parent_int,
+                             const float* boxes, const uint32_t* __restrict__ start, int n_leaves, float4* out,
+                             unsigned* err)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n - 1 || (i > 0 && last[i] - first[i] + 1 <= kLeafMax)) return;
+    const int32_t cl = child_l[i], cr = child_r[i];
+    const bool ll = child_size(cl, first, last) <= kLeafMax, lr = child_size(cr, first, last) <= kLeafMax;
+    if (!ll && !lr) return;
+    int at = 0, c = i;
+    int p = i > 0 ? parent_int[i] : -1;
+    // the tree is at most 62 levels deep; the cap only guards against a
+    // malformed parent chain
+    for (int level = 0; p >= 0; ++level) {
+        if (level > 128) {
+            atomicOr(err, 4u);
+            return;
+        }
+        const int32_t pl = child_l[p], pr = child_r[p];
+        if (c == pr) {
+            at += child_size(pl, first, last) <= kLeafMax ? 1 : leaves_in(pl, first, last, start);
+        } else if (child_size(pr, first, last) <= kLeafMax) {
+            ++at;
+        }
+        c = p;
+        p = p > 0 ? parent_int[p] : -1;
     }
-    *out0 = make_float4(lo[0], lo[1], lo[2], __int_as_float(ref));
-    *out1 = make_float4(hi[0], hi[1], hi[2], __int_as_float(cnt));
+    float lo[3], hi[3];
+    for (int q = 0; q < 2; ++q) {
+        if (!(q == 0 ? ll : lr)) continue;
+        const int32_t ch = q == 0 ? cl : cr;
+        const int e = at + (q == 1 && ll ? 1 : 0);
+        if (e < 0 || e >= n_leaves) {              // never true for a well-formed tree
+            atomicOr(err, 4u);
+            return;
+        }
+        child_box(ch, xyzh, boxes, lo, hi);
+        out[2 * (int64_t)e] = make_float4(lo[0], lo[1], lo[2], __int_as_float(child_first(ch, first)));
+        out[2 * (int64_t)e + 1] =
+            make_float4(hi[0], hi[1], hi[2], __int_as_float(child_size(ch, first, last)));
+    }
 }
 
-__global__ void k_pack(const float4* __restrict__ xyzh, int n, const int32_t* child_l,
-                       const int32_t* child_r, const int32_t* first, const int32_t* last,
-                       const float* boxes, float4* nodes)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n - 1) return;
-    float4 a, b, c, d;
-    pack_child(child_l[i], xyzh, boxes, first, last, &a, &b);
-    pack_child(child_r[i], xyzh, boxes, first, last, &c, &d);
-    nodes[4 * (int64_t)i + 0] = a;
-    nodes[4 * (int64_t)i + 1] = b;
-    nodes[4 * (int64_t)i + 2] = c;
-    nodes[4 * (int64_t)i + 3] = d;
-}
-
-// n == 1: one root whose left child is the single particle, right child empty
-__global__ void k_pack_single(const float4* __restrict__ xyzh, float4* nodes)
+// n == 1: one leaf
+__global__ void k_leaf_single(const float4* __restrict__ xyzh, float4* out)
 {
     float lo[3], hi[3];
     sphere_box(xyzh[0], lo, hi);
-    nodes[0] = make_float4(lo[0], lo[1], lo[2], __int_as_float(0));
-    nodes[1] = make_float4(hi[0], hi[1], hi[2], __int_as_float(1));
-    nodes[2] = make_float4(1.f, 1.f, 1.f, __int_as_float(0));
-    nodes[3] = make_float4(-1.f, -1.f, -1.f, __int_as_float(-1));   // count < 0: no child
+    out[0] = make_float4(lo[0], lo[1], lo[2], __int_as_float(0));
+    out[1] = make_float4(hi[0], hi[1], hi[2], __int_as_float(1));
+}
+
+// One level of the 32-ary tree: a warp bounds 32 entries of the level below.
+__global__ void k_level(const float4* __restrict__ in, int n_in, float4* out, int n_out)
+{
+    const int g = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (g >= n_out) return;
+    const int e = 32 * g + lane;
+    float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f), hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+    if (e < n_in) {
+        lo = in[2 * (int64_t)e];
+        hi = in[2 * (int64_t)e + 1];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o));
+        lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o));
+        lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o));
+        hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o));
+        hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o));
+        hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o));
+    }
+    if (lane == 0) {
+        lo.w = hi.w = 0.f;
+        out[2 * (int64_t)g] = lo;
+        out[2 * (int64_t)g + 1] = hi;
+    }
 }
 
 void free_bvh_arrays(urchin_bvh* b)
 {
     if (!b) return;
-    cudaFree(b->nodes);
+    cudaFree(b->boxes);
     cudaFree(b->xyzh);
     cudaFree(b->A32);
     cudaFree(b->A64);
@@ -306,7 +379,7 @@ void free_bvh_arrays(urchin_bvh* b)
     cudaFree(b->inv);
     cudaFree(b->ktab);
     b->ktab = nullptr;
-    b->nodes = nullptr;
+    b->boxes = nullptr;
     b->xyzh = nullptr;
     b->A32 = nullptr;
     b->A64 = nullptr;
@@ -322,8 +395,6 @@ int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaS
     b->L = box->L;
     b->unit_cm = box->unit_cm;
     URCHIN_TRY_CUDA(cudaGetDevice(&b->device));
-    b->n_nodes = (int)std::max<int64_t>(1, n - 1);
-    URCHIN_TRY_CUDA(cudaMalloc(&b->nodes, sizeof(float4) * 4 * (size_t)b->n_nodes));
     URCHIN_TRY_CUDA(cudaMalloc(&b->xyzh, sizeof(float4) * (size_t)n));
     URCHIN_TRY_CUDA(cudaMalloc(&b->A32, sizeof(float) * (size_t)n));
     URCHIN_TRY_CUDA(cudaMalloc(&b->A64, sizeof(double) * (size_t)n));
@@ -358,6 +429,8 @@ int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaS
     size_t o_pleaf = lay.take((size_t)n * 4);
     size_t o_boxes = lay.take((size_t)ni * 6 * 4);
     size_t o_visits = lay.take((size_t)ni * 4);
+    size_t o_flags = lay.take((size_t)(n + 1) * 4);
+    size_t o_stmp = lay.take(scan_tmp_bytes(n + 1));
     Scratch scr;
     URCHIN_TRY(scr.alloc(lay.bytes, s));
     unsigned* bounds = scr.at<unsigned>(o_bounds);
@@ -390,41 +463,73 @@ int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaS
                                   bounds + 7);
     URCHIN_TRY(launched());
 
-    if (n == 1) {
-        k_pack_single<<<1, 1, 0, s>>>(b->xyzh, b->nodes);
-        URCHIN_TRY(launched());
-    } else {
-        int32_t* cl = scr.at<int32_t>(o_cl);
-        int32_t* cr = scr.at<int32_t>(o_cr);
-        int32_t* first = scr.at<int32_t>(o_first);
-        int32_t* last = scr.at<int32_t>(o_last);
-        int32_t* pint = scr.at<int32_t>(o_pint);
+    int n_leaves = 1;
+    int32_t* cl = scr.at<int32_t>(o_cl);
+    int32_t* cr = scr.at<int32_t>(o_cr);
+    int32_t* first = scr.at<int32_t>(o_first);
+    int32_t* last = scr.at<int32_t>(o_last);
+    int32_t* pint = scr.at<int32_t>(o_pint);
+    float* boxes = scr.at<float>(o_boxes);
+    uint32_t* start = scr.at<uint32_t>(o_flags);
+    const unsigned gi = (unsigned)((ni + 255) / 256);
+    if (n > 1) {
         int32_t* pleaf = scr.at<int32_t>(o_pleaf);
-        float* boxes = scr.at<float>(o_boxes);
         unsigned* visits = scr.at<unsigned>(o_visits);
-        int ninode = (int)(n - 1);
-        unsigned gi = (unsigned)((ninode + 255) / 256);
         unsigned gl = (unsigned)((n + 255) / 256);
-        URCHIN_TRY_CUDA(cudaMemsetAsync(visits, 0, (size_t)ninode * 4, s));
+        URCHIN_TRY_CUDA(cudaMemsetAsync(visits, 0, (size_t)ni * 4, s));
+        URCHIN_TRY_CUDA(cudaMemsetAsync(start, 0, (size_t)(n + 1) * 4, s));
         k_karras<<<gi, 256, 0, s>>>(codes, (int)n, cl, cr, first, last, pint, pleaf);
         URCHIN_TRY(launched());
+        k_leaf_flags<<<gi, 256, 0, s>>>((int)n, cl, cr, first, last, start);
+        URCHIN_TRY(launched());
+        // start[p] = leaves before particle p; start[n] = all (its flag is 0)
+        URCHIN_TRY(scan_exclusive_u32(start, start, n + 1, scr.at<void>(o_stmp), nullptr, s));
+        uint32_t total = 0;
+        URCHIN_TRY_CUDA(cudaMemcpyAsync(&total, start + n, sizeof(total), cudaMemcpyDeviceToHost, s));
         k_refit<<<gl, 256, 0, s>>>(b->xyzh, (int)n, cl, cr, pint, pleaf, boxes, visits, bounds + 7);
         URCHIN_TRY(launched());
-        k_pack<<<gi, 256, 0, s>>>(b->xyzh, (int)n, cl, cr, first, last, boxes, b->nodes);
+        URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
+        if (total < 1 || (int64_t)total > n)
+            return set_error(URCHIN_ERR_CUDA, "urchin_build_bvh: %u leaves for %lld particles", total, (long long)n);
+        n_leaves = (int)total;
+    }
+    // levels up to the first of one entry above the leaves
+    int64_t entries = 0;
+    b->n_lev = 0;
+    for (int l = 0, c = n_leaves;; ++l, c = (c + 31) / 32) {
+        if (l >= kMaxLevels) return set_error(URCHIN_ERR_CUDA, "urchin_build_bvh: too many tree levels");
+        b->lev_off[l] = (int)entries;
+        b->lev_cnt[l] = c;
+        b->n_lev = l;
+        entries += c;
+        if (l > 0 && c == 1) break;
+    }
+    URCHIN_TRY_CUDA(cudaMalloc(&b->boxes, sizeof(float4) * 2 * (size_t)entries));
+    if (n > 1)
+        k_leaf_place<<<gi, 256, 0, s>>>(b->xyzh, (int)n, cl, cr, first, last, pint, boxes, start, n_leaves, b->boxes,
+                                        bounds + 7);
+    else
+        k_leaf_single<<<1, 1, 0, s>>>(b->xyzh, b->boxes);
+    URCHIN_TRY(launched());
+    for (int l = 1; l <= b->n_lev; ++l) {
+        const int c = b->lev_cnt[l];
+        k_level<<<(unsigned)((c + 7) / 8), 256, 0, s>>>(b->boxes + 2 * (int64_t)b->lev_off[l - 1], b->lev_cnt[l - 1],
+                                                        b->boxes + 2 * (int64_t)b->lev_off[l], c);
         URCHIN_TRY(launched());
     }
-    float4 root[4];
-    URCHIN_TRY_CUDA(cudaMemcpyAsync(root, b->nodes, sizeof(root), cudaMemcpyDeviceToHost, s));
+    float4 root[2];
+    URCHIN_TRY_CUDA(cudaMemcpyAsync(root, b->boxes + 2 * (int64_t)b->lev_off[b->n_lev], sizeof(root),
+                                    cudaMemcpyDeviceToHost, s));
     URCHIN_TRY_CUDA(cudaMemcpyAsync(hb, bounds, sizeof(hb), cudaMemcpyDeviceToHost, s));
     URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
     if (hb[7] & 12u) return set_error(URCHIN_ERR_CUDA, "urchin_build_bvh: internal consistency check failed (%u)",
                                       hb[7]);
-    b->root_lo[0] = std::min(root[0].x, root[2].x);
-    b->root_lo[1] = std::min(root[0].y, root[2].y);
-    b->root_lo[2] = std::min(root[0].z, root[2].z);
-    b->root_hi[0] = std::max(root[1].x, root[3].x);
-    b->root_hi[1] = std::max(root[1].y, root[3].y);
-    b->root_hi[2] = std::max(root[1].z, root[3].z);
+    b->root_lo[0] = root[0].x;
+    b->root_lo[1] = root[0].y;
+    b->root_lo[2] = root[0].z;
+    b->root_hi[0] = root[1].x;
+    b->root_hi[1] = root[1].y;
+    b->root_hi[2] = root[1].z;
     scr.release();
     URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
     return URCHIN_OK;

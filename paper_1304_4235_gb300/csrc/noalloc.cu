@@ -132,7 +132,5 @@ extern "C" int urchin_trace_columns_noalloc(const urchin_bvh* bvh, const double*
     URCHIN_TRY_CUDA(cudaMemcpyAsync(&st, ctr + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
     if (st & kStOrigin) return set_error(URCHIN_ERR_ARG, "urchin_trace_columns_noalloc: origin index out of range");
-    if (st & kStStack) return set_error(URCHIN_ERR_CUDA, "urchin_trace_columns_noalloc: traversal stack overflow");
-    if (st & kStVisit) return set_error(URCHIN_ERR_CUDA, "urchin_trace_columns_noalloc: malformed tree");
     return URCHIN_OK;
 }

@@ -1337,7 +1337,6 @@ int Solver::read_scalars(double* maxrel, unsigned* st)
     *st = (unsigned)(h[1] >> 32);
     last_above = (int64_t)h[7];
     if (*st & kStNonfinite) return set_error(URCHIN_ERR_NONFINITE, "urchin_solve: non-finite neutral fraction");
-    if (*st & (kStStack | kStVisit)) return set_error(URCHIN_ERR_CUDA, "urchin_solve: traversal stack/visit limit hit");
     if (*st & kStSegment) return set_error(URCHIN_ERR_CUDA, "urchin_solve: segment fill disagrees with its count");
     return URCHIN_OK;
 }

@@ -7,14 +7,17 @@
 // of Eq. Gt via the erf form I(h,b,z1,z2).
 //
 // Work distribution: a persistent grid; each warp takes tasks of 32
-// Morton-consecutive origins in one direction from an atomic queue, so the
-// 32 rays of a warp are parallel and start close together.  The warp walks
-// the tree as one packet: a child is entered when any lane's segment crosses
-// its box (warp vote), so every lane follows the same path and stack and the
-// node fetches are broadcasts; at a leaf each lane tests its own segment
-// against the leaf's spheres.  The packet visits the union of the lanes'
-// nodes (a beam about as wide as the 32 origins' spread, comparable to h),
-// in exchange for uniform control flow.
+// neighbouring origins in one direction from an atomic queue, so the 32 rays
+// of a warp are parallel and start close together (a beam).  The beam walks
+// the 32-ary box tree as one packet, each lane testing one child of the
+// current entry against the beam; at a leaf each lane tests one sphere
+// against the beam, and the spheres that pass are staged in shared memory.
+// Every 32 staged spheres, each lane tests them against its own ray in the
+// beam's frame (a handful of packed FP32 operations per sphere, conservative)
+// and keeps the ones it may cross as a bit mask; the exact hit test and the
+// chord integral then run with every lane on its own next candidate, so that
+// the expensive part works on (nearly) full warps while each ray still sums
+// its hits in the tree's fixed order.
 #include <algorithm>
 #include <cmath>
 
@@ -26,8 +29,9 @@ namespace {
 
 struct TraceParams {
     const float2* ktab;           // [kKTab + 1] full-chord M4 table (value, slope x dt)
-    const float4* nodes;
-    int n_nodes;
+    const float4* boxes;          // 32-ary tree (urchin_bvh::boxes)
+    int n_lev;
+    int lev_off[kMaxLevels], lev_cnt[kMaxLevels];
     int n;
     const float4* xyzh;
     const float* w32;
@@ -94,6 +98,7 @@ struct Sink {
     Real coef;                    // MODE_SCATTER
     Real near, near_c;            // near/far: near column and its compensation
     double ox, oy, oz;            // near/far: shifted origin in double (the near test)
+    Real sx, sy, sz;              // (image-shifted) origin
     uint32_t lo_pend, hi_pend;    // MODE_FILL, split indices: halves / bytes of the current word
     int64_t ray;                  // MODE_CHUNK: row k n + origin slot
     int2* cw;                     // MODE_CHUNK: the ray's current chunk
@@ -237,53 +242,6 @@ __device__ __forceinline__ float m4_full_tab(const float2* tab, float t)
            (f3 - f2) * b.y;
 }
 
-__device__ __forceinline__ float m4_inner_prim_f(float b2, float a)
-{
-    float q = sqrtf(b2 + a * a);
-    float L = b2 > 0.f ? logf(a + q) - 0.5f * logf(b2) : 0.f;
-    return a * (1.f - 6.f * b2 - 2.f * a * a) + 1.5f * a * q * q * q + 2.25f * b2 * a * q + 2.25f * b2 * b2 * L;
-}
-
-// Gauss-Legendre nodes and weights on [-1, 1], n = 8
-__constant__ float kGLx[8] = {-0.9602898564975363f, -0.7966664774136267f, -0.5255324099163290f,
-                              -0.1834346424956498f, 0.1834346424956498f,  0.5255324099163290f,
-                              0.7966664774136267f,  0.9602898564975363f};
-__constant__ float kGLw[8] = {0.1012285362903763f, 0.2223810344533745f, 0.3137066458778873f,
-                              0.3626837833783620f, 0.3626837833783620f, 0.3137066458778873f,
-                              0.2223810344533745f, 0.1012285362903763f};
-
-__device__ __forceinline__ float m4_outer_gl(float b2, float a1, float a2)
-{
-    const float m = 0.5f * (a1 + a2), r = 0.5f * (a2 - a1);
-    float acc = 0.f;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        float u = fmaf(r, kGLx[g], m);
-        float v = 1.f - sqrtf(fmaf(u, u, b2));
-        acc = fmaf(kGLw[g], v * v * v, acc);
-    }
-    return 2.f * r * acc;
-}
-
-// int_{a1}^{a2} M4shape du for 0 <= a1 < a2 <= c
-__device__ __forceinline__ float m4_piece_f(float b2, float a1, float a2)
-{
-    const float s = b2 < 0.25f ? sqrtf(0.25f - b2) : 0.f;
-    float r = 0.f;
-    if (a1 < s) r += m4_inner_prim_f(b2, fminf(a2, s)) - m4_inner_prim_f(b2, a1);
-    const float lo = fmaxf(a1, s);
-    if (a2 > lo) r += m4_outer_gl(b2, lo, a2);
-    return r;
-}
-
-__device__ __forceinline__ float m4_part_f(float b2, float u1, float u2)
-{
-    float t = 0.f;
-    if (u1 < 0.f) t += m4_piece_f(b2, fmaxf(0.f, -u2), -u1);
-    if (u2 > 0.f) t += m4_piece_f(b2, fmaxf(0.f, u1), u2);
-    return t;
-}
-
 // int_{a1}^{a2} M4shape(sqrt(b2 + u^2)) du for 0 <= a1 <= a2 <= sqrt(1 - b2):
 // the inner piece (q <= 1/2) by its antiderivative Fi (Fi(0) = 0), the
 // outer piece by 6-point Gauss-Legendre quadrature of 2(1 - q)^3 (within
@@ -373,42 +331,26 @@ struct Kahan {
     }
 };
 
-// Segment [0, L] of o + t d against an axis-aligned box (float slab test).
-__device__ __forceinline__ bool seg_box(float ox, float oy, float oz, float ix, float iy, float iz,
-                                        float L, float4 lo, float4 hi)
-{
-    float tx0 = (lo.x - ox) * ix, tx1 = (hi.x - ox) * ix;
-    float ty0 = (lo.y - oy) * iy, ty1 = (hi.y - oy) * iy;
-    float tz0 = (lo.z - oz) * iz, tz1 = (hi.z - oz) * iz;
-    float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.f));
-    float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fminf(fmaxf(tz0, tz1), L));
-    return tn <= tf;
-}
-
-__device__ __forceinline__ float safe_inv(double d)
-{
-    return fabs(d) > 1e-20 ? (float)(1.0 / d) : copysignf(1e30f, (float)d);
-}
-
 // ---- the packet's beam ------------------------------------------------------
-// The 32 rays of a packet are parallel (one direction d).  In a frame
-// (e1, e2, d) anchored at one live lane's origin B, a lane's segment is the
-// point (u_i, v_i) across the direction and the depth interval
-// [t_i, t_i + l_ray] along it; the beam is the box [u_lo, u_hi] x [v_lo, v_hi]
-// of the live lanes' points and the depth range [t_lo, t_hi + l_ray].  A
-// particle can only be crossed by some lane if its sphere reaches that box:
-// lateral distance from (u_j, v_j) to the box below h_j and depth range
-// [t_j - h_j, t_j + h_j] overlapping.  At a leaf, lanes 0..cnt-1 test one
-// particle each against the beam (one warp instruction stream for the whole
-// leaf) and only the particles that pass are tested per lane.  The test is
-// made conservative by a margin of a few float roundings of the coordinates,
-// so it never drops a crossing: every lane's hits, and the order in which it
-// sums them, are those of the unfiltered loop.
+// The 32 rays of a packet are parallel (one direction d).  In the frame
+// (e1, e2, d) anchored at C, a lane's segment is the point (u_i, v_i) across
+// the direction and the depths [t_i, t_i + l_ray]; the beam is the box
+// |u| <= hu, |v| <= hv, |t| <= ht that holds the live lanes' segments.
+// Everything decided in this frame (child boxes, spheres against the beam,
+// spheres against a lane's ray) is a conservative filter in front of the exact
+// hit test: distances carry a margin of several times the roundings of the
+// projections (each coordinate difference is rounded once and projected with
+// a frame orthonormal to ~3e-7, together below 2e-6 of the distances
+// involved; the margin is 4e-6 of them, plus 3e-7 of the coordinates for an
+// origin held in double), so no crossing is dropped and the hits are those of
+// testing every sphere.
 struct Beam {
-    float bx, by, bz;             // anchor B
-    float e1x, e1y, e1z, e2x, e2y, e2z, dx, dy, dz;
-    float ulo, uhi, vlo, vhi, tlo, thi;
-    float eps;                    // absolute margin of the projections
+    float4 c;                     // C, ht
+    float4 e1;                    // e1, hu
+    float4 e2;                    // e2, hv
+    float4 d;                     // d, margin
+    float4 o;                     // half extents of the beam's axis-aligned bounds, margin included; 0
+    float4 r;                     // its radii along d x (x, y, z), margin included; 0
 };
 
 __device__ __forceinline__ float wmin(float v)
@@ -422,22 +364,16 @@ __device__ __forceinline__ float wmax(float v)
     return v;
 }
 
-// Called by all 32 lanes with the same direction; (fx, fy, fz) is the
-// lane's (shifted) origin.  Writes the warp's beam to shared memory (out,
-// one per warp) and returns false when no lane is live.
-__device__ __forceinline__ bool make_beam(Beam* out, bool live, float fx, float fy, float fz, float dx, float dy,
-                                          float dz, float L)
+// Called by all 32 lanes with the same direction d and length L; (sx, sy, sz)
+// is the lane's (shifted) origin.  Writes the warp's beam to shared memory and
+// the lane's point and depth to (u, v, t); at least one lane is live.
+template <typename Real>
+__device__ __forceinline__ void make_beam(Beam* out, unsigned lv, bool live, Real sx, Real sy, Real sz, float dx,
+                                          float dy, float dz, float L, float& u, float& v, float& t)
 {
-    const unsigned lv = __ballot_sync(0xffffffffu, live);
-    if (!lv) return false;
-    Beam B;
     const int a = __ffs(lv) - 1;
-    B.bx = __shfl_sync(0xffffffffu, fx, a);
-    B.by = __shfl_sync(0xffffffffu, fy, a);
-    B.bz = __shfl_sync(0xffffffffu, fz, a);
-    B.dx = dx;
-    B.dy = dy;
-    B.dz = dz;
+    const Real bx = __shfl_sync(0xffffffffu, sx, a), by = __shfl_sync(0xffffffffu, sy, a),
+               bz = __shfl_sync(0xffffffffu, sz, a);
     // e1 perpendicular to d, from the coordinate axis least aligned with it
     float ax = 0.f, ay = 0.f, az = 0.f;
     if (fabsf(dx) <= fabsf(dy) && fabsf(dx) <= fabsf(dz)) ax = 1.f;
@@ -448,51 +384,112 @@ __device__ __forceinline__ bool make_beam(Beam* out, bool live, float fx, float 
     e1x *= inv;
     e1y *= inv;
     e1z *= inv;
-    B.e1x = e1x;
-    B.e1y = e1y;
-    B.e1z = e1z;
-    B.e2x = dy * e1z - dz * e1y;
-    B.e2y = dz * e1x - dx * e1z;
-    B.e2z = dx * e1y - dy * e1x;
-    const float rx = fx - B.bx, ry = fy - B.by, rz = fz - B.bz;
-    const float u = rx * B.e1x + ry * B.e1y + rz * B.e1z;
-    const float v = rx * B.e2x + ry * B.e2y + rz * B.e2z;
-    const float t = rx * dx + ry * dy + rz * dz;
-    B.ulo = wmin(live ? u : INFINITY);
-    B.uhi = wmax(live ? u : -INFINITY);
-    B.vlo = wmin(live ? v : INFINITY);
-    B.vhi = wmax(live ? v : -INFINITY);
-    B.tlo = wmin(live ? t : INFINITY);
-    B.thi = wmax(live ? t : -INFINITY) + L;
-    // roundings of the projections: a few ulp of the coordinates' magnitude
-    const float span = fmaxf(fmaxf(B.uhi - B.ulo, B.vhi - B.vlo), B.thi - B.tlo);
-    B.eps = 1e-5f * (span + fabsf(B.bx) + fabsf(B.by) + fabsf(B.bz));
+    const float e2x = dy * e1z - dz * e1y, e2y = dz * e1x - dx * e1z, e2z = dx * e1y - dy * e1x;
+    // the live lanes' bounds relative to lane a's origin give the centre
+    float rx = (float)(sx - bx), ry = (float)(sy - by), rz = (float)(sz - bz);
+    u = rx * e1x + ry * e1y + rz * e1z;
+    v = rx * e2x + ry * e2y + rz * e2z;
+    t = rx * dx + ry * dy + rz * dz;
+    const float um = 0.5f * (wmin(live ? u : INFINITY) + wmax(live ? u : -INFINITY));
+    const float vm = 0.5f * (wmin(live ? v : INFINITY) + wmax(live ? v : -INFINITY));
+    const float tm = 0.5f * (wmin(live ? t : INFINITY) + wmax(live ? t : -INFINITY) + L);
+    const float cx = (float)bx + (um * e1x + vm * e2x + tm * dx);
+    const float cy = (float)by + (um * e1y + vm * e2y + tm * dy);
+    const float cz = (float)bz + (um * e1z + vm * e2z + tm * dz);
+    rx = (float)(sx - Real(cx));
+    ry = (float)(sy - Real(cy));
+    rz = (float)(sz - Real(cz));
+    u = rx * e1x + ry * e1y + rz * e1z;
+    v = rx * e2x + ry * e2y + rz * e2z;
+    t = rx * dx + ry * dy + rz * dz;
+    float hu = wmax(live ? fabsf(u) : 0.f), hv = wmax(live ? fabsf(v) : 0.f);
+    float ht = wmax(live ? fmaxf(fabsf(t), fabsf(t + L)) : 0.f);
+    const float eps = 4e-6f * (hu + hv + ht) + 3e-7f * (fabsf(cx) + fabsf(cy) + fabsf(cz));
+    hu += eps;
+    hv += eps;
+    ht += eps;
     __syncwarp();                    // the previous beam's readers are done
-    if ((threadIdx.x & 31) == 0) *out = B;
+    if ((threadIdx.x & 31) == 0) {
+        out->c = make_float4(cx, cy, cz, ht);
+        out->e1 = make_float4(e1x, e1y, e1z, hu);
+        out->e2 = make_float4(e2x, e2y, e2z, hv);
+        out->d = make_float4(dx, dy, dz, eps);
+        out->o = make_float4(hu * fabsf(e1x) + hv * fabsf(e2x) + ht * fabsf(dx) + eps,
+                             hu * fabsf(e1y) + hv * fabsf(e2y) + ht * fabsf(dy) + eps,
+                             hu * fabsf(e1z) + hv * fabsf(e2z) + ht * fabsf(dz) + eps, 0.f);
+        // d x axis lies in the (e1, e2) plane: its components are those of the axis on e2 and e1
+        out->r = make_float4(hu * fabsf(e2x) + hv * fabsf(e1x) + eps, hu * fabsf(e2y) + hv * fabsf(e1y) + eps,
+                             hu * fabsf(e2z) + hv * fabsf(e1z) + eps, 0.f);
+    }
     __syncwarp();
-    return true;
 }
 
-// Mask of the leaf's particles (bit l for particle ref + l) that the beam can
-// reach.  Every lane calls it; lanes 0..cnt-1 test one particle each.
-__device__ __forceinline__ unsigned beam_mask(const TraceParams& P, const Beam& B, int ref, int cnt)
+// Whether the beam may reach the box [lo, hi]: separating axes x, y, z (on
+// the differences to C, so that near-touching faces are exact), e1, e2, d and
+// d x (x, y, z).  Comparisons are written so that a NaN passes.
+__device__ __forceinline__ bool beam_box(const Beam& B, float4 lo, float4 hi)
 {
-    const int lane = threadIdx.x & 31;
-    bool pass = false;
-    if (lane < cnt && ref >= 0 && cnt <= kLeafMax && ref + cnt <= P.n) {
-        const float4 q = __ldg(P.xyzh + ref + lane);
-        const float rx = q.x - B.bx, ry = q.y - B.by, rz = q.z - B.bz;
-        const float u = rx * B.e1x + ry * B.e1y + rz * B.e1z;
-        const float v = rx * B.e2x + ry * B.e2y + rz * B.e2z;
-        const float t = rx * B.dx + ry * B.dy + rz * B.dz;
-        const float hh = q.w * 1.00001f + B.eps + 1e-5f * (fabsf(rx) + fabsf(ry) + fabsf(rz));
-        const float du = fmaxf(fmaxf(B.ulo - u, u - B.uhi), 0.f);
-        const float dv = fmaxf(fmaxf(B.vlo - v, v - B.vhi), 0.f);
-        pass = du * du + dv * dv < hh * hh && t + hh > B.tlo && t - hh < B.thi;
-    }
-    return __ballot_sync(0xffffffffu, pass);
+    const float4 c4 = B.c, o4 = B.o;
+    const float lx = lo.x - c4.x, ly = lo.y - c4.y, lz = lo.z - c4.z;
+    const float hx = hi.x - c4.x, hy = hi.y - c4.y, hz = hi.z - c4.z;
+    if (lx > o4.x || ly > o4.y || lz > o4.z || hx < -o4.x || hy < -o4.y || hz < -o4.z) return false;
+    const float4 d4 = B.d, a4 = B.e1, b4 = B.e2, r4 = B.r;
+    const float cx = 0.5f * (lx + hx), cy = 0.5f * (ly + hy), cz = 0.5f * (lz + hz);
+    const float ex = 0.5f * (hx - lx), ey = 0.5f * (hy - ly), ez = 0.5f * (hz - lz);
+    const float m = 2e-6f * (ex + ey + ez + fabsf(cx) + fabsf(cy) + fabsf(cz));
+    const float adx = fabsf(d4.x), ady = fabsf(d4.y), adz = fabsf(d4.z);
+    bool out = fabsf(cx * a4.x + cy * a4.y + cz * a4.z) > ex * fabsf(a4.x) + ey * fabsf(a4.y) + ez * fabsf(a4.z) + a4.w + m;
+    out = out || fabsf(cx * b4.x + cy * b4.y + cz * b4.z) > ex * fabsf(b4.x) + ey * fabsf(b4.y) + ez * fabsf(b4.z) + b4.w + m;
+    out = out || fabsf(cx * d4.x + cy * d4.y + cz * d4.z) > ex * adx + ey * ady + ez * adz + c4.w + m;
+    out = out || fabsf(cy * d4.z - cz * d4.y) > ey * adz + ez * ady + r4.x + m;
+    out = out || fabsf(cz * d4.x - cx * d4.z) > ez * adx + ex * adz + r4.y + m;
+    out = out || fabsf(cx * d4.y - cy * d4.x) > ex * ady + ey * adx + r4.z + m;
+    return !out;
 }
-static_assert(kLeafMax <= 32, "a leaf's particles are filtered one per lane");
+
+// ---- staged spheres -----------------------------------------------------------
+// kSlots blocks of 32 spheres per warp: one being filled, the others holding
+// candidates that some lane has not evaluated yet (kSlots - 1 candidate masks
+// per lane).  A lane ahead of the others works on the later blocks instead of
+// waiting, which keeps the evaluation rounds full: rays of one beam differ in
+// their hits per block by more than their mean.
+constexpr int kSlots = 3;
+struct Staged {
+    float u[32], v[32], t[32], hh[32];      // the block being filled, in the beam's frame; hh = (h + margin)^2
+    float4 q[32 * kSlots];                  // x, y, z, h
+    float2 aw[32 * kSlots];                 // FP32: A_j and the tracer weight A_j x_j
+    int j[32 * kSlots];                     // Morton slot
+};
+
+// The lanes' candidates among the block's first m spheres (bit e: sphere e):
+// the lane's segment comes within h + margin of the sphere's centre,
+//   (u_e - u)^2 + (v_e - v)^2 + dt^2 < hh,  dt the distance of t_e to [t, t + L].
+// Two spheres per packed FP32 operation.
+__device__ __forceinline__ unsigned candidates(const Staged& S, int m, float u, float v, float t, float L)
+{
+    const float2 nu = make_float2(-u, -u), nv = make_float2(-v, -v), nt = make_float2(-t, -t), nL = make_float2(-L, -L);
+    unsigned mask = 0u;
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+        if (e >= m) break;
+        const float4 u4 = *reinterpret_cast<const float4*>(S.u + e), v4 = *reinterpret_cast<const float4*>(S.v + e);
+        const float4 t4 = *reinterpret_cast<const float4*>(S.t + e), h4 = *reinterpret_cast<const float4*>(S.hh + e);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const float2 du = __fadd2_rn(p ? make_float2(u4.z, u4.w) : make_float2(u4.x, u4.y), nu);
+            const float2 dv = __fadd2_rn(p ? make_float2(v4.z, v4.w) : make_float2(v4.x, v4.y), nv);
+            const float2 a = __fadd2_rn(p ? make_float2(t4.z, t4.w) : make_float2(t4.x, t4.y), nt);
+            const float2 b = __fadd2_rn(a, nL);
+            const float2 w = make_float2(fmaxf(fmaxf(-a.x, b.x), 0.f), fmaxf(fmaxf(-a.y, b.y), 0.f));
+            float2 r = __fmul2_rn(dv, dv);
+            r = __ffma2_rn(du, du, r);
+            r = __ffma2_rn(w, w, r);
+            if (!(r.x >= (p ? h4.z : h4.x))) mask |= 1u << (e + 2 * p);
+            if (!(r.y >= (p ? h4.w : h4.y))) mask |= 2u << (e + 2 * p);
+        }
+    }
+    return m < 32 ? mask & ((1u << m) - 1u) : mask;
+}
 
 // Particle index of stored segment pos: an int32, or split into 16 + 8 bits.
 // A lane writes its ray's segments at consecutive positions from a multiple
@@ -527,15 +524,13 @@ constexpr int kPQ = 64;           // queue capacity per warp; a round takes 32
 constexpr int kPQNear = 32;       // owner flag: a near particle (near/far split)
 constexpr int kPQClipLo = 64;     // owner flag: the segment's start cuts the chord
 constexpr int kPQClipHi = 128;    // owner flag: the segment's end cuts the chord
-struct PartItem {
-    float beta2, u1, u2;          // chord in units of h: b^2/h^2 and [u1, u2]
-    int j;                        // particle (Morton slot)
-    int owner;                    // lane of the ray | kPQNear | kPQClipLo | kPQClipHi
-    float coef;                   // MODE_SCATTER: the ray's coefficient
-    int64_t pos;                  // MODE_FILL: the segment's position
-};
 struct PartQueue {
-    PartItem item[kPQ];
+    float beta2[kPQ], u1[kPQ], u2[kPQ];   // chord in units of h: b^2/h^2 and [u1, u2]
+    float A[kPQ];                 // A_j
+    float w[kPQ];                 // the tracer weight A_j x_j (MODE_SCATTER: the ray's coefficient)
+    int j[kPQ];                   // particle (Morton slot)
+    int owner[kPQ];               // lane of the ray | kPQNear | kPQClipLo | kPQClipHi
+    int64_t pos[kPQ];             // MODE_FILL, MODE_CHUNK: the segment's position
     float val[32];                // results of the round being flushed
     unsigned own[64];             // per owner (lane, lane + kPQNear): items of the round
 };
@@ -561,20 +556,19 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
     int owner = -1;
     float v = 0.f;
     if (lane < n) {
-        const PartItem it = pq->item[lane];
-        const float F = KERNEL == URCHIN_KERNEL_M4
-                            ? m4_part_q(tab, it.beta2, it.u1, it.u2, (it.owner & kPQClipLo) != 0,
-                                        (it.owner & kPQClipHi) != 0)
-                            : gt_chord<float>(P, it.beta2, it.u1, it.u2);
-        const float A = __ldg(P.A32 + it.j);
+        const int ow = pq->owner[lane], j = pq->j[lane];
+        const float b2 = pq->beta2[lane], u1 = pq->u1[lane], u2 = pq->u2[lane];
+        const float F = KERNEL == URCHIN_KERNEL_M4 ? m4_part_q(tab, b2, u1, u2, (ow & kPQClipLo) != 0, (ow & kPQClipHi) != 0)
+                                                   : gt_chord<float>(P, b2, u1, u2);
+        const float A = pq->A[lane];
         if (MODE == MODE_SCATTER) {
-            atomicAdd(P.xbar + it.j, (double)(it.coef * (A * F)));
+            atomicAdd(P.xbar + j, (double)(pq->w[lane] * (A * F)));
         } else {
-            const bool near = NF && (it.owner & kPQNear);
-            v = near ? A * F : __ldg(P.w32 + it.j) * F;
-            if (MODE == MODE_FILL && !near) static_cast<float*>(P.seg_val)[it.pos] = A * F;
-            if (MODE == MODE_CHUNK && it.pos >= 0) P.chunk_seg[it.pos] = make_int2(it.j, __float_as_int(A * F));
-            owner = it.owner & (31 | kPQNear);
+            const bool near = NF && (ow & kPQNear);
+            v = near ? A * F : pq->w[lane] * F;
+            if (MODE == MODE_FILL && !near) static_cast<float*>(P.seg_val)[pq->pos[lane]] = A * F;
+            if (MODE == MODE_CHUNK && pq->pos[lane] >= 0) P.chunk_seg[pq->pos[lane]] = make_int2(j, __float_as_int(A * F));
+            owner = ow & (31 | kPQNear);
         }
     }
     if (MODE != MODE_SCATTER) {
@@ -591,10 +585,33 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
         pq->own[lane + kPQNear] = 0u;
     }
     const int rest = count - n;
-    PartItem tail;
-    if (lane < rest) tail = pq->item[n + lane];
-    __syncwarp();
-    if (lane < rest) pq->item[lane] = tail;
+    if (rest > 0) {
+        __syncwarp();
+        float b2 = 0.f, u1 = 0.f, u2 = 0.f, A = 0.f, w = 0.f;
+        int j = 0, ow = 0;
+        int64_t pos = 0;
+        if (lane < rest) {
+            b2 = pq->beta2[n + lane];
+            u1 = pq->u1[n + lane];
+            u2 = pq->u2[n + lane];
+            A = pq->A[n + lane];
+            w = pq->w[n + lane];
+            j = pq->j[n + lane];
+            ow = pq->owner[n + lane];
+            if (MODE == MODE_FILL || MODE == MODE_CHUNK) pos = pq->pos[n + lane];
+        }
+        __syncwarp();
+        if (lane < rest) {
+            pq->beta2[lane] = b2;
+            pq->u1[lane] = u1;
+            pq->u2[lane] = u2;
+            pq->A[lane] = A;
+            pq->w[lane] = w;
+            pq->j[lane] = j;
+            pq->owner[lane] = ow;
+            if (MODE == MODE_FILL || MODE == MODE_CHUNK) pq->pos[lane] = pos;
+        }
+    }
     __syncwarp();
     count = rest;
 }
@@ -614,278 +631,414 @@ __device__ __forceinline__ unsigned long long chunk_block(const TraceParams& P, 
     return b;
 }
 
-// FP32 hit evaluation: cheap rejection, then the impact parameter from an
-// error-free cross product; full chords from the table at once, partial
-// chords queued for flush_partials.  Every lane of the warp calls it (the
-// queue is shared); lanes that are not live only take part in the queue.
+// FP32 evaluation of one candidate per lane (act: the lane has one): the
+// impact parameter from an error-free cross product decides the hit; full
+// chords from the table at once, partial chords queued for flush_partials.
+// Every lane of the warp calls it (the queue and the chunks are shared).
 template <int KERNEL, int MODE, bool NF>
-__device__ __forceinline__ void leaf_hits_f32(const TraceParams& P, const float2* tab, PartQueue* pq, int& pq_count,
-                                              unsigned long long* stash, int ref, int cnt, unsigned mask, bool live,
-                                              float sx, float sy, float sz, float dx, float dy, float dz, float L,
-                                              Sink<float>& k, unsigned& err)
+__device__ __forceinline__ void eval_f32(const TraceParams& P, const float2* tab, PartQueue* pq, int& pq_count,
+                                         unsigned long long* stash, bool act, const Staged& S, int at, float dx,
+                                         float dy, float dz, float L, Sink<float>& k, unsigned& err)
 {
-    if (ref < 0 || cnt > kLeafMax || ref + cnt > P.n) return;   // never true for a well-formed tree
-    if (live) k.ntest += (unsigned)__popc(mask);
     const int lane = threadIdx.x & 31;
-    for (unsigned m = mask; m; m &= m - 1) {
-        const int j = ref + __ffs(m) - 1;
-        bool part = false, near = false, store = false;
-        int clip = 0;
-        float beta2 = 0.f, u1 = 0.f, u2 = 0.f, segv = 0.f;
-        int64_t spos = 0;
-        if (live) {
-            // The hit decision is written with explicit roundings (no
-            // multiply-add contraction left to the compiler), so that the
-            // counting and the filling traversal, separate instantiations,
-            // find exactly the same hits.
-            const float4 q = __ldg(P.xyzh + j);
-            const float ex = q.x - sx, ey = q.y - sy, ez = q.z - sz;
-            float cx = __fsub_rn(__fmul_rn(ey, dz), __fmul_rn(ez, dy));
-            float cy = __fsub_rn(__fmul_rn(ez, dx), __fmul_rn(ex, dz));
-            float cz = __fsub_rn(__fmul_rn(ex, dy), __fmul_rn(ey, dx));
-            const float h2 = __fmul_rn(q.w, q.w);
-            bool hit = fmaf(cz, cz, fmaf(cy, cy, __fmul_rn(cx, cx))) < __fmul_rn(1.0001f, h2);
-            float b2 = 0.f, tc = 0.f, ch = 0.f;
-            if (hit) {
-                cx = dop(ey, dz, ez, dy);
-                cy = dop(ez, dx, ex, dz);
-                cz = dop(ex, dy, ey, dx);
-                b2 = fmaf(cz, cz, fmaf(cy, cy, __fmul_rn(cx, cx)));
-                hit = b2 < h2;
-            }
-            if (hit) {
-                tc = fmaf(ez, dz, fmaf(ey, dy, __fmul_rn(ex, dx)));
-                ch = sqrtf(__fsub_rn(h2, b2));
-                hit = __fadd_rn(tc, ch) > 0.f && __fsub_rn(tc, ch) < L;
-            }
-            if (hit) {
-                near = NF && is_near(k, q, tc, ch);
-                if (!near) ++k.nhit;
-                if (MODE == MODE_CHUNK && !near) store = true;
-                if (MODE != MODE_COUNT) {
-                    const float ih = 1.f / q.w;
-                    beta2 = b2 * ih * ih;
-                    if (MODE == MODE_FILL && !near) {
-                        // the index is written now, in order; a partial chord's value at the flush
-                        if (k.pos < k.end) {
-                            store_index(P, k, k.pos, j);
-                            spos = k.pos++;
-                        } else {
-                            err |= kStSegment;
-                            hit = false;
-                        }
-                    }
-                    if (hit && __fsub_rn(tc, ch) >= 0.f && __fadd_rn(tc, ch) <= L) {
-                        const float F = KERNEL == URCHIN_KERNEL_M4 ? m4_full_tab(tab, beta2)
-                                                                   : gt_chord<float>(P, beta2, -ch * ih, ch * ih);
-                        const float A = __ldg(P.A32 + j);
-                        if (MODE == MODE_SCATTER) {
-                            atomicAdd(P.xbar + j, (double)(k.coef * (A * F)));
-                        } else if (near) {
-                            Kahan::add(k.near, k.near_c, A * F);
-                        } else {
-                            Kahan::add(k.sum, k.comp, __ldg(P.w32 + j) * F);
-                            if (MODE == MODE_FILL) static_cast<float*>(P.seg_val)[spos] = A * F;
-                            if (MODE == MODE_CHUNK) segv = A * F;
-                        }
-                    } else if (hit) {
-                        part = true;
-                        clip = (__fsub_rn(tc, ch) < 0.f ? kPQClipLo : 0) | (__fadd_rn(tc, ch) > L ? kPQClipHi : 0);
-                        u1 = (fmaxf(0.f, tc - ch) - tc) * ih;
-                        u2 = (fminf(L, tc + ch) - tc) * ih;
-                    }
-                }
-            }
+    bool part = false, near = false, store = false;
+    int clip = 0, j = 0;
+    float beta2 = 0.f, u1 = 0.f, u2 = 0.f, segv = 0.f;
+    float2 aw = make_float2(0.f, 0.f);
+    int64_t spos = 0;
+    if (act) {
+        // The hit decision is written with explicit roundings (no
+        // multiply-add contraction left to the compiler), so that the
+        // counting and the filling traversal, separate instantiations,
+        // find exactly the same hits.
+        const float4 q = S.q[at];
+        j = S.j[at];
+        const float ex = q.x - k.sx, ey = q.y - k.sy, ez = q.z - k.sz;
+        const float cx = dop(ey, dz, ez, dy);
+        const float cy = dop(ez, dx, ex, dz);
+        const float cz = dop(ex, dy, ey, dx);
+        const float h2 = __fmul_rn(q.w, q.w);
+        const float b2 = fmaf(cz, cz, fmaf(cy, cy, __fmul_rn(cx, cx)));
+        bool hit = b2 < h2;
+        float tc = 0.f, ch = 0.f;
+        if (hit) {
+            tc = fmaf(ez, dz, fmaf(ey, dy, __fmul_rn(ex, dx)));
+            ch = sqrtf(__fsub_rn(h2, b2));
+            hit = __fadd_rn(tc, ch) > 0.f && __fsub_rn(tc, ch) < L;
         }
-        if (MODE == MODE_COUNT) continue;
-        if constexpr (MODE == MODE_CHUNK) {
-            // with the warp converged: a new chunk for every ray whose chunk
-            // is full (or that has none yet), then the segment's index (and a
-            // full chord's value; a partial chord's at the flush)
-            const bool need = store && k.coff == kChunk;
-            const unsigned nm = __ballot_sync(0xffffffffu, need);
-            if (nm) {
-                unsigned long long base = 0;
-                if (lane == 0) base = chunk_block(P, stash, __popc(nm));
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if (need) {
-                    const unsigned long long c = base + (unsigned long long)__popc(nm & ((1u << lane) - 1u));
-                    if (c < P.chunk_cap) {
-                        if (k.cur == kNoChunk) P.chunk_head[k.ray] = (uint32_t)c;
-                        else P.chunk_next[k.cur] = (uint32_t)c;
-                        k.cur = (uint32_t)c;
-                        k.cw = P.chunk_seg + c * (unsigned long long)kChunk;
-                        k.coff = 0;
+        if (hit) {
+            near = NF && is_near(k, q, tc, ch);
+            if (!near) ++k.nhit;
+            if (MODE == MODE_CHUNK && !near) store = true;
+            if (MODE != MODE_COUNT) {
+                aw = S.aw[at];
+                const float ih = 1.f / q.w;
+                beta2 = b2 * ih * ih;
+                if (MODE == MODE_FILL && !near) {
+                    // the index is written now, in order; a partial chord's value at the flush
+                    if (k.pos < k.end) {
+                        store_index(P, k, k.pos, j);
+                        spos = k.pos++;
                     } else {
-                        k.coff = kChunk + 1;        // the pool is exhausted: this ray stores no more
+                        err |= kStSegment;
+                        hit = false;
                     }
                 }
-            }
-            spos = -1;
-            if (store && k.coff < kChunk) {
-                // a partial chord's entry is written whole at the flush
-                if (!part) k.cw[k.coff] = make_int2(j, __float_as_int(segv));
-                else spos = (int64_t)k.cur * kChunk + k.coff;
-                ++k.coff;
+                if (hit && __fsub_rn(tc, ch) >= 0.f && __fadd_rn(tc, ch) <= L) {
+                    const float F = KERNEL == URCHIN_KERNEL_M4 ? m4_full_tab(tab, beta2)
+                                                               : gt_chord<float>(P, beta2, -ch * ih, ch * ih);
+                    if (MODE == MODE_SCATTER) {
+                        atomicAdd(P.xbar + j, (double)(k.coef * (aw.x * F)));
+                    } else if (near) {
+                        Kahan::add(k.near, k.near_c, aw.x * F);
+                    } else {
+                        Kahan::add(k.sum, k.comp, aw.y * F);
+                        if (MODE == MODE_FILL) static_cast<float*>(P.seg_val)[spos] = aw.x * F;
+                        if (MODE == MODE_CHUNK) segv = aw.x * F;
+                    }
+                } else if (hit) {
+                    part = true;
+                    clip = (__fsub_rn(tc, ch) < 0.f ? kPQClipLo : 0) | (__fadd_rn(tc, ch) > L ? kPQClipHi : 0);
+                    u1 = (fmaxf(0.f, tc - ch) - tc) * ih;
+                    u2 = (fminf(L, tc + ch) - tc) * ih;
+                }
             }
         }
-        const unsigned pb = __ballot_sync(0xffffffffu, part);
-        if (!pb) continue;
-        if (part) {
-            PartItem& it = pq->item[pq_count + __popc(pb & ((1u << lane) - 1u))];
-            it.beta2 = beta2;
-            it.u1 = u1;
-            it.u2 = u2;
-            it.j = j;
-            it.owner = lane | (near ? kPQNear : 0) | clip;
-            it.coef = MODE == MODE_SCATTER ? k.coef : 0.f;
-            it.pos = spos;
-        }
-        pq_count += __popc(pb);
-        __syncwarp();
-        if (pq_count >= 32) flush_partials<KERNEL, MODE, NF>(P, tab, pq, pq_count, 32, k);
     }
+    if (MODE == MODE_COUNT) return;
+    if constexpr (MODE == MODE_CHUNK) {
+        // with the warp converged: a new chunk for every ray whose chunk
+        // is full (or that has none yet), then the segment's index (and a
+        // full chord's value; a partial chord's at the flush)
+        const bool need = store && k.coff == kChunk;
+        const unsigned nm = __ballot_sync(0xffffffffu, need);
+        if (nm) {
+            unsigned long long base = 0;
+            if (lane == 0) base = chunk_block(P, stash, __popc(nm));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (need) {
+                const unsigned long long c = base + (unsigned long long)__popc(nm & ((1u << lane) - 1u));
+                if (c < P.chunk_cap) {
+                    if (k.cur == kNoChunk) P.chunk_head[k.ray] = (uint32_t)c;
+                    else P.chunk_next[k.cur] = (uint32_t)c;
+                    k.cur = (uint32_t)c;
+                    k.cw = P.chunk_seg + c * (unsigned long long)kChunk;
+                    k.coff = 0;
+                } else {
+                    k.coff = kChunk + 1;        // the pool is exhausted: this ray stores no more
+                }
+            }
+        }
+        spos = -1;
+        if (store && k.coff < kChunk) {
+            // a partial chord's entry is written whole at the flush
+            if (!part) k.cw[k.coff] = make_int2(j, __float_as_int(segv));
+            else spos = (int64_t)k.cur * kChunk + k.coff;
+            ++k.coff;
+        }
+    }
+    const unsigned pb = __ballot_sync(0xffffffffu, part);
+    if (!pb) return;
+    if (part) {
+        const int i = pq_count + __popc(pb & ((1u << lane) - 1u));
+        pq->beta2[i] = beta2;
+        pq->u1[i] = u1;
+        pq->u2[i] = u2;
+        pq->A[i] = aw.x;
+        pq->w[i] = MODE == MODE_SCATTER ? k.coef : aw.y;
+        pq->j[i] = j;
+        pq->owner[i] = lane | (near ? kPQNear : 0) | clip;
+        if (MODE == MODE_FILL || MODE == MODE_CHUNK) pq->pos[i] = spos;
+    }
+    pq_count += __popc(pb);
+    __syncwarp();
+    if (pq_count >= 32) flush_partials<KERNEL, MODE, NF>(P, tab, pq, pq_count, 32, k);
 }
 
+// The same in double, chords evaluated in place.
 template <typename Real, int KERNEL, int MODE, bool NF>
-__device__ __forceinline__ void leaf_hits(const TraceParams& P, int ref, int cnt, unsigned mask, Real sx, Real sy,
-                                          Real sz, Real dx, Real dy, Real dz, Real L, Sink<Real>& k, unsigned& err)
+__device__ __forceinline__ void eval_f64(const TraceParams& P, const Staged& S, int at, Real dx, Real dy, Real dz,
+                                         Real L, Sink<Real>& k, unsigned& err)
 {
     using O = RealOps<Real>;
-    if (ref < 0 || cnt > kLeafMax || ref + cnt > P.n) return;   // never true for a well-formed tree
-    k.ntest += (unsigned)__popc(mask);
-    for (unsigned m = mask; m; m &= m - 1) {
-        const int j = ref + __ffs(m) - 1;
-        // explicit roundings in the hit decision, as in leaf_hits_f32
-        float4 q = __ldg(P.xyzh + j);
-        Real ex = Real(q.x) - sx, ey = Real(q.y) - sy, ez = Real(q.z) - sz;
-        Real tc = fma(ez, dz, fma(ey, dy, mul_rn(ex, dx)));
-        Real cx = sub_rn(mul_rn(ey, dz), mul_rn(ez, dy));
-        Real cy = sub_rn(mul_rn(ez, dx), mul_rn(ex, dz));
-        Real cz = sub_rn(mul_rn(ex, dy), mul_rn(ey, dx));
-        Real b2 = fma(cz, cz, fma(cy, cy, mul_rn(cx, cx)));
-        Real h = Real(q.w);
-        Real h2 = mul_rn(h, h);
-        if (b2 >= h2) continue;
-        Real ch = O::sqrt_(sub_rn(h2, b2));
-        if (add_rn(tc, ch) <= Real(0) || sub_rn(tc, ch) >= L) continue;
-        const bool near = NF && is_near(k, q, tc, ch);
-        if (!near) ++k.nhit;
-        if (MODE == MODE_COUNT) continue;
-        Real ih = Real(1) / h;
-        Real beta2 = b2 * ih * ih;
-        Real F;
-        if (sub_rn(tc, ch) >= Real(0) && add_rn(tc, ch) <= L) {
-            Real c = ch * ih;
-            if (KERNEL == URCHIN_KERNEL_M4) F = m4_full(beta2, c);
-            else F = gt_chord(P, beta2, -c, c);
+    // explicit roundings in the hit decision, as in eval_f32
+    const float4 q = S.q[at];
+    const int j = S.j[at];
+    Real ex = Real(q.x) - k.sx, ey = Real(q.y) - k.sy, ez = Real(q.z) - k.sz;
+    Real tc = fma(ez, dz, fma(ey, dy, mul_rn(ex, dx)));
+    Real cx = sub_rn(mul_rn(ey, dz), mul_rn(ez, dy));
+    Real cy = sub_rn(mul_rn(ez, dx), mul_rn(ex, dz));
+    Real cz = sub_rn(mul_rn(ex, dy), mul_rn(ey, dx));
+    Real b2 = fma(cz, cz, fma(cy, cy, mul_rn(cx, cx)));
+    Real h = Real(q.w);
+    Real h2 = mul_rn(h, h);
+    if (b2 >= h2) return;
+    Real ch = O::sqrt_(sub_rn(h2, b2));
+    if (add_rn(tc, ch) <= Real(0) || sub_rn(tc, ch) >= L) return;
+    const bool near = NF && is_near(k, q, tc, ch);
+    if (!near) ++k.nhit;
+    if (MODE == MODE_COUNT) return;
+    Real ih = Real(1) / h;
+    Real beta2 = b2 * ih * ih;
+    Real F;
+    if (sub_rn(tc, ch) >= Real(0) && add_rn(tc, ch) <= L) {
+        Real c = ch * ih;
+        if (KERNEL == URCHIN_KERNEL_M4) F = m4_full(beta2, c);
+        else F = gt_chord(P, beta2, -c, c);
+    } else {
+        Real u1 = (fmax(Real(0), tc - ch) - tc) * ih;
+        Real u2 = (fmin(L, tc + ch) - tc) * ih;
+        if (KERNEL == URCHIN_KERNEL_M4) F = m4_part(beta2, u1, u2);
+        else F = gt_chord(P, beta2, u1, u2);
+    }
+    if (MODE == MODE_SCATTER) {
+        atomicAdd(P.xbar + j, (double)(k.coef * (Real(__ldg(P.A64 + j)) * F)));
+        return;
+    }
+    if (near) {
+        Kahan::add(k.near, k.near_c, Real(__ldg(P.A64 + j)) * F);
+        return;
+    }
+    Kahan::add(k.sum, k.comp, O::weight(P, j) * F);
+    if (MODE == MODE_FILL) {
+        if (k.pos < k.end) {
+            store_index(P, k, k.pos, j);
+            static_cast<Real*>(P.seg_val)[k.pos] = Real(__ldg(P.A64 + j)) * F;
+            ++k.pos;
         } else {
-            Real u1 = (fmax(Real(0), tc - ch) - tc) * ih;
-            Real u2 = (fmin(L, tc + ch) - tc) * ih;
-            if (KERNEL == URCHIN_KERNEL_M4) F = m4_part(beta2, u1, u2);
-            else F = gt_chord(P, beta2, u1, u2);
-        }
-        if (MODE == MODE_SCATTER) {
-            const Real A = sizeof(Real) == 4 ? Real(__ldg(P.A32 + j)) : Real(__ldg(P.A64 + j));
-            atomicAdd(P.xbar + j, (double)(k.coef * (A * F)));
-            continue;
-        }
-        if (near) {
-            const Real A = sizeof(Real) == 4 ? Real(__ldg(P.A32 + j)) : Real(__ldg(P.A64 + j));
-            Kahan::add(k.near, k.near_c, A * F);
-            continue;
-        }
-        Kahan::add(k.sum, k.comp, O::weight(P, j) * F);
-        if (MODE == MODE_FILL) {
-            if (k.pos < k.end) {
-                store_index(P, k, k.pos, j);
-                const Real A = sizeof(Real) == 4 ? Real(__ldg(P.A32 + j)) : Real(__ldg(P.A64 + j));
-                static_cast<Real*>(P.seg_val)[k.pos] = A * F;
-                ++k.pos;
-            } else {
-                err |= kStSegment;
-            }
+            err |= kStSegment;
         }
     }
 }
 
+// The tree walk of one packet: next() gives the leaves that the beam may
+// reach, in the list's order, one after the other.
+struct Walk {
+    int lev, node;                // current entry: number `node` of level `lev`
+    unsigned mask;                // its children still to be entered
+    unsigned pend;                // lane l holds level l's mask while its subtrees are walked
+    int lref, lcnt;               // children that are leaves: the lane's leaf
+    unsigned visits;
+
+    __device__ __forceinline__ void children(const TraceParams& P, const Beam& B)
+    {
+        const int c = 32 * node + (int)(threadIdx.x & 31);
+        bool pass = false;
+        if (c < P.lev_cnt[lev - 1]) {
+            const float4* b = P.boxes + 2 * ((int64_t)P.lev_off[lev - 1] + c);
+            const float4 lo = __ldg(b), hi = __ldg(b + 1);
+            lref = __float_as_int(lo.w);
+            lcnt = __float_as_int(hi.w);
+            pass = beam_box(B, lo, hi);
+        }
+        mask = __ballot_sync(0xffffffffu, pass);
+        ++visits;
+    }
+
+    __device__ __forceinline__ void start(const TraceParams& P, const Beam& B)
+    {
+        lev = P.n_lev;
+        node = 0;
+        pend = 0u;
+        children(P, B);
+    }
+
+    // false at the end of the walk
+    __device__ __forceinline__ bool next(const TraceParams& P, const Beam& B, int& ref, int& cnt)
+    {
+        for (;;) {
+            if (mask == 0u) {
+                if (lev == P.n_lev) return false;
+                ++lev;
+                node >>= 5;
+                mask = __shfl_sync(0xffffffffu, pend, lev);
+                continue;
+            }
+            const int c = __ffs(mask) - 1;
+            mask &= mask - 1u;
+            if (lev == 1) {
+                ref = __shfl_sync(0xffffffffu, lref, c);
+                cnt = __shfl_sync(0xffffffffu, lcnt, c);
+                return true;
+            }
+            if ((int)(threadIdx.x & 31) == lev) pend = mask;
+            node = 32 * node + c;
+            --lev;
+            children(P, B);
+        }
+    }
+};
+
+// One image of the packet's rays: walk, stage, filter, evaluate (file comment).
 template <typename Real, int KERNEL, int MODE, bool NF>
-__device__ void ray_column(const TraceParams& P, const float2* tab, Beam* beam, PartQueue* pq, int& pq_count,
-                           unsigned long long* stash, float4 o, Real dx, Real dy, Real dz, bool live, Sink<Real>& sk,
-                           unsigned& err, unsigned& nvisit)
+__device__ __forceinline__ void packet_image(const TraceParams& P, const float2* tab, const Beam& B, Staged& S,
+                                             PartQueue* pq, int& pq_count, unsigned long long* stash, float u, float v,
+                                             float t, float Lf, Real dx, Real dy, Real dz, bool live, Sink<Real>& sk,
+                                             unsigned& err, unsigned& nvisit)
 {
     const Real L = Real(P.l_ray);
-    const float Lf = (float)P.l_ray * 1.000001f + 1e-30f;
-    const float ix = safe_inv((double)dx), iy = safe_inv((double)dy), iz = safe_inv((double)dz);
-    const int nimg = P.periodic ? P.nimg : 0;
-    const float4 rlo = make_float4(P.root_lo[0], P.root_lo[1], P.root_lo[2], 0.f);
-    const float4 rhi = make_float4(P.root_hi[0], P.root_hi[1], P.root_hi[2], 0.f);
-    int stack[kStackMax];
-    for (int ax = -nimg; ax <= nimg; ++ax)
-    for (int ay = -nimg; ay <= nimg; ++ay)
-    for (int az = -nimg; az <= nimg; ++az) {
-        // images of the particles at r_j + a L are reached by shifting the
-        // origin to r_i - a L
-        Real sx = Real(o.x) - Real(ax) * Real(P.Lbox);
-        Real sy = Real(o.y) - Real(ay) * Real(P.Lbox);
-        Real sz = Real(o.z) - Real(az) * Real(P.Lbox);
-        float fx = (float)sx, fy = (float)sy, fz = (float)sz;
-        if (!__any_sync(0xffffffffu, live && seg_box(fx, fy, fz, ix, iy, iz, Lf, rlo, rhi))) continue;
-        if (!make_beam(beam, live, fx, fy, fz, (float)dx, (float)dy, (float)dz, Lf)) continue;
-        if (NF) {
-            sk.ox = (double)o.x - (double)ax * P.Lbox;
-            sk.oy = (double)o.y - (double)ay * P.Lbox;
-            sk.oz = (double)o.z - (double)az * P.Lbox;
+    const int lane = threadIdx.x & 31;
+    constexpr bool kF32 = sizeof(Real) == 4;
+    constexpr bool kWantW = kF32 && MODE != MODE_COUNT && MODE != MODE_SCATTER;
+    constexpr bool kWantA = kF32 && MODE != MODE_COUNT && (MODE != MODE_TAU || NF);
+    Walk W;
+    W.visits = 0u;
+    W.start(P, B);
+    int ref = 0, cnt = 0;
+    bool more = W.next(P, B, ref, cnt);
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 aw = make_float2(0.f, 0.f);
+    auto fetch = [&](int r, int c) {
+        if (lane < c && r >= 0 && r + lane < P.n) {
+            q = __ldg(P.xyzh + r + lane);
+            if (kWantA) aw.x = __ldg(P.A32 + r + lane);
+            if (kWantW) aw.y = __ldg(P.w32 + r + lane);
         }
-        int sp = 0;
-        int node = 0;
-        // a traversal visits every internal node at most once; the cap only
-        // guards against a malformed tree
-        int budget = P.n_nodes + 1;
+    };
+    if (more) fetch(ref, cnt);
+    unsigned m0 = 0u, m1 = 0u;       // candidates in the oldest and the newer full block
+    int st = 0, ns = 0;              // block being filled (0, 32, 64) and its spheres
+    for (;;) {
+        const bool last = !more;
+        unsigned pm = 0u;
+        float su = 0.f, sv = 0.f, stt = 0.f, shh = 0.f;
+        const float4 cq = q;
+        const float2 caw = aw;
+        const int cj = ref + lane;
+        if (!last) {
+            // sphere (one per lane) against the beam
+            bool pass = false;
+            if (lane < cnt) {
+                const float4 c4 = B.c, a4 = B.e1, b4 = B.e2, d4 = B.d;
+                const float rx = cq.x - c4.x, ry = cq.y - c4.y, rz = cq.z - c4.z;
+                su = rx * a4.x + ry * a4.y + rz * a4.z;
+                sv = rx * b4.x + ry * b4.y + rz * b4.z;
+                stt = rx * d4.x + ry * d4.y + rz * d4.z;
+                const float hh = cq.w * 1.00001f + d4.w + 4e-6f * (fabsf(rx) + fabsf(ry) + fabsf(rz));
+                shh = hh * hh;
+                const float du = fmaxf(fabsf(su) - a4.w, 0.f), dv = fmaxf(fabsf(sv) - b4.w, 0.f),
+                            dt = fmaxf(fabsf(stt) - c4.w, 0.f);
+                pass = !(fmaf(dt, dt, fmaf(dv, dv, du * du)) >= shh) && cj >= 0 && cj < P.n;
+            }
+            pm = __ballot_sync(0xffffffffu, pass);
+            more = W.next(P, B, ref, cnt);
+            if (more) fetch(ref, cnt);
+            if (pm == 0u) continue;
+        }
+        const bool mine = (pm >> lane) & 1u;
+        const int rank = __popc(pm & ((1u << lane) - 1u)), room = 32 - ns, pc = __popc(pm);
+        if (mine && rank < room) {
+            S.u[ns + rank] = su;
+            S.v[ns + rank] = sv;
+            S.t[ns + rank] = stt;
+            S.hh[ns + rank] = shh;
+            S.q[st + ns + rank] = cq;
+            S.j[st + ns + rank] = cj;
+            if (kWantA || kWantW) S.aw[st + ns + rank] = caw;
+        }
+        if (!last && pc < room) {
+            ns += pc;
+            continue;
+        }
+        // the block is full (or the walk over): the lanes' candidates in it
+        const int m = last ? ns : 32;
+        __syncwarp();
+        unsigned m2 = candidates(S, m, u, v, t, Lf);
+        if (live) sk.ntest += (unsigned)m;
+        else m2 = 0u;
+        // evaluate until the oldest block is done (at the end: all of them)
         for (;;) {
-            if (--budget < 0) {
-                err |= kStVisit;
-                break;
+            const unsigned all = m0 | m1 | m2;
+            if (!__any_sync(0xffffffffu, (last ? all : m0) != 0u)) break;
+            int at = st >= 32 ? st - 32 : st + 64;          // the newer block
+            unsigned b = m1;
+            if (m0) {
+                b = m0;
+                at = st >= 64 ? st - 64 : st + 32;          // the oldest
+            } else if (!b) {
+                b = m2;
+                at = st;
             }
-            if ((unsigned)node >= (unsigned)P.n_nodes) {   // never true for a well-formed tree
-                err |= kStVisit;
-                break;
-            }
-            ++nvisit;
-            const float4* nd = P.nodes + 4 * (int64_t)node;
-            float4 a = __ldg(nd), b = __ldg(nd + 1), c = __ldg(nd + 2), d = __ldg(nd + 3);
-            int lref = __float_as_int(a.w), lcnt = __float_as_int(b.w);
-            int rref = __float_as_int(c.w), rcnt = __float_as_int(d.w);
-            bool hl = __any_sync(0xffffffffu, live && seg_box(fx, fy, fz, ix, iy, iz, Lf, a, b));
-            bool hr = __any_sync(0xffffffffu, live && rcnt >= 0 && seg_box(fx, fy, fz, ix, iy, iz, Lf, c, d));
-            // leaf children: left then right, through one call site
-            const bool leaf_l = hl && lcnt > 0, leaf_r = hr && rcnt > 0;
-#pragma unroll 1
-            for (int q = leaf_l ? 0 : 1; q < (leaf_r ? 2 : 1); ++q) {
-                const int ref = q == 0 ? lref : rref, cnt = q == 0 ? lcnt : rcnt;
-                const unsigned mask = beam_mask(P, *beam, ref, cnt);
-                if (mask) {
-                    if constexpr (sizeof(Real) == 4)
-                        leaf_hits_f32<KERNEL, MODE, NF>(P, tab, pq, pq_count, stash, ref, cnt, mask, live, sx, sy,
-                                                        sz, dx, dy, dz, L, sk, err);
-                    else if (live)
-                        leaf_hits<Real, KERNEL, MODE, NF>(P, ref, cnt, mask, sx, sy, sz, dx, dy, dz, L, sk, err);
-                }
-            }
-            hl = hl && !leaf_l;
-            hr = hr && !leaf_r;
-            if (hl && hr) {
-                if (sp < kStackMax) stack[sp++] = rref;
-                else err |= kStStack;
-                node = lref;
-            } else if (hl) {
-                node = lref;
-            } else if (hr) {
-                node = rref;
+            const unsigned rest = b & (b - 1u);
+            at += __ffs(b) - 1;
+            if (m0) m0 = rest;
+            else if (m1) m1 = rest;
+            else m2 = rest;
+            if constexpr (kF32) {
+                eval_f32<KERNEL, MODE, NF>(P, tab, pq, pq_count, stash, all != 0u, S, all ? at : 0, dx, dy, dz, L, sk, err);
             } else {
-                if (sp == 0) break;
-                node = stack[--sp];
+                if (all) eval_f64<Real, KERNEL, MODE, NF>(P, S, at, dx, dy, dz, L, sk, err);
+                __syncwarp();
             }
+        }
+        if (last) break;
+        m0 = m1;
+        m1 = m2;
+        st = st >= 64 ? 0 : st + 32;
+        ns = pc - room;
+        __syncwarp();                // the block's readers are done
+        if (mine && rank >= room) {
+            S.u[rank - room] = su;
+            S.v[rank - room] = sv;
+            S.t[rank - room] = stt;
+            S.hh[rank - room] = shh;
+            S.q[st + rank - room] = cq;
+            S.j[st + rank - room] = cj;
+            if (kWantA || kWantW) S.aw[st + rank - room] = caw;
+        }
+    }
+    nvisit += W.visits;
+    __syncwarp();
+}
+
+template <typename Real, int KERNEL, int MODE, bool NF>
+__device__ __forceinline__ void ray_column(const TraceParams& P, const float2* tab, Beam* beam, Staged& S,
+                                           PartQueue* pq, int& pq_count, unsigned long long* stash, float4 o, Real dx,
+                                           Real dy, Real dz, bool live, Sink<Real>& sk, unsigned& err,
+                                           unsigned& nvisit)
+{
+    const unsigned lv = __ballot_sync(0xffffffffu, live);
+    if (!lv) return;
+    const float Lf = (float)P.l_ray * 1.000001f + 1e-30f;
+    const int nimg = P.periodic ? P.nimg : 0;
+    const int side = 2 * nimg + 1;
+    const int images = side * side * side;
+    float u, v, t;
+    // the images of the box that the unshifted beam may reach, 32 at a time,
+    // then one after the other in the order of their indices
+    for (int i0 = 0; i0 < images; i0 += 32) {
+        unsigned im = 1u;
+        if (images > 1) {
+            make_beam(beam, lv, live, Real(o.x), Real(o.y), Real(o.z), (float)dx, (float)dy, (float)dz, Lf, u, v, t);
+            const int i = i0 + (int)(threadIdx.x & 31);
+            bool pass = false;
+            if (i < images) {
+                const float ax = (float)(i / (side * side) - nimg) * (float)P.Lbox,
+                            ay = (float)((i / side) % side - nimg) * (float)P.Lbox,
+                            az = (float)(i % side - nimg) * (float)P.Lbox;
+                // the shifted faces and the shifted origins are each rounded
+                const float m = 1e-6f * (fabsf(ax) + fabsf(ay) + fabsf(az) + (float)P.Lbox);
+                pass = beam_box(*beam, make_float4(P.root_lo[0] + ax - m, P.root_lo[1] + ay - m, P.root_lo[2] + az - m, 0.f),
+                                make_float4(P.root_hi[0] + ax + m, P.root_hi[1] + ay + m, P.root_hi[2] + az + m, 0.f));
+            }
+            im = __ballot_sync(0xffffffffu, pass);
+        }
+        for (; im; im &= im - 1u) {
+            const int i = i0 + __ffs(im) - 1;
+            const int ax = i / (side * side) - nimg, ay = (i / side) % side - nimg, az = i % side - nimg;
+            // images of the particles at r_j + a L are reached by shifting the
+            // origin to r_i - a L
+            sk.sx = Real(o.x) - Real(ax) * Real(P.Lbox);
+            sk.sy = Real(o.y) - Real(ay) * Real(P.Lbox);
+            sk.sz = Real(o.z) - Real(az) * Real(P.Lbox);
+            if (NF) {
+                sk.ox = (double)o.x - (double)ax * P.Lbox;
+                sk.oy = (double)o.y - (double)ay * P.Lbox;
+                sk.oz = (double)o.z - (double)az * P.Lbox;
+            }
+            make_beam(beam, lv, live, sk.sx, sk.sy, sk.sz, (float)dx, (float)dy, (float)dz, Lf, u, v, t);
+            packet_image<Real, KERNEL, MODE, NF>(P, tab, *beam, S, pq, pq_count, stash, u, v, t, Lf, dx, dy, dz, live,
+                                                 sk, err, nvisit);
         }
     }
 }
@@ -900,6 +1053,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
     extern __shared__ double s_dirs[];
     float2* s_tab = reinterpret_cast<float2*>(s_dirs + 3 * P.R);
     __shared__ Beam s_beam[256 / 32];
+    __shared__ Staged s_staged[256 / 32];
     __shared__ unsigned long long s_stash[256 / 32][2];   // MODE_CHUNK: the warp's block of chunks
     // the warps' partial-chord queues (FP32 modes that evaluate chords), after the table
     constexpr bool kQueue = sizeof(Real) == 4 && MODE != MODE_COUNT;
@@ -940,7 +1094,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
         float4 o = __ldg(P.xyzh + org);
         Real dx = Real(s_dirs[3 * k]), dy = Real(s_dirs[3 * k + 1]), dz = Real(s_dirs[3 * k + 2]);
         unsigned nvisit = 0;
-        Sink<Real> sk{Real(0), Real(0), Real(0), Real(0), 0u, 0u, 0, 0, Real(0), Real(0), Real(0), 0.0, 0.0, 0.0};
+        Sink<Real> sk{};
         // stored-segment rows are indexed by direction and Morton slot (rows
         // of particles not in the item list stay empty)
         const int64_t ray = (int64_t)k * P.n + org;
@@ -957,8 +1111,8 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
             sk.coef = static_cast<const Real*>(P.coef)[orow * P.row_stride + (int64_t)k * P.k_stride];
             live = sk.coef != Real(0);
         }
-        ray_column<Real, KERNEL, MODE, NF>(P, s_tab, s_beam + (threadIdx.x >> 5), pq, pq_count,
-                                           s_stash[threadIdx.x >> 5], o, dx, dy, dz, live, sk, err, nvisit);
+        ray_column<Real, KERNEL, MODE, NF>(P, s_tab, s_beam + (threadIdx.x >> 5), s_staged[threadIdx.x >> 5], pq,
+                                           pq_count, s_stash[threadIdx.x >> 5], o, dx, dy, dz, live, sk, err, nvisit);
         if constexpr (kQueue) {
             if (pq_count > 0) flush_partials<KERNEL, MODE, NF>(P, s_tab, pq, pq_count, pq_count, sk);
         }
@@ -1017,7 +1171,9 @@ int launch_one(const TraceParams& P, cudaStream_t s)
                             ? trace_queue_offset(P.R, KERNEL) + sizeof(PartQueue) * (256 / 32)
                             : sizeof(double) * 3 * (size_t)P.R +
                                   ((sizeof(Real) == 4 && KERNEL == URCHIN_KERNEL_M4) ? sizeof(float2) * (kKTab + 1) : 0);
-    if (smem > 48 * 1024) URCHIN_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // with the static arrays (beams, staged spheres) beyond the default 48 KB
+    if (smem + sizeof(Staged) * 8 + 2048 > 48 * 1024)
+        URCHIN_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int grid = 0;
     URCHIN_TRY(grid_for(fn, 256, smem, &grid));
     int64_t tasks = P.n_chunks * P.R;
@@ -1096,8 +1252,12 @@ int launch_trace(const TraceJob& job, cudaStream_t s)
     const urchin_bvh* b = job.bvh;
     TraceParams P;
     P.ktab = b->ktab;
-    P.nodes = b->nodes;
-    P.n_nodes = b->n_nodes;
+    P.boxes = b->boxes;
+    P.n_lev = b->n_lev;
+    for (int l = 0; l < kMaxLevels; ++l) {
+        P.lev_off[l] = b->lev_off[l];
+        P.lev_cnt[l] = b->lev_cnt[l];
+    }
     P.n = (int)b->n;
     P.xyzh = b->xyzh;
     P.w32 = job.w32;
@@ -1427,8 +1587,6 @@ int trace_columns_impl(const char* fn, const urchin_bvh* bvh, const double* x, c
     scr.release();
     URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
     if (st & kStOrigin) return set_error(URCHIN_ERR_ARG, "%s: origin index out of range", fn);
-    if (st & kStStack) return set_error(URCHIN_ERR_CUDA, "%s: traversal stack overflow", fn);
-    if (st & kStVisit) return set_error(URCHIN_ERR_CUDA, "%s: malformed tree (visit limit)", fn);
     return URCHIN_OK;
 }
 
@@ -1516,7 +1674,5 @@ extern "C" int urchin_trace_columns_vjp(const urchin_bvh* bvh, const double* dir
     scr.release();
     URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
     if (st & kStOrigin) return set_error(URCHIN_ERR_ARG, "urchin_trace_columns_vjp: origin index out of range");
-    if (st & kStStack) return set_error(URCHIN_ERR_CUDA, "urchin_trace_columns_vjp: traversal stack overflow");
-    if (st & kStVisit) return set_error(URCHIN_ERR_CUDA, "urchin_trace_columns_vjp: malformed tree (visit limit)");
     return URCHIN_OK;
 }
