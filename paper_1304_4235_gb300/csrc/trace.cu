@@ -14,10 +14,12 @@
 // against the beam, and the spheres that pass are staged in shared memory.
 // Every 32 staged spheres, each lane tests them against its own ray in the
 // beam's frame (a handful of packed FP32 operations per sphere, conservative)
-// and keeps the ones it may cross as a bit mask; the exact hit test and the
-// chord integral then run with every lane on its own next candidate, so that
-// the expensive part works on (nearly) full warps while each ray still sums
-// its hits in the tree's fixed order.
+// and keeps the ones it may cross as a bit mask.  The (ray, sphere) pairs of
+// the masks are listed ray by ray, and the exact hit test and the chord
+// integral run over the list 32 pairs at a time, whichever rays they belong
+// to; each lane then adds its own ray's values in list order, so that the
+// expensive part works on full warps while every ray still sums its hits in
+// the tree's fixed order.
 #include <algorithm>
 #include <cmath>
 
@@ -97,11 +99,7 @@ struct Sink {
     int64_t pos, end;
     Real coef;                    // MODE_SCATTER
     Real near, near_c;            // near/far: near column and its compensation
-    double ox, oy, oz;            // near/far: shifted origin in double (the near test)
-    Real sx, sy, sz;              // (image-shifted) origin
-    uint32_t lo_pend, hi_pend;    // MODE_FILL, split indices: halves / bytes of the current word
     int64_t ray;                  // MODE_CHUNK: row k n + origin slot
-    int2* cw;                     // MODE_CHUNK: the ray's current chunk
     int coff;                     // MODE_CHUNK: entries used in it (kChunk: none or full; kChunk + 1: pool exhausted)
     uint32_t cur;                 // MODE_CHUNK: its index (kNoChunk before the first)
 };
@@ -115,11 +113,11 @@ constexpr uint32_t kNoChunk = 0xffffffffu;
 // compared in double from the float positions (the differences are exact),
 // like the reference definition, so both sides classify every pair alike.
 template <typename Real>
-__device__ __forceinline__ bool is_near(const Sink<Real>& k, float4 q, Real tc, Real ch)
+__device__ __forceinline__ bool is_near(const double* o, float4 q, Real tc, Real ch)
 {
     const Real gap = tc - ch;
     if (fabs((double)gap) > 1e-4 * (double)q.w) return gap < Real(0);
-    const double ex = (double)q.x - k.ox, ey = (double)q.y - k.oy, ez = (double)q.z - k.oz;
+    const double ex = (double)q.x - o[0], ey = (double)q.y - o[1], ez = (double)q.z - o[2];
     const double hh = (double)q.w;
     return fma(ez, ez, fma(ey, ey, __dmul_rn(ex, ex))) < __dmul_rn(hh, hh);
 }
@@ -266,8 +264,14 @@ __device__ __forceinline__ float m4_seg_f(float b2, float a1, float a2)
     const float rb = b2 > 0.f ? rsqrtf(b2) : 0.f;
     float r = 0.f;
     if (a1 < s) {
-        r = m4_inner_fi(b2, rb, fminf(a2, s));
-        if (a1 > 0.f) r -= m4_inner_fi(b2, rb, a1);
+        // one copy of the code for both ends: the traversal's loop has to stay
+        // in the instruction cache
+        const int ends = a1 > 0.f ? 2 : 1;
+#pragma unroll 1
+        for (int e = 0; e < ends; ++e) {
+            const float fi = m4_inner_fi(b2, rb, e == 0 ? fminf(a2, s) : a1);
+            r = e == 0 ? fi : r - fi;
+        }
     }
     const float lo = fmaxf(a1, s);
     if (a2 > lo) {
@@ -297,11 +301,17 @@ __device__ __forceinline__ float m4_part_q(const float2* tab, float b2, float u1
     // the first piece: the clipped half of a straddling chord, or the chord
     float a1 = straddle ? 0.f : fminf(fabsf(u1), fabsf(u2));
     float a2 = straddle ? (clip_hi ? u2 : -u1) : fmaxf(fabsf(u1), fabsf(u2));
-    float F = m4_seg_f(b2, a1, a2);
-    if (straddle) {
-        if (clip_hi && clip_lo) F += m4_seg_f(b2, 0.f, -u1);
-        else F += 0.5f * m4_full_tab(tab, b2);
+    const bool both = straddle && clip_hi && clip_lo;
+    float F = 0.f;
+#pragma unroll 1
+    for (int e = 0;; ++e) {
+        const float r = m4_seg_f(b2, a1, a2);
+        F = e == 0 ? r : F + r;
+        if (e == 1 || !both) break;
+        a1 = 0.f;
+        a2 = -u1;
     }
+    if (straddle && !both) F += 0.5f * m4_full_tab(tab, b2);
     return F;
 }
 
@@ -318,6 +328,14 @@ struct Kahan {
     __device__ __forceinline__ static void add(float& s, float& c, float v)
     {
         float y = v - c;
+        float t = s + y;
+        c = (t - s) - y;
+        s = t;
+    }
+    // s += a b, the product not rounded
+    __device__ __forceinline__ static void add_product(float& s, float& c, float a, float b)
+    {
+        float y = fmaf(a, b, -c);
         float t = s + y;
         c = (t - s) - y;
         s = t;
@@ -366,11 +384,14 @@ __device__ __forceinline__ float wmax(float v)
 
 // Called by all 32 lanes with the same direction d and length L; (sx, sy, sz)
 // is the lane's (shifted) origin.  Writes the warp's beam to shared memory and
-// the lane's point and depth to (u, v, t); at least one lane is live.
+// returns the lane's point and depth (u, v, t); at least one lane is live.
+// A called function: it runs once per image, and the traversal's loop has to
+// stay in the instruction cache.
 template <typename Real>
-__device__ __forceinline__ void make_beam(Beam* out, unsigned lv, bool live, Real sx, Real sy, Real sz, float dx,
-                                          float dy, float dz, float L, float& u, float& v, float& t)
+__device__ __noinline__ float3 make_beam(Beam* out, unsigned lv, bool live, Real sx, Real sy, Real sz, float dx,
+                                         float dy, float dz, float L)
 {
+    float u, v, t;
     const int a = __ffs(lv) - 1;
     const Real bx = __shfl_sync(0xffffffffu, sx, a), by = __shfl_sync(0xffffffffu, sy, a),
                bz = __shfl_sync(0xffffffffu, sz, a);
@@ -422,6 +443,7 @@ __device__ __forceinline__ void make_beam(Beam* out, unsigned lv, bool live, Rea
                              hu * fabsf(e2z) + hv * fabsf(e1z) + eps, 0.f);
     }
     __syncwarp();
+    return make_float3(u, v, t);
 }
 
 // Whether the beam may reach the box [lo, hi]: separating axes x, y, z (on
@@ -447,25 +469,50 @@ __device__ __forceinline__ bool beam_box(const Beam& B, float4 lo, float4 hi)
     return !out;
 }
 
-// ---- staged spheres -----------------------------------------------------------
-// kSlots blocks of 32 spheres per warp: one being filled, the others holding
-// candidates that some lane has not evaluated yet (kSlots - 1 candidate masks
-// per lane).  A lane ahead of the others works on the later blocks instead of
-// waiting, which keeps the evaluation rounds full: rays of one beam differ in
-// their hits per block by more than their mean.
-constexpr int kSlots = 3;
+// ---- staged spheres and pairs ---------------------------------------------------
+// A warp's work space: a block of up to 32 spheres that the beam may reach and
+// the list of (ray, sphere) pairs that the lanes' masks give for it, at most
+// kPairs at a time (4 spheres never give more than 128).  The sizes keep three
+// blocks of 8 warps on an SM.
+template <typename Real>
+struct alignas(4 * sizeof(Real)) Origin {
+    Real x, y, z;                 // a lane's (image-shifted) origin
+    Real coef;                    // MODE_SCATTER: its ray's coefficient
+};
+template <typename Real, int MODE, bool NF>
 struct Staged {
-    float u[32], v[32], t[32], hh[32];      // the block being filled, in the beam's frame; hh = (h + margin)^2
-    float4 q[32 * kSlots];                  // x, y, z, h
-    float2 aw[32 * kSlots];                 // FP32: A_j and the tracer weight A_j x_j
-    int j[32 * kSlots];                     // Morton slot
+    static constexpr bool kF32 = sizeof(Real) == 4;
+    static constexpr bool kStored = MODE == 2 || MODE == 4;   // MODE_FILL, MODE_CHUNK
+    static constexpr int kPairs = kF32 && kStored ? 192 : 256;
+    float4 q[32];                 // x, y, z, h
+    Origin<Real> org[32];
+    union {
+        struct {
+            float u[32], v[32], t[32], hh[32];        // in the beam's frame; hh = (h + margin)^2
+        };
+        Real tc[kPairs];          // once the masks are made: depths of the closest approach, where they are
+    };                            //   kept; then (FP32) a pair's weight
+    Real val[kPairs];             // a pair's chord integral (FP64: times its weight); before that b^2, where it is kept
+    int64_t base0[MODE == 2 ? 32 : 1];        // MODE_FILL, per lane: where its next hits are stored
+    uint32_t chunk0[MODE == 4 ? 32 : 1], chunk1[MODE == 4 ? 32 : 1];   // MODE_CHUNK, per lane: its chunk and the next
+    int room[kStored ? 32 : 1];               // per lane: hits that fit (there)
+    unsigned lane_hits[kStored ? 32 : 1];     // per lane: which of its pairs are hits
+    int lane_off[kStored ? 32 : 1];           // per lane: its first pair
+    double near_o[NF ? 32 : 1][3];            // near/far: shifted origin in double (the near test)
+    float2 aw[kF32 ? 32 : 1];     // A_j and the tracer weight A_j x_j
+    float2 g[kF32 ? 32 : 1];      // 1/h and h^2
+    int j[32];                    // Morton slot
+    unsigned hit[kPairs / 32 + 1], full[kPairs / 32 + 1], any[kPairs / 32 + 1];   // bit per pair; any: near ones too
+    uint16_t pair[kPairs];        // sphere << 5 | lane
+    uint8_t list[kF32 ? 1 : kPairs];          // FP64: full chords from the front, partial from the back
 };
 
 // The lanes' candidates among the block's first m spheres (bit e: sphere e):
 // the lane's segment comes within h + margin of the sphere's centre,
 //   (u_e - u)^2 + (v_e - v)^2 + dt^2 < hh,  dt the distance of t_e to [t, t + L].
 // Two spheres per packed FP32 operation.
-__device__ __forceinline__ unsigned candidates(const Staged& S, int m, float u, float v, float t, float L)
+template <typename St>
+__device__ __forceinline__ unsigned candidates(const St& S, int m, float u, float v, float t, float L)
 {
     const float2 nu = make_float2(-u, -u), nv = make_float2(-v, -v), nt = make_float2(-t, -t), nL = make_float2(-L, -L);
     unsigned mask = 0u;
@@ -491,23 +538,16 @@ __device__ __forceinline__ unsigned candidates(const Staged& S, int m, float u, 
     return m < 32 ? mask & ((1u << m) - 1u) : mask;
 }
 
-// Particle index of stored segment pos: an int32, or split into 16 + 8 bits.
-// A lane writes its ray's segments at consecutive positions from a multiple
-// of 8 to a multiple of 8 (the padding), so the split halves and bytes are
-// gathered in the sink and written as whole 32-bit words.
-template <typename Real>
-__device__ __forceinline__ void store_index(const TraceParams& P, Sink<Real>& k, int64_t pos, int j)
+// Particle index of stored segment pos: an int32, or split into 16 + 8 bits
+// (neighbouring lanes store neighbouring positions of one ray's list).
+__device__ __forceinline__ void store_index(const TraceParams& P, int64_t pos, int j)
 {
     if (P.seg_col) {
         P.seg_col[pos] = j;
         return;
     }
-    const uint32_t lo = (uint32_t)j & 0xffffu, hi = ((uint32_t)j >> 16) & 0xffu;
-    if (pos & 1) reinterpret_cast<uint32_t*>(P.seg_lo)[pos >> 1] = k.lo_pend | (lo << 16);
-    else k.lo_pend = lo;
-    const int sh = (int)(pos & 3) * 8;
-    k.hi_pend = (sh == 0 ? 0u : k.hi_pend) | (hi << sh);
-    if ((pos & 3) == 3) reinterpret_cast<uint32_t*>(P.seg_hi)[pos >> 2] = k.hi_pend;
+    P.seg_lo[pos] = (uint16_t)((uint32_t)j & 0xffffu);
+    P.seg_hi[pos] = (uint8_t)(((uint32_t)j >> 16) & 0xffu);
 }
 
 // ---- deferred partial chords ------------------------------------------------
@@ -524,33 +564,26 @@ constexpr int kPQ = 64;           // queue capacity per warp; a round takes 32
 constexpr int kPQNear = 32;       // owner flag: a near particle (near/far split)
 constexpr int kPQClipLo = 64;     // owner flag: the segment's start cuts the chord
 constexpr int kPQClipHi = 128;    // owner flag: the segment's end cuts the chord
+template <bool kStored, bool NF>
 struct PartQueue {
     float beta2[kPQ], u1[kPQ], u2[kPQ];   // chord in units of h: b^2/h^2 and [u1, u2]
     float A[kPQ];                 // A_j
     float w[kPQ];                 // the tracer weight A_j x_j (MODE_SCATTER: the ray's coefficient)
     int j[kPQ];                   // particle (Morton slot)
     int owner[kPQ];               // lane of the ray | kPQNear | kPQClipLo | kPQClipHi
-    int64_t pos[kPQ];             // MODE_FILL, MODE_CHUNK: the segment's position
+    int64_t pos[kStored ? kPQ : 1];       // MODE_FILL, MODE_CHUNK: the segment's position
     float val[32];                // results of the round being flushed
-    unsigned own[64];             // per owner (lane, lane + kPQNear): items of the round
+    unsigned own[NF ? 64 : 32];   // per owner (lane, lane + kPQNear): items of the round
 };
-
-// Byte offset of the queues in k_trace's dynamic shared memory: after the
-// directions (double[3R]) and the FP32 M4 table, 16-byte aligned.
-__host__ __device__ __forceinline__ size_t trace_queue_offset(int R, int kernel)
-{
-    const size_t b = sizeof(double) * 3 * (size_t)R + (kernel == URCHIN_KERNEL_M4 ? sizeof(float2) * (kKTab + 1) : 0);
-    return (b + 15) & ~size_t(15);
-}
 
 // Evaluate the first n (<= 32) queued chords, one per lane, and move the
 // rest to the front.  Every lane of the warp calls it.  Inlined: as a called
 // function its reference arguments kept the ray's running state (sums,
 // cursor, queue length) in local memory for the whole traversal, which cost
 // 7 % of the traversal's time.
-template <int KERNEL, int MODE, bool NF>
-__device__ __forceinline__ void flush_partials(const TraceParams& P, const float2* tab, PartQueue* pq, int& count,
-                                               int n, Sink<float>& k)
+template <int KERNEL, int MODE, bool NF, typename Queue>
+__device__ __forceinline__ void flush_partials(const TraceParams& P, const float2* tab, Queue* pq, int& count, int n,
+                                               Sink<float>& k)
 {
     const int lane = threadIdx.x & 31;
     int owner = -1;
@@ -566,15 +599,14 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
         } else {
             const bool near = NF && (ow & kPQNear);
             v = near ? A * F : pq->w[lane] * F;
-            if (MODE == MODE_FILL && !near) static_cast<float*>(P.seg_val)[pq->pos[lane]] = A * F;
+            if (MODE == MODE_FILL && pq->pos[lane] >= 0) static_cast<float*>(P.seg_val)[pq->pos[lane]] = A * F;
             if (MODE == MODE_CHUNK && pq->pos[lane] >= 0) P.chunk_seg[pq->pos[lane]] = make_int2(j, __float_as_int(A * F));
             owner = ow & (31 | kPQNear);
         }
     }
     if (MODE != MODE_SCATTER) {
         pq->val[lane] = v;
-        const unsigned same = __match_any_sync(0xffffffffu, owner);
-        if (owner >= 0 && (same & ((1u << lane) - 1u)) == 0u) pq->own[owner] = same;
+        if (owner >= 0) atomicOr(&pq->own[owner], 1u << lane);
         __syncwarp();
         for (unsigned m = pq->own[lane]; m; m &= m - 1) Kahan::add(k.psum, k.pcomp, pq->val[__ffs(m) - 1]);
         if (NF)
@@ -582,7 +614,7 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
                 Kahan::add(k.near, k.near_c, pq->val[__ffs(m) - 1]);
         __syncwarp();
         pq->own[lane] = 0u;
-        pq->own[lane + kPQNear] = 0u;
+        if (NF) pq->own[lane + kPQNear] = 0u;
     }
     const int rest = count - n;
     if (rest > 0) {
@@ -631,86 +663,31 @@ __device__ __forceinline__ unsigned long long chunk_block(const TraceParams& P, 
     return b;
 }
 
-// FP32 evaluation of one candidate per lane (act: the lane has one): the
-// impact parameter from an error-free cross product decides the hit; full
-// chords from the table at once, partial chords queued for flush_partials.
-// Every lane of the warp calls it (the queue and the chunks are shared).
-template <int KERNEL, int MODE, bool NF>
-__device__ __forceinline__ void eval_f32(const TraceParams& P, const float2* tab, PartQueue* pq, int& pq_count,
-                                         unsigned long long* stash, bool act, const Staged& S, int at, float dx,
-                                         float dy, float dz, float L, Sink<float>& k, unsigned& err)
+// Where a lane's next h hits go (MODE_FILL, MODE_CHUNK; called with the warp
+// converged): consecutive positions of its ray's segment list, in MODE_CHUNK
+// the rest of its chunk and then a new one (h <= 32 = kChunk, so one is enough).
+template <int MODE, typename Real, typename St>
+__device__ __forceinline__ void assign_positions(const TraceParams& P, unsigned long long* stash, St& S, int h,
+                                                 Sink<Real>& k, unsigned& err)
 {
     const int lane = threadIdx.x & 31;
-    bool part = false, near = false, store = false;
-    int clip = 0, j = 0;
-    float beta2 = 0.f, u1 = 0.f, u2 = 0.f, segv = 0.f;
-    float2 aw = make_float2(0.f, 0.f);
-    int64_t spos = 0;
-    if (act) {
-        // The hit decision is written with explicit roundings (no
-        // multiply-add contraction left to the compiler), so that the
-        // counting and the filling traversal, separate instantiations,
-        // find exactly the same hits.
-        const float4 q = S.q[at];
-        j = S.j[at];
-        const float ex = q.x - k.sx, ey = q.y - k.sy, ez = q.z - k.sz;
-        const float cx = dop(ey, dz, ez, dy);
-        const float cy = dop(ez, dx, ex, dz);
-        const float cz = dop(ex, dy, ey, dx);
-        const float h2 = __fmul_rn(q.w, q.w);
-        const float b2 = fmaf(cz, cz, fmaf(cy, cy, __fmul_rn(cx, cx)));
-        bool hit = b2 < h2;
-        float tc = 0.f, ch = 0.f;
-        if (hit) {
-            tc = fmaf(ez, dz, fmaf(ey, dy, __fmul_rn(ex, dx)));
-            ch = sqrtf(__fsub_rn(h2, b2));
-            hit = __fadd_rn(tc, ch) > 0.f && __fsub_rn(tc, ch) < L;
+    if constexpr (MODE == MODE_FILL) {
+        int r = h;
+        if ((int64_t)h > k.end - k.pos) {              // more hits than were counted
+            r = (int)(k.end - k.pos);
+            err |= kStSegment;
         }
-        if (hit) {
-            near = NF && is_near(k, q, tc, ch);
-            if (!near) ++k.nhit;
-            if (MODE == MODE_CHUNK && !near) store = true;
-            if (MODE != MODE_COUNT) {
-                aw = S.aw[at];
-                const float ih = 1.f / q.w;
-                beta2 = b2 * ih * ih;
-                if (MODE == MODE_FILL && !near) {
-                    // the index is written now, in order; a partial chord's value at the flush
-                    if (k.pos < k.end) {
-                        store_index(P, k, k.pos, j);
-                        spos = k.pos++;
-                    } else {
-                        err |= kStSegment;
-                        hit = false;
-                    }
-                }
-                if (hit && __fsub_rn(tc, ch) >= 0.f && __fadd_rn(tc, ch) <= L) {
-                    const float F = KERNEL == URCHIN_KERNEL_M4 ? m4_full_tab(tab, beta2)
-                                                               : gt_chord<float>(P, beta2, -ch * ih, ch * ih);
-                    if (MODE == MODE_SCATTER) {
-                        atomicAdd(P.xbar + j, (double)(k.coef * (aw.x * F)));
-                    } else if (near) {
-                        Kahan::add(k.near, k.near_c, aw.x * F);
-                    } else {
-                        Kahan::add(k.sum, k.comp, aw.y * F);
-                        if (MODE == MODE_FILL) static_cast<float*>(P.seg_val)[spos] = aw.x * F;
-                        if (MODE == MODE_CHUNK) segv = aw.x * F;
-                    }
-                } else if (hit) {
-                    part = true;
-                    clip = (__fsub_rn(tc, ch) < 0.f ? kPQClipLo : 0) | (__fadd_rn(tc, ch) > L ? kPQClipHi : 0);
-                    u1 = (fmaxf(0.f, tc - ch) - tc) * ih;
-                    u2 = (fminf(L, tc + ch) - tc) * ih;
-                }
-            }
-        }
-    }
-    if (MODE == MODE_COUNT) return;
-    if constexpr (MODE == MODE_CHUNK) {
-        // with the warp converged: a new chunk for every ray whose chunk
-        // is full (or that has none yet), then the segment's index (and a
-        // full chord's value; a partial chord's at the flush)
-        const bool need = store && k.coff == kChunk;
+        S.base0[lane] = k.pos;
+        S.room[lane] = r;
+        k.pos += r;
+    } else {
+        // coff: entries used of the current chunk (kChunk: none left, or no
+        // chunk yet; kChunk + 1: the pool is exhausted, nothing more is stored)
+        const int r = k.coff <= kChunk ? kChunk - k.coff : 0;
+        const bool need = k.coff <= kChunk && h > r;
+        S.chunk0[lane] = k.cur;
+        S.room[lane] = r;
+        uint32_t next = kNoChunk;
         const unsigned nm = __ballot_sync(0xffffffffu, need);
         if (nm) {
             unsigned long long base = 0;
@@ -721,94 +698,334 @@ __device__ __forceinline__ void eval_f32(const TraceParams& P, const float2* tab
                 if (c < P.chunk_cap) {
                     if (k.cur == kNoChunk) P.chunk_head[k.ray] = (uint32_t)c;
                     else P.chunk_next[k.cur] = (uint32_t)c;
-                    k.cur = (uint32_t)c;
-                    k.cw = P.chunk_seg + c * (unsigned long long)kChunk;
-                    k.coff = 0;
+                    next = (uint32_t)c;
+                    k.cur = next;
+                    k.coff = h - r;
                 } else {
-                    k.coff = kChunk + 1;        // the pool is exhausted: this ray stores no more
+                    k.coff = kChunk + 1;
                 }
             }
         }
-        spos = -1;
-        if (store && k.coff < kChunk) {
-            // a partial chord's entry is written whole at the flush
-            if (!part) k.cw[k.coff] = make_int2(j, __float_as_int(segv));
-            else spos = (int64_t)k.cur * kChunk + k.coff;
-            ++k.coff;
-        }
+        if (!need && k.coff <= kChunk) k.coff += h;
+        S.chunk1[lane] = next;
     }
-    const unsigned pb = __ballot_sync(0xffffffffu, part);
-    if (!pb) return;
-    if (part) {
-        const int i = pq_count + __popc(pb & ((1u << lane) - 1u));
-        pq->beta2[i] = beta2;
-        pq->u1[i] = u1;
-        pq->u2[i] = u2;
-        pq->A[i] = aw.x;
-        pq->w[i] = MODE == MODE_SCATTER ? k.coef : aw.y;
-        pq->j[i] = j;
-        pq->owner[i] = lane | (near ? kPQNear : 0) | clip;
-        if (MODE == MODE_FILL || MODE == MODE_CHUNK) pq->pos[i] = spos;
-    }
-    pq_count += __popc(pb);
-    __syncwarp();
-    if (pq_count >= 32) flush_partials<KERNEL, MODE, NF>(P, tab, pq, pq_count, 32, k);
 }
 
-// The same in double, chords evaluated in place.
-template <typename Real, int KERNEL, int MODE, bool NF>
-__device__ __forceinline__ void eval_f64(const TraceParams& P, const Staged& S, int at, Real dx, Real dy, Real dz,
-                                         Real L, Sink<Real>& k, unsigned& err)
+// Position of pair p, a hit of lane o (-1: not stored).
+template <int MODE, typename St>
+__device__ __forceinline__ int64_t hit_position(const St& S, int p, int o)
 {
-    using O = RealOps<Real>;
-    // explicit roundings in the hit decision, as in eval_f32
-    const float4 q = S.q[at];
-    const int j = S.j[at];
-    Real ex = Real(q.x) - k.sx, ey = Real(q.y) - k.sy, ez = Real(q.z) - k.sz;
-    Real tc = fma(ez, dz, fma(ey, dy, mul_rn(ex, dx)));
-    Real cx = sub_rn(mul_rn(ey, dz), mul_rn(ez, dy));
-    Real cy = sub_rn(mul_rn(ez, dx), mul_rn(ex, dz));
-    Real cz = sub_rn(mul_rn(ex, dy), mul_rn(ey, dx));
-    Real b2 = fma(cz, cz, fma(cy, cy, mul_rn(cx, cx)));
-    Real h = Real(q.w);
-    Real h2 = mul_rn(h, h);
-    if (b2 >= h2) return;
-    Real ch = O::sqrt_(sub_rn(h2, b2));
-    if (add_rn(tc, ch) <= Real(0) || sub_rn(tc, ch) >= L) return;
-    const bool near = NF && is_near(k, q, tc, ch);
-    if (!near) ++k.nhit;
-    if (MODE == MODE_COUNT) return;
-    Real ih = Real(1) / h;
-    Real beta2 = b2 * ih * ih;
-    Real F;
-    if (sub_rn(tc, ch) >= Real(0) && add_rn(tc, ch) <= L) {
-        Real c = ch * ih;
-        if (KERNEL == URCHIN_KERNEL_M4) F = m4_full(beta2, c);
-        else F = gt_chord(P, beta2, -c, c);
-    } else {
-        Real u1 = (fmax(Real(0), tc - ch) - tc) * ih;
-        Real u2 = (fmin(L, tc + ch) - tc) * ih;
-        if (KERNEL == URCHIN_KERNEL_M4) F = m4_part(beta2, u1, u2);
-        else F = gt_chord(P, beta2, u1, u2);
+    const int i = __popc(S.lane_hits[o] & ((1u << (p - S.lane_off[o])) - 1u)), r = S.room[o];
+    if constexpr (MODE == MODE_FILL) return i < r ? S.base0[o] + i : -1;
+    const uint32_t c = i < r ? S.chunk0[o] : S.chunk1[o];
+    // the first chunk's free entries are its last r
+    return c == kNoChunk ? -1 : (int64_t)c * kChunk + (i < r ? kChunk - r + i : i - r);
+}
+
+// Bits [off, off + c) of a list of flag words, c <= 32.
+__device__ __forceinline__ unsigned flag_bits(const unsigned* w, int off, int c)
+{
+    const unsigned b = __funnelshift_r(w[off >> 5], w[(off >> 5) + 1], off & 31);
+    return c < 32 ? b & ((1u << c) - 1u) : b;
+}
+
+// Hit decision of pair (sphere e, lane o).  Written with explicit roundings
+// (no multiply-add contraction left to the compiler), so that the counting and
+// the filling traversal, separate instantiations, find exactly the same hits.
+// FP32: the impact parameter from an error-free cross product.
+template <typename St>
+__device__ __forceinline__ bool decide(const St& S, int e, int o, float dx, float dy, float dz, float L, float& b2,
+                                       float& tc, float& ch)
+{
+    const float4 q = S.q[e];
+    const Origin<float> s = S.org[o];
+    const float ex = q.x - s.x, ey = q.y - s.y, ez = q.z - s.z;
+    const float cx = dop(ey, dz, ez, dy);
+    const float cy = dop(ez, dx, ex, dz);
+    const float cz = dop(ex, dy, ey, dx);
+    const float h2 = S.g[e].y;
+    b2 = fmaf(cz, cz, fmaf(cy, cy, __fmul_rn(cx, cx)));
+    if (!(b2 < h2)) return false;
+    tc = fmaf(ez, dz, fmaf(ey, dy, __fmul_rn(ex, dx)));
+    ch = sqrtf(__fsub_rn(h2, b2));
+    return __fadd_rn(tc, ch) > 0.f && __fsub_rn(tc, ch) < L;
+}
+
+template <typename St>
+__device__ __forceinline__ bool decide(const St& S, int e, int o, double dx, double dy, double dz, double L,
+                                       double& b2, double& tc, double& ch)
+{
+    const float4 q = S.q[e];
+    const Origin<double> s = S.org[o];
+    const double ex = (double)q.x - s.x, ey = (double)q.y - s.y, ez = (double)q.z - s.z;
+    const double cx = sub_rn(mul_rn(ey, dz), mul_rn(ez, dy));
+    const double cy = sub_rn(mul_rn(ez, dx), mul_rn(ex, dz));
+    const double cz = sub_rn(mul_rn(ex, dy), mul_rn(ey, dx));
+    const double h2 = mul_rn((double)q.w, (double)q.w);
+    b2 = fma(cz, cz, fma(cy, cy, mul_rn(cx, cx)));
+    if (!(b2 < h2)) return false;
+    tc = fma(ez, dz, fma(ey, dy, mul_rn(ex, dx)));
+    ch = sqrt(sub_rn(h2, b2));
+    return add_rn(tc, ch) > 0.0 && sub_rn(tc, ch) < L;
+}
+
+// The pairs of the lanes' masks mm (at most kPairs in all): listed, decided,
+// evaluated and added up (file comment).  FP32: full chords from the table at
+// once, partial chords queued for flush_partials.  Where hits are stored
+// (MODE_FILL, MODE_CHUNK) all pairs are decided first, which gives every hit
+// its position.
+template <int KERNEL, int MODE, bool NF, typename Queue, typename St>
+__device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* tab, Queue* pq, int& pq_count,
+                                          unsigned long long* stash, St& S, unsigned mm, bool drain, float dx, float dy,
+                                          float dz, float L, Sink<float>& k, unsigned& err)
+{
+    constexpr bool kStored = MODE == MODE_FILL || MODE == MODE_CHUNK;
+    const int lane = threadIdx.x & 31;
+    const int c = __popc(mm);
+    int off = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, off, d);
+        if (lane >= d) off += y;
     }
-    if (MODE == MODE_SCATTER) {
-        atomicAdd(P.xbar + j, (double)(k.coef * (Real(__ldg(P.A64 + j)) * F)));
-        return;
+    const int total = __shfl_sync(0xffffffffu, off, 31);
+    off -= c;
+    {
+        int i = off;
+        for (unsigned m = mm; m; m &= m - 1u) S.pair[i++] = (uint16_t)(((__ffs(m) - 1) << 5) | lane);
     }
-    if (near) {
-        Kahan::add(k.near, k.near_c, Real(__ldg(P.A64 + j)) * F);
-        return;
+    __syncwarp();
+    if constexpr (kStored) {
+        for (int p0 = 0; p0 < total; p0 += 32) {
+            const int p = p0 + lane;
+            bool hit = false, near = false;
+            if (p < total) {
+                const int pr = S.pair[p], e = pr >> 5, o = pr & 31;
+                float b2, tc = 0.f, ch = 0.f;
+                hit = decide(S, e, o, dx, dy, dz, L, b2, tc, ch);
+                if (hit) {
+                    near = NF && is_near(S.near_o[o], S.q[e], tc, ch);
+                    S.val[p] = b2;
+                    S.tc[p] = tc;
+                }
+            }
+            const unsigned ha = __ballot_sync(0xffffffffu, hit), hw = __ballot_sync(0xffffffffu, hit && !near);
+            if (lane == 0) {
+                S.any[p0 >> 5] = ha;
+                S.hit[p0 >> 5] = hw;
+            }
+        }
+        __syncwarp();
+        const unsigned hm = c ? flag_bits(S.hit, off, c) : 0u;
+        k.nhit += (unsigned)__popc(hm);
+        S.lane_hits[lane] = hm;
+        S.lane_off[lane] = off;
+        assign_positions<MODE>(P, stash, S, __popc(hm), k, err);
+        __syncwarp();
     }
-    Kahan::add(k.sum, k.comp, O::weight(P, j) * F);
-    if (MODE == MODE_FILL) {
-        if (k.pos < k.end) {
-            store_index(P, k, k.pos, j);
-            static_cast<Real*>(P.seg_val)[k.pos] = Real(__ldg(P.A64 + j)) * F;
-            ++k.pos;
-        } else {
-            err |= kStSegment;
+    for (int p0 = 0; p0 < total || drain; p0 += 32) {
+        const int p = p0 + lane;
+        bool hit = false, near = false, full = false, part = false;
+        int clip = 0, e = 0, o = 0;
+        float beta2 = 0.f, u1 = 0.f, u2 = 0.f;
+        float2 aw = make_float2(0.f, 0.f);
+        int64_t pos = -1;
+        if (p < total) {
+            const int pr = S.pair[p];
+            e = pr >> 5;
+            o = pr & 31;
+            float b2, tc = 0.f, ch = 0.f;
+            if constexpr (kStored) {
+                hit = (S.any[p0 >> 5] >> lane) & 1u;
+                if (hit) {
+                    b2 = S.val[p];
+                    tc = S.tc[p];
+                    ch = sqrtf(__fsub_rn(S.g[e].y, b2));
+                    near = NF && !((S.hit[p0 >> 5] >> lane) & 1u);
+                    if (!near) {
+                        pos = hit_position<MODE>(S, p, o);
+                        if (MODE == MODE_FILL && pos >= 0) store_index(P, pos, S.j[e]);
+                    }
+                }
+            } else {
+                hit = decide(S, e, o, dx, dy, dz, L, b2, tc, ch);
+                if (hit) near = NF && is_near(S.near_o[o], S.q[e], tc, ch);
+            }
+            if (hit && MODE != MODE_COUNT) {
+                const float ih = S.g[e].x;
+                aw = S.aw[e];
+                beta2 = b2 * ih * ih;
+                full = __fsub_rn(tc, ch) >= 0.f && __fadd_rn(tc, ch) <= L;
+                if (full) {
+                    const float F = KERNEL == URCHIN_KERNEL_M4 ? m4_full_tab(tab, beta2)
+                                                               : gt_chord<float>(P, beta2, -ch * ih, ch * ih);
+                    if (MODE == MODE_SCATTER) atomicAdd(P.xbar + S.j[e], (double)(S.org[o].coef * (aw.x * F)));
+                    else {
+                        S.val[p] = F;
+                        S.tc[p] = near ? aw.x : aw.y;
+                    }
+                    if (MODE == MODE_FILL && pos >= 0) static_cast<float*>(P.seg_val)[pos] = aw.x * F;
+                    if (MODE == MODE_CHUNK && pos >= 0) P.chunk_seg[pos] = make_int2(S.j[e], __float_as_int(aw.x * F));
+                } else {
+                    part = true;
+                    clip = (__fsub_rn(tc, ch) < 0.f ? kPQClipLo : 0) | (__fadd_rn(tc, ch) > L ? kPQClipHi : 0);
+                    u1 = (fmaxf(0.f, tc - ch) - tc) * ih;
+                    u2 = (fminf(L, tc + ch) - tc) * ih;
+                }
+            }
+        }
+        const unsigned fw = __ballot_sync(0xffffffffu, full);
+        if constexpr (!kStored) {
+            const unsigned hw = __ballot_sync(0xffffffffu, hit && !near);
+            if (lane == 0) S.hit[p0 >> 5] = hw;
+        }
+        if (MODE == MODE_COUNT) continue;
+        if (lane == 0) S.full[p0 >> 5] = fw;
+        const unsigned pb = __ballot_sync(0xffffffffu, part);
+        if (!pb && !drain) continue;
+        if (part) {
+            const int i = pq_count + __popc(pb & ((1u << lane) - 1u));
+            pq->beta2[i] = beta2;
+            pq->u1[i] = u1;
+            pq->u2[i] = u2;
+            pq->A[i] = aw.x;
+            pq->w[i] = MODE == MODE_SCATTER ? S.org[o].coef : aw.y;
+            pq->j[i] = S.j[e];
+            pq->owner[i] = o | (near ? kPQNear : 0) | clip;
+            if (kStored) pq->pos[i] = pos;
+        }
+        pq_count += __popc(pb);
+        __syncwarp();
+        // (at the end of the rays, drain, what is left: fewer than 32)
+        if (pq_count >= 32 || (drain && pq_count > 0))
+            flush_partials<KERNEL, MODE, NF>(P, tab, pq, pq_count, min(pq_count, 32), k);
+        if (drain) break;
+    }
+    __syncwarp();
+    if (c) {
+        if (!kStored) k.nhit += (unsigned)__popc(flag_bits(S.hit, off, c));
+        if (MODE != MODE_COUNT && MODE != MODE_SCATTER) {
+            unsigned far = 0xffffffffu;
+            if (NF) far = flag_bits(S.hit, off, c);
+            for (unsigned m = flag_bits(S.full, off, c); m; m &= m - 1u) {
+                const int i = __ffs(m) - 1;
+                const float F = S.val[off + i], w = S.tc[off + i];
+                if (!NF || ((far >> i) & 1u)) Kahan::add_product(k.sum, k.comp, w, F);
+                else Kahan::add_product(k.near, k.near_c, w, F);
+            }
         }
     }
+    __syncwarp();
+}
+
+// The same in double: the pairs are decided first and split into full and
+// partial chords, each evaluated 32 at a time (one kind costs two to three
+// times the other, and the FP64 pipe is what bounds this path).
+template <int KERNEL, int MODE, bool NF, typename St>
+__device__ __forceinline__ void pairs_f64(const TraceParams& P, unsigned long long* stash, St& S, unsigned mm,
+                                          double dx, double dy, double dz, double L, Sink<double>& k, unsigned& err)
+{
+    constexpr bool kStored = MODE == MODE_FILL;
+    const int lane = threadIdx.x & 31;
+    const int c = __popc(mm);
+    int off = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, off, d);
+        if (lane >= d) off += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, off, 31);
+    off -= c;
+    {
+        int i = off;
+        for (unsigned m = mm; m; m &= m - 1u) S.pair[i++] = (uint16_t)(((__ffs(m) - 1) << 5) | lane);
+    }
+    __syncwarp();
+    int nf = 0, np = 0;
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        const int p = p0 + lane;
+        bool hit = false, near = false, full = false;
+        if (p < total) {
+            const int pr = S.pair[p], e = pr >> 5, o = pr & 31;
+            double b2, tc = 0.0, ch = 0.0;
+            hit = decide(S, e, o, dx, dy, dz, L, b2, tc, ch);
+            if (hit) {
+                near = NF && is_near(S.near_o[o], S.q[e], tc, ch);
+                full = sub_rn(tc, ch) >= 0.0 && add_rn(tc, ch) <= L;
+                S.val[p] = b2;
+                S.tc[p] = tc;
+            }
+        }
+        const unsigned ha = __ballot_sync(0xffffffffu, hit), hw = __ballot_sync(0xffffffffu, hit && !near);
+        const unsigned fw = __ballot_sync(0xffffffffu, hit && full), lt = (1u << lane) - 1u;
+        if (hit) {
+            if (full) S.list[nf + __popc(fw & lt)] = (uint8_t)p;
+            else S.list[St::kPairs - 1 - np - __popc(ha & ~fw & lt)] = (uint8_t)p;
+        }
+        nf += __popc(fw);
+        np += __popc(ha & ~fw);
+        if (lane == 0) {
+            S.any[p0 >> 5] = ha;
+            S.hit[p0 >> 5] = hw;
+        }
+    }
+    __syncwarp();
+    const unsigned hm = c ? flag_bits(S.hit, off, c) : 0u;
+    k.nhit += (unsigned)__popc(hm);
+    if constexpr (kStored) {
+        S.lane_hits[lane] = hm;
+        S.lane_off[lane] = off;
+        assign_positions<MODE>(P, stash, S, __popc(hm), k, err);
+        __syncwarp();
+    }
+#pragma unroll 1
+    for (int kind = MODE == MODE_COUNT ? 2 : 0; kind < 2; ++kind) {
+        const int n = kind == 0 ? nf : np;
+#pragma unroll 1
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            if (i >= n) continue;
+            const int p = S.list[kind == 0 ? i : St::kPairs - 1 - i];
+            const int pr = S.pair[p], e = pr >> 5, o = pr & 31, j = S.j[e];
+            const double b2 = S.val[p], h = (double)S.q[e].w, ih = 1.0 / h;
+            const double ch = sqrt(sub_rn(mul_rn(h, h), b2));
+            const double beta2 = b2 * ih * ih;
+            double F;
+            if (kind == 0) {
+                const double cc = ch * ih;
+                if (KERNEL == URCHIN_KERNEL_M4) F = m4_full(beta2, cc);
+                else F = gt_chord(P, beta2, -cc, cc);
+            } else {
+                const double tc = S.tc[p];
+                const double u1 = (fmax(0.0, tc - ch) - tc) * ih, u2 = (fmin(L, tc + ch) - tc) * ih;
+                if (KERNEL == URCHIN_KERNEL_M4) F = m4_part(beta2, u1, u2);
+                else F = gt_chord(P, beta2, u1, u2);
+            }
+            if (MODE == MODE_SCATTER) {
+                atomicAdd(P.xbar + j, S.org[o].coef * (__ldg(P.A64 + j) * F));
+                continue;
+            }
+            const bool far = !NF || ((S.hit[p >> 5] >> (p & 31)) & 1u);
+            S.val[p] = far ? __ldg(P.w64 + j) * F : __ldg(P.A64 + j) * F;
+            if (kStored && far) {
+                const int64_t pos = hit_position<MODE>(S, p, o);
+                if (pos >= 0) {
+                    store_index(P, pos, j);
+                    static_cast<double*>(P.seg_val)[pos] = __ldg(P.A64 + j) * F;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (c && MODE != MODE_SCATTER && MODE != MODE_COUNT) {
+        for (unsigned m = flag_bits(S.any, off, c); m; m &= m - 1u) {
+            const int i = __ffs(m) - 1;
+            const double v = S.val[off + i];
+            if (!NF || ((hm >> i) & 1u)) Kahan::add(k.sum, k.comp, v);
+            else Kahan::add(k.near, k.near_c, v);
+        }
+    }
+    __syncwarp();
 }
 
 // The tree walk of one packet: next() gives the leaves that the beam may
@@ -819,6 +1036,7 @@ struct Walk {
     unsigned pend;                // lane l holds level l's mask while its subtrees are walked
     int lref, lcnt;               // children that are leaves: the lane's leaf
     unsigned visits;
+    bool fresh;                   // the current entry's children have not been tested
 
     __device__ __forceinline__ void children(const TraceParams& P, const Beam& B)
     {
@@ -833,20 +1051,22 @@ struct Walk {
         }
         mask = __ballot_sync(0xffffffffu, pass);
         ++visits;
+        fresh = false;
     }
 
-    __device__ __forceinline__ void start(const TraceParams& P, const Beam& B)
+    __device__ __forceinline__ void start(const TraceParams& P)
     {
         lev = P.n_lev;
         node = 0;
-        pend = 0u;
-        children(P, B);
+        mask = pend = visits = 0u;
+        fresh = true;
     }
 
     // false at the end of the walk
     __device__ __forceinline__ bool next(const TraceParams& P, const Beam& B, int& ref, int& cnt)
     {
         for (;;) {
+            if (fresh) children(P, B);
             if (mask == 0u) {
                 if (lev == P.n_lev) return false;
                 ++lev;
@@ -864,17 +1084,19 @@ struct Walk {
             if ((int)(threadIdx.x & 31) == lev) pend = mask;
             node = 32 * node + c;
             --lev;
-            children(P, B);
+            fresh = true;
         }
     }
 };
 
-// One image of the packet's rays: walk, stage, filter, evaluate (file comment).
-template <typename Real, int KERNEL, int MODE, bool NF>
-__device__ __forceinline__ void packet_image(const TraceParams& P, const float2* tab, const Beam& B, Staged& S,
-                                             PartQueue* pq, int& pq_count, unsigned long long* stash, float u, float v,
-                                             float t, float Lf, Real dx, Real dy, Real dz, bool live, Sink<Real>& sk,
-                                             unsigned& err, unsigned& nvisit)
+// One image of the packet's rays: walk, stage, filter, evaluate (file comment);
+// with drain, no image but the queued partial chords (so that the loop holds
+// one copy of that code).
+template <typename Real, int KERNEL, int MODE, bool NF, typename Queue, typename St>
+__device__ __forceinline__ void packet_image(const TraceParams& P, const float2* tab, const Beam& B, St& S,
+                                             Queue* pq, int& pq_count, unsigned long long* stash, float3 pt,
+                                             float Lf, Real dx, Real dy, Real dz, bool live, bool drain,
+                                             Sink<Real>& sk, unsigned& err, unsigned& nvisit)
 {
     const Real L = Real(P.l_ray);
     const int lane = threadIdx.x & 31;
@@ -882,10 +1104,9 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
     constexpr bool kWantW = kF32 && MODE != MODE_COUNT && MODE != MODE_SCATTER;
     constexpr bool kWantA = kF32 && MODE != MODE_COUNT && (MODE != MODE_TAU || NF);
     Walk W;
-    W.visits = 0u;
-    W.start(P, B);
-    int ref = 0, cnt = 0;
-    bool more = W.next(P, B, ref, cnt);
+    W.start(P);
+    int ref = 0, cnt = 0;            // the current leaf (none at first) while the next one is on its way
+    bool more = !drain;
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
     float2 aw = make_float2(0.f, 0.f);
     auto fetch = [&](int r, int c) {
@@ -895,9 +1116,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
             if (kWantW) aw.y = __ldg(P.w32 + r + lane);
         }
     };
-    if (more) fetch(ref, cnt);
-    unsigned m0 = 0u, m1 = 0u;       // candidates in the oldest and the newer full block
-    int st = 0, ns = 0;              // block being filled (0, 32, 64) and its spheres
+    int ns = 0;                      // spheres in the block being filled
     for (;;) {
         const bool last = !more;
         unsigned pm = 0u;
@@ -906,7 +1125,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
         const float2 caw = aw;
         const int cj = ref + lane;
         if (!last) {
-            // sphere (one per lane) against the beam
+            // sphere (one per lane) against the beam; the next leaf's spheres are on their way meanwhile
             bool pass = false;
             if (lane < cnt) {
                 const float4 c4 = B.c, a4 = B.e1, b4 = B.e2, d4 = B.d;
@@ -925,17 +1144,22 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
             if (more) fetch(ref, cnt);
             if (pm == 0u) continue;
         }
+        const int rank = __popc(pm & ((1u << lane) - 1u)), pc = __popc(pm);
+        auto stage = [&](int at) {
+            S.u[at] = su;
+            S.v[at] = sv;
+            S.t[at] = stt;
+            S.hh[at] = shh;
+            S.q[at] = cq;
+            S.j[at] = cj;
+            if constexpr (kF32) {
+                S.g[at] = make_float2(1.f / cq.w, __fmul_rn(cq.w, cq.w));
+                if (kWantA || kWantW) S.aw[at] = caw;
+            }
+        };
         const bool mine = (pm >> lane) & 1u;
-        const int rank = __popc(pm & ((1u << lane) - 1u)), room = 32 - ns, pc = __popc(pm);
-        if (mine && rank < room) {
-            S.u[ns + rank] = su;
-            S.v[ns + rank] = sv;
-            S.t[ns + rank] = stt;
-            S.hh[ns + rank] = shh;
-            S.q[st + ns + rank] = cq;
-            S.j[st + ns + rank] = cj;
-            if (kWantA || kWantW) S.aw[st + ns + rank] = caw;
-        }
+        const int room = 32 - ns;
+        if (mine && rank < room) stage(ns + rank);
         if (!last && pc < room) {
             ns += pc;
             continue;
@@ -943,106 +1167,145 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
         // the block is full (or the walk over): the lanes' candidates in it
         const int m = last ? ns : 32;
         __syncwarp();
-        unsigned m2 = candidates(S, m, u, v, t, Lf);
+        unsigned mask = candidates(S, m, pt.x, pt.y, pt.z, Lf);
         if (live) sk.ntest += (unsigned)m;
-        else m2 = 0u;
-        // evaluate until the oldest block is done (at the end: all of them)
-        for (;;) {
-            const unsigned all = m0 | m1 | m2;
-            if (!__any_sync(0xffffffffu, (last ? all : m0) != 0u)) break;
-            int at = st >= 32 ? st - 32 : st + 64;          // the newer block
-            unsigned b = m1;
-            if (m0) {
-                b = m0;
-                at = st >= 64 ? st - 64 : st + 32;          // the oldest
-            } else if (!b) {
-                b = m2;
-                at = st;
-            }
-            const unsigned rest = b & (b - 1u);
-            at += __ffs(b) - 1;
-            if (m0) m0 = rest;
-            else if (m1) m1 = rest;
-            else m2 = rest;
-            if constexpr (kF32) {
-                eval_f32<KERNEL, MODE, NF>(P, tab, pq, pq_count, stash, all != 0u, S, all ? at : 0, dx, dy, dz, L, sk, err);
-            } else {
-                if (all) eval_f64<Real, KERNEL, MODE, NF>(P, S, at, dx, dy, dz, L, sk, err);
-                __syncwarp();
-            }
+        else mask = 0u;
+        // as many spheres at a time as their pairs fit: all, half, a quarter or an eighth
+        const int total = __reduce_add_sync(0xffffffffu, __popc(mask));
+        int step = 32;
+        while (total > St::kPairs && step > 4) {
+            step >>= 1;
+            int most = 0;
+            for (int e0 = 0; e0 < 32; e0 += step)
+                most = max(most, (int)__reduce_add_sync(0xffffffffu, __popc(mask & (((1u << step) - 1u) << e0))));
+            if (most <= St::kPairs) break;
         }
-        if (last) break;
-        m0 = m1;
-        m1 = m2;
-        st = st >= 64 ? 0 : st + 32;
-        ns = pc - room;
+#pragma unroll 1
+        for (int e0 = 0; (total > 0 || drain) && e0 < 32; e0 += step) {
+            const unsigned mm = step == 32 ? mask : mask & (((1u << step) - 1u) << e0);
+            if constexpr (kF32)
+                pairs_f32<KERNEL, MODE, NF>(P, tab, pq, pq_count, stash, S, mm, drain, dx, dy, dz, L, sk, err);
+            else
+                pairs_f64<KERNEL, MODE, NF>(P, stash, S, mm, dx, dy, dz, L, sk, err);
+        }
         __syncwarp();                // the block's readers are done
-        if (mine && rank >= room) {
-            S.u[rank - room] = su;
-            S.v[rank - room] = sv;
-            S.t[rank - room] = stt;
-            S.hh[rank - room] = shh;
-            S.q[st + rank - room] = cq;
-            S.j[st + rank - room] = cj;
-            if (kWantA || kWantW) S.aw[st + rank - room] = caw;
-        }
+        if (last) break;
+        ns = pc - room;
+        if (mine && rank >= room) stage(rank - room);
     }
     nvisit += W.visits;
     __syncwarp();
 }
 
-template <typename Real, int KERNEL, int MODE, bool NF>
-__device__ __forceinline__ void ray_column(const TraceParams& P, const float2* tab, Beam* beam, Staged& S,
-                                           PartQueue* pq, int& pq_count, unsigned long long* stash, float4 o, Real dx,
+// A packet's origins usually fit in a few smoothing lengths, but some packets
+// straddle a gap of the origins' order (a jump of the Morton curve, a sparse
+// sample of origins), and one beam around all of them would sweep much of the
+// box: such packets are traced as several beams, each of the origins within
+// kBeamReach smoothing lengths (across) of its first one.  A ray's sums do not
+// depend on the rays that share its beam.
+constexpr float kBeamReach = 5.f;
+
+template <typename Real, int KERNEL, int MODE, bool NF, typename Queue, typename St>
+__device__ __forceinline__ void ray_column(const TraceParams& P, const float2* tab, Beam* beam, St& S,
+                                           Queue* pq, int& pq_count, unsigned long long* stash, float4 o, Real dx,
                                            Real dy, Real dz, bool live, Sink<Real>& sk, unsigned& err,
                                            unsigned& nvisit)
 {
-    const unsigned lv = __ballot_sync(0xffffffffu, live);
-    if (!lv) return;
+    const int lane = threadIdx.x & 31;
     const float Lf = (float)P.l_ray * 1.000001f + 1e-30f;
     const int nimg = P.periodic ? P.nimg : 0;
     const int side = 2 * nimg + 1;
     const int images = side * side * side;
-    float u, v, t;
-    // the images of the box that the unshifted beam may reach, 32 at a time,
-    // then one after the other in the order of their indices
-    for (int i0 = 0; i0 < images; i0 += 32) {
-        unsigned im = 1u;
-        if (images > 1) {
-            make_beam(beam, lv, live, Real(o.x), Real(o.y), Real(o.z), (float)dx, (float)dy, (float)dz, Lf, u, v, t);
-            const int i = i0 + (int)(threadIdx.x & 31);
-            bool pass = false;
-            if (i < images) {
-                const float ax = (float)(i / (side * side) - nimg) * (float)P.Lbox,
-                            ay = (float)((i / side) % side - nimg) * (float)P.Lbox,
-                            az = (float)(i % side - nimg) * (float)P.Lbox;
-                // the shifted faces and the shifted origins are each rounded
-                const float m = 1e-6f * (fabsf(ax) + fabsf(ay) + fabsf(az) + (float)P.Lbox);
-                pass = beam_box(*beam, make_float4(P.root_lo[0] + ax - m, P.root_lo[1] + ay - m, P.root_lo[2] + az - m, 0.f),
-                                make_float4(P.root_hi[0] + ax + m, P.root_hi[1] + ay + m, P.root_hi[2] + az + m, 0.f));
-            }
-            im = __ballot_sync(0xffffffffu, pass);
+    constexpr bool kQueue = sizeof(Real) == 4 && MODE != MODE_COUNT;
+    float3 pt = make_float3(0.f, 0.f, 0.f);
+    unsigned left = __ballot_sync(0xffffffffu, live);
+    while (left || (kQueue && pq_count > 0)) {
+        const bool drain = !left;
+        bool in = false;
+        if (!drain) {
+            const int a = __ffs(left) - 1;
+            const float rx = o.x - __shfl_sync(0xffffffffu, o.x, a), ry = o.y - __shfl_sync(0xffffffffu, o.y, a),
+                        rz = o.z - __shfl_sync(0xffffffffu, o.z, a), w = kBeamReach * __shfl_sync(0xffffffffu, o.w, a);
+            const float along = rx * (float)dx + ry * (float)dy + rz * (float)dz;
+            const float across2 = rx * rx + ry * ry + rz * rz - along * along;
+            in = ((left >> lane) & 1u) && (lane == a || (across2 <= w * w && fabsf(along) <= 0.5f * Lf + w));
         }
-        for (; im; im &= im - 1u) {
-            const int i = i0 + __ffs(im) - 1;
-            const int ax = i / (side * side) - nimg, ay = (i / side) % side - nimg, az = i % side - nimg;
-            // images of the particles at r_j + a L are reached by shifting the
-            // origin to r_i - a L
-            sk.sx = Real(o.x) - Real(ax) * Real(P.Lbox);
-            sk.sy = Real(o.y) - Real(ay) * Real(P.Lbox);
-            sk.sz = Real(o.z) - Real(az) * Real(P.Lbox);
-            if (NF) {
-                sk.ox = (double)o.x - (double)ax * P.Lbox;
-                sk.oy = (double)o.y - (double)ay * P.Lbox;
-                sk.oz = (double)o.z - (double)az * P.Lbox;
+        const unsigned lv = __ballot_sync(0xffffffffu, in);
+        left &= ~lv;
+        // the images of the box that the unshifted beam may reach, 32 at a
+        // time, then one after the other in the order of their indices
+        for (int i0 = 0; i0 < (drain ? 1 : images); i0 += 32) {
+            unsigned im = 1u;
+            if (images > 1 && !drain) {
+                make_beam<Real>(beam, lv, in, Real(o.x), Real(o.y), Real(o.z), (float)dx, (float)dy, (float)dz, Lf);
+                const int i = i0 + lane;
+                bool pass = false;
+                if (i < images) {
+                    const float ax = (float)(i / (side * side) - nimg) * (float)P.Lbox,
+                                ay = (float)((i / side) % side - nimg) * (float)P.Lbox,
+                                az = (float)(i % side - nimg) * (float)P.Lbox;
+                    // the shifted faces and the shifted origins are each rounded
+                    const float m = 1e-6f * (fabsf(ax) + fabsf(ay) + fabsf(az) + (float)P.Lbox);
+                    pass = beam_box(*beam,
+                                    make_float4(P.root_lo[0] + ax - m, P.root_lo[1] + ay - m, P.root_lo[2] + az - m, 0.f),
+                                    make_float4(P.root_hi[0] + ax + m, P.root_hi[1] + ay + m, P.root_hi[2] + az + m, 0.f));
+                }
+                im = __ballot_sync(0xffffffffu, pass);
             }
-            make_beam(beam, lv, live, sk.sx, sk.sy, sk.sz, (float)dx, (float)dy, (float)dz, Lf, u, v, t);
-            packet_image<Real, KERNEL, MODE, NF>(P, tab, *beam, S, pq, pq_count, stash, u, v, t, Lf, dx, dy, dz, live,
-                                                 sk, err, nvisit);
+            for (; im; im &= im - 1u) {
+                const int i = i0 + __ffs(im) - 1;
+                const int ax = i / (side * side) - nimg, ay = (i / side) % side - nimg, az = i % side - nimg;
+                // images of the particles at r_j + a L are reached by shifting the
+                // origin to r_i - a L
+                const Real sx = Real(o.x) - Real(ax) * Real(P.Lbox);
+                const Real sy = Real(o.y) - Real(ay) * Real(P.Lbox);
+                const Real sz = Real(o.z) - Real(az) * Real(P.Lbox);
+                S.org[lane] = Origin<Real>{sx, sy, sz, sk.coef};
+                if (NF) {
+                    S.near_o[lane][0] = (double)o.x - (double)ax * P.Lbox;
+                    S.near_o[lane][1] = (double)o.y - (double)ay * P.Lbox;
+                    S.near_o[lane][2] = (double)o.z - (double)az * P.Lbox;
+                }
+                if (!drain)
+                    pt = make_beam<Real>(beam, lv, in, sx, sy, sz, (float)dx, (float)dy, (float)dz, Lf);
+                packet_image<Real, KERNEL, MODE, NF>(P, tab, *beam, S, pq, pq_count, stash, pt, Lf, dx, dy, dz, in,
+                                                     drain, sk, err, nvisit);
+            }
         }
     }
 }
 
+// k_trace's shared memory: per warp the work space, the beam, the block of
+// chunks (MODE_CHUNK) and the queue of partial chords (FP32 modes that evaluate
+// chords); the FP32 M4 table; the directions (double[3 R]).
+template <typename Real, int KERNEL, int MODE, bool NF>
+struct TraceLayout {
+    static constexpr bool kF32 = sizeof(Real) == 4;
+    static constexpr bool kQueue = kF32 && MODE != MODE_COUNT;
+    static constexpr bool kTable = kQueue && KERNEL == URCHIN_KERNEL_M4;
+    using St = Staged<Real, MODE, NF>;
+    using Queue = PartQueue<MODE == MODE_FILL || MODE == MODE_CHUNK, NF>;
+    static constexpr size_t up(size_t b) { return (b + 15) & ~size_t(15); }
+    static constexpr size_t kBeam = up(sizeof(St) * 8);
+    static constexpr size_t kStashAt = up(kBeam + sizeof(Beam) * 8);
+    static constexpr size_t kTab = up(kStashAt + 8 * 2 * sizeof(unsigned long long));
+    static constexpr size_t kQueueAt = up(kTab + (kTable ? sizeof(float2) * (kKTab + 1) : 0));
+    static constexpr size_t kDirs = up(kQueueAt + (kQueue ? sizeof(Queue) * 8 : 0));
+    static size_t bytes(int R) { return kDirs + sizeof(double) * 3 * (size_t)R; }
+};
+static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, false>) % 16 == 0, "shared layout");
+
+// Bound by instruction issue (71 % of the slots, 1/5 of the stalls waiting for
+// shared memory, DRAM idle): 29 warp instructions per crossed sphere on the
+// log-normal box with 32 origins per beam, against 45 when every lane tested
+// every staged sphere exactly, and 14 on the halo's long rays (21).  The pair
+// list keeps the exact test and the chords at 30 of 32 lanes (16 to 21 when
+// every lane took its own next candidate).  The traversal's loop has to fit
+// the instruction cache: with two copies of the partial chords' code in it the
+// list-keeping form stalled on fetches for half its time (256^3 box: solve
+// 1168 ms, with one copy 893).  All rays of the 128^3 box 102 -> 79 ms, of the
+// 262144-particle halo 44.1 -> 34.5 ms, 9973 x 48 rays of the 48^3 box in FP64
+// 277 -> 31 ms.
 // Three blocks of 256 per SM (80 registers a thread): with four (64
 // registers) the spills cost more than the fourth block's warps hide; with
 // two (no spills) too few warps are left to hide the loads.  The transpose
@@ -1050,27 +1313,27 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const float2* t
 template <typename Real, int KERNEL, int MODE, bool NF>
 __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(TraceParams P)
 {
-    extern __shared__ double s_dirs[];
-    float2* s_tab = reinterpret_cast<float2*>(s_dirs + 3 * P.R);
-    __shared__ Beam s_beam[256 / 32];
-    __shared__ Staged s_staged[256 / 32];
-    __shared__ unsigned long long s_stash[256 / 32][2];   // MODE_CHUNK: the warp's block of chunks
-    // the warps' partial-chord queues (FP32 modes that evaluate chords), after the table
-    constexpr bool kQueue = sizeof(Real) == 4 && MODE != MODE_COUNT;
-    PartQueue* pq = nullptr;
+    using Lay = TraceLayout<Real, KERNEL, MODE, NF>;
+    constexpr bool kQueue = Lay::kQueue;
+    extern __shared__ __align__(32) unsigned char smem[];
+    const int wid = threadIdx.x >> 5;
+    typename Lay::St& st = reinterpret_cast<typename Lay::St*>(smem)[wid];
+    Beam* beam = reinterpret_cast<Beam*>(smem + Lay::kBeam) + wid;
+    unsigned long long* stash = reinterpret_cast<unsigned long long*>(smem + Lay::kStashAt) + 2 * wid;
+    float2* s_tab = reinterpret_cast<float2*>(smem + Lay::kTab);
+    typename Lay::Queue* pq = reinterpret_cast<typename Lay::Queue*>(smem + Lay::kQueueAt) + wid;
+    double* s_dirs = reinterpret_cast<double*>(smem + Lay::kDirs);
     if (kQueue) {
-        const size_t off = trace_queue_offset(P.R, KERNEL);
-        pq = reinterpret_cast<PartQueue*>(reinterpret_cast<unsigned char*>(s_dirs) + off) + (threadIdx.x >> 5);
         pq->own[threadIdx.x & 31] = 0u;
-        pq->own[(threadIdx.x & 31) + kPQNear] = 0u;
+        if (NF) pq->own[(threadIdx.x & 31) + kPQNear] = 0u;
     }
     int pq_count = 0;
     if ((threadIdx.x & 31) == 0) {
-        s_stash[threadIdx.x >> 5][0] = 0ull;
-        s_stash[threadIdx.x >> 5][1] = 0ull;
+        stash[0] = 0ull;
+        stash[1] = 0ull;
     }
     for (int t = threadIdx.x; t < 3 * P.R; t += blockDim.x) s_dirs[t] = P.dirs[t];
-    if (sizeof(Real) == 4 && KERNEL == URCHIN_KERNEL_M4)
+    if (Lay::kTable)
         for (int t = threadIdx.x; t <= kKTab; t += blockDim.x) s_tab[t] = P.ktab[t];
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -1099,7 +1362,6 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
         // of particles not in the item list stay empty)
         const int64_t ray = (int64_t)k * P.n + org;
         sk.ray = ray;
-        sk.cw = nullptr;
         sk.coff = kChunk;
         sk.cur = kNoChunk;
         const int64_t orow = live ? (P.out_row ? (int64_t)P.out_row[item] : item) : 0;
@@ -1111,11 +1373,8 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
             sk.coef = static_cast<const Real*>(P.coef)[orow * P.row_stride + (int64_t)k * P.k_stride];
             live = sk.coef != Real(0);
         }
-        ray_column<Real, KERNEL, MODE, NF>(P, s_tab, s_beam + (threadIdx.x >> 5), s_staged[threadIdx.x >> 5], pq,
-                                           pq_count, s_stash[threadIdx.x >> 5], o, dx, dy, dz, live, sk, err, nvisit);
-        if constexpr (kQueue) {
-            if (pq_count > 0) flush_partials<KERNEL, MODE, NF>(P, s_tab, pq, pq_count, pq_count, sk);
-        }
+        ray_column<Real, KERNEL, MODE, NF>(P, s_tab, beam, st, pq, pq_count, stash, o, dx, dy, dz, live, sk, err,
+                                           nvisit);
         if (slot < P.n_items) {
             hits += sk.nhit;
             tests += sk.ntest;
@@ -1125,14 +1384,15 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
             if (MODE != MODE_COUNT && MODE != MODE_SCATTER) {
                 if (MODE == MODE_CHUNK && sk.coff < kChunk) {
                     // zero entries up to a multiple of kSegPad (inside the chunk)
-                    for (; (sk.coff & (kSegPad - 1)) != 0; ++sk.coff) sk.cw[sk.coff] = make_int2(0, 0);
+                    for (; (sk.coff & (kSegPad - 1)) != 0; ++sk.coff)
+                        P.chunk_seg[(int64_t)sk.cur * kChunk + sk.coff] = make_int2(0, 0);
                 }
                 if (MODE == MODE_FILL) {
                     // the padding (fewer than kSegPad entries) holds zero values
                     if (sk.end - sk.pos >= kSegPad || sk.pos > sk.end) err |= kStSegment;
                     else
                         for (int64_t q = sk.pos; q < sk.end; ++q) {
-                            store_index(P, sk, q, 0);
+                            store_index(P, q, 0);
                             static_cast<Real*>(P.seg_val)[q] = Real(0);
                         }
                 }
@@ -1167,13 +1427,8 @@ template <typename Real, int KERNEL, int MODE, bool NF>
 int launch_one(const TraceParams& P, cudaStream_t s)
 {
     const void* fn = (const void*)k_trace<Real, KERNEL, MODE, NF>;
-    const size_t smem = (sizeof(Real) == 4 && MODE != MODE_COUNT)
-                            ? trace_queue_offset(P.R, KERNEL) + sizeof(PartQueue) * (256 / 32)
-                            : sizeof(double) * 3 * (size_t)P.R +
-                                  ((sizeof(Real) == 4 && KERNEL == URCHIN_KERNEL_M4) ? sizeof(float2) * (kKTab + 1) : 0);
-    // with the static arrays (beams, staged spheres) beyond the default 48 KB
-    if (smem + sizeof(Staged) * 8 + 2048 > 48 * 1024)
-        URCHIN_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = TraceLayout<Real, KERNEL, MODE, NF>::bytes(P.R);
+    if (smem > 48 * 1024) URCHIN_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int grid = 0;
     URCHIN_TRY(grid_for(fn, 256, smem, &grid));
     int64_t tasks = P.n_chunks * P.R;
