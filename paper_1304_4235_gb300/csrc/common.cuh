@@ -98,10 +98,11 @@ size_t scan64_tmp_bytes(int64_t n);
 int scan_counts_u64(const uint32_t* in, uint64_t* out, int64_t n, void* tmp, uint64_t* total_dev,
                     cudaStream_t s);
 
-// Stable LSD radix sort of (key, value) pairs on the low `bits` bits of key.
-size_t radix_tmp_bytes(int64_t n);
-int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, void* tmp,
-                     cudaStream_t s);
+// Stable LSD radix sort of (key, value) pairs on the low `bits` bits of key,
+// for `segs` arrays of n pairs that lie one after the other (each sorted by
+// itself; segs * n below 2^32).
+size_t radix_tmp_bytes(int64_t n, int64_t segs = 1);
+int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, void* tmp, cudaStream_t s, int64_t segs = 1);
 
 // Stream compaction: out[m] = i for every i with flags[i] != 0, in order;
 // *count_dev = m.  `tmp` needs compact_tmp_bytes(n).
@@ -212,23 +213,22 @@ struct TraceJob {
 int launch_trace(const TraceJob& job, cudaStream_t s);
 
 // Per-direction traversal order of the items: for each direction k the
-// origins sorted by a 63-bit Morton code in the frame (e1, e2, d_k) with the
-// axis along d_k compressed by a factor E, so that 32 consecutive origins
-// form a beam along the ray direction, about E times longer than wide.
-// Rays share their sphere crossings when the beam is narrow against h and
-// short against l_ray, so E = l_ray / (2 h_geo), h_geo the geometric mean of
-// h, clamped to [1, 64].  Measured traversal of all rays: 262144-particle
-// halo (l_ray / 2h_geo ~ 20) E = 16: 43 ms, 4: 51, 1: 58; the 256^3
-// log-normal box (~2) E = 16: 1.06 s, 4: 0.90, 1: 0.87 (30-bit keys, E = 16:
-// 1.34 s).  On the 4096-particle lattice the order costs more than it saves
-// (sort launches, and 9.1 instead of 7.4 sphere tests per hit), so short
-// lists keep item order.  order needs R * n_items int32; tmp needs
-// ray_order_tmp_bytes(n_items).
+// origins sorted by a 32-bit Morton code (11 bits across, 10 along) in the
+// frame (e1, e2, d_k) with the axis along d_k compressed by a factor E, so
+// that 32 consecutive origins form a beam along the ray direction, about E
+// times longer than wide; equal codes keep the items' order (Morton order of
+// the particles).  Rays share their sphere crossings when the beam is narrow
+// against h and short against l_ray, so E = l_ray / (2 h_geo), h_geo the
+// geometric mean of h, clamped to [1, 64].  Several directions are sorted in
+// one set of launches, up to kRayOrderBatch keys.  Short lists keep item
+// order (kRayOrderMinItems).  order needs R * n_items int32; tmp needs
+// ray_order_tmp_bytes(n_items, R).
 constexpr int64_t kRayOrderMinItems = 16384;
+constexpr int64_t kRayOrderBatch = int64_t(1) << 23;
 double ray_order_elongation(const urchin_bvh* bvh, double l_ray);
-size_t ray_order_tmp_bytes(int64_t n_items);
-int ray_order(const urchin_bvh* bvh, const int32_t* items, int64_t n_items, const double* dirs_host, int R,
-              double l_ray, int32_t* order, void* tmp, cudaStream_t s);
+size_t ray_order_tmp_bytes(int64_t n_items, int R);
+int ray_order(const urchin_bvh* bvh, const int32_t* items, int64_t n_items, const double* dirs_dev, int R,
+              double l_ray, int32_t* order, void* tmp, size_t tmp_bytes, cudaStream_t s);
 
 // w_bar[b] += sum_r sg[r] exp(lc[r] - s_b tau[r]) over n_rays rays (tau in
 // the precision's type; the coefficient of ray r is sg[r] exp(lc[r]))

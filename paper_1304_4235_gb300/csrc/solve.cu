@@ -830,7 +830,7 @@ int Solver::order_for(const int32_t* items, int64_t n_items, const int32_t** out
         ord_cap = 2 * (int64_t)P.R * n;
         Layout lay;
         const size_t o_o = lay.take(sizeof(int32_t) * (size_t)ord_cap);
-        const size_t o_t = lay.take(ray_order_tmp_bytes(n));
+        const size_t o_t = lay.take(ray_order_tmp_bytes(n, P.R));
         URCHIN_TRY(ord.alloc(lay.bytes, s));
         ord_base = ord.at<int32_t>(o_o);
         ord_tmp = ord.at<void>(o_t);
@@ -839,7 +839,7 @@ int Solver::order_for(const int32_t* items, int64_t n_items, const int32_t** out
     if (n_items > n || n_items < kRayOrderMinItems) return URCHIN_OK;   // item order
     if (ord_used + need > ord_cap) items_changed();
     int32_t* o = ord_base + ord_used;
-    URCHIN_TRY(ray_order(bvh, items, n_items, P.dirs, P.R, P.l_ray, o, ord_tmp, s));
+    URCHIN_TRY(ray_order(bvh, items, n_items, dirs, P.R, P.l_ray, o, ord_tmp, ray_order_tmp_bytes(n, P.R), s));
     ord_used += need;
     orders.push_back(OrderEntry{items, n_items, o});
     *out = o;

@@ -1588,50 +1588,61 @@ __device__ __forceinline__ uint64_t spread21(uint32_t v)
     return x;
 }
 
-__device__ __forceinline__ uint32_t quant21(float f)
-{
-    return (uint32_t)fminf(fmaxf(f * 2097152.f, 0.f), 2097151.f);
-}
-
-// keys of the items for one direction: the 63-bit Morton code of
-// (u, v, t / E) in the frame (e1, e2, d), coordinates relative to c scaled by
-// inv into [0, 1), as its low 32 bits (lo) and high 31 bits (hi)
+// keys of the items for directions k0 + blockIdx.y: the Morton code of
+// (u, v, t / E) in the frame (e1, e2, d), 11 bits each over the widest of the
+// three extents of the box (the last bit, of t, dropped)
 __global__ void k_ray_keys(const float4* __restrict__ xyzh, const int32_t* __restrict__ items, int64_t n_items,
-                           float3 e1, float3 e2, float3 d, float3 c, float inv, float inv_E, uint32_t* lo,
-                           uint32_t* hi, int32_t* vals)
+                           const double* __restrict__ dirs, int k0, float3 c, float3 ext, float inv_E,
+                           uint32_t* __restrict__ keys, int32_t* __restrict__ vals)
 {
+    const int k = k0 + blockIdx.y;
+    const float dx = (float)dirs[3 * k], dy = (float)dirs[3 * k + 1], dz = (float)dirs[3 * k + 2];
+    // e1 perpendicular to d, from the coordinate axis least aligned with it
+    float ax = 0.f, ay = 0.f, az = 0.f;
+    if (fabsf(dx) <= fabsf(dy) && fabsf(dx) <= fabsf(dz)) ax = 1.f;
+    else if (fabsf(dy) <= fabsf(dz)) ay = 1.f;
+    else az = 1.f;
+    float e1x = dy * az - dz * ay, e1y = dz * ax - dx * az, e1z = dx * ay - dy * ax;
+    const float r = rsqrtf(e1x * e1x + e1y * e1y + e1z * e1z);
+    e1x *= r;
+    e1y *= r;
+    e1z *= r;
+    const float e2x = dy * e1z - dz * e1y, e2y = dz * e1x - dx * e1z, e2z = dx * e1y - dy * e1x;
+    const float su = fabsf(e1x) * ext.x + fabsf(e1y) * ext.y + fabsf(e1z) * ext.z;
+    const float sv = fabsf(e2x) * ext.x + fabsf(e2y) * ext.y + fabsf(e2z) * ext.z;
+    const float st = (fabsf(dx) * ext.x + fabsf(dy) * ext.y + fabsf(dz) * ext.z) * inv_E;
+    const float inv = 2048.f / fmaxf(fmaxf(fmaxf(su, sv), st), 1e-30f);
+    auto q11 = [](float f) { return (uint32_t)fminf(fmaxf(f, 0.f), 2047.f); };
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_items;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float4 p = __ldg(xyzh + (items ? items[i] : (int32_t)i));
         const float rx = p.x - c.x, ry = p.y - c.y, rz = p.z - c.z;
-        const float u = (rx * e1.x + ry * e1.y + rz * e1.z) * inv + 0.5f;
-        const float v = (rx * e2.x + ry * e2.y + rz * e2.z) * inv + 0.5f;
-        const float t = (rx * d.x + ry * d.y + rz * d.z) * inv * inv_E + 0.5f;
-        const uint64_t key = (spread21(quant21(u)) << 2) | (spread21(quant21(v)) << 1) | spread21(quant21(t));
-        lo[i] = (uint32_t)key;
-        hi[i] = (uint32_t)(key >> 32);
-        vals[i] = (int32_t)i;
+        const float u = (rx * e1x + ry * e1y + rz * e1z + 0.5f * su) * inv;
+        const float v = (rx * e2x + ry * e2y + rz * e2z + 0.5f * sv) * inv;
+        const float t = ((rx * dx + ry * dy + rz * dz) * inv_E + 0.5f * st) * inv;
+        const uint64_t code = (spread21(q11(u)) << 2) | (spread21(q11(v)) << 1) | spread21(q11(t));
+        keys[(int64_t)blockIdx.y * n_items + i] = (uint32_t)(code >> 1);
+        vals[(int64_t)blockIdx.y * n_items + i] = (int32_t)i;
     }
 }
 
-// key[p] = hi[vals[p]]: the high words in the order of the first sort
-__global__ void k_gather_hi(const uint32_t* __restrict__ hi, const int32_t* __restrict__ vals, int64_t n,
-                            uint32_t* key)
+size_t order_bytes(int64_t n_items, int64_t g)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
-        key[p] = hi[vals[p]];
+    Layout lay;
+    lay.take(sizeof(uint32_t) * (size_t)(g * n_items));
+    lay.take(radix_tmp_bytes(n_items, g));
+    return lay.bytes;
+}
+
+// directions sorted at a time
+int64_t order_batch(int64_t n_items, int R)
+{
+    return std::max<int64_t>(1, std::min<int64_t>(R, kRayOrderBatch / std::max<int64_t>(n_items, 1)));
 }
 
 }  // namespace
 
-size_t ray_order_tmp_bytes(int64_t n_items)
-{
-    Layout lay;
-    lay.take(sizeof(uint32_t) * (size_t)n_items);
-    lay.take(sizeof(uint32_t) * (size_t)n_items);
-    lay.take(radix_tmp_bytes(n_items));
-    return lay.bytes;
-}
+size_t ray_order_tmp_bytes(int64_t n_items, int R) { return order_bytes(n_items, order_batch(n_items, R)); }
 
 double ray_order_elongation(const urchin_bvh* b, double l_ray)
 {
@@ -1639,50 +1650,32 @@ double ray_order_elongation(const urchin_bvh* b, double l_ray)
     return std::min(64.0, std::max(1.0, l_ray / (2.0 * hg)));
 }
 
-int ray_order(const urchin_bvh* b, const int32_t* items, int64_t n_items, const double* dirs, int R, double l_ray,
-              int32_t* order, void* tmp, cudaStream_t s)
+int ray_order(const urchin_bvh* b, const int32_t* items, int64_t n_items, const double* dirs_dev, int R, double l_ray,
+              int32_t* order, void* tmp, size_t tmp_bytes, cudaStream_t s)
 {
     if (n_items <= 0) return URCHIN_OK;
+    // as many directions at a time as the work space holds (it may be sized for another number of items)
+    int64_t g = order_batch(n_items, R);
+    while (g > 1 && order_bytes(n_items, g) > tmp_bytes) --g;
+    if (order_bytes(n_items, g) > tmp_bytes) return set_error(URCHIN_ERR_ARG, "ray_order: work space too small");
     Layout lay;
-    const size_t o_lo = lay.take(sizeof(uint32_t) * (size_t)n_items);
-    const size_t o_hi = lay.take(sizeof(uint32_t) * (size_t)n_items);
-    const size_t o_t = lay.take(radix_tmp_bytes(n_items));
-    uint32_t* lo = reinterpret_cast<uint32_t*>(static_cast<char*>(tmp) + o_lo);
-    uint32_t* hi = reinterpret_cast<uint32_t*>(static_cast<char*>(tmp) + o_hi);
+    const size_t o_k = lay.take(sizeof(uint32_t) * (size_t)(g * n_items));
+    const size_t o_t = lay.take(radix_tmp_bytes(n_items, g));
+    uint32_t* keys = reinterpret_cast<uint32_t*>(static_cast<char*>(tmp) + o_k);
     void* rt = static_cast<char*>(tmp) + o_t;
     const double E = ray_order_elongation(b, l_ray);
     const float3 c = make_float3(0.5f * (b->root_lo[0] + b->root_hi[0]), 0.5f * (b->root_lo[1] + b->root_hi[1]),
                                  0.5f * (b->root_lo[2] + b->root_hi[2]));
-    const double ex = b->root_hi[0] - b->root_lo[0], ey = b->root_hi[1] - b->root_lo[1],
-                 ez = b->root_hi[2] - b->root_lo[2];
-    const double diam = std::sqrt(ex * ex + ey * ey + ez * ez);
-    const float inv = (float)(1.0 / std::max(diam, 1e-30));
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_items + 255) / 256, 4096));
-    for (int k = 0; k < R; ++k) {
-        const double dx = dirs[3 * k], dy = dirs[3 * k + 1], dz = dirs[3 * k + 2];
-        // e1 perpendicular to d, from the coordinate axis least aligned with it
-        double ax = 0, ay = 0, az = 0;
-        if (std::fabs(dx) <= std::fabs(dy) && std::fabs(dx) <= std::fabs(dz)) ax = 1;
-        else if (std::fabs(dy) <= std::fabs(dz)) ay = 1;
-        else az = 1;
-        double e1x = dy * az - dz * ay, e1y = dz * ax - dx * az, e1z = dx * ay - dy * ax;
-        const double nn = std::sqrt(e1x * e1x + e1y * e1y + e1z * e1z);
-        e1x /= nn;
-        e1y /= nn;
-        e1z /= nn;
-        const double e2x = dy * e1z - dz * e1y, e2y = dz * e1x - dx * e1z, e2z = dx * e1y - dy * e1x;
+    const float3 ext = make_float3(b->root_hi[0] - b->root_lo[0], b->root_hi[1] - b->root_lo[1],
+                                   b->root_hi[2] - b->root_lo[2]);
+    const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_items + 255) / 256, 4096));
+    for (int k = 0; k < R; k += (int)g) {
+        const int m = (int)std::min<int64_t>(g, R - k);
         int32_t* vals = order + (size_t)k * n_items;
-        k_ray_keys<<<grid, 256, 0, s>>>(b->xyzh, items, n_items, make_float3((float)e1x, (float)e1y, (float)e1z),
-                                        make_float3((float)e2x, (float)e2y, (float)e2z),
-                                        make_float3((float)dx, (float)dy, (float)dz), c, inv, (float)(1.0 / E),
-                                        lo, hi, vals);
+        k_ray_keys<<<dim3(gx, (unsigned)m), 256, 0, s>>>(b->xyzh, items, n_items, dirs_dev, k, c, ext, (float)(1.0 / E),
+                                                         keys, vals);
         URCHIN_TRY(launched());
-        // least significant word first; the radix sort is stable, so the
-        // second pass leaves equal high words in low-word order
-        URCHIN_TRY(radix_sort_pairs(lo, vals, n_items, 32, rt, s));
-        k_gather_hi<<<grid, 256, 0, s>>>(hi, vals, n_items, lo);
-        URCHIN_TRY(launched());
-        URCHIN_TRY(radix_sort_pairs(lo, vals, n_items, 31, rt, s));
+        URCHIN_TRY(radix_sort_pairs(keys, vals, n_items, 32, rt, s, m));
     }
     return URCHIN_OK;
 }
@@ -1796,7 +1789,7 @@ int trace_columns_impl(const char* fn, const urchin_bvh* bvh, const double* x, c
     size_t o_items = lay.take(origins ? sizeof(int32_t) * (size_t)n_orig : 0);
     const bool ordered = n_orig >= kRayOrderMinItems;
     size_t o_ord = lay.take(ordered ? sizeof(int32_t) * (size_t)R * (size_t)n_orig : 0);
-    size_t o_otmp = lay.take(ordered ? ray_order_tmp_bytes(n_orig) : 0);
+    size_t o_otmp = lay.take(ordered ? ray_order_tmp_bytes(n_orig, R) : 0);
     Scratch scr;
     URCHIN_TRY(scr.alloc(lay.bytes, s));
     unsigned* ctr = scr.at<unsigned>(o_ctr);
@@ -1829,8 +1822,9 @@ int trace_columns_impl(const char* fn, const urchin_bvh* bvh, const double* x, c
         job.items = nullptr;
         job.out_row = bvh->perm;
     }
-    if (n_orig >= kRayOrderMinItems) {
-        URCHIN_TRY(ray_order(bvh, job.items, n_orig, dirs, R, l_ray, scr.at<int32_t>(o_ord), scr.at<void>(o_otmp), s));
+    if (ordered) {
+        URCHIN_TRY(ray_order(bvh, job.items, n_orig, job.dirs_dev, R, l_ray, scr.at<int32_t>(o_ord),
+                             scr.at<void>(o_otmp), ray_order_tmp_bytes(n_orig, R), s));
         job.order = scr.at<int32_t>(o_ord);
     }
     job.near_far = near_out ? 1 : 0;
@@ -1888,6 +1882,9 @@ extern "C" int urchin_trace_columns_vjp(const urchin_bvh* bvh, const double* dir
     size_t o_dirs = lay.take(sizeof(double) * 3 * (size_t)R);
     size_t o_xm = lay.take(sizeof(double) * (size_t)n);
     size_t o_items = lay.take(origins ? sizeof(int32_t) * (size_t)n_orig : 0);
+    const bool ordered = n_orig >= kRayOrderMinItems;
+    size_t o_ord = lay.take(ordered ? sizeof(int32_t) * (size_t)R * (size_t)n_orig : 0);
+    size_t o_otmp = lay.take(ordered ? ray_order_tmp_bytes(n_orig, R) : 0);
     Scratch scr;
     URCHIN_TRY(scr.alloc(lay.bytes, s));
     unsigned* ctr = scr.at<unsigned>(o_ctr);
@@ -1919,6 +1916,11 @@ extern "C" int urchin_trace_columns_vjp(const urchin_bvh* bvh, const double* dir
     } else {
         job.items = nullptr;
         job.out_row = bvh->perm;
+    }
+    if (ordered) {
+        URCHIN_TRY(ray_order(bvh, job.items, n_orig, job.dirs_dev, R, l_ray, scr.at<int32_t>(o_ord),
+                             scr.at<void>(o_otmp), ray_order_tmp_bytes(n_orig, R), s));
+        job.order = scr.at<int32_t>(o_ord);
     }
     URCHIN_TRY(launch_trace(job, s));
     unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096));

@@ -259,115 +259,182 @@ int scan_counts_u64(const uint32_t* in, uint64_t* out, int64_t n, void* tmp, uin
 }
 
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort, 4-bit digits, 256 threads x 16 items per tile.
+// Stable LSD radix sort, 8-bit digits, of `segs` independent arrays of n pairs
+// that lie one after the other (the ray orders of several directions at once):
+// per digit a histogram of every tile, one scan over [segment][digit][tile]
+// (its values are the pairs' final places, segment offsets included), and a
+// scatter that ranks a tile's pairs with warp matches, puts them in order in
+// shared memory and writes runs of equal digits.  A tile holds kRadixThreads x
+// ITEMS pairs.  4-bit digits with 16 dependent rounds per tile and one segment
+// per launch had spent 33 us per digit whatever n was (262144 keys: 16
+// launches of 64 blocks each for the histogram, the scan and the scatter).
 // ---------------------------------------------------------------------------
 constexpr int kRadixThreads = 256;
-constexpr int kRadixRounds = 16;
-constexpr int kRadixTile = kRadixThreads * kRadixRounds;
-constexpr int kRadixDigits = 16;
+constexpr int kRadixDigits = 256;
+constexpr int kRadixItemsSmall = 4, kRadixItemsLarge = 16;
+// tiles of 4096 pairs once they fill the GPU, of 1024 below (more blocks)
+constexpr int64_t kRadixLarge = int64_t(1) << 21;
 
-__global__ void k_radix_hist(const uint32_t* keys, int64_t n, int shift, uint32_t* hist, int nblocks)
+static int radix_items(int64_t n, int64_t segs) { return n * segs >= kRadixLarge ? kRadixItemsLarge : kRadixItemsSmall; }
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift,
+                                                              uint32_t* __restrict__ hist, int tiles)
 {
     __shared__ uint32_t cnt[kRadixDigits];
-    if (threadIdx.x < kRadixDigits) cnt[threadIdx.x] = 0;
+    cnt[threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    for (int r = 0; r < kRadixRounds; ++r) {
-        int64_t i = base + (int64_t)r * kRadixThreads + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 15u], 1u);
+    const int seg = blockIdx.x / tiles, tile = blockIdx.x - seg * tiles;
+    const uint32_t* k = keys + (int64_t)seg * n;
+    const int64_t base = (int64_t)tile * (kRadixThreads * ITEMS);
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t i = base + r * kRadixThreads + threadIdx.x;
+        if (i < n) atomicAdd(&cnt[(k[i] >> shift) & (kRadixDigits - 1)], 1u);
     }
     __syncthreads();
-    if (threadIdx.x < kRadixDigits) hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
+    hist[((int64_t)seg * kRadixDigits + threadIdx.x) * tiles + tile] = cnt[threadIdx.x];
 }
 
-__global__ void k_radix_scatter(const uint32_t* kin, const int32_t* vin, uint32_t* kout, int32_t* vout,
-                                int64_t n, int shift, const uint32_t* offsets, int nblocks)
+template <int ITEMS>
+__global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(const uint32_t* __restrict__ kin,
+                                                                 const int32_t* __restrict__ vin,
+                                                                 uint32_t* __restrict__ kout,
+                                                                 int32_t* __restrict__ vout, int64_t n, int64_t total,
+                                                                 int shift, const uint32_t* __restrict__ offsets,
+                                                                 int tiles)
 {
     constexpr int W = kRadixThreads / 32;
-    __shared__ uint32_t running[kRadixDigits];
-    __shared__ uint32_t wcnt[W][kRadixDigits + 1];
-    __shared__ uint32_t wpre[W][kRadixDigits + 1];
-    __shared__ uint32_t rtot[kRadixDigits];
+    constexpr int kTile = kRadixThreads * ITEMS;
+    __shared__ uint32_t wcnt[W][kRadixDigits];    // per warp and digit: count, then the warp's first place in the tile
+    __shared__ uint32_t dst[kRadixDigits];        // global place of the tile's first pair of a digit, minus its place in the tile
+    __shared__ uint32_t wsum[W];
+    __shared__ uint32_t skey[kTile];
+    __shared__ int32_t sval[kTile];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x < kRadixDigits)
-        running[threadIdx.x] = offsets[(int64_t)threadIdx.x * nblocks + blockIdx.x];
+    const int seg = blockIdx.x / tiles, tile = blockIdx.x - seg * tiles;
+    const int64_t base = (int64_t)tile * kTile;
+    const int m = (int)(n - base < kTile ? n - base : kTile);      // pairs of this tile
+    for (int t = threadIdx.x; t < W * kRadixDigits; t += kRadixThreads) (&wcnt[0][0])[t] = 0;
+    __syncthreads();
+    // a warp's pairs are consecutive; ranks among the equal digits of the warp, in order
+    uint32_t key[ITEMS], rank[ITEMS];
+    int32_t val[ITEMS];
     const uint32_t lt = (1u << lane) - 1u;
-    int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    for (int r = 0; r < kRadixRounds; ++r) {
-        for (int t = threadIdx.x; t < W * (kRadixDigits + 1); t += blockDim.x)
-            (&wcnt[0][0])[t] = 0;
-        __syncthreads();
-        int64_t i = base + (int64_t)r * kRadixThreads + threadIdx.x;
-        bool valid = i < n;
-        uint32_t key = valid ? kin[i] : 0u;
-        int32_t val = valid ? vin[i] : 0;
-        uint32_t d = valid ? ((key >> shift) & 15u) : (uint32_t)kRadixDigits;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        uint32_t rank = __popc(peers & lt);
-        if (rank == 0) wcnt[wid][d] = __popc(peers);
-        __syncthreads();
-        if (threadIdx.x < kRadixDigits) {
-            uint32_t acc = 0;
-            for (int w = 0; w < W; ++w) {
-                wpre[w][threadIdx.x] = acc;
-                acc += wcnt[w][threadIdx.x];
-            }
-            rtot[threadIdx.x] = acc;
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int i = wid * (32 * ITEMS) + r * 32 + lane;
+        const bool valid = i < m;
+        key[r] = valid ? kin[(int64_t)seg * n + base + i] : 0xffffffffu;
+        val[r] = valid ? vin[(int64_t)seg * n + base + i] : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const bool valid = wid * (32 * ITEMS) + r * 32 + lane < m;
+        const uint32_t d = valid ? (key[r] >> shift) & (kRadixDigits - 1) : (uint32_t)kRadixDigits;
+        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = __popc(peers & lt);
+        uint32_t have = 0;
+        if (valid) have = wcnt[wid][d];
+        __syncwarp();
+        if (valid && before == 0) wcnt[wid][d] = have + __popc(peers);
+        __syncwarp();
+        rank[r] = have + before;
+    }
+    __syncthreads();
+    {
+        // thread = digit: the warps' counts to first places, then over the digits
+        const int d = threadIdx.x;
+        uint32_t acc = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const uint32_t c = wcnt[w][d];
+            wcnt[w][d] = acc;
+            acc += c;
         }
+        uint32_t incl = warp_incl_scan(acc);
+        if (lane == 31) wsum[wid] = incl;
         __syncthreads();
-        if (valid) {
-            uint32_t pos = running[d] + wpre[wid][d] + rank;
-            if (pos < n) {          // always true for a consistent histogram
-                kout[pos] = key;
-                vout[pos] = val;
-            }
+        uint32_t pre = incl - acc;
+        for (int w = 0; w < wid; ++w) pre += wsum[w];
+#pragma unroll
+        for (int w = 0; w < W; ++w) wcnt[w][d] += pre;
+        dst[d] = offsets[((int64_t)seg * kRadixDigits + d) * tiles + tile] - pre;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        if (wid * (32 * ITEMS) + r * 32 + lane >= m) continue;
+        const uint32_t at = wcnt[wid][(key[r] >> shift) & (kRadixDigits - 1)] + rank[r];
+        if (at < (uint32_t)kTile) {              // always true: ranks within a tile
+            skey[at] = key[r];
+            sval[at] = val[r];
         }
-        __syncthreads();
-        if (threadIdx.x < kRadixDigits) running[threadIdx.x] += rtot[threadIdx.x];
-        __syncthreads();
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < m; t += kRadixThreads) {
+        const uint32_t k = skey[t];
+        const uint32_t pos = dst[(k >> shift) & (kRadixDigits - 1)] + (uint32_t)t;
+        if ((int64_t)pos < total) {              // always true for a consistent histogram
+            kout[pos] = k;
+            vout[pos] = sval[t];
+        }
     }
 }
 
-size_t radix_tmp_bytes(int64_t n)
+size_t radix_tmp_bytes(int64_t n, int64_t segs)
 {
-    int64_t nblocks = ceil_div(n, kRadixTile);
+    const int64_t all = n * segs;
+    const int64_t tiles = ceil_div(n, kRadixThreads * radix_items(n, segs));
     size_t b = 0;
-    b += ((size_t)n * 4 + 255) & ~size_t(255);                      // alt keys
-    b += ((size_t)n * 4 + 255) & ~size_t(255);                      // alt vals
-    b += ((size_t)nblocks * kRadixDigits * 4 + 255) & ~size_t(255); // histogram
-    b += scan_tmp_bytes(nblocks * kRadixDigits);
+    b += ((size_t)all * 4 + 255) & ~size_t(255);                                  // alt keys
+    b += ((size_t)all * 4 + 255) & ~size_t(255);                                  // alt vals
+    b += ((size_t)(segs * tiles) * kRadixDigits * 4 + 255) & ~size_t(255);        // histogram
+    b += scan_tmp_bytes(segs * tiles * kRadixDigits);
     return b;
 }
 
-int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, void* tmp, cudaStream_t s)
+template <int ITEMS>
+static int radix_pass(const uint32_t* ka, const int32_t* va, uint32_t* kb, int32_t* vb, int64_t n, int64_t segs,
+                      int shift, uint32_t* hist, void* stmp, cudaStream_t s)
 {
-    if (n <= 1) return URCHIN_OK;
-    int64_t nblocks = ceil_div(n, kRadixTile);
+    const int64_t tiles = ceil_div(n, kRadixThreads * ITEMS);
+    const unsigned grid = (unsigned)(segs * tiles);
+    k_radix_hist<ITEMS><<<grid, kRadixThreads, 0, s>>>(ka, n, shift, hist, (int)tiles);
+    URCHIN_TRY(launched());
+    URCHIN_TRY(scan_exclusive_u32(hist, hist, segs * tiles * kRadixDigits, stmp, nullptr, s));
+    k_radix_scatter<ITEMS><<<grid, kRadixThreads, 0, s>>>(ka, va, kb, vb, n, n * segs, shift, hist, (int)tiles);
+    return launched();
+}
+
+int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, void* tmp, cudaStream_t s, int64_t segs)
+{
+    if (n <= 1 || segs < 1) return URCHIN_OK;
+    const int64_t all = n * segs;
+    const int items = radix_items(n, segs);
+    const int64_t tiles = ceil_div(n, kRadixThreads * items);
     char* p = static_cast<char*>(tmp);
     uint32_t* k2 = reinterpret_cast<uint32_t*>(p);
-    p += ((size_t)n * 4 + 255) & ~size_t(255);
+    p += ((size_t)all * 4 + 255) & ~size_t(255);
     int32_t* v2 = reinterpret_cast<int32_t*>(p);
-    p += ((size_t)n * 4 + 255) & ~size_t(255);
+    p += ((size_t)all * 4 + 255) & ~size_t(255);
     uint32_t* hist = reinterpret_cast<uint32_t*>(p);
-    p += ((size_t)nblocks * kRadixDigits * 4 + 255) & ~size_t(255);
+    p += ((size_t)(segs * tiles) * kRadixDigits * 4 + 255) & ~size_t(255);
     void* stmp = p;
-    int passes = (bits + 3) / 4;
+    const int passes = (bits + 7) / 8;
     uint32_t *ka = keys, *kb = k2;
     int32_t *va = vals, *vb = v2;
     for (int pass = 0; pass < passes; ++pass) {
-        int shift = 4 * pass;
-        k_radix_hist<<<(unsigned)nblocks, kRadixThreads, 0, s>>>(ka, n, shift, hist, (int)nblocks);
-        URCHIN_TRY(launched());
-        URCHIN_TRY(scan_exclusive_u32(hist, hist, nblocks * kRadixDigits, stmp, nullptr, s));
-        k_radix_scatter<<<(unsigned)nblocks, kRadixThreads, 0, s>>>(ka, va, kb, vb, n, shift, hist,
-                                                                    (int)nblocks);
-        URCHIN_TRY(launched());
+        if (items == kRadixItemsLarge)
+            URCHIN_TRY(radix_pass<kRadixItemsLarge>(ka, va, kb, vb, n, segs, 8 * pass, hist, stmp, s));
+        else
+            URCHIN_TRY(radix_pass<kRadixItemsSmall>(ka, va, kb, vb, n, segs, 8 * pass, hist, stmp, s));
         uint32_t* tk = ka; ka = kb; kb = tk;
         int32_t* tv = va; va = vb; vb = tv;
     }
     if (ka != keys) {
-        URCHIN_TRY_CUDA(cudaMemcpyAsync(keys, ka, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
-        URCHIN_TRY_CUDA(cudaMemcpyAsync(vals, va, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
+        URCHIN_TRY_CUDA(cudaMemcpyAsync(keys, ka, (size_t)all * 4, cudaMemcpyDeviceToDevice, s));
+        URCHIN_TRY_CUDA(cudaMemcpyAsync(vals, va, (size_t)all * 4, cudaMemcpyDeviceToDevice, s));
     }
     return URCHIN_OK;
 }
