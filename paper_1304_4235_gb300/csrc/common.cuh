@@ -221,9 +221,15 @@ int launch_trace(const TraceJob& job, cudaStream_t s);
 // against h and short against l_ray, so E = l_ray / (2 h_geo), h_geo the
 // geometric mean of h, clamped to [1, 64].  Several directions are sorted in
 // one set of launches, up to kRayOrderBatch keys.  Short lists keep item
-// order (kRayOrderMinItems).  order needs R * n_items int32; tmp needs
+// order (kRayOrderMinItems, kRayOrderMinSample).  order needs R * n_items int32; tmp needs
 // ray_order_tmp_bytes(n_items, R).
 constexpr int64_t kRayOrderMinItems = 16384;
+// A caller's list of origins is a sample of the particles (or in any order),
+// so its neighbours lie apart and the order pays much earlier: 3000 of 64^3
+// box particles 2.2 -> 1.6 ms, 12000 4.1 -> 2.6, 5000 of a 200000-particle
+// halo 11.3 -> 3.0 ms; all particles of a 20^3 / 25^3 box (Morton order as it
+// is) 0.65 -> 0.84 / 0.88 -> 1.29 ms.
+constexpr int64_t kRayOrderMinSample = 1024;
 constexpr int64_t kRayOrderBatch = int64_t(1) << 23;
 double ray_order_elongation(const urchin_bvh* bvh, double l_ray);
 size_t ray_order_tmp_bytes(int64_t n_items, int R);

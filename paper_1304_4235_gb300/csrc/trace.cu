@@ -54,7 +54,8 @@ struct TraceParams {
     int nimg;
     float root_lo[3], root_hi[3];
     double gt_t2, gt_t, gt_pref;
-    int64_t n_chunks;
+    int64_t n_chunks;             // packets per direction
+    int packet;                   // origins per packet (32, or fewer where 32 leave warps idle)
     // stored-segment modes
     uint32_t* counts;             // MODE_COUNT: hits per ray, index k * n_items + item
     const uint64_t* row_ptr;      // MODE_FILL: first segment of each ray (same index), size + 1
@@ -1347,11 +1348,12 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
         if ((unsigned long long)task >= total) break;
         const int k = (int)(task / P.n_chunks);
         const int64_t chunk = (int64_t)(task % P.n_chunks);
-        const int64_t slot = chunk * 32 + lane;
+        const int64_t slot = chunk * P.packet + lane;
         // every lane takes part in the packet's votes; lanes past the end of
         // the origin list (and, in the transpose, rays with a zero
         // coefficient) are carried along without a segment
-        bool live = slot < P.n_items;
+        bool live = lane < P.packet && slot < P.n_items;
+        const bool mine = live;
         const int64_t item = !live ? 0 : (P.order ? (int64_t)P.order[(int64_t)k * P.n_items + slot] : slot);
         const int32_t org = live ? (P.items ? P.items[item] : (int32_t)item) : 0;
         float4 o = __ldg(P.xyzh + org);
@@ -1375,7 +1377,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
         }
         ray_column<Real, KERNEL, MODE, NF>(P, s_tab, beam, st, pq, pq_count, stash, o, dx, dy, dz, live, sk, err,
                                            nvisit);
-        if (slot < P.n_items) {
+        if (mine) {
             hits += sk.nhit;
             tests += sk.ntest;
             visits += nvisit;
@@ -1541,7 +1543,21 @@ int launch_trace(const TraceJob& job, cudaStream_t s)
     P.gt_t2 = g.t2;
     P.gt_t = g.t;
     P.gt_pref = g.pref;
-    P.n_chunks = (job.n_items + 31) / 32;
+    {
+        // 32 origins per packet share most spheres; few rays are spread over
+        // more warps instead, down to 8 per packet, while 3/4 of the 24 warps an
+        // SM holds (FP64, whose evaluation outweighs the walk: all) would be
+        // idle.  9^3 lattice, 12 rays: 32, 16, 8, 4 per packet 0.49, 0.34, 0.27,
+        // 0.26 ms; 16^3: 0.43, 0.34, 0.38, 0.47 ms; FP64 9^3: 3.3, 1.9, 1.24,
+        // 1.37 ms.
+        int dev = 0, sms = 0;
+        URCHIN_TRY_CUDA(cudaGetDevice(&dev));
+        URCHIN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const int64_t enough = (int64_t)sms * (job.precision == URCHIN_F64 ? 24 : 18);
+        P.packet = 32;
+        while (P.packet > 8 && (job.n_items + P.packet - 1) / P.packet * job.R < enough) P.packet >>= 1;
+    }
+    P.n_chunks = (job.n_items + P.packet - 1) / P.packet;
     if ((unsigned long long)P.n_chunks * (unsigned long long)job.R >= 0xffffffffull)
         return set_error(URCHIN_ERR_ARG, "trace: too many rays for one launch");
     URCHIN_TRY_CUDA(cudaMemsetAsync(job.counter, 0, sizeof(unsigned), s));
@@ -1787,7 +1803,7 @@ int trace_columns_impl(const char* fn, const urchin_bvh* bvh, const double* x, c
     size_t o_dirs = lay.take(sizeof(double) * 3 * (size_t)R);
     size_t o_w = lay.take((f64 ? sizeof(double) : sizeof(float)) * (size_t)n);
     size_t o_items = lay.take(origins ? sizeof(int32_t) * (size_t)n_orig : 0);
-    const bool ordered = n_orig >= kRayOrderMinItems;
+    const bool ordered = n_orig >= (origins ? kRayOrderMinSample : kRayOrderMinItems);
     size_t o_ord = lay.take(ordered ? sizeof(int32_t) * (size_t)R * (size_t)n_orig : 0);
     size_t o_otmp = lay.take(ordered ? ray_order_tmp_bytes(n_orig, R) : 0);
     Scratch scr;
@@ -1882,7 +1898,7 @@ extern "C" int urchin_trace_columns_vjp(const urchin_bvh* bvh, const double* dir
     size_t o_dirs = lay.take(sizeof(double) * 3 * (size_t)R);
     size_t o_xm = lay.take(sizeof(double) * (size_t)n);
     size_t o_items = lay.take(origins ? sizeof(int32_t) * (size_t)n_orig : 0);
-    const bool ordered = n_orig >= kRayOrderMinItems;
+    const bool ordered = n_orig >= (origins ? kRayOrderMinSample : kRayOrderMinItems);
     size_t o_ord = lay.take(ordered ? sizeof(int32_t) * (size_t)R * (size_t)n_orig : 0);
     size_t o_otmp = lay.take(ordered ? ray_order_tmp_bytes(n_orig, R) : 0);
     Scratch scr;
