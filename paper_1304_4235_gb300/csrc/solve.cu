@@ -170,42 +170,28 @@ __device__ __forceinline__ void sweep_counters(const SweepArgs& A, double my_max
     }
 }
 
-// The plain sweep without tangent, one thread per particle: its R rays are
-// folded in turn (Eq. gamma_shld, fold_ray) with a running log-sum-exp over
-// the rays, then every lane takes its particle's FP64 update at once (the
-// ray-parallel layout of k_sweep leaves all but one warp of the block idle
-// during the FP64 part).
+// The plain sweep without tangent: fold_rows over the particles, each
+// particle's FP64 update (Eq. xroots) by one thread.
 template <typename Real>
-__global__ void __launch_bounds__(kSweepThreads) k_sweep_pp(SweepArgs A)
+__global__ void __launch_bounds__(kFoldThreads) k_sweep_pp(SweepArgs A, FoldSplit sp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr bool kF32 = sizeof(Real) == 4;
-    // FP32: the packed coefficients {e2, e2t, wn, 0} of fold_ray_q4; FP64:
-    // e2 and wn
-    float4* q4 = kF32 ? reinterpret_cast<float4*>(smem_raw) : nullptr;
-    Real* e2 = kF32 ? nullptr : reinterpret_cast<Real*>(smem_raw);
-    Real* wn = kF32 ? nullptr : e2 + A.F;
+    FoldTable<Real> T(smem_raw, A.F);
+    double* lk = reinterpret_cast<double*>(smem_raw + FoldTable<Real>::kBytes * (size_t)((A.F + 1) & ~1));
     __shared__ double sh[2];
-    fold_prepare<Real>(A.s, A.w, A.F, e2, nullptr, wn, nullptr, sh, q4);
+    T.prepare(A.s, A.w, A.F, sh);
     const double gthin = sh[0];
-    const double smin = sh[1];
     const Real* tau = static_cast<const Real*>(A.tau);
     double my_max = 0.0;
     unsigned long long my_above = 0, my_switch = 0;
     unsigned err = 0;
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < A.n_items;
-         row += (int64_t)gridDim.x * blockDim.x) {
-        RayMean<Real> lse;
-        for (int k = 0; k < A.R; ++k) {
-            const Real t = tau[row + (int64_t)k * A.k_stride];
-            Real S, S2;
-            if constexpr (kF32) S = fold_ray_q4(t, q4, A.F);
-            else fold_ray<false>(t, e2, nullptr, wn, nullptr, A.F, S, S2);
-            lse.add(ray_lnrate(smin, t, S));
-        }
-        double xn, G, alpha;
-        particle_update(A, row, lse.mean(A.R), gthin, &xn, &G, &alpha, my_max, my_above, my_switch, err);
-    }
+    fold_rows<Real>(
+        sp, A.n_items, A.R, A.F, T, gthin, sh[1], lk,
+        [&](int64_t row, int k) { return tau[row + (int64_t)k * A.k_stride]; },
+        [&](int64_t row, double lmean) {
+            double xn, G, alpha;
+            particle_update(A, row, lmean, gthin, &xn, &G, &alpha, my_max, my_above, my_switch, err);
+        });
     sweep_counters(A, my_max, my_above, my_switch, err);
 }
 
@@ -619,20 +605,23 @@ int launch_sweep(const SweepArgs& A, cudaStream_t s)
 {
     if (A.n_items <= 0) return URCHIN_OK;
     const size_t rsz = A.precision == URCHIN_F64 ? sizeof(double) : sizeof(float);
-    // plain sweeps without tangent: one thread per particle (0.152 ms against
-    // 0.184 ms per sweep of the 262144-particle halo for the ray-parallel layout)
+    // plain sweeps without tangent
     if (!A.he && !A.near_far && !A.want_tangent) {
-        // e2 and wn (FP64), or the packed {e2, e2t, wn, 0} (FP32)
-        const size_t sm = (A.precision == URCHIN_F64 ? 2 : 4) * (size_t)A.F * rsz;
-        const void* fp = A.precision == URCHIN_F64 ? (const void*)k_sweep_pp<double> : (const void*)k_sweep_pp<float>;
+        int dev = 0, sms = 0;
+        URCHIN_TRY_CUDA(cudaGetDevice(&dev));
+        URCHIN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const bool d = A.precision == URCHIN_F64;
+        FoldSplit sp = fold_split(A.n_items, A.R, sms, d);
+        const size_t sm = (d ? FoldTable<double>::kBytes : FoldTable<float>::kBytes) * (size_t)((A.F + 1) & ~1) + sp.lk_bytes;
+        const void* fp = d ? (const void*)k_sweep_pp<double> : (const void*)k_sweep_pp<float>;
         if (sm > 48 * 1024)
             URCHIN_TRY_CUDA(cudaFuncSetAttribute(fp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         int g = 0;
-        URCHIN_TRY(grid_for(fp, kSweepThreads, sm, &g));
-        const int64_t need = (A.n_items + kSweepThreads - 1) / kSweepThreads;
+        URCHIN_TRY(grid_for(fp, kFoldThreads, sm, &g));
+        const int64_t need = (A.n_items + sp.rows - 1) / sp.rows;
         if (need < g) g = (int)std::max<int64_t>(need, 1);
-        void* args[] = {const_cast<SweepArgs*>(&A)};
-        URCHIN_TRY_CUDA(cudaLaunchKernel(fp, dim3(g), dim3(kSweepThreads), args, sm, s));
+        void* args[] = {const_cast<SweepArgs*>(&A), &sp};
+        URCHIN_TRY_CUDA(cudaLaunchKernel(fp, dim3(g), dim3(kFoldThreads), args, sm, s));
         return launched();
     }
     const bool f64 = A.precision == URCHIN_F64;

@@ -18,64 +18,41 @@ namespace urchin {
 
 namespace {
 
-constexpr int kGammaThreads = 256;
-
-// Threads (local, k) fold ray k of row `local` (fold_ray: the exponent of
-// every bin formed without rounding error); the per-row log-sum-exp runs with
-// one thread per row packed into the first lanes.
 template <typename Real>
-__global__ void __launch_bounds__(kGammaThreads) k_gamma(GammaJob J)
+__global__ void __launch_bounds__(kFoldThreads) k_gamma(GammaJob J, FoldSplit sp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr bool kF32 = sizeof(Real) == 4;
-    double* lk = reinterpret_cast<double*>(smem_raw);
-    Real* e2 = reinterpret_cast<Real*>(lk + kGammaThreads);
-    Real* wn = e2 + J.F;
-    Real* e2t = kF32 ? wn + J.F : nullptr;
+    FoldTable<Real> T(smem_raw, J.F);
+    double* lk = reinterpret_cast<double*>(smem_raw + FoldTable<Real>::kBytes * (size_t)((J.F + 1) & ~1));
     __shared__ double sh[2];
-    fold_prepare<Real>(J.s, J.w, J.F, e2, e2t, wn, nullptr, sh);
-    const int rows_per_block = kGammaThreads / J.R;
-    const int local = threadIdx.x / J.R;
-    const int k = threadIdx.x % J.R;
+    T.prepare(J.s, J.w, J.F, sh);
     const double gthin = sh[0];
-    const double smin = sh[1];
-    for (int64_t row0 = (int64_t)blockIdx.x * rows_per_block; row0 < J.n_rows;
-         row0 += (int64_t)gridDim.x * rows_per_block) {
-        const int64_t row = row0 + local;
-        if (local < rows_per_block && row < J.n_rows) {
-            const Real tau = static_cast<const Real*>(J.tau)[row * J.row_stride + (int64_t)k * J.k_stride];
-            Real S, S2;
-            fold_ray<false>(tau, e2, e2t, wn, nullptr, J.F, S, S2);
-            lk[local * J.R + k] = ray_lnrate(smin, tau, S);
-        }
-        __syncthreads();
-        const int p = threadIdx.x;
-        const int64_t prow = row0 + p;
-        if (p < rows_per_block && prow < J.n_rows) {
-            RayMean<Real> lse;
-            for (int r = 0; r < J.R; ++r) lse.add(lk[p * J.R + r]);
-            const double lmean = lse.mean(J.R);     // ln(Gamma / Gamma_thin)
-            J.gamma_out[prow] = gthin * exp(lmean);
-            if (J.tau_eff_out) J.tau_eff_out[prow] = (float)(-lmean);
-        }
-        __syncthreads();
-    }
+    const Real* tau = static_cast<const Real*>(J.tau);
+    fold_rows<Real>(
+        sp, J.n_rows, J.R, J.F, T, gthin, sh[1], lk,
+        [&](int64_t row, int k) { return tau[row * J.row_stride + (int64_t)k * J.k_stride]; },
+        [&](int64_t row, double lmean) {
+            J.gamma_out[row] = gthin * exp(lmean);
+            if (J.tau_eff_out) J.tau_eff_out[row] = (float)(-lmean);
+        });
 }
 
 template <typename Real>
 int launch_gamma_t(const GammaJob& J, cudaStream_t s)
 {
-    // per-ray log rates (double), then e2, wn and (FP32) the tail e2t
-    const size_t smem = sizeof(double) * kGammaThreads + (sizeof(Real) == 4 ? 3 : 2) * (size_t)J.F * sizeof(Real);
+    int dev = 0, sms = 0;
+    URCHIN_TRY_CUDA(cudaGetDevice(&dev));
+    URCHIN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const FoldSplit sp = fold_split(J.n_rows, J.R, sms, sizeof(Real) == 8);
+    const size_t smem = FoldTable<Real>::kBytes * (size_t)((J.F + 1) & ~1) + sp.lk_bytes;
     auto fn = k_gamma<Real>;
     if (smem > 48 * 1024)
         URCHIN_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int rows_per_block = kGammaThreads / J.R;
-    int64_t need = (J.n_rows + rows_per_block - 1) / rows_per_block;
+    const int64_t need = (J.n_rows + sp.rows - 1) / sp.rows;
     int grid = 0;
-    URCHIN_TRY(grid_for((const void*)fn, kGammaThreads, smem, &grid));
+    URCHIN_TRY(grid_for((const void*)fn, kFoldThreads, smem, &grid));
     if (need < grid) grid = (int)std::max<int64_t>(need, 1);
-    fn<<<grid, kGammaThreads, smem, s>>>(J);
+    fn<<<grid, kFoldThreads, smem, s>>>(J, sp);
     URCHIN_TRY(launched());
     return URCHIN_OK;
 }

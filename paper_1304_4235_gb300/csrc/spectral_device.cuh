@@ -2,7 +2,11 @@
 // standalone equilibrium kernel and the solver's fused sweep kernels.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
+
 #include "common.cuh"
+
 
 namespace urchin {
 
@@ -31,11 +35,12 @@ __device__ __forceinline__ double log_p(double x) { return log(x); }
 // Block-wide preparation in shared memory (every thread of the block calls
 // it; at most 1024 threads): sh[0] = Gamma_thin = sum_j w_j, sh[1] = s_min,
 // e2 and wn as above, e2t the FP32 tail (NULL in FP64), sj = s_j (or NULL).
-// With q4 (FP32), the same e2, e2t and wn are written packed, q4[j] =
-// {e2, e2t, wn, 0}, for fold_ray_q4, and e2, e2t and wn are not written.
+// With a2 and z2 (FP32), the same e2, e2t and wn are written for fold_pair,
+// a2[j] = {-e2, -e2, e2t, e2t} and z2[j] = {wn, wn}, and e2, e2t and wn are not
+// written.
 template <typename Real>
 __device__ void fold_prepare(const double* s, const double* w, int F, Real* e2, Real* e2t, Real* wn, Real* sj,
-                             double* sh, float4* q4 = nullptr)
+                             double* sh, float4* a2 = nullptr, float2* z2 = nullptr)
 {
     __shared__ double red[32][2];
     double tot = 0.0, smin = 1e300;
@@ -65,9 +70,10 @@ __device__ void fold_prepare(const double* s, const double* w, int F, Real* e2, 
     const double g = sh[0], m = sh[1];
     for (int j = threadIdx.x; j < F; j += blockDim.x) {
         const double c = (s[j] - m) * 1.4426950408889634;
-        if (q4) {
-            const float h = (float)c;
-            q4[j] = make_float4(h, (float)(c - (double)h), (float)(w[j] / g), 0.f);
+        if (a2) {
+            const float h = (float)c, t = (float)(c - (double)h), q = (float)(w[j] / g);
+            a2[j] = make_float4(-h, -h, t, t);
+            z2[j] = make_float2(q, q);
         } else {
             e2[j] = (Real)c;
             if (e2t) e2t[j] = (Real)(c - (double)(Real)c);
@@ -107,27 +113,6 @@ __device__ __forceinline__ void fold_ray(float tau, const float* e2, const float
     }
     S_out = S;
     S2_out = S2;
-}
-
-// fold_ray<false> in FP32 with each bin's three coefficients read as one
-// 16-byte word, q = {e2, e2t, wn, 0} (the same arithmetic in the same order,
-// so the same S bit for bit; one shared-memory load per bin instead of three).
-__device__ __forceinline__ float fold_ray_q4(float tau, const float4* q4, int F)
-{
-    tau = tau < 1e30f ? tau : (tau == tau ? 1e30f : tau);
-    float S = 0.f, c = 0.f;
-    for (int j = 0; j < F; ++j) {
-        const float4 q = q4[j];
-        const float p = q.x * tau;
-        const float err = fmaf(q.y, tau, fmaf(q.x, tau, -p));
-        const float v0 = q.z * exp2f(-p);
-        const float v = fmaf(-v0, err * 0.6931471805599453f, v0);
-        const float yy = v - c;
-        const float t = S + yy;
-        c = (t - S) - yy;
-        S = t;
-    }
-    return S;
 }
 
 template <bool kTan>
@@ -239,6 +224,154 @@ struct RayMean {
     }
     __device__ __forceinline__ double mean(int R) const { return m + log_split(acc / (Real)R); }
 };
+
+// ---- a row's rays folded by one or several threads ------------------------------
+// Rows (particles, origins) of R rays each: a group of G threads folds a row,
+// `per` rays a thread (two at a time), and one thread combines them.  One
+// thread per row where the rows fill the GPU; the fewer the rows, the more
+// threads share one (fold_split), so that a few thousand rows still use every
+// SM.  The rays are combined in their order either way, so the result does
+// not depend on G.  Bound by the FP32 pipe and issue (FP64: its pipe): packed
+// operations take 10 issue slots per ray and bin instead of 15.  12 rays, 100
+// bins, FP32 / ms: 400003 rows with the equilibrium 0.58 -> 0.50, a sweep of
+// 65536 particles 0.067 -> 0.055; FP64, a sweep of 4096 particles and 50 bins
+// 0.93 -> 0.10 (16 blocks before).
+struct FoldSplit {
+    int G;                        // threads per row
+    int per;                      // rays per thread
+    int rows;                     // rows per block of kFoldThreads
+    size_t lk_bytes;              // shared memory for the log rates (G > 1)
+};
+constexpr int kFoldThreads = 256;
+
+// Threads wanted per SM: 768 (FP64 1536).  ms with 256 / 768 / 1536 / 3072:
+// 50003 rows of 12 rays and 100 bins 0.130 / 0.113 / 0.119 / 0.148, solve of a
+// 65536-particle halo 195.3 / 192.9 / 194.7 / 203.6; FP64, 60003 rows 3.84 /
+// 3.82 / 3.26 / 3.25.
+inline FoldSplit fold_split(int64_t n_rows, int R, int sms, bool f64)
+{
+    FoldSplit f;
+    const int64_t want = (int64_t)sms * (f64 ? 1536 : 768);
+    int64_t g = std::min<int64_t>(R, (want + n_rows - 1) / std::max<int64_t>(n_rows, 1));
+    // the log rates of a block's rows within 24 KB
+    if (g > 1) g = std::min<int64_t>(R, std::max<int64_t>(g, (R + 11) / 12));
+    f.per = (int)(R / g);
+    if (g > 1 && f.per > 1) f.per &= ~1;           // rays are folded two at a time
+    f.G = (R + f.per - 1) / f.per;
+    f.rows = kFoldThreads / f.G;
+    f.lk_bytes = f.G > 1 ? sizeof(double) * (size_t)R * f.rows : 0;
+    return f;
+}
+
+// The spectrum in shared memory: FP32 a2 and z2, FP64 e2 and wn (fold_prepare).
+template <typename Real> struct FoldTable;
+template <> struct FoldTable<float> {
+    float4* a2;
+    float2* z2;
+    static constexpr size_t kBytes = sizeof(float4) + sizeof(float2);   // per bin
+    __device__ __forceinline__ FoldTable(unsigned char* smem, int F)
+        : a2(reinterpret_cast<float4*>(smem)), z2(reinterpret_cast<float2*>(a2 + F)) {}
+    __device__ __forceinline__ void prepare(const double* s, const double* w, int F, double* sh)
+    {
+        fold_prepare<float>(s, w, F, nullptr, nullptr, nullptr, nullptr, sh, a2, z2);
+    }
+};
+template <> struct FoldTable<double> {
+    double* e2;
+    double* wn;
+    static constexpr size_t kBytes = 2 * sizeof(double);
+    __device__ __forceinline__ FoldTable(unsigned char* smem, int F)
+        : e2(reinterpret_cast<double*>(smem)), wn(e2 + F) {}
+    __device__ __forceinline__ void prepare(const double* s, const double* w, int F, double* sh)
+    {
+        fold_prepare<double>(s, w, F, e2, nullptr, wn, nullptr, sh);
+    }
+};
+
+// S of two rays: the arithmetic of fold_ray<false> in its order (the same bits),
+// both rays in packed FP32 operations, one read of a bin's coefficients for the
+// two.  Every lane of the warp calls it.  With skip (finite weights), leading
+// bins whose exponentials underflow to zero for every ray of the warp (p >= 152:
+// 2^-p below half the smallest denormal) are passed over: they leave the sum
+// and its compensation at zero.
+__device__ __forceinline__ void fold_pair(const FoldTable<float>& T, int F, bool skip, bool, float t0, float t1,
+                                          float& S0, float& S1)
+{
+    t0 = t0 < 1e30f ? t0 : (t0 == t0 ? 1e30f : t0);
+    t1 = t1 < 1e30f ? t1 : (t1 == t1 ? 1e30f : t1);
+    const float2 t = make_float2(t0, t1), nt = make_float2(-t0, -t1);
+    const float2 mln2 = make_float2(-0.6931471805599453f, -0.6931471805599453f), m1 = make_float2(-1.f, -1.f);
+    float2 S = make_float2(0.f, 0.f), nc = make_float2(0.f, 0.f);      // the sum, minus its compensation
+    int j = 0;
+    if (skip) {
+        const float tm = fminf(t0, t1);
+        const bool nan = t0 != t0 || t1 != t1;
+        while (j < F && __all_sync(0xffffffffu, !nan && T.a2[j].x * tm <= -152.f)) ++j;
+    }
+    for (; j < F; ++j) {
+        const float4 q = T.a2[j];
+        const float2 a = make_float2(q.x, q.y), b = make_float2(q.z, q.w), z = T.z2[j];
+        const float2 np = __fmul2_rn(a, t);                                   // -p
+        const float2 err = __ffma2_rn(b, t, __ffma2_rn(a, nt, np));
+        const float2 v0 = __fmul2_rn(z, make_float2(exp2f(np.x), exp2f(np.y)));
+        const float2 v = __ffma2_rn(v0, __fmul2_rn(err, mln2), v0);
+        const float2 y = __fadd2_rn(v, nc);
+        const float2 u = __fadd2_rn(S, y);
+        nc = __ffma2_rn(__ffma2_rn(S, m1, u), m1, y);                         // y - (u - S)
+        S = u;
+    }
+    S0 = S.x;
+    S1 = S.y;
+}
+
+__device__ __forceinline__ void fold_pair(const FoldTable<double>& T, int F, bool, bool two, double t0, double t1,
+                                          double& S0, double& S1)
+{
+    double S2;
+    fold_ray<false>(t0, T.e2, nullptr, T.wn, nullptr, F, S0, S2);
+    if (two) fold_ray<false>(t1, T.e2, nullptr, T.wn, nullptr, F, S1, S2);
+}
+
+// Every row of [0, n_rows): its rays' columns tau(row, k), and fin(row,
+// ln(Gamma / Gamma_thin)) once per row.  Called by all threads of the block
+// (kFoldThreads); lk: sp.lk_bytes of shared memory.
+template <typename Real, typename Tau, typename Fin>
+__device__ __forceinline__ void fold_rows(const FoldSplit sp, int64_t n_rows, int R, int F, const FoldTable<Real>& T,
+                                          double gthin, double smin, double* lk, Tau tau, Fin fin)
+{
+    const int g = threadIdx.x / sp.rows, local = threadIdx.x - g * sp.rows;
+    const bool skip = isfinite(gthin);
+    for (int64_t row0 = (int64_t)blockIdx.x * sp.rows; row0 < n_rows; row0 += (int64_t)gridDim.x * sp.rows) {
+        const int64_t row = row0 + local;
+        const bool act = g < sp.G && row < n_rows;
+        RayMean<Real> lse;
+        for (int i = 0; i < sp.per; i += 2) {
+            const int k0 = g * sp.per + i, k1 = k0 + 1;
+            const bool in0 = act && k0 < R, in1 = act && i + 1 < sp.per && k1 < R;
+            const Real t0 = in0 ? tau(row, k0) : Real(1e30);
+            const Real t1 = in1 ? tau(row, k1) : t0;
+            Real S0 = Real(0), S1 = Real(0);
+            if (sizeof(Real) == 4 || in0) fold_pair(T, F, skip, in1, t0, t1, S0, S1);
+            if (sp.G == 1) {
+                if (in0) lse.add(ray_lnrate(smin, t0, S0));
+                if (in1) lse.add(ray_lnrate(smin, t1, S1));
+            } else {
+                if (in0) lk[k0 * sp.rows + local] = ray_lnrate(smin, t0, S0);
+                if (in1) lk[k1 * sp.rows + local] = ray_lnrate(smin, t1, S1);
+            }
+        }
+        if (sp.G == 1) {
+            if (act) fin(row, lse.mean(R));
+        } else {
+            __syncthreads();
+            if (threadIdx.x < sp.rows && row0 + threadIdx.x < n_rows) {
+                for (int k = 0; k < R; ++k) lse.add(lk[k * sp.rows + threadIdx.x]);
+                fin(row0 + threadIdx.x, lse.mean(R));
+            }
+            __syncthreads();
+        }
+    }
+}
 
 struct Rates {
     double alphaA, alphaB, gamma_c;   // cm^3 s^-1
