@@ -22,6 +22,7 @@
 // the tree's fixed order.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -130,18 +131,12 @@ __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(
 
 template <typename Real> struct RealOps;
 template <> struct RealOps<float> {
-    static __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
-    static __device__ __forceinline__ float log_(float x) { return logf(x); }
     static __device__ __forceinline__ float exp_(float x) { return expf(x); }
     static __device__ __forceinline__ float erf_(float x) { return erff(x); }
-    static __device__ __forceinline__ float weight(const TraceParams& P, int j) { return __ldg(P.w32 + j); }
 };
 template <> struct RealOps<double> {
-    static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-    static __device__ __forceinline__ double log_(double x) { return log(x); }
     static __device__ __forceinline__ double exp_(double x) { return exp(x); }
     static __device__ __forceinline__ double erf_(double x) { return erf(x); }
-    static __device__ __forceinline__ double weight(const TraceParams& P, int j) { return __ldg(P.w64 + j); }
 };
 
 // ---- M4 chord integrals in units of h -------------------------------------
@@ -155,58 +150,77 @@ template <> struct RealOps<double> {
 //   Fi(s) - Fo(s) = -s(1/4 + 13/2 b2) + (3 b2 + 3 b2^2) L(s).
 // At the chord end a = c = sqrt(1 - b2) (q = 1):
 //   Fo(c) = c(1/2 + 13/4 b2) - (3 b2 + 3/4 b2^2) L(c).
-template <typename Real>
-__device__ __forceinline__ Real m4_join(Real b2, Real lb, Real& s_out)
-{
-    using O = RealOps<Real>;
-    Real s = O::sqrt_(Real(0.25) - b2);
-    s_out = s;
-    Real Ls = b2 > Real(0) ? O::log_(s + Real(0.5)) - lb : Real(0);
-    return -s * (Real(0.25) + Real(6.5) * b2) + (Real(3) * b2 + Real(3) * b2 * b2) * Ls;
-}
+// In double (the FP32 chords are below).  The FP64 pipe bounds this path (2
+// results per clock and SM), so a chord takes as few FP64 operations as it can:
+// one ln b and one join for both ends, the two pieces' polynomials as one with
+// selected coefficients, and logarithms from a table (after Tang, 1990):
+// x = 2^e m, c about 1 / m from the top 7 bits of m, r = m c - 1 exactly,
+// ln x = e ln 2 - ln c + log1p(r), |r| < 0.004, the series to r^7; absolute
+// error about 1e-16, 11 operations where log() takes some 27.
+constexpr int kLogTab = 128;
 
-template <typename Real>
-__device__ __forceinline__ Real m4_full(Real b2, Real c)
+__device__ __forceinline__ void log_table(double2* tab)
 {
-    using O = RealOps<Real>;
-    Real lb = b2 > Real(0) ? Real(0.5) * O::log_(b2) : Real(0);
-    Real Lc = b2 > Real(0) ? O::log_(c + Real(1)) - lb : Real(0);
-    Real H = c * (Real(0.5) + Real(3.25) * b2) - (Real(3) * b2 + Real(0.75) * b2 * b2) * Lc;
-    if (b2 < Real(0.25)) {
-        Real s;
-        H += m4_join(b2, lb, s);
+    for (int i = threadIdx.x; i < kLogTab; i += blockDim.x) {
+        const double c = (double)(float)(1.0 / (1.0 + (i + 0.5) / kLogTab));
+        tab[i] = make_double2(c, -log(c));
     }
-    return Real(2) * H;
 }
 
-template <typename Real>
-__device__ __forceinline__ Real m4_H(Real b2, Real lb, Real a)
+__device__ __forceinline__ double log_tab(const double2* tab, double x)
 {
-    using O = RealOps<Real>;
-    Real q = O::sqrt_(b2 + a * a);
-    Real La = b2 > Real(0) ? O::log_(a + q) - lb : Real(0);
-    Real q3 = q * q * q;
-    if (b2 < Real(0.25)) {
-        Real s;
-        Real join = m4_join(b2, lb, s);
-        if (a <= s)
-            return a * (Real(1) - Real(6) * b2 - Real(2) * a * a) + Real(1.5) * a * q3 +
-                   Real(2.25) * b2 * a * q + Real(2.25) * b2 * b2 * La;
-        return a * (Real(2) + Real(6) * b2 + Real(2) * a * a) - Real(3) * a * q - Real(0.5) * a * q3 -
-               Real(0.75) * b2 * a * q - (Real(3) * b2 + Real(0.75) * b2 * b2) * La + join;
+    const int hi = __double2hiint(x);
+    if (hi < 0x00100000 || hi >= 0x7ff00000) return log(x);        // zero, denormal, negative, infinite, NaN
+    const double2 T = tab[(hi >> 13) & (kLogTab - 1)];
+    const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
+    const double r = fma(m, T.x, -1.0);
+    double p = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+    p = fma(r, p, 0.2);
+    p = fma(r, p, -0.25);
+    p = fma(r, p, 1.0 / 3.0);
+    p = fma(r, p, -0.5);
+    return fma((double)((hi >> 20) - 1023), 0.6931471805599453, T.y) + fma(r * r, p, r);
+}
+
+// ln b of b^2, and Fi(s) - Fo(s) with s = sqrt(1/4 - b^2) (b^2 < 1/4)
+__device__ __forceinline__ double m4_join(const double2* lt, double b2, double lb, double& s)
+{
+    s = sqrt(0.25 - b2);
+    const double Ls = b2 > 0.0 ? log_tab(lt, s + 0.5) - lb : 0.0;
+    return fma(fma(3.0 * b2, b2, 3.0 * b2), Ls, -s * fma(6.5, b2, 0.25));
+}
+
+__device__ __forceinline__ double m4_full(const double2* lt, double b2, double c)
+{
+    const double lb = b2 > 0.0 ? 0.5 * log_tab(lt, b2) : 0.0;
+    const double Lc = b2 > 0.0 ? log_tab(lt, c + 1.0) - lb : 0.0;
+    double H = c * fma(3.25, b2, 0.5) - fma(0.75 * b2, b2, 3.0 * b2) * Lc;
+    if (b2 < 0.25) {
+        double s;
+        H += m4_join(lt, b2, lb, s);
     }
-    return a * (Real(2) + Real(6) * b2 + Real(2) * a * a) - Real(3) * a * q - Real(0.5) * a * q3 -
-           Real(0.75) * b2 * a * q - (Real(3) * b2 + Real(0.75) * b2 * b2) * La;
+    return 2.0 * H;
 }
 
-template <typename Real>
-__device__ __forceinline__ Real m4_part(Real b2, Real u1, Real u2)
+__device__ __forceinline__ double m4_part(const double2* lt, double b2, double u1, double u2)
 {
-    using O = RealOps<Real>;
-    Real lb = b2 > Real(0) ? Real(0.5) * O::log_(b2) : Real(0);
-    Real g2 = u2 >= Real(0) ? m4_H(b2, lb, u2) : -m4_H(b2, lb, -u2);
-    Real g1 = u1 >= Real(0) ? m4_H(b2, lb, u1) : -m4_H(b2, lb, -u1);
-    return g2 - g1;
+    const double lb = b2 > 0.0 ? 0.5 * log_tab(lt, b2) : 0.0;
+    double s = -1.0, join = 0.0;
+    if (b2 < 0.25) join = m4_join(lt, b2, lb, s);
+    const double kLo = fma(0.75 * b2, b2, 3.0 * b2), kLi = 2.25 * b2 * b2, kqo = -fma(0.75, b2, 3.0), kqi = 2.25 * b2;
+    double H[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const double a = fabs(e == 0 ? u1 : u2), q2 = fma(a, a, b2), q = sqrt(q2);
+        const double L = b2 > 0.0 ? log_tab(lt, a + q) - lb : 0.0;
+        const bool in = a <= s;
+        // a (k0 + k1 (6 b2 + 2 a^2) + q (kq + k3 q^2)) + kL L
+        const double g = fma(4.0, b2, 2.0 * q2);
+        const double P = (in ? 1.0 - g : 2.0 + g) + q * fma(in ? 1.5 : -0.5, q2, in ? kqi : kqo);
+        const double v = fma(a, P, (in ? kLi : -kLo) * L) + (in ? 0.0 : join);
+        H[e] = (e == 0 ? u1 : u2) >= 0.0 ? v : -v;
+    }
+    return H[1] - H[0];
 }
 
 // ---- truncated Gaussian (Eq. Gt, I(h,b,z1,z2)) ----------------------------
@@ -491,21 +505,21 @@ struct Staged {
         struct {
             float u[32], v[32], t[32], hh[32];        // in the beam's frame; hh = (h + margin)^2
         };
-        Real tc[kPairs];          // once the masks are made: depths of the closest approach, where they are
-    };                            //   kept; then (FP32) a pair's weight
-    Real val[kPairs];             // a pair's chord integral (FP64: times its weight); before that b^2, where it is kept
+        Real tc[kF32 || kStored ? kPairs : 1];        // once the masks are made: depths of the closest approach,
+    };                                                //   where they are kept; then (FP32) a pair's weight
+    Real val[kF32 || kStored ? kPairs : 1];   // b^2, where it is kept; then (FP32) a pair's chord integral
     int64_t base0[MODE == 2 ? 32 : 1];        // MODE_FILL, per lane: where its next hits are stored
     uint32_t chunk0[MODE == 4 ? 32 : 1], chunk1[MODE == 4 ? 32 : 1];   // MODE_CHUNK, per lane: its chunk and the next
     int room[kStored ? 32 : 1];               // per lane: hits that fit (there)
     unsigned lane_hits[kStored ? 32 : 1];     // per lane: which of its pairs are hits
     int lane_off[kStored ? 32 : 1];           // per lane: its first pair
+    double ih[kF32 ? 1 : 32];     // FP64: 1/h
     double near_o[NF ? 32 : 1][3];            // near/far: shifted origin in double (the near test)
     float2 aw[kF32 ? 32 : 1];     // A_j and the tracer weight A_j x_j
     float2 g[kF32 ? 32 : 1];      // 1/h and h^2
     int j[32];                    // Morton slot
     unsigned hit[kPairs / 32 + 1], full[kPairs / 32 + 1], any[kPairs / 32 + 1];   // bit per pair; any: near ones too
     uint16_t pair[kPairs];        // sphere << 5 | lane
-    uint8_t list[kF32 ? 1 : kPairs];          // FP64: full chords from the front, partial from the back
 };
 
 // The lanes' candidates among the block's first m spheres (bit e: sphere e):
@@ -649,6 +663,98 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
     count = rest;
 }
 
+struct Queued {
+    int part, full;               // hits waiting (full: FP64 only)
+};
+
+// FP64: hits wait in two queues, full chords and partial ones (which cost
+// twice as much), and either is evaluated 32 at a time.  Each ray's values are
+// added in its queues' orders, full and partial chords apart, as in FP32.
+template <bool kStored, bool NF>
+struct HitQueue {
+    double b2[2][kPQ];            // [0] full, [1] partial chords: b^2
+    double tc[kPQ];               // partial: depth of the closest approach
+    int64_t pos[2][kStored ? kPQ : 1];    // MODE_FILL: the segment's position
+    double val[32];
+    double ih[2][kPQ];            // 1/h
+    float h[2][kPQ];
+    int j[2][kPQ];                // particle (Morton slot)
+    int owner[2][kPQ];            // lane of the ray | kPQNear
+    unsigned own[NF ? 64 : 32];   // as PartQueue::own
+};
+
+template <int KERNEL, int MODE, bool NF, int KIND, typename Queue, typename St>
+__device__ __forceinline__ void flush_hits(const TraceParams& P, const double2* lt, Queue* hq, const St& S, int& count,
+                                           int n, double L, Sink<double>& k)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane < n) {
+        const int j = hq->j[KIND][lane], ow = hq->owner[KIND][lane];
+        const double b2 = hq->b2[KIND][lane], h = (double)hq->h[KIND][lane], ih = hq->ih[KIND][lane];
+        const double ch = sqrt(__fma_rn(h, h, -b2));
+        const double beta2 = b2 * ih * ih;
+        double F;
+        if (KIND == 0) {
+            const double c = ch * ih;
+            // erf is odd: both ends of a full chord from one
+            F = KERNEL == URCHIN_KERNEL_M4 ? m4_full(lt, beta2, c)
+                                           : P.gt_pref * exp(-P.gt_t2 * beta2) * (2.0 * erf(P.gt_t * c));
+        } else {
+            const double tc = hq->tc[lane];
+            const double u1 = (fmax(0.0, tc - ch) - tc) * ih, u2 = (fmin(L, tc + ch) - tc) * ih;
+            F = KERNEL == URCHIN_KERNEL_M4 ? m4_part(lt, beta2, u1, u2) : gt_chord(P, beta2, u1, u2);
+        }
+        if (MODE == MODE_SCATTER) {
+            atomicAdd(P.xbar + j, S.org[ow].coef * (__ldg(P.A64 + j) * F));
+        } else {
+            const bool near = NF && (ow & kPQNear);
+            hq->val[lane] = near ? __ldg(P.A64 + j) * F : __ldg(P.w64 + j) * F;
+            if (MODE == MODE_FILL && hq->pos[KIND][lane] >= 0)
+                static_cast<double*>(P.seg_val)[hq->pos[KIND][lane]] = __ldg(P.A64 + j) * F;
+            atomicOr(&hq->own[ow & (31 | kPQNear)], 1u << lane);
+        }
+    }
+    __syncwarp();
+    if (MODE != MODE_SCATTER) {
+        for (unsigned m = hq->own[lane]; m; m &= m - 1) {
+            if (KIND == 0) Kahan::add(k.sum, k.comp, hq->val[__ffs(m) - 1]);
+            else Kahan::add(k.psum, k.pcomp, hq->val[__ffs(m) - 1]);
+        }
+        if (NF)
+            for (unsigned m = hq->own[lane + kPQNear]; m; m &= m - 1)
+                Kahan::add(k.near, k.near_c, hq->val[__ffs(m) - 1]);
+        __syncwarp();
+        hq->own[lane] = 0u;
+        if (NF) hq->own[lane + kPQNear] = 0u;
+    }
+    const int rest = count - n;
+    double b2 = 0.0, tc = 0.0, ih = 0.0;
+    float h = 0.f;
+    int j = 0, ow = 0;
+    int64_t pos = 0;
+    if (lane < rest) {
+        b2 = hq->b2[KIND][n + lane];
+        ih = hq->ih[KIND][n + lane];
+        if (KIND == 1) tc = hq->tc[n + lane];
+        h = hq->h[KIND][n + lane];
+        j = hq->j[KIND][n + lane];
+        ow = hq->owner[KIND][n + lane];
+        if (MODE == MODE_FILL) pos = hq->pos[KIND][n + lane];
+    }
+    __syncwarp();
+    if (lane < rest) {
+        hq->b2[KIND][lane] = b2;
+        hq->ih[KIND][lane] = ih;
+        if (KIND == 1) hq->tc[lane] = tc;
+        hq->h[KIND][lane] = h;
+        hq->j[KIND][lane] = j;
+        hq->owner[KIND][lane] = ow;
+        if (MODE == MODE_FILL) hq->pos[KIND][lane] = pos;
+    }
+    __syncwarp();
+    count = rest;
+}
+
 // MODE_CHUNK: `want` consecutive chunks from the warp's block of chunks in
 // shared memory, a new block of kStash (or more) from the global counter when
 // it runs out.  Called by lane 0 with the warp converged.
@@ -752,22 +858,25 @@ __device__ __forceinline__ bool decide(const St& S, int e, int o, float dx, floa
     return __fadd_rn(tc, ch) > 0.f && __fsub_rn(tc, ch) < L;
 }
 
+// In double the half chord ch stays squared, w = h^2 - b^2 = ch^2: tc + ch > 0,
+// tc - ch < L, and (full) tc - ch >= 0, tc + ch <= L by comparing squares.
 template <typename St>
 __device__ __forceinline__ bool decide(const St& S, int e, int o, double dx, double dy, double dz, double L,
-                                       double& b2, double& tc, double& ch)
+                                       double& b2, double& tc, bool& full)
 {
     const float4 q = S.q[e];
     const Origin<double> s = S.org[o];
     const double ex = (double)q.x - s.x, ey = (double)q.y - s.y, ez = (double)q.z - s.z;
-    const double cx = sub_rn(mul_rn(ey, dz), mul_rn(ez, dy));
-    const double cy = sub_rn(mul_rn(ez, dx), mul_rn(ex, dz));
-    const double cz = sub_rn(mul_rn(ex, dy), mul_rn(ey, dx));
-    const double h2 = mul_rn((double)q.w, (double)q.w);
-    b2 = fma(cz, cz, fma(cy, cy, mul_rn(cx, cx)));
-    if (!(b2 < h2)) return false;
-    tc = fma(ez, dz, fma(ey, dy, mul_rn(ex, dx)));
-    ch = sqrt(sub_rn(h2, b2));
-    return add_rn(tc, ch) > 0.0 && sub_rn(tc, ch) < L;
+    const double cx = __fma_rn(ey, dz, -mul_rn(ez, dy));
+    const double cy = __fma_rn(ez, dx, -mul_rn(ex, dz));
+    const double cz = __fma_rn(ex, dy, -mul_rn(ey, dx));
+    b2 = __fma_rn(cz, cz, __fma_rn(cy, cy, mul_rn(cx, cx)));
+    const double w = __fma_rn((double)q.w, (double)q.w, -b2);
+    if (!(w > 0.0)) return false;
+    tc = __fma_rn(ez, dz, __fma_rn(ey, dy, mul_rn(ex, dx)));
+    const double d = sub_rn(L, tc), t2 = mul_rn(tc, tc), d2 = mul_rn(d, d);
+    full = tc >= 0.0 && d >= 0.0 && w <= t2 && w <= d2;
+    return (tc > 0.0 || w > t2) && (d > 0.0 || w > d2);
 }
 
 // The pairs of the lanes' masks mm (at most kPairs in all): listed, decided,
@@ -919,12 +1028,16 @@ __device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* ta
     __syncwarp();
 }
 
-// The same in double: the pairs are decided first and split into full and
-// partial chords, each evaluated 32 at a time (one kind costs two to three
-// times the other, and the FP64 pipe is what bounds this path).
-template <int KERNEL, int MODE, bool NF, typename St>
-__device__ __forceinline__ void pairs_f64(const TraceParams& P, unsigned long long* stash, St& S, unsigned mm,
-                                          double dx, double dy, double dz, double L, Sink<double>& k, unsigned& err)
+__device__ __forceinline__ double half_chord(float h, double b2)
+{
+    return sqrt(__fma_rn((double)h, (double)h, -b2));
+}
+
+// The same in double: hits go to the queues of full and of partial chords.
+template <int KERNEL, int MODE, bool NF, typename Queue, typename St>
+__device__ __forceinline__ void pairs_f64(const TraceParams& P, const double2* lt, Queue* hq, Queued& qn,
+                                          unsigned long long* stash, St& S, unsigned mm, bool drain, double dx,
+                                          double dy, double dz, double L, Sink<double>& k, unsigned& err)
 {
     constexpr bool kStored = MODE == MODE_FILL;
     const int lane = threadIdx.x & 31;
@@ -942,90 +1055,92 @@ __device__ __forceinline__ void pairs_f64(const TraceParams& P, unsigned long lo
         for (unsigned m = mm; m; m &= m - 1u) S.pair[i++] = (uint16_t)(((__ffs(m) - 1) << 5) | lane);
     }
     __syncwarp();
-    int nf = 0, np = 0;
-    for (int p0 = 0; p0 < total; p0 += 32) {
-        const int p = p0 + lane;
-        bool hit = false, near = false, full = false;
-        if (p < total) {
-            const int pr = S.pair[p], e = pr >> 5, o = pr & 31;
-            double b2, tc = 0.0, ch = 0.0;
-            hit = decide(S, e, o, dx, dy, dz, L, b2, tc, ch);
-            if (hit) {
-                near = NF && is_near(S.near_o[o], S.q[e], tc, ch);
-                full = sub_rn(tc, ch) >= 0.0 && add_rn(tc, ch) <= L;
-                S.val[p] = b2;
-                S.tc[p] = tc;
+    if constexpr (kStored) {
+        for (int p0 = 0; p0 < total; p0 += 32) {
+            const int p = p0 + lane;
+            bool hit = false, near = false, full = false;
+            if (p < total) {
+                const int pr = S.pair[p], e = pr >> 5, o = pr & 31;
+                double b2, tc = 0.0;
+                hit = decide(S, e, o, dx, dy, dz, L, b2, tc, full);
+                if (hit) {
+                    near = NF && is_near(S.near_o[o], S.q[e], tc, half_chord(S.q[e].w, b2));
+                    S.val[p] = b2;
+                    S.tc[p] = tc;
+                }
+            }
+            const unsigned fw = __ballot_sync(0xffffffffu, hit && full);
+            const unsigned ha = __ballot_sync(0xffffffffu, hit), hw = __ballot_sync(0xffffffffu, hit && !near);
+            if (lane == 0) {
+                S.any[p0 >> 5] = ha;
+                S.hit[p0 >> 5] = hw;
+                S.full[p0 >> 5] = fw;
             }
         }
-        const unsigned ha = __ballot_sync(0xffffffffu, hit), hw = __ballot_sync(0xffffffffu, hit && !near);
-        const unsigned fw = __ballot_sync(0xffffffffu, hit && full), lt = (1u << lane) - 1u;
-        if (hit) {
-            if (full) S.list[nf + __popc(fw & lt)] = (uint8_t)p;
-            else S.list[St::kPairs - 1 - np - __popc(ha & ~fw & lt)] = (uint8_t)p;
-        }
-        nf += __popc(fw);
-        np += __popc(ha & ~fw);
-        if (lane == 0) {
-            S.any[p0 >> 5] = ha;
-            S.hit[p0 >> 5] = hw;
-        }
-    }
-    __syncwarp();
-    const unsigned hm = c ? flag_bits(S.hit, off, c) : 0u;
-    k.nhit += (unsigned)__popc(hm);
-    if constexpr (kStored) {
+        __syncwarp();
+        const unsigned hm = c ? flag_bits(S.hit, off, c) : 0u;
+        k.nhit += (unsigned)__popc(hm);
         S.lane_hits[lane] = hm;
         S.lane_off[lane] = off;
         assign_positions<MODE>(P, stash, S, __popc(hm), k, err);
         __syncwarp();
     }
-#pragma unroll 1
-    for (int kind = MODE == MODE_COUNT ? 2 : 0; kind < 2; ++kind) {
-        const int n = kind == 0 ? nf : np;
-#pragma unroll 1
-        for (int i0 = 0; i0 < n; i0 += 32) {
-            const int i = i0 + lane;
-            if (i >= n) continue;
-            const int p = S.list[kind == 0 ? i : St::kPairs - 1 - i];
-            const int pr = S.pair[p], e = pr >> 5, o = pr & 31, j = S.j[e];
-            const double b2 = S.val[p], h = (double)S.q[e].w, ih = 1.0 / h;
-            const double ch = sqrt(sub_rn(mul_rn(h, h), b2));
-            const double beta2 = b2 * ih * ih;
-            double F;
-            if (kind == 0) {
-                const double cc = ch * ih;
-                if (KERNEL == URCHIN_KERNEL_M4) F = m4_full(beta2, cc);
-                else F = gt_chord(P, beta2, -cc, cc);
-            } else {
-                const double tc = S.tc[p];
-                const double u1 = (fmax(0.0, tc - ch) - tc) * ih, u2 = (fmin(L, tc + ch) - tc) * ih;
-                if (KERNEL == URCHIN_KERNEL_M4) F = m4_part(beta2, u1, u2);
-                else F = gt_chord(P, beta2, u1, u2);
-            }
-            if (MODE == MODE_SCATTER) {
-                atomicAdd(P.xbar + j, S.org[o].coef * (__ldg(P.A64 + j) * F));
-                continue;
-            }
-            const bool far = !NF || ((S.hit[p >> 5] >> (p & 31)) & 1u);
-            S.val[p] = far ? __ldg(P.w64 + j) * F : __ldg(P.A64 + j) * F;
-            if (kStored && far) {
-                const int64_t pos = hit_position<MODE>(S, p, o);
-                if (pos >= 0) {
-                    store_index(P, pos, j);
-                    static_cast<double*>(P.seg_val)[pos] = __ldg(P.A64 + j) * F;
+    for (int p0 = 0; p0 < total || drain; p0 += 32) {
+        const int p = p0 + lane;
+        bool hit = false, near = false, full = false;
+        int e = 0, o = 0;
+        double b2 = 0.0, tc = 0.0;
+        int64_t pos = -1;
+        if (p < total) {
+            const int pr = S.pair[p];
+            e = pr >> 5;
+            o = pr & 31;
+            if constexpr (kStored) {
+                hit = (S.any[p0 >> 5] >> lane) & 1u;
+                if (hit) {
+                    b2 = S.val[p];
+                    tc = S.tc[p];
+                    full = (S.full[p0 >> 5] >> lane) & 1u;
+                    near = NF && !((S.hit[p0 >> 5] >> lane) & 1u);
+                    if (!near) {
+                        pos = hit_position<MODE>(S, p, o);
+                        if (pos >= 0) store_index(P, pos, S.j[e]);
+                    }
                 }
+            } else {
+                hit = decide(S, e, o, dx, dy, dz, L, b2, tc, full);
+                full = full && hit;
+                if (hit) near = NF && is_near(S.near_o[o], S.q[e], tc, half_chord(S.q[e].w, b2));
             }
         }
+        if constexpr (!kStored) {
+            const unsigned hw = __ballot_sync(0xffffffffu, hit && !near);
+            if (lane == 0) S.hit[p0 >> 5] = hw;
+        }
+        if (MODE == MODE_COUNT) continue;
+        const unsigned fb = __ballot_sync(0xffffffffu, full), pb = __ballot_sync(0xffffffffu, hit && !full);
+        const unsigned lt_mask = (1u << lane) - 1u;
+        if (hit) {
+            const int kind = full ? 0 : 1, i = full ? qn.full + __popc(fb & lt_mask) : qn.part + __popc(pb & lt_mask);
+            hq->b2[kind][i] = b2;
+            if (!full) hq->tc[i] = tc;
+            hq->h[kind][i] = S.q[e].w;
+            hq->ih[kind][i] = S.ih[e];
+            hq->j[kind][i] = S.j[e];
+            hq->owner[kind][i] = o | (near ? kPQNear : 0);
+            if (kStored) hq->pos[kind][i] = pos;
+        }
+        qn.full += __popc(fb);
+        qn.part += __popc(pb);
+        __syncwarp();
+        if (qn.full >= 32 || (drain && qn.full > 0))
+            flush_hits<KERNEL, MODE, NF, 0>(P, lt, hq, S, qn.full, min(qn.full, 32), L, k);
+        if (qn.part >= 32 || (drain && qn.part > 0))
+            flush_hits<KERNEL, MODE, NF, 1>(P, lt, hq, S, qn.part, min(qn.part, 32), L, k);
+        if (drain) break;
     }
     __syncwarp();
-    if (c && MODE != MODE_SCATTER && MODE != MODE_COUNT) {
-        for (unsigned m = flag_bits(S.any, off, c); m; m &= m - 1u) {
-            const int i = __ffs(m) - 1;
-            const double v = S.val[off + i];
-            if (!NF || ((hm >> i) & 1u)) Kahan::add(k.sum, k.comp, v);
-            else Kahan::add(k.near, k.near_c, v);
-        }
-    }
+    if (!kStored && c) k.nhit += (unsigned)__popc(flag_bits(S.hit, off, c));
     __syncwarp();
 }
 
@@ -1094,8 +1209,8 @@ struct Walk {
 // with drain, no image but the queued partial chords (so that the loop holds
 // one copy of that code).
 template <typename Real, int KERNEL, int MODE, bool NF, typename Queue, typename St>
-__device__ __forceinline__ void packet_image(const TraceParams& P, const float2* tab, const Beam& B, St& S,
-                                             Queue* pq, int& pq_count, unsigned long long* stash, float3 pt,
+__device__ __forceinline__ void packet_image(const TraceParams& P, const unsigned char* tab, const Beam& B, St& S,
+                                             Queue* pq, Queued& qn, unsigned long long* stash, float3 pt,
                                              float Lf, Real dx, Real dy, Real dz, bool live, bool drain,
                                              Sink<Real>& sk, unsigned& err, unsigned& nvisit)
 {
@@ -1156,6 +1271,8 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
             if constexpr (kF32) {
                 S.g[at] = make_float2(1.f / cq.w, __fmul_rn(cq.w, cq.w));
                 if (kWantA || kWantW) S.aw[at] = caw;
+            } else {
+                S.ih[at] = 1.0 / (double)cq.w;
             }
         };
         const bool mine = (pm >> lane) & 1u;
@@ -1185,9 +1302,11 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
         for (int e0 = 0; (total > 0 || drain) && e0 < 32; e0 += step) {
             const unsigned mm = step == 32 ? mask : mask & (((1u << step) - 1u) << e0);
             if constexpr (kF32)
-                pairs_f32<KERNEL, MODE, NF>(P, tab, pq, pq_count, stash, S, mm, drain, dx, dy, dz, L, sk, err);
+                pairs_f32<KERNEL, MODE, NF>(P, reinterpret_cast<const float2*>(tab), pq, qn.part, stash, S, mm, drain, dx,
+                                            dy, dz, L, sk, err);
             else
-                pairs_f64<KERNEL, MODE, NF>(P, stash, S, mm, dx, dy, dz, L, sk, err);
+                pairs_f64<KERNEL, MODE, NF>(P, reinterpret_cast<const double2*>(tab), pq, qn, stash, S, mm, drain, dx, dy,
+                                            dz, L, sk, err);
         }
         __syncwarp();                // the block's readers are done
         if (last) break;
@@ -1207,8 +1326,8 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const float2*
 constexpr float kBeamReach = 5.f;
 
 template <typename Real, int KERNEL, int MODE, bool NF, typename Queue, typename St>
-__device__ __forceinline__ void ray_column(const TraceParams& P, const float2* tab, Beam* beam, St& S,
-                                           Queue* pq, int& pq_count, unsigned long long* stash, float4 o, Real dx,
+__device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned char* tab, Beam* beam, St& S,
+                                           Queue* pq, Queued& qn, unsigned long long* stash, float4 o, Real dx,
                                            Real dy, Real dz, bool live, Sink<Real>& sk, unsigned& err,
                                            unsigned& nvisit)
 {
@@ -1217,10 +1336,10 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const float2* t
     const int nimg = P.periodic ? P.nimg : 0;
     const int side = 2 * nimg + 1;
     const int images = side * side * side;
-    constexpr bool kQueue = sizeof(Real) == 4 && MODE != MODE_COUNT;
+    constexpr bool kQueue = MODE != MODE_COUNT;
     float3 pt = make_float3(0.f, 0.f, 0.f);
     unsigned left = __ballot_sync(0xffffffffu, live);
-    while (left || (kQueue && pq_count > 0)) {
+    while (left || (kQueue && (qn.part > 0 || qn.full > 0))) {
         const bool drain = !left;
         bool in = false;
         if (!drain) {
@@ -1269,7 +1388,7 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const float2* t
                 }
                 if (!drain)
                     pt = make_beam<Real>(beam, lv, in, sx, sy, sz, (float)dx, (float)dy, (float)dz, Lf);
-                packet_image<Real, KERNEL, MODE, NF>(P, tab, *beam, S, pq, pq_count, stash, pt, Lf, dx, dy, dz, in,
+                packet_image<Real, KERNEL, MODE, NF>(P, tab, *beam, S, pq, qn, stash, pt, Lf, dx, dy, dz, in,
                                                      drain, sk, err, nvisit);
             }
         }
@@ -1277,20 +1396,22 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const float2* t
 }
 
 // k_trace's shared memory: per warp the work space, the beam, the block of
-// chunks (MODE_CHUNK) and the queue of partial chords (FP32 modes that evaluate
-// chords); the FP32 M4 table; the directions (double[3 R]).
+// chunks (MODE_CHUNK) and the queue of partial chords (FP64: of hits) in modes
+// that evaluate chords; the M4 table (FP64: of logarithms); the directions (double[3 R]).
 template <typename Real, int KERNEL, int MODE, bool NF>
 struct TraceLayout {
     static constexpr bool kF32 = sizeof(Real) == 4;
-    static constexpr bool kQueue = kF32 && MODE != MODE_COUNT;
+    static constexpr bool kQueue = MODE != MODE_COUNT;
     static constexpr bool kTable = kQueue && KERNEL == URCHIN_KERNEL_M4;
+    static constexpr bool kStored = MODE == MODE_FILL || MODE == MODE_CHUNK;
     using St = Staged<Real, MODE, NF>;
-    using Queue = PartQueue<MODE == MODE_FILL || MODE == MODE_CHUNK, NF>;
+    using Queue = std::conditional_t<kF32, PartQueue<kStored, NF>, HitQueue<kStored, NF>>;
     static constexpr size_t up(size_t b) { return (b + 15) & ~size_t(15); }
     static constexpr size_t kBeam = up(sizeof(St) * 8);
     static constexpr size_t kStashAt = up(kBeam + sizeof(Beam) * 8);
     static constexpr size_t kTab = up(kStashAt + 8 * 2 * sizeof(unsigned long long));
-    static constexpr size_t kQueueAt = up(kTab + (kTable ? sizeof(float2) * (kKTab + 1) : 0));
+    static constexpr size_t kQueueAt =
+        up(kTab + (!kTable ? 0 : kF32 ? sizeof(float2) * (kKTab + 1) : sizeof(double2) * kLogTab));
     static constexpr size_t kDirs = up(kQueueAt + (kQueue ? sizeof(Queue) * 8 : 0));
     static size_t bytes(int R) { return kDirs + sizeof(double) * 3 * (size_t)R; }
 };
@@ -1311,8 +1432,12 @@ static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, 
 // registers) the spills cost more than the fourth block's warps hide; with
 // two (no spills) too few warps are left to hide the loads.  The transpose
 // keeps four: its FP64 atomic adds want the warps more than the registers.
+// FP64: bound by the FP64 pipe (84 % busy before the queues of full and partial
+// chords, at 17 of 32 lanes), two blocks; 16^3 lattice solve 18.3 -> 11.4 ms,
+// 24^3 box 10.7 -> 5.2 ms, 8000-particle halo 13.1 -> 8.8 ms, 9973 x 48 rays of
+// the 48^3 box (G_t) 25.3 -> 18.7 ms with queues and table logarithms.
 template <typename Real, int KERNEL, int MODE, bool NF>
-__global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(TraceParams P)
+__global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 2 : MODE == MODE_SCATTER ? 4 : 3) k_trace(TraceParams P)
 {
     using Lay = TraceLayout<Real, KERNEL, MODE, NF>;
     constexpr bool kQueue = Lay::kQueue;
@@ -1321,21 +1446,22 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
     typename Lay::St& st = reinterpret_cast<typename Lay::St*>(smem)[wid];
     Beam* beam = reinterpret_cast<Beam*>(smem + Lay::kBeam) + wid;
     unsigned long long* stash = reinterpret_cast<unsigned long long*>(smem + Lay::kStashAt) + 2 * wid;
-    float2* s_tab = reinterpret_cast<float2*>(smem + Lay::kTab);
+    unsigned char* s_tab = smem + Lay::kTab;
     typename Lay::Queue* pq = reinterpret_cast<typename Lay::Queue*>(smem + Lay::kQueueAt) + wid;
     double* s_dirs = reinterpret_cast<double*>(smem + Lay::kDirs);
     if (kQueue) {
         pq->own[threadIdx.x & 31] = 0u;
         if (NF) pq->own[(threadIdx.x & 31) + kPQNear] = 0u;
     }
-    int pq_count = 0;
+    Queued qn{0, 0};
     if ((threadIdx.x & 31) == 0) {
         stash[0] = 0ull;
         stash[1] = 0ull;
     }
     for (int t = threadIdx.x; t < 3 * P.R; t += blockDim.x) s_dirs[t] = P.dirs[t];
-    if (Lay::kTable)
-        for (int t = threadIdx.x; t <= kKTab; t += blockDim.x) s_tab[t] = P.ktab[t];
+    if (Lay::kTable && Lay::kF32)
+        for (int t = threadIdx.x; t <= kKTab; t += blockDim.x) reinterpret_cast<float2*>(s_tab)[t] = P.ktab[t];
+    if (Lay::kTable && !Lay::kF32) log_table(reinterpret_cast<double2*>(s_tab));
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const unsigned long long total = (unsigned long long)P.n_chunks * (unsigned long long)P.R;
@@ -1375,7 +1501,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_SCATTER ? 4 : 3) k_trace(Tra
             sk.coef = static_cast<const Real*>(P.coef)[orow * P.row_stride + (int64_t)k * P.k_stride];
             live = sk.coef != Real(0);
         }
-        ray_column<Real, KERNEL, MODE, NF>(P, s_tab, beam, st, pq, pq_count, stash, o, dx, dy, dz, live, sk, err,
+        ray_column<Real, KERNEL, MODE, NF>(P, s_tab, beam, st, pq, qn, stash, o, dx, dy, dz, live, sk, err,
                                            nvisit);
         if (mine) {
             hits += sk.nhit;
