@@ -126,7 +126,6 @@ __device__ __forceinline__ bool is_near(const double* o, float4 q, Real tc, Real
 
 // Rounded arithmetic the compiler may not contract into multiply-adds.
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 
 template <typename Real> struct RealOps;
@@ -498,7 +497,7 @@ template <typename Real, int MODE, bool NF>
 struct Staged {
     static constexpr bool kF32 = sizeof(Real) == 4;
     static constexpr bool kStored = MODE == 2 || MODE == 4;   // MODE_FILL, MODE_CHUNK
-    static constexpr int kPairs = kF32 && kStored ? 192 : 256;
+    static constexpr int kPairs = kF32 && kStored ? (NF ? 128 : 192) : 256;
     float4 q[32];                 // x, y, z, h
     Origin<Real> org[32];
     union {
@@ -574,55 +573,67 @@ __device__ __forceinline__ void store_index(const TraceParams& P, int64_t pos, i
 // whose ray met one.  Instead the warp appends its partial chords to a queue
 // in shared memory and evaluates them 32 at a time, one per lane; every ray
 // then adds its own results in queue order (the lanes of one ray's items
-// found with a match), so the sums stay deterministic.
+// found by a bit mask per ray), so the sums stay deterministic.
 constexpr int kPQ = 64;           // queue capacity per warp; a round takes 32
 constexpr int kPQNear = 32;       // owner flag: a near particle (near/far split)
 constexpr int kPQClipLo = 64;     // owner flag: the segment's start cuts the chord
 constexpr int kPQClipHi = 128;    // owner flag: the segment's end cuts the chord
-template <bool kStored, bool NF>
+template <int MODE, bool NF>
 struct PartQueue {
-    float beta2[kPQ], u1[kPQ], u2[kPQ];   // chord in units of h: b^2/h^2 and [u1, u2]
-    float A[kPQ];                 // A_j
-    float w[kPQ];                 // the tracer weight A_j x_j (MODE_SCATTER: the ray's coefficient)
-    int j[kPQ];                   // particle (Morton slot)
-    int owner[kPQ];               // lane of the ray | kPQNear | kPQClipLo | kPQClipHi
-    int64_t pos[kStored ? kPQ : 1];       // MODE_FILL, MODE_CHUNK: the segment's position
+    static constexpr bool kAux = MODE != 0;   // every mode but MODE_TAU, of whose items the near ones need A_j
+    float4 item[kPQ];             // b^2/h^2 and [u1, u2] in units of h; the tracer weight A_j x_j (MODE_SCATTER: the ray's coefficient)
+    int4 aux[kAux ? kPQ : 1];     // particle (Morton slot), low half of the segment's position, bits of A_j; 0
+    float A[NF && !kAux ? kPQ : 1];
+    int owner[kPQ];               // lane of the ray | kPQNear | kPQClipLo | kPQClipHi | high half of the position << 16
     float val[32];                // results of the round being flushed
     unsigned own[NF ? 64 : 32];   // per owner (lane, lane + kPQNear): items of the round
 };
 
-// Evaluate the first n (<= 32) queued chords, one per lane, and move the
-// rest to the front.  Every lane of the warp calls it.  Inlined: as a called
-// function its reference arguments kept the ray's running state (sums,
-// cursor, queue length) in local memory for the whole traversal, which cost
-// 7 % of the traversal's time.
+// Items waiting in a ring of kPQ and where it begins (full: FP64 only).
+struct Queued {
+    int part, full, part_head, full_head;
+};
+
+// Position of a stored segment in a queue item: 47 bits and "nowhere" (-1).
+__device__ __forceinline__ int pos_hi(int64_t pos) { return pos < 0 ? (int)0xffff0000 : (int)(pos >> 32) << 16; }
+__device__ __forceinline__ int64_t pos_of(int owner, int lo)
+{
+    const int hi = (owner >> 16) & 0xffff;
+    return hi == 0xffff ? -1 : ((int64_t)hi << 32) | (uint32_t)lo;
+}
+
+// Evaluate the first n (<= 32) queued chords, one per lane.  Every lane of the
+// warp calls it.  Inlined: as a called function its reference arguments kept
+// the ray's running state (sums, cursor, queue length) in local memory for the
+// whole traversal, which cost 7 % of the traversal's time.
 template <int KERNEL, int MODE, bool NF, typename Queue>
-__device__ __forceinline__ void flush_partials(const TraceParams& P, const float2* tab, Queue* pq, int& count, int n,
+__device__ __forceinline__ void flush_partials(const TraceParams& P, const float2* tab, Queue* pq, Queued& qn, int n,
                                                Sink<float>& k)
 {
     const int lane = threadIdx.x & 31;
-    int owner = -1;
-    float v = 0.f;
     if (lane < n) {
-        const int ow = pq->owner[lane], j = pq->j[lane];
-        const float b2 = pq->beta2[lane], u1 = pq->u1[lane], u2 = pq->u2[lane];
-        const float F = KERNEL == URCHIN_KERNEL_M4 ? m4_part_q(tab, b2, u1, u2, (ow & kPQClipLo) != 0, (ow & kPQClipHi) != 0)
-                                                   : gt_chord<float>(P, b2, u1, u2);
-        const float A = pq->A[lane];
+        const int at = (qn.part_head + lane) & (kPQ - 1);
+        const int ow = pq->owner[at];
+        const float4 q = pq->item[at];
+        const float F = KERNEL == URCHIN_KERNEL_M4 ? m4_part_q(tab, q.x, q.y, q.z, (ow & kPQClipLo) != 0, (ow & kPQClipHi) != 0)
+                                                   : gt_chord<float>(P, q.x, q.y, q.z);
+        int4 x = make_int4(0, 0, 0, 0);
+        if (Queue::kAux) x = pq->aux[at];
+        const float A = NF && !Queue::kAux ? pq->A[at] : __int_as_float(x.z);
         if (MODE == MODE_SCATTER) {
-            atomicAdd(P.xbar + j, (double)(pq->w[lane] * (A * F)));
+            atomicAdd(P.xbar + x.x, (double)(q.w * (A * F)));
         } else {
-            const bool near = NF && (ow & kPQNear);
-            v = near ? A * F : pq->w[lane] * F;
-            if (MODE == MODE_FILL && pq->pos[lane] >= 0) static_cast<float*>(P.seg_val)[pq->pos[lane]] = A * F;
-            if (MODE == MODE_CHUNK && pq->pos[lane] >= 0) P.chunk_seg[pq->pos[lane]] = make_int2(j, __float_as_int(A * F));
-            owner = ow & (31 | kPQNear);
+            pq->val[lane] = NF && (ow & kPQNear) ? A * F : q.w * F;
+            if (MODE == MODE_FILL || MODE == MODE_CHUNK) {
+                const int64_t pos = pos_of(ow, x.y);
+                if (MODE == MODE_FILL && pos >= 0) static_cast<float*>(P.seg_val)[pos] = A * F;
+                if (MODE == MODE_CHUNK && pos >= 0) P.chunk_seg[pos] = make_int2(x.x, __float_as_int(A * F));
+            }
+            atomicOr(&pq->own[ow & (NF ? 31 | kPQNear : 31)], 1u << lane);
         }
     }
+    __syncwarp();
     if (MODE != MODE_SCATTER) {
-        pq->val[lane] = v;
-        if (owner >= 0) atomicOr(&pq->own[owner], 1u << lane);
-        __syncwarp();
         for (unsigned m = pq->own[lane]; m; m &= m - 1) Kahan::add(k.psum, k.pcomp, pq->val[__ffs(m) - 1]);
         if (NF)
             for (unsigned m = pq->own[lane + kPQNear]; m; m &= m - 1)
@@ -630,42 +641,11 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
         __syncwarp();
         pq->own[lane] = 0u;
         if (NF) pq->own[lane + kPQNear] = 0u;
-    }
-    const int rest = count - n;
-    if (rest > 0) {
         __syncwarp();
-        float b2 = 0.f, u1 = 0.f, u2 = 0.f, A = 0.f, w = 0.f;
-        int j = 0, ow = 0;
-        int64_t pos = 0;
-        if (lane < rest) {
-            b2 = pq->beta2[n + lane];
-            u1 = pq->u1[n + lane];
-            u2 = pq->u2[n + lane];
-            A = pq->A[n + lane];
-            w = pq->w[n + lane];
-            j = pq->j[n + lane];
-            ow = pq->owner[n + lane];
-            if (MODE == MODE_FILL || MODE == MODE_CHUNK) pos = pq->pos[n + lane];
-        }
-        __syncwarp();
-        if (lane < rest) {
-            pq->beta2[lane] = b2;
-            pq->u1[lane] = u1;
-            pq->u2[lane] = u2;
-            pq->A[lane] = A;
-            pq->w[lane] = w;
-            pq->j[lane] = j;
-            pq->owner[lane] = ow;
-            if (MODE == MODE_FILL || MODE == MODE_CHUNK) pq->pos[lane] = pos;
-        }
     }
-    __syncwarp();
-    count = rest;
+    qn.part_head = (qn.part_head + n) & (kPQ - 1);
+    qn.part -= n;
 }
-
-struct Queued {
-    int part, full;               // hits waiting (full: FP64 only)
-};
 
 // FP64: hits wait in two queues, full chords and partial ones (which cost
 // twice as much), and either is evaluated 32 at a time.  Each ray's values are
@@ -684,13 +664,14 @@ struct HitQueue {
 };
 
 template <int KERNEL, int MODE, bool NF, int KIND, typename Queue, typename St>
-__device__ __forceinline__ void flush_hits(const TraceParams& P, const double2* lt, Queue* hq, const St& S, int& count,
-                                           int n, double L, Sink<double>& k)
+__device__ __forceinline__ void flush_hits(const TraceParams& P, const double2* lt, Queue* hq, const St& S,
+                                           int& count, int& head, int n, double L, Sink<double>& k)
 {
     const int lane = threadIdx.x & 31;
     if (lane < n) {
-        const int j = hq->j[KIND][lane], ow = hq->owner[KIND][lane];
-        const double b2 = hq->b2[KIND][lane], h = (double)hq->h[KIND][lane], ih = hq->ih[KIND][lane];
+        const int at = (head + lane) & (kPQ - 1);
+        const int j = hq->j[KIND][at], ow = hq->owner[KIND][at];
+        const double b2 = hq->b2[KIND][at], h = (double)hq->h[KIND][at], ih = hq->ih[KIND][at];
         const double ch = sqrt(__fma_rn(h, h, -b2));
         const double beta2 = b2 * ih * ih;
         double F;
@@ -700,7 +681,7 @@ __device__ __forceinline__ void flush_hits(const TraceParams& P, const double2* 
             F = KERNEL == URCHIN_KERNEL_M4 ? m4_full(lt, beta2, c)
                                            : P.gt_pref * exp(-P.gt_t2 * beta2) * (2.0 * erf(P.gt_t * c));
         } else {
-            const double tc = hq->tc[lane];
+            const double tc = hq->tc[at];
             const double u1 = (fmax(0.0, tc - ch) - tc) * ih, u2 = (fmin(L, tc + ch) - tc) * ih;
             F = KERNEL == URCHIN_KERNEL_M4 ? m4_part(lt, beta2, u1, u2) : gt_chord(P, beta2, u1, u2);
         }
@@ -709,8 +690,8 @@ __device__ __forceinline__ void flush_hits(const TraceParams& P, const double2* 
         } else {
             const bool near = NF && (ow & kPQNear);
             hq->val[lane] = near ? __ldg(P.A64 + j) * F : __ldg(P.w64 + j) * F;
-            if (MODE == MODE_FILL && hq->pos[KIND][lane] >= 0)
-                static_cast<double*>(P.seg_val)[hq->pos[KIND][lane]] = __ldg(P.A64 + j) * F;
+            if (MODE == MODE_FILL && hq->pos[KIND][at] >= 0)
+                static_cast<double*>(P.seg_val)[hq->pos[KIND][at]] = __ldg(P.A64 + j) * F;
             atomicOr(&hq->own[ow & (31 | kPQNear)], 1u << lane);
         }
     }
@@ -727,32 +708,9 @@ __device__ __forceinline__ void flush_hits(const TraceParams& P, const double2* 
         hq->own[lane] = 0u;
         if (NF) hq->own[lane + kPQNear] = 0u;
     }
-    const int rest = count - n;
-    double b2 = 0.0, tc = 0.0, ih = 0.0;
-    float h = 0.f;
-    int j = 0, ow = 0;
-    int64_t pos = 0;
-    if (lane < rest) {
-        b2 = hq->b2[KIND][n + lane];
-        ih = hq->ih[KIND][n + lane];
-        if (KIND == 1) tc = hq->tc[n + lane];
-        h = hq->h[KIND][n + lane];
-        j = hq->j[KIND][n + lane];
-        ow = hq->owner[KIND][n + lane];
-        if (MODE == MODE_FILL) pos = hq->pos[KIND][n + lane];
-    }
     __syncwarp();
-    if (lane < rest) {
-        hq->b2[KIND][lane] = b2;
-        hq->ih[KIND][lane] = ih;
-        if (KIND == 1) hq->tc[lane] = tc;
-        hq->h[KIND][lane] = h;
-        hq->j[KIND][lane] = j;
-        hq->owner[KIND][lane] = ow;
-        if (MODE == MODE_FILL) hq->pos[KIND][lane] = pos;
-    }
-    __syncwarp();
-    count = rest;
+    head = (head + n) & (kPQ - 1);
+    count -= n;
 }
 
 // MODE_CHUNK: `want` consecutive chunks from the warp's block of chunks in
@@ -885,7 +843,7 @@ __device__ __forceinline__ bool decide(const St& S, int e, int o, double dx, dou
 // (MODE_FILL, MODE_CHUNK) all pairs are decided first, which gives every hit
 // its position.
 template <int KERNEL, int MODE, bool NF, typename Queue, typename St>
-__device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* tab, Queue* pq, int& pq_count,
+__device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* tab, Queue* pq, Queued& qn,
                                           unsigned long long* stash, St& S, unsigned mm, bool drain, float dx, float dy,
                                           float dz, float L, Sink<float>& k, unsigned& err)
 {
@@ -994,21 +952,17 @@ __device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* ta
         const unsigned pb = __ballot_sync(0xffffffffu, part);
         if (!pb && !drain) continue;
         if (part) {
-            const int i = pq_count + __popc(pb & ((1u << lane) - 1u));
-            pq->beta2[i] = beta2;
-            pq->u1[i] = u1;
-            pq->u2[i] = u2;
-            pq->A[i] = aw.x;
-            pq->w[i] = MODE == MODE_SCATTER ? S.org[o].coef : aw.y;
-            pq->j[i] = S.j[e];
-            pq->owner[i] = o | (near ? kPQNear : 0) | clip;
-            if (kStored) pq->pos[i] = pos;
+            const int i = (qn.part_head + qn.part + __popc(pb & ((1u << lane) - 1u))) & (kPQ - 1);
+            pq->item[i] = make_float4(beta2, u1, u2, MODE == MODE_SCATTER ? S.org[o].coef : aw.y);
+            if (Queue::kAux) pq->aux[i] = make_int4(S.j[e], (int)(uint32_t)pos, __float_as_int(aw.x), 0);
+            if (NF && !Queue::kAux) pq->A[i] = aw.x;
+            pq->owner[i] = o | (near ? kPQNear : 0) | clip | (kStored ? pos_hi(pos) : 0);
         }
-        pq_count += __popc(pb);
+        qn.part += __popc(pb);
         __syncwarp();
         // (at the end of the rays, drain, what is left: fewer than 32)
-        if (pq_count >= 32 || (drain && pq_count > 0))
-            flush_partials<KERNEL, MODE, NF>(P, tab, pq, pq_count, min(pq_count, 32), k);
+        if (qn.part >= 32 || (drain && qn.part > 0))
+            flush_partials<KERNEL, MODE, NF>(P, tab, pq, qn, min(qn.part, 32), k);
         if (drain) break;
     }
     __syncwarp();
@@ -1121,7 +1075,8 @@ __device__ __forceinline__ void pairs_f64(const TraceParams& P, const double2* l
         const unsigned fb = __ballot_sync(0xffffffffu, full), pb = __ballot_sync(0xffffffffu, hit && !full);
         const unsigned lt_mask = (1u << lane) - 1u;
         if (hit) {
-            const int kind = full ? 0 : 1, i = full ? qn.full + __popc(fb & lt_mask) : qn.part + __popc(pb & lt_mask);
+            const int kind = full ? 0 : 1, i = (full ? qn.full_head + qn.full + __popc(fb & lt_mask)
+                                                     : qn.part_head + qn.part + __popc(pb & lt_mask)) & (kPQ - 1);
             hq->b2[kind][i] = b2;
             if (!full) hq->tc[i] = tc;
             hq->h[kind][i] = S.q[e].w;
@@ -1134,9 +1089,9 @@ __device__ __forceinline__ void pairs_f64(const TraceParams& P, const double2* l
         qn.part += __popc(pb);
         __syncwarp();
         if (qn.full >= 32 || (drain && qn.full > 0))
-            flush_hits<KERNEL, MODE, NF, 0>(P, lt, hq, S, qn.full, min(qn.full, 32), L, k);
+            flush_hits<KERNEL, MODE, NF, 0>(P, lt, hq, S, qn.full, qn.full_head, min(qn.full, 32), L, k);
         if (qn.part >= 32 || (drain && qn.part > 0))
-            flush_hits<KERNEL, MODE, NF, 1>(P, lt, hq, S, qn.part, min(qn.part, 32), L, k);
+            flush_hits<KERNEL, MODE, NF, 1>(P, lt, hq, S, qn.part, qn.part_head, min(qn.part, 32), L, k);
         if (drain) break;
     }
     __syncwarp();
@@ -1269,10 +1224,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
             S.q[at] = cq;
             S.j[at] = cj;
             if constexpr (kF32) {
-                S.g[at] = make_float2(1.f / cq.w, __fmul_rn(cq.w, cq.w));
                 if (kWantA || kWantW) S.aw[at] = caw;
-            } else {
-                S.ih[at] = 1.0 / (double)cq.w;
             }
         };
         const bool mine = (pm >> lane) & 1u;
@@ -1285,6 +1237,11 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
         // the block is full (or the walk over): the lanes' candidates in it
         const int m = last ? ns : 32;
         __syncwarp();
+        {
+            const float h = lane < m ? S.q[lane].w : 1.f;
+            if constexpr (kF32) S.g[lane] = make_float2(MODE == MODE_COUNT ? 0.f : 1.f / h, __fmul_rn(h, h));
+            else if (MODE != MODE_COUNT) S.ih[lane] = 1.0 / (double)h;
+        }
         unsigned mask = candidates(S, m, pt.x, pt.y, pt.z, Lf);
         if (live) sk.ntest += (unsigned)m;
         else mask = 0u;
@@ -1302,7 +1259,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
         for (int e0 = 0; (total > 0 || drain) && e0 < 32; e0 += step) {
             const unsigned mm = step == 32 ? mask : mask & (((1u << step) - 1u) << e0);
             if constexpr (kF32)
-                pairs_f32<KERNEL, MODE, NF>(P, reinterpret_cast<const float2*>(tab), pq, qn.part, stash, S, mm, drain, dx,
+                pairs_f32<KERNEL, MODE, NF>(P, reinterpret_cast<const float2*>(tab), pq, qn, stash, S, mm, drain, dx,
                                             dy, dz, L, sk, err);
             else
                 pairs_f64<KERNEL, MODE, NF>(P, reinterpret_cast<const double2*>(tab), pq, qn, stash, S, mm, drain, dx, dy,
@@ -1405,7 +1362,7 @@ struct TraceLayout {
     static constexpr bool kTable = kQueue && KERNEL == URCHIN_KERNEL_M4;
     static constexpr bool kStored = MODE == MODE_FILL || MODE == MODE_CHUNK;
     using St = Staged<Real, MODE, NF>;
-    using Queue = std::conditional_t<kF32, PartQueue<kStored, NF>, HitQueue<kStored, NF>>;
+    using Queue = std::conditional_t<kF32, PartQueue<MODE, NF>, HitQueue<kStored, NF>>;
     static constexpr size_t up(size_t b) { return (b + 15) & ~size_t(15); }
     static constexpr size_t kBeam = up(sizeof(St) * 8);
     static constexpr size_t kStashAt = up(kBeam + sizeof(Beam) * 8);
@@ -1430,14 +1387,14 @@ static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, 
 // 277 -> 31 ms.
 // Three blocks of 256 per SM (80 registers a thread): with four (64
 // registers) the spills cost more than the fourth block's warps hide; with
-// two (no spills) too few warps are left to hide the loads.  The transpose
-// keeps four: its FP64 atomic adds want the warps more than the registers.
+// two (no spills) too few warps are left to hide the loads (128^3 box 69.6 and
+// 76.8 ms, transpose of the 65536-particle halo 6.3 and 6.3 ms).
 // FP64: bound by the FP64 pipe (84 % busy before the queues of full and partial
 // chords, at 17 of 32 lanes), two blocks; 16^3 lattice solve 18.3 -> 11.4 ms,
 // 24^3 box 10.7 -> 5.2 ms, 8000-particle halo 13.1 -> 8.8 ms, 9973 x 48 rays of
 // the 48^3 box (G_t) 25.3 -> 18.7 ms with queues and table logarithms.
 template <typename Real, int KERNEL, int MODE, bool NF>
-__global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 2 : MODE == MODE_SCATTER ? 4 : 3) k_trace(TraceParams P)
+__global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 2 : 3) k_trace(TraceParams P)
 {
     using Lay = TraceLayout<Real, KERNEL, MODE, NF>;
     constexpr bool kQueue = Lay::kQueue;
@@ -1453,7 +1410,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 2 : MODE == MODE_SCAT
         pq->own[threadIdx.x & 31] = 0u;
         if (NF) pq->own[(threadIdx.x & 31) + kPQNear] = 0u;
     }
-    Queued qn{0, 0};
+    Queued qn{0, 0, 0, 0};
     if ((threadIdx.x & 31) == 0) {
         stash[0] = 0ull;
         stash[1] = 0ull;
