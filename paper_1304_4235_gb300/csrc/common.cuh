@@ -104,25 +104,25 @@ int scan_counts_u64(const uint32_t* in, uint64_t* out, int64_t n, void* tmp, uin
 size_t radix_tmp_bytes(int64_t n, int64_t segs = 1);
 int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, void* tmp, cudaStream_t s, int64_t segs = 1);
 
-// Stream compaction: out[m] = i for every i with flags[i] != 0, in order;
-// *count_dev = m.  `tmp` needs compact_tmp_bytes(n).
+// Stream compaction: out[m] = i for every i with flags[i] != 0, in order, or,
+// with a permutation seq of [0, n), in the order of seq; *count_dev = m.  `tmp`
+// needs compact_tmp_bytes(n).
 size_t compact_tmp_bytes(int64_t n);
 int compact_indices(const uint8_t* flags, int64_t n, int32_t* out, uint32_t* count_dev, void* tmp,
-                    cudaStream_t s);
+                    cudaStream_t s, const int32_t* seq = nullptr);
 
 }  // namespace urchin
 
 // ---- the BVH object --------------------------------------------------------
-// Leaves are the subtrees of at most kLeafMax particles of the binary radix
-// tree, listed in the order of a depth-first walk that takes a node's leaf
-// children before its inner ones (the order in which a ray sums its hits).
-// Above them stands an implicit 32-ary tree over that list: entry g of level
-// l + 1 bounds entries [32 g, 32 g + 32) of level l.  An entry is two float4:
-//   boxes[2e] = (lo.xyz, first particle)   boxes[2e + 1] = (hi.xyz, particles)
-// (particle range in Morton order, as int bit patterns; levels above 0 hold
-// boxes only).  Level l starts at entry lev_off[l] and has lev_cnt[l]
-// entries; the top level (at least 1) has one.
-constexpr int kMaxLevels = 8;     // 32^6 = 2^30 particles, one per leaf, plus level 0 and a spare
+// Particles are kept in the order of a depth-first walk of the binary radix
+// tree that takes a node's leaf children (subtrees of at most kLeafMax
+// particles) before its inner ones: Morton order but for those swaps, and the
+// order in which a ray sums its hits ("Morton slot" below).  Above them stands
+// an implicit 32-ary tree: entry g of level 0 bounds the spheres of slots
+// [32 g, 32 g + 32), entry g of level l + 1 entries [32 g, 32 g + 32) of level
+// l.  An entry is two float4, lo.xyz and hi.xyz.  Level l starts at entry
+// lev_off[l] and has lev_cnt[l] entries; the top level (at least 1) has one.
+constexpr int kMaxLevels = 8;     // 2^30 particles: levels 0 to 5
 struct urchin_bvh {
     int64_t n = 0;
     int periodic = 0;
@@ -142,6 +142,7 @@ struct urchin_bvh {
     double* A64 = nullptr;        // [n]
     int32_t* perm = nullptr;      // [n] Morton slot -> original index
     int32_t* inv = nullptr;       // [n] original index -> Morton slot
+    int32_t* mslot = nullptr;     // [n] the slots in Morton order
     float2* ktab = nullptr;       // [kKTab + 1] full-chord M4 table
 };
 
@@ -154,7 +155,7 @@ constexpr unsigned kStInput = 8u;       // n_H or T not finite and > 0
 constexpr unsigned kStWarm = 16u;       // warm-start x outside (0, 1]
 constexpr unsigned kStSegment = 64u;    // stored-segment fill disagrees with its count
 
-constexpr int kLeafMax = 32;      // subtrees with <= kLeafMax particles become leaves
+constexpr int kLeafMax = 32;      // subtrees with <= kLeafMax particles are leaves of the particle order
 constexpr int kSegPad = 8;        // stored rays are padded to a multiple of kSegPad segments (zero
                                   // values, particle 0) so the SpMV reads 8 segments per lane
 constexpr int kKTab = 2048;       // intervals of the full-chord M4 table in t = b^2/h^2

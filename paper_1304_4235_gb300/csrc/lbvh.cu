@@ -3,11 +3,10 @@
 // The paper does not describe its search structure; this is a Morton-code
 // LBVH: 30-bit Morton codes of the sphere centres, stable radix sort, the
 // binary radix tree of Karras (2012, "Maximizing parallelism in the
-// construction of BVHs, octrees and k-d trees"), bottom-up refit of sphere
-// bounds.  Subtrees of at most kLeafMax particles become leaves, listed in a
-// fixed depth-first order, and an implicit 32-ary tree of boxes over that list
-// is what the traversal reads (one lane tests one child).  The particle data
-// are copied into Morton order so that a leaf is a contiguous range.
+// construction of BVHs, octrees and k-d trees").  The radix tree only orders
+// the particles (k_leaf_order); the traversal reads an implicit 32-ary tree of
+// boxes over the ordered particles, 32 to a block (one lane tests one sphere
+// or one child).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -162,7 +161,7 @@ __device__ __forceinline__ int delta(const uint32_t* __restrict__ codes, int n, 
 // splits it at the highest differing bit.  Children are encoded >= 0 for an
 // internal node, ~leaf for a leaf (particle).
 __global__ void k_karras(const uint32_t* __restrict__ codes, int n, int32_t* child_l, int32_t* child_r,
-                         int32_t* first, int32_t* last, int32_t* parent_int, int32_t* parent_leaf)
+                         int32_t* first, int32_t* last, int32_t* parent_int)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
@@ -185,9 +184,9 @@ __global__ void k_karras(const uint32_t* __restrict__ codes, int n, int32_t* chi
     int lo = min(i, j), hi = max(i, j);
     first[i] = lo;
     last[i] = hi;
-    if (lo == g) { child_l[i] = ~g; parent_leaf[g] = i; }
+    if (lo == g) child_l[i] = ~g;
     else { child_l[i] = g; parent_int[g] = i; }
-    if (hi == g + 1) { child_r[i] = ~(g + 1); parent_leaf[g + 1] = i; }
+    if (hi == g + 1) child_r[i] = ~(g + 1);
     else { child_r[i] = g + 1; parent_int[g + 1] = i; }
     if (i == 0) parent_int[0] = -1;
 }
@@ -205,52 +204,6 @@ __device__ __forceinline__ void sphere_box(float4 p, float lo[3], float hi[3])
     hi[2] = __fadd_ru(__fadd_ru(p.z, p.w), pad);
 }
 
-__device__ __forceinline__ void child_box(int32_t c, const float4* __restrict__ xyzh, const float* boxes,
-                                          float lo[3], float hi[3])
-{
-    if (c < 0) {
-        sphere_box(xyzh[~c], lo, hi);
-    } else {
-        const float* b = boxes + 6 * (int64_t)c;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = __ldcg(b + a);
-            hi[a] = __ldcg(b + 3 + a);
-        }
-    }
-}
-
-__global__ void k_refit(const float4* __restrict__ xyzh, int n, const int32_t* child_l,
-                        const int32_t* child_r, const int32_t* parent_int, const int32_t* parent_leaf,
-                        float* boxes, unsigned* visits, unsigned* err)
-{
-    int leaf = blockIdx.x * blockDim.x + threadIdx.x;
-    if (leaf >= n) return;
-    int p = parent_leaf[leaf];
-    // the tree is at most 62 levels deep (30-bit codes, 32-bit index
-    // tie-break); the cap only guards against a malformed parent chain
-    for (int level = 0; p >= 0; ++level) {
-        if (level > 128) {
-            atomicOr(err, 4u);
-            return;
-        }
-        __threadfence();
-        unsigned old = atomicAdd(&visits[p], 1u);
-        if (old == 0) return;          // sibling subtree not finished yet
-        __threadfence();
-        float llo[3], lhi[3], rlo[3], rhi[3];
-        child_box(child_l[p], xyzh, boxes, llo, lhi);
-        child_box(child_r[p], xyzh, boxes, rlo, rhi);
-        float* b = boxes + 6 * (int64_t)p;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            __stcg(b + a, fminf(llo[a], rlo[a]));
-            __stcg(b + 3 + a, fmaxf(lhi[a], rhi[a]));
-        }
-        p = parent_int[p];
-    }
-}
-
 // Particles of child c of an inner node (c < 0: the single particle ~c).
 __device__ __forceinline__ int child_size(int32_t c, const int32_t* __restrict__ first,
                                           const int32_t* __restrict__ last)
@@ -258,45 +211,22 @@ __device__ __forceinline__ int child_size(int32_t c, const int32_t* __restrict__
     return c < 0 ? 1 : last[c] - first[c] + 1;
 }
 
-__device__ __forceinline__ int child_first(int32_t c, const int32_t* __restrict__ first)
-{
-    return c < 0 ? ~c : first[c];
-}
-
-// flags[p] = 1 where a leaf starts at particle p: the children of at most
-// kLeafMax particles of the root and of every larger inner node
-__global__ void k_leaf_flags(int n, const int32_t* __restrict__ child_l, const int32_t* __restrict__ child_r,
-                             const int32_t* __restrict__ first, const int32_t* __restrict__ last, uint32_t* flags)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n - 1 || (i > 0 && last[i] - first[i] + 1 <= kLeafMax)) return;
-    const int32_t l = child_l[i], r = child_r[i];
-    if (child_size(l, first, last) <= kLeafMax) flags[child_first(l, first)] = 1u;
-    if (child_size(r, first, last) <= kLeafMax) flags[child_first(r, first)] = 1u;
-}
-
-// Leaves in subtree c, from the exclusive scan of the flags (start[n] = all)
-__device__ __forceinline__ int leaves_in(int32_t c, const int32_t* __restrict__ first,
-                                         const int32_t* __restrict__ last, const uint32_t* __restrict__ start)
-{
-    const int lo = child_first(c, first);
-    return (int)(start[lo + child_size(c, first, last)] - start[lo]);
-}
-
-// Every leaf to its place in the depth-first list (leaf children before
-// inner ones, left before right): the leaves that precede it below each of
-// its ancestors, summed on the way up.
-__global__ void k_leaf_place(const float4* __restrict__ xyzh, int n, const int32_t* __restrict__ child_l,
-                             const int32_t* __restrict__ child_r, const int32_t* __restrict__ first,
-                             const int32_t* __restrict__ last, const int32_t* __restrict__ parent_int,
-                             const float* boxes, const uint32_t* __restrict__ start, int n_leaves, float4* out,
-                             unsigned* err)
+// order[s] = the particle of slot s (and mslot, the slots in Morton order): the subtrees of at most kLeafMax
+// particles ("leaves": the children of at most kLeafMax particles of the root
+// and of every larger inner node) in the order of a depth-first walk that
+// takes a node's leaf children before its inner ones, left before right, a
+// leaf's particles in Morton order.  A leaf's first slot is the sum, over its
+// ancestors, of the particles that precede it below each.
+__global__ void k_leaf_order(int n, const int32_t* __restrict__ child_l, const int32_t* __restrict__ child_r,
+                             const int32_t* __restrict__ first, const int32_t* __restrict__ last,
+                             const int32_t* __restrict__ parent_int, const int32_t* __restrict__ idx, int32_t* order,
+                             int32_t* mslot, unsigned* err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1 || (i > 0 && last[i] - first[i] + 1 <= kLeafMax)) return;
     const int32_t cl = child_l[i], cr = child_r[i];
-    const bool ll = child_size(cl, first, last) <= kLeafMax, lr = child_size(cr, first, last) <= kLeafMax;
-    if (!ll && !lr) return;
+    const int nl = child_size(cl, first, last), nr = child_size(cr, first, last);
+    if (nl > kLeafMax && nr > kLeafMax) return;
     int at = 0, c = i;
     int p = i > 0 ? parent_int[i] : -1;
     // the tree is at most 62 levels deep; the cap only guards against a
@@ -308,36 +238,50 @@ __global__ void k_leaf_place(const float4* __restrict__ xyzh, int n, const int32
         }
         const int32_t pl = child_l[p], pr = child_r[p];
         if (c == pr) {
-            at += child_size(pl, first, last) <= kLeafMax ? 1 : leaves_in(pl, first, last, start);
-        } else if (child_size(pr, first, last) <= kLeafMax) {
-            ++at;
+            at += child_size(pl, first, last);
+        } else {
+            const int m = child_size(pr, first, last);
+            if (m <= kLeafMax) at += m;
         }
         c = p;
         p = p > 0 ? parent_int[p] : -1;
     }
-    float lo[3], hi[3];
-    for (int q = 0; q < 2; ++q) {
-        if (!(q == 0 ? ll : lr)) continue;
-        const int32_t ch = q == 0 ? cl : cr;
-        const int e = at + (q == 1 && ll ? 1 : 0);
-        if (e < 0 || e >= n_leaves) {              // never true for a well-formed tree
-            atomicOr(err, 4u);
-            return;
-        }
-        child_box(ch, xyzh, boxes, lo, hi);
-        out[2 * (int64_t)e] = make_float4(lo[0], lo[1], lo[2], __int_as_float(child_first(ch, first)));
-        out[2 * (int64_t)e + 1] =
-            make_float4(hi[0], hi[1], hi[2], __int_as_float(child_size(ch, first, last)));
+    const int f = first[i];
+    if (at < 0 || at + (nl <= kLeafMax ? nl : 0) + (nr <= kLeafMax ? nr : 0) > n) {   // never true for a well-formed tree
+        atomicOr(err, 4u);
+        return;
     }
+    if (nl <= kLeafMax)
+        for (int q = 0; q < nl; ++q, ++at) {
+            order[at] = idx[f + q];
+            mslot[f + q] = at;
+        }
+    if (nr <= kLeafMax)
+        for (int q = nl; q < nl + nr; ++q, ++at) {
+            order[at] = idx[f + q];
+            mslot[f + q] = at;
+        }
 }
 
-// n == 1: one leaf
-__global__ void k_leaf_single(const float4* __restrict__ xyzh, float4* out)
+// Level 0 of the 32-ary tree: a warp bounds the spheres of 32 slots.
+__global__ void k_blocks(const float4* __restrict__ xyzh, int n, float4* out, int n_out)
 {
-    float lo[3], hi[3];
-    sphere_box(xyzh[0], lo, hi);
-    out[0] = make_float4(lo[0], lo[1], lo[2], __int_as_float(0));
-    out[1] = make_float4(hi[0], hi[1], hi[2], __int_as_float(1));
+    const int g = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (g >= n_out) return;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    if (32 * g + lane < n) sphere_box(xyzh[32 * g + lane], lo, hi);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+        }
+    if (lane == 0) {
+        out[2 * (int64_t)g] = make_float4(lo[0], lo[1], lo[2], 0.f);
+        out[2 * (int64_t)g + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+    }
 }
 
 // One level of the 32-ary tree: a warp bounds 32 entries of the level below.
@@ -377,6 +321,7 @@ void free_bvh_arrays(urchin_bvh* b)
     cudaFree(b->A64);
     cudaFree(b->perm);
     cudaFree(b->inv);
+    cudaFree(b->mslot);
     cudaFree(b->ktab);
     b->ktab = nullptr;
     b->boxes = nullptr;
@@ -385,6 +330,7 @@ void free_bvh_arrays(urchin_bvh* b)
     b->A64 = nullptr;
     b->perm = nullptr;
     b->inv = nullptr;
+    b->mslot = nullptr;
 }
 
 int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaStream_t s)
@@ -400,6 +346,7 @@ int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaS
     URCHIN_TRY_CUDA(cudaMalloc(&b->A64, sizeof(double) * (size_t)n));
     URCHIN_TRY_CUDA(cudaMalloc(&b->perm, sizeof(int32_t) * (size_t)n));
     URCHIN_TRY_CUDA(cudaMalloc(&b->inv, sizeof(int32_t) * (size_t)n));
+    URCHIN_TRY_CUDA(cudaMalloc(&b->mslot, sizeof(int32_t) * (size_t)n));
     URCHIN_TRY_CUDA(cudaMalloc(&b->ktab, sizeof(float2) * (kKTab + 1)));
     {
         static float2 table[kKTab + 1];
@@ -426,11 +373,7 @@ int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaS
     size_t o_first = lay.take((size_t)ni * 4);
     size_t o_last = lay.take((size_t)ni * 4);
     size_t o_pint = lay.take((size_t)ni * 4);
-    size_t o_pleaf = lay.take((size_t)n * 4);
-    size_t o_boxes = lay.take((size_t)ni * 6 * 4);
-    size_t o_visits = lay.take((size_t)ni * 4);
-    size_t o_flags = lay.take((size_t)(n + 1) * 4);
-    size_t o_stmp = lay.take(scan_tmp_bytes(n + 1));
+    size_t o_order = lay.take((size_t)n * 4);
     Scratch scr;
     URCHIN_TRY(scr.alloc(lay.bytes, s));
     unsigned* bounds = scr.at<unsigned>(o_bounds);
@@ -457,46 +400,30 @@ int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaS
     k_morton<<<grid, 256, 0, s>>>(p->pos_x, p->pos_y, p->pos_z, n, bounds, codes, idx);
     URCHIN_TRY(launched());
     URCHIN_TRY(radix_sort_pairs(codes, idx, n, 30, scr.at<void>(o_radix), s));
+    int32_t* order = idx;
+    if (n == 1) URCHIN_TRY_CUDA(cudaMemsetAsync(b->mslot, 0, sizeof(int32_t), s));
+    if (n > 1) {
+        int32_t* cl = scr.at<int32_t>(o_cl);
+        int32_t* cr = scr.at<int32_t>(o_cr);
+        int32_t* first = scr.at<int32_t>(o_first);
+        int32_t* last = scr.at<int32_t>(o_last);
+        int32_t* pint = scr.at<int32_t>(o_pint);
+        const unsigned gi = (unsigned)((ni + 255) / 256);
+        order = scr.at<int32_t>(o_order);
+        k_karras<<<gi, 256, 0, s>>>(codes, (int)n, cl, cr, first, last, pint);
+        URCHIN_TRY(launched());
+        k_leaf_order<<<gi, 256, 0, s>>>((int)n, cl, cr, first, last, pint, idx, order, b->mslot, bounds + 7);
+        URCHIN_TRY(launched());
+    }
     const double mass_to_A = sigma_th_cm2() * 8.0 / kPi;
-    k_gather<<<grid, 256, 0, s>>>(p->pos_x, p->pos_y, p->pos_z, p->h, p->mass_H, idx, n, mass_to_A,
+    k_gather<<<grid, 256, 0, s>>>(p->pos_x, p->pos_y, p->pos_z, p->h, p->mass_H, order, n, mass_to_A,
                                   b->unit_cm, b->xyzh, b->A32, b->A64, b->perm, b->inv,
                                   bounds + 7);
     URCHIN_TRY(launched());
-
-    int n_leaves = 1;
-    int32_t* cl = scr.at<int32_t>(o_cl);
-    int32_t* cr = scr.at<int32_t>(o_cr);
-    int32_t* first = scr.at<int32_t>(o_first);
-    int32_t* last = scr.at<int32_t>(o_last);
-    int32_t* pint = scr.at<int32_t>(o_pint);
-    float* boxes = scr.at<float>(o_boxes);
-    uint32_t* start = scr.at<uint32_t>(o_flags);
-    const unsigned gi = (unsigned)((ni + 255) / 256);
-    if (n > 1) {
-        int32_t* pleaf = scr.at<int32_t>(o_pleaf);
-        unsigned* visits = scr.at<unsigned>(o_visits);
-        unsigned gl = (unsigned)((n + 255) / 256);
-        URCHIN_TRY_CUDA(cudaMemsetAsync(visits, 0, (size_t)ni * 4, s));
-        URCHIN_TRY_CUDA(cudaMemsetAsync(start, 0, (size_t)(n + 1) * 4, s));
-        k_karras<<<gi, 256, 0, s>>>(codes, (int)n, cl, cr, first, last, pint, pleaf);
-        URCHIN_TRY(launched());
-        k_leaf_flags<<<gi, 256, 0, s>>>((int)n, cl, cr, first, last, start);
-        URCHIN_TRY(launched());
-        // start[p] = leaves before particle p; start[n] = all (its flag is 0)
-        URCHIN_TRY(scan_exclusive_u32(start, start, n + 1, scr.at<void>(o_stmp), nullptr, s));
-        uint32_t total = 0;
-        URCHIN_TRY_CUDA(cudaMemcpyAsync(&total, start + n, sizeof(total), cudaMemcpyDeviceToHost, s));
-        k_refit<<<gl, 256, 0, s>>>(b->xyzh, (int)n, cl, cr, pint, pleaf, boxes, visits, bounds + 7);
-        URCHIN_TRY(launched());
-        URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
-        if (total < 1 || (int64_t)total > n)
-            return set_error(URCHIN_ERR_CUDA, "urchin_build_bvh: %u leaves for %lld particles", total, (long long)n);
-        n_leaves = (int)total;
-    }
-    // levels up to the first of one entry above the leaves
+    // levels up to the first of one entry above the blocks
     int64_t entries = 0;
     b->n_lev = 0;
-    for (int l = 0, c = n_leaves;; ++l, c = (c + 31) / 32) {
+    for (int l = 0, c = (int)((n + 31) / 32);; ++l, c = (c + 31) / 32) {
         if (l >= kMaxLevels) return set_error(URCHIN_ERR_CUDA, "urchin_build_bvh: too many tree levels");
         b->lev_off[l] = (int)entries;
         b->lev_cnt[l] = c;
@@ -505,11 +432,7 @@ int build(const urchin_particles* p, const urchin_box* box, urchin_bvh* b, cudaS
         if (l > 0 && c == 1) break;
     }
     URCHIN_TRY_CUDA(cudaMalloc(&b->boxes, sizeof(float4) * 2 * (size_t)entries));
-    if (n > 1)
-        k_leaf_place<<<gi, 256, 0, s>>>(b->xyzh, (int)n, cl, cr, first, last, pint, boxes, start, n_leaves, b->boxes,
-                                        bounds + 7);
-    else
-        k_leaf_single<<<1, 1, 0, s>>>(b->xyzh, b->boxes);
+    k_blocks<<<(unsigned)((b->lev_cnt[0] + 7) / 8), 256, 0, s>>>(b->xyzh, (int)n, b->boxes, b->lev_cnt[0]);
     URCHIN_TRY(launched());
     for (int l = 1; l <= b->n_lev; ++l) {
         const int c = b->lev_cnt[l];

@@ -1346,7 +1346,7 @@ int Solver::first_sweep()
     URCHIN_TRY(columns(nullptr, n, 1));
     URCHIN_TRY(timed_sweep(sweep_args(nullptr, n, 1), s));
     uint32_t* cnt = reinterpret_cast<uint32_t*>(misc + 2);
-    URCHIN_TRY(compact_indices(active, n, list, cnt, comp_tmp, s));
+    URCHIN_TRY(compact_indices(active, n, list, cnt, comp_tmp, s, bvh->mslot));
     const int32_t* full = nullptr;                // sweep 0's ray order of all particles
     for (const OrderEntry& e : orders)
         if (e.items == nullptr && e.n == n) full = e.order;
@@ -1751,7 +1751,7 @@ int Solver::adjoint(const uint8_t* state_orig, const double* xbar_orig, int cold
     k_state_in<<<gn, 256, 0, s>>>(bvh->perm, state_orig, n, active, latch, status);
     URCHIN_TRY(launched());
     uint32_t* cnt = reinterpret_cast<uint32_t*>(misc + 2);
-    URCHIN_TRY(compact_indices(active, n, list, cnt, comp_tmp, s));
+    URCHIN_TRY(compact_indices(active, n, list, cnt, comp_tmp, s, bvh->mslot));
     items_changed();
     uint32_t hc = 0;
     URCHIN_TRY_CUDA(cudaMemcpyAsync(&hc, cnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));

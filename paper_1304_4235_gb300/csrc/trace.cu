@@ -10,7 +10,7 @@
 // neighbouring origins in one direction from an atomic queue, so the 32 rays
 // of a warp are parallel and start close together (a beam).  The beam walks
 // the 32-ary box tree as one packet, each lane testing one child of the
-// current entry against the beam; at a leaf each lane tests one sphere
+// current entry against the beam; at a block of 32 each lane tests one sphere
 // against the beam, and the spheres that pass are staged in shared memory.
 // Every 32 staged spheres, each lane tests them against its own ray in the
 // beam's frame (a handful of packed FP32 operations per sphere, conservative)
@@ -1099,13 +1099,12 @@ __device__ __forceinline__ void pairs_f64(const TraceParams& P, const double2* l
     __syncwarp();
 }
 
-// The tree walk of one packet: next() gives the leaves that the beam may
-// reach, in the list's order, one after the other.
+// The tree walk of one packet: next() gives the blocks of 32 spheres that the
+// beam may reach, in their order, one after the other.
 struct Walk {
     int lev, node;                // current entry: number `node` of level `lev`
     unsigned mask;                // its children still to be entered
     unsigned pend;                // lane l holds level l's mask while its subtrees are walked
-    int lref, lcnt;               // children that are leaves: the lane's leaf
     unsigned visits;
     bool fresh;                   // the current entry's children have not been tested
 
@@ -1116,8 +1115,6 @@ struct Walk {
         if (c < P.lev_cnt[lev - 1]) {
             const float4* b = P.boxes + 2 * ((int64_t)P.lev_off[lev - 1] + c);
             const float4 lo = __ldg(b), hi = __ldg(b + 1);
-            lref = __float_as_int(lo.w);
-            lcnt = __float_as_int(hi.w);
             pass = beam_box(B, lo, hi);
         }
         mask = __ballot_sync(0xffffffffu, pass);
@@ -1148,8 +1145,8 @@ struct Walk {
             const int c = __ffs(mask) - 1;
             mask &= mask - 1u;
             if (lev == 1) {
-                ref = __shfl_sync(0xffffffffu, lref, c);
-                cnt = __shfl_sync(0xffffffffu, lcnt, c);
+                ref = 32 * (32 * node + c);
+                cnt = min(32, P.n - ref);
                 return true;
             }
             if ((int)(threadIdx.x & 31) == lev) pend = mask;
@@ -1176,7 +1173,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
     constexpr bool kWantA = kF32 && MODE != MODE_COUNT && (MODE != MODE_TAU || NF);
     Walk W;
     W.start(P);
-    int ref = 0, cnt = 0;            // the current leaf (none at first) while the next one is on its way
+    int ref = 0, cnt = 0;            // the current block (none at first) while the next one is on its way
     bool more = !drain;
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
     float2 aw = make_float2(0.f, 0.f);
@@ -1196,7 +1193,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
         const float2 caw = aw;
         const int cj = ref + lane;
         if (!last) {
-            // sphere (one per lane) against the beam; the next leaf's spheres are on their way meanwhile
+            // sphere (one per lane) against the beam; the next block of spheres is on its way meanwhile
             bool pass = false;
             if (lane < cnt) {
                 const float4 c4 = B.c, a4 = B.e1, b4 = B.e2, d4 = B.d;

@@ -442,16 +442,19 @@ int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, void* t
 // ---------------------------------------------------------------------------
 // Compaction
 // ---------------------------------------------------------------------------
-__global__ void k_flags_u32(const uint8_t* flags, uint32_t* out, int64_t n)
+__global__ void k_flags_u32(const uint8_t* flags, const int32_t* seq, uint32_t* out, int64_t n)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = flags[i] ? 1u : 0u;
+        out[i] = flags[seq ? seq[i] : i] ? 1u : 0u;
 }
 
-__global__ void k_compact_scatter(const uint8_t* flags, const uint32_t* pos, int64_t n, int32_t* out)
+__global__ void k_compact_scatter(const uint8_t* flags, const int32_t* seq, const uint32_t* pos, int64_t n,
+                                  int32_t* out)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (flags[i] && pos[i] < n) out[pos[i]] = (int32_t)i;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t q = seq ? seq[i] : (int32_t)i;
+        if (flags[q] && pos[i] < n) out[pos[i]] = q;
+    }
 }
 
 size_t compact_tmp_bytes(int64_t n)
@@ -460,16 +463,16 @@ size_t compact_tmp_bytes(int64_t n)
 }
 
 int compact_indices(const uint8_t* flags, int64_t n, int32_t* out, uint32_t* count_dev, void* tmp,
-                    cudaStream_t s)
+                    cudaStream_t s, const int32_t* seq)
 {
     uint32_t* pos = static_cast<uint32_t*>(tmp);
     void* stmp = static_cast<char*>(tmp) + (((size_t)n * 4 + 255) & ~size_t(255));
     unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, 256), 4096);
     if (grid == 0) grid = 1;
-    k_flags_u32<<<grid, 256, 0, s>>>(flags, pos, n);
+    k_flags_u32<<<grid, 256, 0, s>>>(flags, seq, pos, n);
     URCHIN_TRY(launched());
     URCHIN_TRY(scan_exclusive_u32(pos, pos, n, stmp, count_dev, s));
-    k_compact_scatter<<<grid, 256, 0, s>>>(flags, pos, n, out);
+    k_compact_scatter<<<grid, 256, 0, s>>>(flags, seq, pos, n, out);
     URCHIN_TRY(launched());
     return URCHIN_OK;
 }
