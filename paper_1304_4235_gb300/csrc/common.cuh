@@ -192,7 +192,7 @@ struct TraceJob {
     const uint64_t* row_ptr;      // mode 2: [R * n + 1] offsets of each ray's segments (same index)
     int32_t* seg_col;             // mode 2: Morton index of the particle per segment, or NULL:
     uint16_t* seg_lo;             //    its low 16 bits and
-    uint8_t* seg_hi;              //    its high 8 bits (FP32 segments, every index below 2^24)
+    uint8_t* seg_hi;              //    its high 8 bits (FP32 segments, every index below 2^24; NULL: below 2^16)
     void* seg_val;                // mode 2: A_j * chord integral per segment (precision's type)
     const void* coef;             // mode 3: per-ray coefficient (precision's type), indexed like out
     double* xbar;                 // mode 3: [n] Morton order, accumulated with atomics

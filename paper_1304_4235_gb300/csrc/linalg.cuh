@@ -12,7 +12,7 @@ struct SpmvArgs {
     const uint64_t* row_ptr;     // [R * n_rows_per_k + 1], multiples of kSegPad
     const int32_t* col;          // [nnz] Morton particle index (padding: 0), or NULL:
     const uint16_t* lo;          //   its low 16 bits
-    const uint8_t* hi;           //   and high 8 bits (FP32 only)
+    const uint8_t* hi;           //   and high 8 bits (FP32 only; NULL: every index below 2^16)
     const void* val;             // [nnz] A_j * chord integral (float or double; padding: 0)
     const void* xvec;            // [n] vector the columns are linear in (Morton order, same type)
     const int32_t* items;        // [n_items] Morton particle of each evaluated ray origin (NULL = identity)

@@ -788,7 +788,8 @@ int Solver::count_spmv(const int32_t* items, int64_t n_items)
         seg = (int64_t)h;
         if (items == list && n_items == n_act) active_nnz = seg;
     }
-    const int64_t isz = (seg_col || chunked) ? (int64_t)sizeof(int32_t) : (int64_t)(sizeof(uint16_t) + sizeof(uint8_t));
+    const int64_t isz = (seg_col || chunked) ? (int64_t)sizeof(int32_t)
+                                             : (int64_t)sizeof(uint16_t) + (seg_hi ? (int64_t)sizeof(uint8_t) : 0);
     stats.spmv_bytes += seg * (isz + (int64_t)vsz) + n_items * P.R * (int64_t)vsz + n * (int64_t)vsz;
     return URCHIN_OK;
 }
@@ -915,6 +916,9 @@ __global__ void k_clear_inactive_rows(const uint8_t* __restrict__ active, int64_
 //     pays one traversal more than storing at once (262144-particle halo:
 //     292 sweeps, 0.86 s; one traversal 0.04 s).
 constexpr int kAutoStoreSweep = 2;
+
+// Up to this many particles a stored index needs its low 16 bits only.
+constexpr int64_t kSegLowOnly = int64_t(1) << 16;
 
 // The stored lists for a product: rows (row_ptr) or linked chunks.
 void Solver::spmv_lists(SpmvArgs& A) const
@@ -1062,7 +1066,8 @@ int Solver::compact_chunks()
     Layout lay;
     const size_t o_col = split ? 0 : lay.take(sizeof(int32_t) * (size_t)nnz);
     const size_t o_lo = split ? lay.take(sizeof(uint16_t) * (size_t)nnz) : 0;
-    const size_t o_hi = split ? lay.take(sizeof(uint8_t) * (size_t)nnz) : 0;
+    const bool high = split && n > kSegLowOnly;
+    const size_t o_hi = high ? lay.take(sizeof(uint8_t) * (size_t)nnz) : 0;
     const size_t o_val = lay.take(sizeof(float) * (size_t)nnz);
     size_t free_b = 0, total_b = 0;
     URCHIN_TRY_CUDA(cudaMemGetInfo(&free_b, &total_b));
@@ -1079,7 +1084,7 @@ int Solver::compact_chunks()
     C.rows = rays;
     C.col = split ? nullptr : seg.at<int32_t>(o_col);
     C.lo = split ? seg.at<uint16_t>(o_lo) : nullptr;
-    C.hi = split ? seg.at<uint8_t>(o_hi) : nullptr;
+    C.hi = high ? seg.at<uint8_t>(o_hi) : nullptr;
     C.val = seg.at<float>(o_val);
     URCHIN_TRY(launch_chunk_compact(C, s));
     seg_col = C.col;
@@ -1182,7 +1187,8 @@ int Solver::columns(const int32_t* items, int64_t n_items, int sweep0, bool buil
     const size_t vsz = f64 ? sizeof(double) : sizeof(float);
     // FP32 segments keep the particle index as 16 + 8 bits (7 bytes per segment)
     const bool split = !f64 && n <= (int64_t(1) << 24);
-    const size_t isz = split ? sizeof(uint16_t) + sizeof(uint8_t) : sizeof(int32_t);
+    const bool high = split && n > kSegLowOnly;
+    const size_t isz = split ? sizeof(uint16_t) + (high ? sizeof(uint8_t) : 0) : sizeof(int32_t);
     const size_t need = (size_t)nnz * (isz + vsz) + 1024;
     bool fits = true;
     if (P.segments == URCHIN_SEG_AUTO) {
@@ -1195,7 +1201,7 @@ int Solver::columns(const int32_t* items, int64_t n_items, int sweep0, bool buil
         Layout lay;
         size_t o_col = split ? 0 : lay.take(sizeof(int32_t) * (size_t)nnz);
         size_t o_lo = split ? lay.take(sizeof(uint16_t) * (size_t)nnz) : 0;
-        size_t o_hi = split ? lay.take(sizeof(uint8_t) * (size_t)nnz) : 0;
+        size_t o_hi = high ? lay.take(sizeof(uint8_t) * (size_t)nnz) : 0;
         size_t o_val = lay.take(vsz * (size_t)nnz);
         int st = seg.alloc(lay.bytes, s);
         if (st != URCHIN_OK) {
@@ -1205,7 +1211,7 @@ int Solver::columns(const int32_t* items, int64_t n_items, int sweep0, bool buil
         } else {
             seg_col = split ? nullptr : seg.at<int32_t>(o_col);
             seg_lo = split ? seg.at<uint16_t>(o_lo) : nullptr;
-            seg_hi = split ? seg.at<uint8_t>(o_hi) : nullptr;
+            seg_hi = high ? seg.at<uint8_t>(o_hi) : nullptr;
             seg_val = seg.at<void>(o_val);
         }
     }

@@ -62,7 +62,7 @@ struct TraceParams {
     const uint64_t* row_ptr;      // MODE_FILL: first segment of each ray (same index), size + 1
     int32_t* seg_col;             // MODE_FILL: Morton index of the particle, or NULL:
     uint16_t* seg_lo;             //   its low 16 bits
-    uint8_t* seg_hi;              //   and high 8 bits (indices below 2^24)
+    uint8_t* seg_hi;              //   and high 8 bits (indices below 2^24; NULL: below 2^16)
     void* seg_val;                // MODE_FILL: A_j * chord integral (float or double)
     const float* A32;
     const double* A64;
@@ -385,15 +385,18 @@ struct Beam {
     float4 r;                     // its radii along d x (x, y, z), margin included; 0
 };
 
+// Smallest and largest of the warp's values (one reduction instruction each).
 __device__ __forceinline__ float wmin(float v)
 {
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 __device__ __forceinline__ float wmax(float v)
 {
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 // Called by all 32 lanes with the same direction d and length L; (sx, sy, sz)
@@ -561,7 +564,7 @@ __device__ __forceinline__ void store_index(const TraceParams& P, int64_t pos, i
         return;
     }
     P.seg_lo[pos] = (uint16_t)((uint32_t)j & 0xffffu);
-    P.seg_hi[pos] = (uint8_t)(((uint32_t)j >> 16) & 0xffu);
+    if (P.seg_hi) P.seg_hi[pos] = (uint8_t)(((uint32_t)j >> 16) & 0xffu);
 }
 
 // ---- deferred partial chords ------------------------------------------------
@@ -1307,24 +1310,38 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
         const unsigned lv = __ballot_sync(0xffffffffu, in);
         left &= ~lv;
         // the images of the box that the unshifted beam may reach, 32 at a
-        // time, then one after the other in the order of their indices
+        // time, then one after the other in the order of their indices; away
+        // from the faces that is the box itself (image `home`), with the same
+        // beam
+        const int home = images / 2;
+        bool have_beam = false;
         for (int i0 = 0; i0 < (drain ? 1 : images); i0 += 32) {
             unsigned im = 1u;
             if (images > 1 && !drain) {
-                make_beam<Real>(beam, lv, in, Real(o.x), Real(o.y), Real(o.z), (float)dx, (float)dy, (float)dz, Lf);
-                const int i = i0 + lane;
-                bool pass = false;
-                if (i < images) {
-                    const float ax = (float)(i / (side * side) - nimg) * (float)P.Lbox,
-                                ay = (float)((i / side) % side - nimg) * (float)P.Lbox,
-                                az = (float)(i % side - nimg) * (float)P.Lbox;
-                    // the shifted faces and the shifted origins are each rounded
-                    const float m = 1e-6f * (fabsf(ax) + fabsf(ay) + fabsf(az) + (float)P.Lbox);
-                    pass = beam_box(*beam,
-                                    make_float4(P.root_lo[0] + ax - m, P.root_lo[1] + ay - m, P.root_lo[2] + az - m, 0.f),
-                                    make_float4(P.root_hi[0] + ax + m, P.root_hi[1] + ay + m, P.root_hi[2] + az + m, 0.f));
+                pt = make_beam<Real>(beam, lv, in, Real(o.x), Real(o.y), Real(o.z), (float)dx, (float)dy, (float)dz, Lf);
+                // the shifted faces and the shifted origins are each rounded
+                const float Lb = (float)P.Lbox, m1 = 2e-6f * (Lb + fabsf(P.root_lo[0]) + fabsf(P.root_hi[0]) + fabsf(P.root_lo[1]) +
+                                                              fabsf(P.root_hi[1]) + fabsf(P.root_lo[2]) + fabsf(P.root_hi[2]));
+                const float4 bc = beam->c, bo = beam->o;
+                if (bc.x + bo.x < P.root_lo[0] + Lb - m1 && bc.x - bo.x > P.root_hi[0] - Lb + m1 &&
+                    bc.y + bo.y < P.root_lo[1] + Lb - m1 && bc.y - bo.y > P.root_hi[1] - Lb + m1 &&
+                    bc.z + bo.z < P.root_lo[2] + Lb - m1 && bc.z - bo.z > P.root_hi[2] - Lb + m1) {
+                    i0 = home & ~31;
+                    im = 1u << (home & 31);
+                    have_beam = true;
+                } else {
+                    const int i = i0 + lane;
+                    bool pass = false;
+                    if (i < images) {
+                        const float ax = (float)(i / (side * side) - nimg) * Lb, ay = (float)((i / side) % side - nimg) * Lb,
+                                    az = (float)(i % side - nimg) * Lb;
+                        const float m = 1e-6f * (fabsf(ax) + fabsf(ay) + fabsf(az) + Lb);
+                        pass = beam_box(*beam,
+                                        make_float4(P.root_lo[0] + ax - m, P.root_lo[1] + ay - m, P.root_lo[2] + az - m, 0.f),
+                                        make_float4(P.root_hi[0] + ax + m, P.root_hi[1] + ay + m, P.root_hi[2] + az + m, 0.f));
+                    }
+                    im = __ballot_sync(0xffffffffu, pass);
                 }
-                im = __ballot_sync(0xffffffffu, pass);
             }
             for (; im; im &= im - 1u) {
                 const int i = i0 + __ffs(im) - 1;
@@ -1340,11 +1357,12 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
                     S.near_o[lane][1] = (double)o.y - (double)ay * P.Lbox;
                     S.near_o[lane][2] = (double)o.z - (double)az * P.Lbox;
                 }
-                if (!drain)
+                if (!drain && !have_beam)
                     pt = make_beam<Real>(beam, lv, in, sx, sy, sz, (float)dx, (float)dy, (float)dz, Lf);
                 packet_image<Real, KERNEL, MODE, NF>(P, tab, *beam, S, pq, qn, stash, pt, Lf, dx, dy, dz, in,
                                                      drain, sk, err, nvisit);
             }
+            if (have_beam) break;
         }
     }
 }
@@ -1661,7 +1679,7 @@ int launch_trace(const TraceJob& job, cudaStream_t s)
     P.chunk_seg = job.chunk_seg;
     if (job.near_far && !job.out_near && job.mode != MODE_COUNT)
         return set_error(URCHIN_ERR_ARG, "trace: near/far split without a near-column output");
-    if (job.mode == MODE_FILL && !job.seg_col && !(job.seg_lo && job.seg_hi && b->n <= (int64_t(1) << 24)))
+    if (job.mode == MODE_FILL && !job.seg_col && !(job.seg_lo && (job.seg_hi ? b->n <= (int64_t(1) << 24) : b->n <= (int64_t(1) << 16))))
         return set_error(URCHIN_ERR_ARG, "trace: segment fill without a particle-index array");
     if (job.mode == MODE_CHUNK && (!job.chunk_head || !job.chunk_next || !job.chunk_counter || !job.counts ||
                                    !job.chunk_seg || job.chunk_cap == 0 || job.chunk_cap > 0xffffffffull))
