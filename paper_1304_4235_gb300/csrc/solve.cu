@@ -916,6 +916,9 @@ __global__ void k_clear_inactive_rows(const uint8_t* __restrict__ active, int64_
 //     pays one traversal more than storing at once (262144-particle halo:
 //     292 sweeps, 0.86 s; one traversal 0.04 s).
 constexpr int kAutoStoreSweep = 2;
+// FP64: in sweep 1 already.  The traversal's arithmetic, not the writing of the
+// lists, is what an FP64 sweep costs (16^3 lattice, 7 sweeps: 10.7 -> 8.1 ms).
+constexpr int kAutoStoreSweep64 = 1;
 
 // Up to this many particles a stored index needs its low 16 bits only.
 constexpr int64_t kSegLowOnly = int64_t(1) << 16;
@@ -1165,7 +1168,7 @@ int Solver::columns(const int32_t* items, int64_t n_items, int sweep0, bool buil
         stats.rays += n_items * P.R;
         return URCHIN_OK;
     }
-    if (deferred && stats.iterations < kAutoStoreSweep) return trace(items, n_items, w32, w64);
+    if (deferred && stats.iterations < (f64 ? kAutoStoreSweep64 : kAutoStoreSweep)) return trace(items, n_items, w32, w64);
     if (!counts_ready || (!counted_all && items == nullptr)) {
         URCHIN_TRY_CUDA(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * (size_t)rays, s));
         job.mode = 1;
