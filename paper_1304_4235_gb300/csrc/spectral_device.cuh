@@ -386,6 +386,8 @@ struct Rates {
 // slow path of this GPU; no pow, no logarithm of a constant): each bracket as
 // exp(-p log1p((lambda/c)^q)), the powers of lambda from ll = ln lambda, and
 // ln T = ln 315614 - ll.
+// WHICH: bit 0 alpha_A, bit 1 alpha_B, bit 2 gamma; what is not asked for is 0.
+template <int WHICH = 7>
 __device__ __forceinline__ Rates hg97_rates(double T)
 {
     constexpr double kLn0522 = -0.6500876910994983;     // ln 0.522
@@ -394,14 +396,25 @@ __device__ __forceinline__ Rates hg97_rates(double T)
     constexpr double kLn2THI = 12.662275226919286;      // ln 315614
     const double lam = 315614.0 / T;
     const double ll = log(lam);
-    const double uA = exp(0.470 * (ll - kLn0522));
-    const double uB = exp(0.407 * (ll - kLn2740));
-    const double uC = exp(0.874 * (ll - kLn0354));
-    Rates r;
-    r.alphaA = 1.269e-13 * exp(1.503 * ll - 1.923 * log1p(uA));
-    r.alphaB = 2.753e-14 * exp(1.500 * ll - 2.242 * log1p(uB));
+    Rates r{0.0, 0.0, 0.0};
+    if (WHICH & 1) r.alphaA = 1.269e-13 * exp(1.503 * ll - 1.923 * log1p(exp(0.470 * (ll - kLn0522))));
+    if (WHICH & 2) r.alphaB = 2.753e-14 * exp(1.500 * ll - 2.242 * log1p(exp(0.407 * (ll - kLn2740))));
     // T^-3/2 lambda^-1.089 = exp(-1.5 (ln 315614 - ll) - 1.089 ll)
-    r.gamma_c = 21.11 * exp(-1.5 * kLn2THI + 0.411 * ll - 0.5 * lam - 1.101 * log1p(uC));
+    if (WHICH & 4)
+        r.gamma_c = 21.11 * exp(-1.5 * kLn2THI + 0.411 * ll - 0.5 * lam - 1.101 * log1p(exp(0.874 * (ll - kLn0354))));
+    return r;
+}
+
+// alpha (in .alphaA) of one recombination case, and gamma: the other case's fit
+// would be a fourth of the FP64 work.  The lanes of a warp that want the other
+// case take its coefficients, not its branch.
+__device__ __forceinline__ Rates hg97_case(double T, bool caseB)
+{
+    constexpr double kLn0522 = -0.6500876910994983, kLn2740 = 1.007957920399979;
+    const double ll = log(315614.0 / T);
+    Rates r = hg97_rates<4>(T);
+    const double u = exp((caseB ? 0.407 : 0.470) * (ll - (caseB ? kLn2740 : kLn0522)));
+    r.alphaA = (caseB ? 2.753e-14 : 1.269e-13) * exp((caseB ? 1.500 : 1.503) * ll - (caseB ? 2.242 : 1.923) * log1p(u));
     return r;
 }
 
