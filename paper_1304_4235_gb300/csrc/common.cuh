@@ -203,6 +203,10 @@ struct TraceJob {
     void* out_near;               // near_far: hydrogen column (x = 1) of the near particles, in tau units,
                                   //    at [origin's Morton slot + k * near_k_stride] (modes 0 and 2)
     int64_t near_k_stride;
+    const float* w32_2;           // modes 0 and 4 (FP32, no near/far), or NULL: weights of two more tracers,
+    const float* w32_3;           //    traced along: their columns go to out_2 and out_3, indexed like out
+    float* out_2;
+    float* out_3;
     uint32_t* chunk_head;         // mode 4: [R * n] first chunk of each ray (index k * n + slot)
     uint32_t* chunk_next;         // mode 4: [chunk_cap] next chunk of the same ray
     unsigned long long* chunk_counter;   // mode 4: chunks handed out, zeroed by the caller; above

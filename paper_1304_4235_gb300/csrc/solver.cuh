@@ -92,6 +92,9 @@ struct Solver {
     void* tau_he1 = nullptr;                     // helium: [R * n] fixed columns, Morton slot + k n
     void* tau_he2 = nullptr;
     int he_columns();
+    Scratch he_mem;                              // weights of the helium columns that sweep 0 traces along
+    float* he_w1 = nullptr;
+    float* he_w2 = nullptr;
     void* comp_tmp = nullptr;
     unsigned long long* hits = nullptr;          // misc[3..5], counted when P.profile
     std::vector<cudaEvent_t> events;             // start/stop pairs of each timed launch

@@ -72,6 +72,10 @@ struct TraceParams {
     const int32_t* order;         // [R * n_items] per-direction item order, or NULL
     // near/far split
     void* out_near;               // [slot + k * near_k_stride] near column (x = 1)
+    const float* w32_2;           // kThree: the other tracers' weights (as w32)
+    const float* w32_3;
+    float* out_2;                 //   and columns (indexed like out)
+    float* out_3;
     int64_t near_k_stride;
     // MODE_CHUNK: segment lists in chunks of kChunk entries taken while tracing
     uint32_t* chunk_head;         // [R * n] first chunk of each ray (rays with hits)
@@ -88,6 +92,9 @@ constexpr int MODE_TAU = 0, MODE_COUNT = 1, MODE_FILL = 2, MODE_SCATTER = 3, MOD
 // known before the traversal); the chunks of a ray are linked through
 // chunk_next.  Used by the solver's first sweep, so that a solve of two sweeps
 // traces once.
+// Flag beside MODE_TAU or MODE_CHUNK (FP32): columns of two more tracers in the
+// same traversal (helium), each summed as a traversal of its own would.
+constexpr int kThree = 8;
 constexpr int kChunk = kChunkEntries;   // entries per chunk (a multiple of kSegPad)
 constexpr int kStash = 64;        // chunks a warp takes from the counter at a time
 
@@ -101,6 +108,7 @@ struct Sink {
     int64_t pos, end;
     Real coef;                    // MODE_SCATTER
     Real near, near_c;            // near/far: near column and its compensation
+    Real sum2, comp2, psum2, pcomp2, sum3, comp3, psum3, pcomp3;   // kThree: the other tracers' sums
     int64_t ray;                  // MODE_CHUNK: row k n + origin slot
     int coff;                     // MODE_CHUNK: entries used in it (kChunk: none or full; kChunk + 1: pool exhausted)
     uint32_t cur;                 // MODE_CHUNK: its index (kNoChunk before the first)
@@ -496,8 +504,10 @@ struct alignas(4 * sizeof(Real)) Origin {
     Real x, y, z;                 // a lane's (image-shifted) origin
     Real coef;                    // MODE_SCATTER: its ray's coefficient
 };
-template <typename Real, int MODE, bool NF>
+template <typename Real, int XMODE, bool NF>
 struct Staged {
+    static constexpr int MODE = XMODE & 7;
+    static constexpr bool k3 = (XMODE & kThree) != 0;
     static constexpr bool kF32 = sizeof(Real) == 4;
     static constexpr bool kStored = MODE == 2 || MODE == 4;   // MODE_FILL, MODE_CHUNK
     static constexpr int kPairs = kF32 && kStored ? (NF ? 128 : 192) : 256;
@@ -519,6 +529,7 @@ struct Staged {
     double near_o[NF ? 32 : 1][3];            // near/far: shifted origin in double (the near test)
     float2 aw[kF32 ? 32 : 1];     // A_j and the tracer weight A_j x_j
     float2 g[kF32 ? 32 : 1];      // 1/h and h^2
+    float2 w23[k3 ? 32 : 1];      // the other tracers' weights
     int j[32];                    // Morton slot
     unsigned hit[kPairs / 32 + 1], full[kPairs / 32 + 1], any[kPairs / 32 + 1];   // bit per pair; any: near ones too
     uint16_t pair[kPairs];        // sphere << 5 | lane
@@ -581,12 +592,16 @@ constexpr int kPQ = 64;           // queue capacity per warp; a round takes 32
 constexpr int kPQNear = 32;       // owner flag: a near particle (near/far split)
 constexpr int kPQClipLo = 64;     // owner flag: the segment's start cuts the chord
 constexpr int kPQClipHi = 128;    // owner flag: the segment's end cuts the chord
-template <int MODE, bool NF>
+template <int XMODE, bool NF>
 struct PartQueue {
+    static constexpr int MODE = XMODE & 7;
+    static constexpr bool k3 = (XMODE & kThree) != 0;
     static constexpr bool kAux = MODE != 0;   // every mode but MODE_TAU, of whose items the near ones need A_j
     float4 item[kPQ];             // b^2/h^2 and [u1, u2] in units of h; the tracer weight A_j x_j (MODE_SCATTER: the ray's coefficient)
     int4 aux[kAux ? kPQ : 1];     // particle (Morton slot), low half of the segment's position, bits of A_j; 0
     float A[NF && !kAux ? kPQ : 1];
+    float2 w23[k3 ? kPQ : 1];     // the other tracers' weights
+    float val2[k3 ? 32 : 1], val3[k3 ? 32 : 1];
     int owner[kPQ];               // lane of the ray | kPQNear | kPQClipLo | kPQClipHi | high half of the position << 16
     float val[32];                // results of the round being flushed
     unsigned own[NF ? 64 : 32];   // per owner (lane, lane + kPQNear): items of the round
@@ -609,10 +624,12 @@ __device__ __forceinline__ int64_t pos_of(int owner, int lo)
 // warp calls it.  Inlined: as a called function its reference arguments kept
 // the ray's running state (sums, cursor, queue length) in local memory for the
 // whole traversal, which cost 7 % of the traversal's time.
-template <int KERNEL, int MODE, bool NF, typename Queue>
+template <int KERNEL, int XMODE, bool NF, typename Queue>
 __device__ __forceinline__ void flush_partials(const TraceParams& P, const float2* tab, Queue* pq, Queued& qn, int n,
                                                Sink<float>& k)
 {
+    constexpr int MODE = XMODE & 7;
+    constexpr bool k3 = (XMODE & kThree) != 0;
     const int lane = threadIdx.x & 31;
     if (lane < n) {
         const int at = (qn.part_head + lane) & (kPQ - 1);
@@ -627,6 +644,11 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
             atomicAdd(P.xbar + x.x, (double)(q.w * (A * F)));
         } else {
             pq->val[lane] = NF && (ow & kPQNear) ? A * F : q.w * F;
+            if constexpr (k3) {
+                const float2 w = pq->w23[at];
+                pq->val2[lane] = w.x * F;
+                pq->val3[lane] = w.y * F;
+            }
             if (MODE == MODE_FILL || MODE == MODE_CHUNK) {
                 const int64_t pos = pos_of(ow, x.y);
                 if (MODE == MODE_FILL && pos >= 0) static_cast<float*>(P.seg_val)[pos] = A * F;
@@ -637,7 +659,13 @@ __device__ __forceinline__ void flush_partials(const TraceParams& P, const float
     }
     __syncwarp();
     if (MODE != MODE_SCATTER) {
-        for (unsigned m = pq->own[lane]; m; m &= m - 1) Kahan::add(k.psum, k.pcomp, pq->val[__ffs(m) - 1]);
+        for (unsigned m = pq->own[lane]; m; m &= m - 1) {
+            Kahan::add(k.psum, k.pcomp, pq->val[__ffs(m) - 1]);
+            if constexpr (k3) {
+                Kahan::add(k.psum2, k.pcomp2, pq->val2[__ffs(m) - 1]);
+                Kahan::add(k.psum3, k.pcomp3, pq->val3[__ffs(m) - 1]);
+            }
+        }
         if (NF)
             for (unsigned m = pq->own[lane + kPQNear]; m; m &= m - 1)
                 Kahan::add(k.near, k.near_c, pq->val[__ffs(m) - 1]);
@@ -845,11 +873,13 @@ __device__ __forceinline__ bool decide(const St& S, int e, int o, double dx, dou
 // once, partial chords queued for flush_partials.  Where hits are stored
 // (MODE_FILL, MODE_CHUNK) all pairs are decided first, which gives every hit
 // its position.
-template <int KERNEL, int MODE, bool NF, typename Queue, typename St>
+template <int KERNEL, int XMODE, bool NF, typename Queue, typename St>
 __device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* tab, Queue* pq, Queued& qn,
                                           unsigned long long* stash, St& S, unsigned mm, bool drain, float dx, float dy,
                                           float dz, float L, Sink<float>& k, unsigned& err)
 {
+    constexpr int MODE = XMODE & 7;
+    constexpr bool k3 = (XMODE & kThree) != 0;
     constexpr bool kStored = MODE == MODE_FILL || MODE == MODE_CHUNK;
     const int lane = threadIdx.x & 31;
     const int c = __popc(mm);
@@ -959,13 +989,14 @@ __device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* ta
             pq->item[i] = make_float4(beta2, u1, u2, MODE == MODE_SCATTER ? S.org[o].coef : aw.y);
             if (Queue::kAux) pq->aux[i] = make_int4(S.j[e], (int)(uint32_t)pos, __float_as_int(aw.x), 0);
             if (NF && !Queue::kAux) pq->A[i] = aw.x;
+            if constexpr (k3) pq->w23[i] = S.w23[e];
             pq->owner[i] = o | (near ? kPQNear : 0) | clip | (kStored ? pos_hi(pos) : 0);
         }
         qn.part += __popc(pb);
         __syncwarp();
         // (at the end of the rays, drain, what is left: fewer than 32)
         if (qn.part >= 32 || (drain && qn.part > 0))
-            flush_partials<KERNEL, MODE, NF>(P, tab, pq, qn, min(qn.part, 32), k);
+            flush_partials<KERNEL, XMODE, NF>(P, tab, pq, qn, min(qn.part, 32), k);
         if (drain) break;
     }
     __syncwarp();
@@ -977,6 +1008,11 @@ __device__ __forceinline__ void pairs_f32(const TraceParams& P, const float2* ta
             for (unsigned m = flag_bits(S.full, off, c); m; m &= m - 1u) {
                 const int i = __ffs(m) - 1;
                 const float F = S.val[off + i], w = S.tc[off + i];
+                if constexpr (k3) {
+                    const float2 q = S.w23[S.pair[off + i] >> 5];
+                    Kahan::add_product(k.sum2, k.comp2, q.x, F);
+                    Kahan::add_product(k.sum3, k.comp3, q.y, F);
+                }
                 if (!NF || ((far >> i) & 1u)) Kahan::add_product(k.sum, k.comp, w, F);
                 else Kahan::add_product(k.near, k.near_c, w, F);
             }
@@ -1163,12 +1199,14 @@ struct Walk {
 // One image of the packet's rays: walk, stage, filter, evaluate (file comment);
 // with drain, no image but the queued partial chords (so that the loop holds
 // one copy of that code).
-template <typename Real, int KERNEL, int MODE, bool NF, typename Queue, typename St>
+template <typename Real, int KERNEL, int XMODE, bool NF, typename Queue, typename St>
 __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigned char* tab, const Beam& B, St& S,
                                              Queue* pq, Queued& qn, unsigned long long* stash, float3 pt,
                                              float Lf, Real dx, Real dy, Real dz, bool live, bool drain,
                                              Sink<Real>& sk, unsigned& err, unsigned& nvisit)
 {
+    constexpr int MODE = XMODE & 7;
+    constexpr bool k3 = (XMODE & kThree) != 0;
     const Real L = Real(P.l_ray);
     const int lane = threadIdx.x & 31;
     constexpr bool kF32 = sizeof(Real) == 4;
@@ -1179,12 +1217,13 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
     int ref = 0, cnt = 0;            // the current block (none at first) while the next one is on its way
     bool more = !drain;
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-    float2 aw = make_float2(0.f, 0.f);
+    float2 aw = make_float2(0.f, 0.f), w23 = make_float2(0.f, 0.f);
     auto fetch = [&](int r, int c) {
         if (lane < c && r >= 0 && r + lane < P.n) {
             q = __ldg(P.xyzh + r + lane);
             if (kWantA) aw.x = __ldg(P.A32 + r + lane);
             if (kWantW) aw.y = __ldg(P.w32 + r + lane);
+            if (k3) w23 = make_float2(__ldg(P.w32_2 + r + lane), __ldg(P.w32_3 + r + lane));
         }
     };
     int ns = 0;                      // spheres in the block being filled
@@ -1193,7 +1232,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
         unsigned pm = 0u;
         float su = 0.f, sv = 0.f, stt = 0.f, shh = 0.f;
         const float4 cq = q;
-        const float2 caw = aw;
+        const float2 caw = aw, cw23 = w23;
         const int cj = ref + lane;
         if (!last) {
             // sphere (one per lane) against the beam; the next block of spheres is on its way meanwhile
@@ -1225,6 +1264,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
             S.j[at] = cj;
             if constexpr (kF32) {
                 if (kWantA || kWantW) S.aw[at] = caw;
+                if constexpr (k3) S.w23[at] = cw23;
             }
         };
         const bool mine = (pm >> lane) & 1u;
@@ -1259,7 +1299,7 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
         for (int e0 = 0; (total > 0 || drain) && e0 < 32; e0 += step) {
             const unsigned mm = step == 32 ? mask : mask & (((1u << step) - 1u) << e0);
             if constexpr (kF32)
-                pairs_f32<KERNEL, MODE, NF>(P, reinterpret_cast<const float2*>(tab), pq, qn, stash, S, mm, drain, dx,
+                pairs_f32<KERNEL, XMODE, NF>(P, reinterpret_cast<const float2*>(tab), pq, qn, stash, S, mm, drain, dx,
                                             dy, dz, L, sk, err);
             else
                 pairs_f64<KERNEL, MODE, NF>(P, reinterpret_cast<const double2*>(tab), pq, qn, stash, S, mm, drain, dx, dy,
@@ -1282,12 +1322,13 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
 // depend on the rays that share its beam.
 constexpr float kBeamReach = 5.f;
 
-template <typename Real, int KERNEL, int MODE, bool NF, typename Queue, typename St>
+template <typename Real, int KERNEL, int XMODE, bool NF, typename Queue, typename St>
 __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned char* tab, Beam* beam, St& S,
                                            Queue* pq, Queued& qn, unsigned long long* stash, float4 o, Real dx,
                                            Real dy, Real dz, bool live, Sink<Real>& sk, unsigned& err,
                                            unsigned& nvisit)
 {
+    constexpr int MODE = XMODE & 7;
     const int lane = threadIdx.x & 31;
     const float Lf = (float)P.l_ray * 1.000001f + 1e-30f;
     const int nimg = P.periodic ? P.nimg : 0;
@@ -1359,7 +1400,7 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
                 }
                 if (!drain && !have_beam)
                     pt = make_beam<Real>(beam, lv, in, sx, sy, sz, (float)dx, (float)dy, (float)dz, Lf);
-                packet_image<Real, KERNEL, MODE, NF>(P, tab, *beam, S, pq, qn, stash, pt, Lf, dx, dy, dz, in,
+                packet_image<Real, KERNEL, XMODE, NF>(P, tab, *beam, S, pq, qn, stash, pt, Lf, dx, dy, dz, in,
                                                      drain, sk, err, nvisit);
             }
             if (have_beam) break;
@@ -1370,14 +1411,15 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
 // k_trace's shared memory: per warp the work space, the beam, the block of
 // chunks (MODE_CHUNK) and the queue of partial chords (FP64: of hits) in modes
 // that evaluate chords; the M4 table (FP64: of logarithms); the directions (double[3 R]).
-template <typename Real, int KERNEL, int MODE, bool NF>
+template <typename Real, int KERNEL, int XMODE, bool NF>
 struct TraceLayout {
+    static constexpr int MODE = XMODE & 7;
     static constexpr bool kF32 = sizeof(Real) == 4;
     static constexpr bool kQueue = MODE != MODE_COUNT;
     static constexpr bool kTable = kQueue && KERNEL == URCHIN_KERNEL_M4;
     static constexpr bool kStored = MODE == MODE_FILL || MODE == MODE_CHUNK;
-    using St = Staged<Real, MODE, NF>;
-    using Queue = std::conditional_t<kF32, PartQueue<MODE, NF>, HitQueue<kStored, NF>>;
+    using St = Staged<Real, XMODE, NF>;
+    using Queue = std::conditional_t<kF32, PartQueue<XMODE, NF>, HitQueue<kStored, NF>>;
     static constexpr size_t up(size_t b) { return (b + 15) & ~size_t(15); }
     static constexpr size_t kBeam = up(sizeof(St) * 8);
     static constexpr size_t kStashAt = up(kBeam + sizeof(Beam) * 8);
@@ -1408,10 +1450,12 @@ static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, 
 // chords, at 17 of 32 lanes), two blocks; 16^3 lattice solve 18.3 -> 11.4 ms,
 // 24^3 box 10.7 -> 5.2 ms, 8000-particle halo 13.1 -> 8.8 ms, 9973 x 48 rays of
 // the 48^3 box (G_t) 25.3 -> 18.7 ms with queues and table logarithms.
-template <typename Real, int KERNEL, int MODE, bool NF>
-__global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 2 : 3) k_trace(TraceParams P)
+template <typename Real, int KERNEL, int XMODE, bool NF>
+__global__ void __launch_bounds__(256, sizeof(Real) == 8 || (XMODE & kThree) ? 2 : 3) k_trace(TraceParams P)
 {
-    using Lay = TraceLayout<Real, KERNEL, MODE, NF>;
+    constexpr int MODE = XMODE & 7;
+    constexpr bool k3 = (XMODE & kThree) != 0;
+    using Lay = TraceLayout<Real, KERNEL, XMODE, NF>;
     constexpr bool kQueue = Lay::kQueue;
     extern __shared__ __align__(32) unsigned char smem[];
     const int wid = threadIdx.x >> 5;
@@ -1473,7 +1517,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 2 : 3) k_trace(TraceP
             sk.coef = static_cast<const Real*>(P.coef)[orow * P.row_stride + (int64_t)k * P.k_stride];
             live = sk.coef != Real(0);
         }
-        ray_column<Real, KERNEL, MODE, NF>(P, s_tab, beam, st, pq, qn, stash, o, dx, dy, dz, live, sk, err,
+        ray_column<Real, KERNEL, XMODE, NF>(P, s_tab, beam, st, pq, qn, stash, o, dx, dy, dz, live, sk, err,
                                            nvisit);
         if (mine) {
             hits += sk.nhit;
@@ -1500,6 +1544,11 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 2 : 3) k_trace(TraceP
                 // depends on the ray alone (not on the rays sharing its warp)
                 static_cast<Real*>(P.out)[orow * P.row_stride + (int64_t)k * P.k_stride] =
                     (sk.sum + sk.psum) - (sk.comp + sk.pcomp);
+                if constexpr (k3) {
+                    const int64_t at = orow * P.row_stride + (int64_t)k * P.k_stride;
+                    P.out_2[at] = (sk.sum2 + sk.psum2) - (sk.comp2 + sk.pcomp2);
+                    P.out_3[at] = (sk.sum3 + sk.psum3) - (sk.comp3 + sk.pcomp3);
+                }
                 if (NF) {
                     const int64_t at = P.near_k_stride > 0 ? (int64_t)org + (int64_t)k * P.near_k_stride
                                                            : orow * P.row_stride + (int64_t)k * P.k_stride;
@@ -1542,6 +1591,13 @@ int launch_one(const TraceParams& P, cudaStream_t s)
 template <typename Real, int KERNEL>
 int dispatch_k(const TraceParams& P, int mode, bool nf, cudaStream_t s)
 {
+    if (P.w32_2) {
+        if constexpr (sizeof(Real) == 4) {
+            if (!nf && mode == MODE_CHUNK) return launch_one<float, KERNEL, MODE_CHUNK | kThree, false>(P, s);
+            if (!nf && mode == MODE_TAU) return launch_one<float, KERNEL, MODE_TAU | kThree, false>(P, s);
+        }
+        return set_error(URCHIN_ERR_ARG, "trace: three tracers need FP32 columns without the near/far split");
+    }
     if (nf) {
         if (mode == MODE_COUNT) return launch_one<Real, KERNEL, MODE_COUNT, true>(P, s);
         if (mode == MODE_FILL) return launch_one<Real, KERNEL, MODE_FILL, true>(P, s);
@@ -1677,6 +1733,12 @@ int launch_trace(const TraceJob& job, cudaStream_t s)
     P.chunk_counter = job.chunk_counter;
     P.chunk_cap = job.chunk_cap;
     P.chunk_seg = job.chunk_seg;
+    P.w32_2 = job.w32_2;
+    P.w32_3 = job.w32_3;
+    P.out_2 = job.out_2;
+    P.out_3 = job.out_3;
+    if ((job.w32_2 != nullptr) != (job.w32_3 && job.out_2 && job.out_3))
+        return set_error(URCHIN_ERR_ARG, "trace: three tracers need two more weights and outputs");
     if (job.near_far && !job.out_near && job.mode != MODE_COUNT)
         return set_error(URCHIN_ERR_ARG, "trace: near/far split without a near-column output");
     if (job.mode == MODE_FILL && !job.seg_col && !(job.seg_lo && (job.seg_hi ? b->n <= (int64_t(1) << 24) : b->n <= (int64_t(1) << 16))))
