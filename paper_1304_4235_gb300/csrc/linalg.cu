@@ -22,6 +22,7 @@ constexpr int kSpmvThreads = 256;
 template <typename Real>
 __global__ void __launch_bounds__(kSpmvThreads) k_spmv(SpmvArgs A)
 {
+    if (A.stop && *A.stop) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (kSpmvThreads / 32);
     const int64_t total = (int64_t)A.R * A.n_items;
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(kSpmvThreads) k_spmv(SpmvArgs A)
 template <bool HI>
 __global__ void __launch_bounds__(kSpmvThreads) k_spmv8(SpmvArgs A)
 {
+    if (A.stop && *A.stop) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (kSpmvThreads / 32);
     const int64_t total = (int64_t)A.R * A.n_items;

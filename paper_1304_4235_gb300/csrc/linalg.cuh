@@ -21,6 +21,7 @@ struct SpmvArgs {
     int R;
     int precision;
     void* out;                   // [R * n_items], index k * n_items + item
+    const int* stop;             // device flag or NULL: the launch does nothing once it is set
     // FP32 lists in linked chunks of kChunkEntries (the traversal's MODE_CHUNK)
     // instead of rows: row_ptr, col, lo, hi and val are then unused
     const uint32_t* chunk_head;  // [R * n_rows_per_k] first chunk of each row, or NULL: row-major lists

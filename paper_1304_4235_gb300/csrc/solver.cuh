@@ -43,6 +43,7 @@ struct SweepArgs {
     unsigned long long* n_above;   // count of updated particles with |dx|/x >= tol
     double tol;
     unsigned* status;
+    const int* stop;           // plain sweeps: device flag or NULL, the launch does nothing once it is set
     double* gamma_out;         // [n_items] optional
     float* tau_eff_out;        // [n_items] optional
     int near_far;              // Sec. 3.3.3 split: tau holds the far columns; the near
@@ -170,6 +171,8 @@ struct Solver {
     std::vector<int64_t> block_lo;               // block b = list[block_lo[b], block_lo[b+1])
     int plain();
     int plain_sweeps(double stop_fraction);
+    int sweep_batch(double stop_fraction, int count, bool* done);
+    Scratch batch_mem;
     int newton();
     int run() { return P.method == URCHIN_METHOD_NEWTON ? newton() : plain(); }
     int finish(double* x_inout);
