@@ -95,6 +95,8 @@ constexpr int MODE_TAU = 0, MODE_COUNT = 1, MODE_FILL = 2, MODE_SCATTER = 3, MOD
 // Flag beside MODE_TAU or MODE_CHUNK (FP32): columns of two more tracers in the
 // same traversal (helium), each summed as a traversal of its own would.
 constexpr int kThree = 8;
+// Flag beside MODE_TAU: the form for many rays (k_trace's comment).
+constexpr int kWide = 16;
 constexpr int kChunk = kChunkEntries;   // entries per chunk (a multiple of kSegPad)
 constexpr int kStash = 64;        // chunks a warp takes from the counter at a time
 
@@ -1420,13 +1422,16 @@ struct TraceLayout {
     static constexpr bool kStored = MODE == MODE_FILL || MODE == MODE_CHUNK;
     using St = Staged<Real, XMODE, NF>;
     using Queue = std::conditional_t<kF32, PartQueue<XMODE, NF>, HitQueue<kStored, NF>>;
+    // warps per block and blocks per SM (k_trace's comment)
+    static constexpr int kWarps = (XMODE & kWide) ? 14 : 8;
+    static constexpr int kBlocks = (XMODE & (kWide | kThree)) || !kF32 ? 2 : 3;
     static constexpr size_t up(size_t b) { return (b + 15) & ~size_t(15); }
-    static constexpr size_t kBeam = up(sizeof(St) * 8);
-    static constexpr size_t kStashAt = up(kBeam + sizeof(Beam) * 8);
-    static constexpr size_t kTab = up(kStashAt + 8 * 2 * sizeof(unsigned long long));
+    static constexpr size_t kBeam = up(sizeof(St) * kWarps);
+    static constexpr size_t kStashAt = up(kBeam + sizeof(Beam) * kWarps);
+    static constexpr size_t kTab = up(kStashAt + kWarps * 2 * sizeof(unsigned long long));
     static constexpr size_t kQueueAt =
         up(kTab + (!kTable ? 0 : kF32 ? sizeof(float2) * (kKTab + 1) : sizeof(double2) * kLogTab));
-    static constexpr size_t kDirs = up(kQueueAt + (kQueue ? sizeof(Queue) * 8 : 0));
+    static constexpr size_t kDirs = up(kQueueAt + (kQueue ? sizeof(Queue) * kWarps : 0));
     static size_t bytes(int R) { return kDirs + sizeof(double) * 3 * (size_t)R; }
 };
 static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, false>) % 16 == 0, "shared layout");
@@ -1442,16 +1447,21 @@ static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, 
 // 1168 ms, with one copy 893).  All rays of the 128^3 box 102 -> 79 ms, of the
 // 262144-particle halo 44.1 -> 34.5 ms, 9973 x 48 rays of the 48^3 box in FP64
 // 277 -> 31 ms.
-// Three blocks of 256 per SM (80 registers a thread): with four (64
-// registers) the spills cost more than the fourth block's warps hide; with
-// two (no spills) too few warps are left to hide the loads (128^3 box 69.6 and
-// 76.8 ms, transpose of the 65536-particle halo 6.3 and 6.3 ms).
+// Three blocks of 8 warps per SM (80 registers a thread).  Plain columns of many
+// rays: two blocks of 14 (72 registers; one M4 table for 14 warps leaves the
+// shared memory for 28 warps).  128^3 box: 28 warps 64.4 ms, 24 warps 67.8, 20
+// warps (96 registers) 72.0, 16 warps (128, no spills) 76.8, 32 warps (64) 66.1;
+// 262144-particle halo 30.2 -> 29.2 ms; but the 16^3 lattice's 3072 packets 0.33
+// -> 0.36 ms, unevenly spread in blocks of 14.  The other FP32 modes need more
+// shared memory per warp (list-keeping 128^3 solve 101.9 ms, with 26 warps
+// 103.6; transpose of the 65536-particle halo 6.3 ms with 16 to 24 warps).
 // FP64: bound by the FP64 pipe (84 % busy before the queues of full and partial
 // chords, at 17 of 32 lanes), two blocks; 16^3 lattice solve 18.3 -> 11.4 ms,
 // 24^3 box 10.7 -> 5.2 ms, 8000-particle halo 13.1 -> 8.8 ms, 9973 x 48 rays of
 // the 48^3 box (G_t) 25.3 -> 18.7 ms with queues and table logarithms.
 template <typename Real, int KERNEL, int XMODE, bool NF>
-__global__ void __launch_bounds__(256, sizeof(Real) == 8 || (XMODE & kThree) ? 2 : 3) k_trace(TraceParams P)
+__global__ void __launch_bounds__(32 * TraceLayout<Real, KERNEL, XMODE, NF>::kWarps, TraceLayout<Real, KERNEL, XMODE, NF>::kBlocks)
+k_trace(TraceParams P)
 {
     constexpr int MODE = XMODE & 7;
     constexpr bool k3 = (XMODE & kThree) != 0;
@@ -1576,14 +1586,15 @@ template <typename Real, int KERNEL, int MODE, bool NF>
 int launch_one(const TraceParams& P, cudaStream_t s)
 {
     const void* fn = (const void*)k_trace<Real, KERNEL, MODE, NF>;
-    const size_t smem = TraceLayout<Real, KERNEL, MODE, NF>::bytes(P.R);
+    using Lay = TraceLayout<Real, KERNEL, MODE, NF>;
+    const size_t smem = Lay::bytes(P.R);
     if (smem > 48 * 1024) URCHIN_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int grid = 0;
-    URCHIN_TRY(grid_for(fn, 256, smem, &grid));
-    int64_t tasks = P.n_chunks * P.R;
-    int64_t need = (tasks + 7) / 8;       // 8 warps per block
+    URCHIN_TRY(grid_for(fn, 32 * Lay::kWarps, smem, &grid));
+    const int64_t tasks = P.n_chunks * P.R;
+    const int64_t need = (tasks + Lay::kWarps - 1) / Lay::kWarps;
     if (need < grid) grid = (int)std::max<int64_t>(need, 1);
-    k_trace<Real, KERNEL, MODE, NF><<<grid, 256, smem, s>>>(P);
+    k_trace<Real, KERNEL, MODE, NF><<<grid, 32 * Lay::kWarps, smem, s>>>(P);
     URCHIN_TRY(launched());
     return URCHIN_OK;
 }
@@ -1611,6 +1622,13 @@ int dispatch_k(const TraceParams& P, int mode, bool nf, cudaStream_t s)
     if (mode == MODE_CHUNK) {
         if constexpr (sizeof(Real) == 4) return launch_one<Real, KERNEL, MODE_CHUNK, false>(P, s);
         return set_error(URCHIN_ERR_ARG, "trace: chunked segment lists are FP32 only");
+    }
+    if constexpr (sizeof(Real) == 4) {
+        // enough packets for two per warp of the wide form
+        int dev = 0, sms = 0;
+        URCHIN_TRY_CUDA(cudaGetDevice(&dev));
+        URCHIN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (P.n_chunks * P.R >= (int64_t)sms * 56) return launch_one<float, KERNEL, MODE_TAU | kWide, false>(P, s);
     }
     return launch_one<Real, KERNEL, MODE_TAU, false>(P, s);
 }
