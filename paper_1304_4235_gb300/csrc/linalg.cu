@@ -246,12 +246,17 @@ __global__ void k_dots(const double* __restrict__ V, int64_t ld, int count, cons
     (void)count;
 }
 
-__global__ void k_dots_reduce(const double* partial, int nb, int count, double* out)
+// out[i] = the sum of dot i's partials in their order: a block fetches them at
+// once, one thread adds (a thread that fetched as it added took 11 us).
+__global__ void k_dots_reduce(const double* partial, int nb, double* out)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
+    __shared__ double v[256];
+    const int i = blockIdx.x;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) v[b] = partial[(int64_t)i * nb + b];
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     double t = 0.0;
-    for (int b = 0; b < nb; ++b) t += partial[(int64_t)i * nb + b];
+    for (int b = 0; b < nb; ++b) t += v[b];
     out[i] = t;
 }
 
@@ -354,7 +359,7 @@ int launch_dots(const double* V, int64_t ld, int count, const double* w, int64_t
     dim3 g((unsigned)nb, (unsigned)count);
     k_dots<<<g, 256, 0, s>>>(V, ld, count, w, n, tmp);
     URCHIN_TRY(launched());
-    k_dots_reduce<<<(count + 63) / 64, 64, 0, s>>>(tmp, nb, count, out);
+    k_dots_reduce<<<count, 256, 0, s>>>(tmp, nb, out);
     return launched();
 }
 
