@@ -325,18 +325,18 @@ def timed(stream, fn):
     return r, a.elapsed_time(b) * 1e-3
 
 
-def roofline_spmv(stats, hbm, peak_kind):
+def roofline_spmv(stats, hbm, peak_kind, n=1 << 24):
     """k_spmv8 (stored-segment columns) against the HBM roofline: 8
     algorithmic bytes per segment (a 4-byte particle index and a 4-byte
-    value; the kernel moves 7, the index split in 16 + 8 bits), plus each
-    ray's 4-byte column and the 4-byte x gather per particle, over the
-    launch's mean duration."""
+    value; the kernel moves 7, the index split in 16 + 8 bits, or 6 up to
+    65536 particles n), plus each ray's 4-byte column and the 4-byte x gather
+    per particle, over the launch's mean duration."""
     launches = sum(st["spmv_launches"] for st in stats)
     spmv_s = sum(st["spmv_s"] for st in stats)
-    moved = sum(st["spmv_bytes"] for st in stats)          # 7 per segment + columns + x
+    moved = sum(st["spmv_bytes"] for st in stats)          # 6 or 7 per segment + columns + x
     st0 = stats[-1]
     extra = launches * (st0["n_active"] * 12 * 4 + st0["n_active"] * 4)
-    seg = max(moved - extra, 0) / 7.0
+    seg = max(moved - extra, 0) / (7.0 if n > 65536 else 6.0)
     per_bytes = (seg * 8 + extra) / max(launches, 1)
     per_s = spmv_s / max(launches, 1)
     achieved = per_bytes / per_s / 1e9 if per_s > 0 else None
@@ -486,7 +486,7 @@ def main():
         "segments_stored": bool(st0["segments_stored"]), "n_active": st0["n_active"], "hits_per_step": st0["hits"],
         "wall_s_to_converged": total_ms * 1e-3 / args.steps,
         "gpu_launches": int(launches),
-        "roofline": (roofline_spmv(stats, hbm, peak_kind) if sum(st["spmv_s"] for st in stats) > trace_s
+        "roofline": (roofline_spmv(stats, hbm, peak_kind, w.n) if sum(st["spmv_s"] for st in stats) > trace_s
                      else roofline(stats, trace_launches, hbm, peak_kind, w.n * len(D.dirs))),
         "kernels": kernels,
         "clocks": clk,
