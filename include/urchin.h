@@ -79,16 +79,18 @@ typedef struct CUstream_st* urchin_stream_t;
 #define URCHIN_SEG_RECOMPUTE    0     /* trace the BVH every sweep              */
 #define URCHIN_SEG_STORE        1     /* store per-ray segment lists once       */
 #define URCHIN_SEG_AUTO         2     /* store when the lists fit in memory     */
-/* A stored segment is the FP32 value and the particle's Morton index split
- * into 16 + 8 bits (7 bytes; n <= 2^24), or FP64 value and int32 index (12
- * bytes); each ray's list is padded with zero entries to a multiple of 8.
+/* A stored segment is the FP32 value and the particle's slot in the tree's
+ * order split into 16 + 8 bits (7 bytes, or 6 without the high byte up to n =
+ * 65536; n <= 2^24), or FP64 value and int32 index (12 bytes); each ray's list
+ * is padded with zero entries to a multiple of 8.
  * URCHIN_SEG_AUTO in FP32 (no near/far split, blocks <= 1) keeps the lists
  * of the first sweep's traversal itself, in linked chunks of 32 (index,
  * value) pairs of 8 bytes sized from a sampled estimate, so that a solve of
  * two sweeps traces once; from the fourth sweep the active rows are copied
- * into the 7-byte row layout when both fit.  When the chunks do not fit or
- * the estimate proves short, the lists are stored from the third sweep (a
- * counting and a filling traversal) where they fit, else every sweep traces. */
+ * into the row layout when both fit.  When the chunks do not fit or the
+ * estimate proves short, the lists are stored from the third sweep (in FP64
+ * from the second; a counting and a filling traversal) where they fit, else
+ * every sweep traces. */
 
 #define URCHIN_MAX_RAYS       192     /* HEALPix N_side <= 4                    */
 #define URCHIN_MAX_BINS      4096     /* frequency bins                         */
@@ -136,7 +138,7 @@ typedef struct {
 } urchin_spectrum;
 
 /* Opaque bounding-volume hierarchy over the particles' smoothing spheres
- * (Morton-ordered copy of the particle data plus a binary radix tree). */
+ * (a copy of the particle data in tree order plus a tree of boxes). */
 typedef struct urchin_bvh urchin_bvh;
 
 /* ---- entry points ------------------------------------------------------ */
@@ -187,7 +189,8 @@ URCHIN_API int urchin_cross_section_ratio(int F, const double* E_edges, int xsec
 
 /* Build the BVH (no counterpart in the paper, which does not describe its
  * search structure): Morton codes of the sphere centres, radix sort, binary
- * radix tree, bottom-up bounds, and a Morton-ordered copy of the particles.
+ * radix tree, a copy of the particles in that tree's depth-first order, and a
+ * 32-way tree of boxes over it.
  * The particle arrays are only read during the call.  `*out` receives a
  * library-owned object; release it with urchin_free_bvh.  The call
  * synchronises `stream`.  Errors: ERR_ARG (NULL, n < 1, h <= 0 or
@@ -237,8 +240,8 @@ URCHIN_API int urchin_trace_columns(const urchin_bvh* bvh, const double* x, cons
  *     its hits in the tree's fixed depth-first order, whichever rays share
  *     its warp), but the rays are traced in the order of the origin list:
  *     the per-direction ray ordering that urchin_trace_columns sorts into
- *     extra memory for 16384 or more origins is skipped, so large calls run
- *     slower.
+ *     extra memory (for 16384 or more particles, and for lists of 1024 or more
+ *     origins) is skipped, so large calls run slower.
  *   - The first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress) and caches it per device ordinal; make that
  *     first call before any stream capture.  The cache assumes the device
@@ -397,8 +400,8 @@ typedef struct {
     int64_t hits;                 /* ray-sphere chord evaluations (profile=1)  */
     double  trace_s;              /* GPU time of the traversals (profile=1)    */
     int     trace_launches;       /* traversal kernel launches                 */
-    int64_t sphere_tests;         /* ray-sphere tests at leaves (profile=1)    */
-    int64_t node_visits;          /* internal nodes visited (profile=1)        */
+    int64_t sphere_tests;         /* spheres filtered against rays (profile=1) */
+    int64_t node_visits;          /* 32-way tree entries visited (profile=1)   */
     int     newton_fallbacks;     /* Newton steps replaced by a plain sweep    */
     int     newton_start;         /* iterations done before Newton took over   */
     double  spmv_s;               /* GPU time of stored-segment sweeps (profile=1) */

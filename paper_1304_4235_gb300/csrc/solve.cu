@@ -1084,7 +1084,7 @@ int Solver::trace_chunked(TraceJob& job)
 }
 
 // From the fourth sweep on, the chunked lists of the active rows are copied
-// into rows (the 7-byte layout of the row product, which streams at the
+// into rows (the 6- or 7-byte layout of the row product, which streams at the
 // bandwidth bound where following chunk links does not) when both fit at
 // once; the chunks are then released.  A solve of two or three sweeps keeps
 // the chunks.
@@ -1225,7 +1225,8 @@ int Solver::columns(const int32_t* items, int64_t n_items, int sweep0, bool buil
     URCHIN_TRY_CUDA(cudaMemcpyAsync(&nnz, total, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
     const size_t vsz = f64 ? sizeof(double) : sizeof(float);
-    // FP32 segments keep the particle index as 16 + 8 bits (7 bytes per segment)
+    // FP32 segments keep the particle index as 16 + 8 bits (7 bytes per
+    // segment), 16 bits up to kSegLowOnly particles (6)
     const bool split = !f64 && n <= (int64_t(1) << 24);
     const bool high = split && n > kSegLowOnly;
     const size_t isz = split ? sizeof(uint16_t) + (high ? sizeof(uint8_t) : 0) : sizeof(int32_t);

@@ -111,7 +111,8 @@ struct Solver {
     void* scan_tmp = nullptr;
     int32_t* seg_col = nullptr;                  // particle index per segment, or NULL when
     uint16_t* seg_lo = nullptr;                  // split into 16 + 8 bits (FP32 segments,
-    uint8_t* seg_hi = nullptr;                   // n <= 2^24: 7 bytes per segment instead of 8)
+    uint8_t* seg_hi = nullptr;                   // n <= 2^24: 7 bytes per segment instead of 8,
+                                                 // NULL up to kSegLowOnly particles: 6)
     void* seg_val = nullptr;
     Scratch seg;
     // segment lists stored by the first sweep's traversal in linked chunks

@@ -233,9 +233,9 @@ struct RayMean {
 // SM.  The rays are combined in their order either way, so the result does
 // not depend on G.  Bound by the FP32 pipe and issue (FP64: its pipe): packed
 // operations take 10 issue slots per ray and bin instead of 15.  12 rays, 100
-// bins, FP32 / ms: 400003 rows with the equilibrium 0.58 -> 0.50, a sweep of
-// 65536 particles 0.067 -> 0.055; FP64, a sweep of 4096 particles and 50 bins
-// 0.93 -> 0.10 (16 blocks before).
+// bins, FP32 / ms: 400003 rows with the equilibrium 0.58 -> 0.50; 200 bins, a
+// sweep of 32768 particles 0.077 -> 0.054; FP64, a sweep of 4096 particles and
+// 50 bins 0.93 -> 0.18 (16 blocks before).
 struct FoldSplit {
     int G;                        // threads per row
     int per;                      // rays per thread

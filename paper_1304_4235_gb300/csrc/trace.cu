@@ -1436,29 +1436,31 @@ struct TraceLayout {
 };
 static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, false>) % 16 == 0, "shared layout");
 
-// Bound by instruction issue (71 % of the slots, 1/5 of the stalls waiting for
-// shared memory, DRAM idle): 29 warp instructions per crossed sphere on the
-// log-normal box with 32 origins per beam, against 45 when every lane tested
+// Bound by instruction issue (75 % of the slots for plain columns, 71 % with the
+// lists; 1/5 of the stalls waiting for shared memory, DRAM idle but for the
+// lists): 28 warp instructions per crossed sphere on the log-normal box with 32
+// origins per beam, 34 with the lists, against 45 and 46 when every lane tested
 // every staged sphere exactly, and 14 on the halo's long rays (21).  The pair
 // list keeps the exact test and the chords at 30 of 32 lanes (16 to 21 when
 // every lane took its own next candidate).  The traversal's loop has to fit
 // the instruction cache: with two copies of the partial chords' code in it the
 // list-keeping form stalled on fetches for half its time (256^3 box: solve
-// 1168 ms, with one copy 893).  All rays of the 128^3 box 102 -> 79 ms, of the
-// 262144-particle halo 44.1 -> 34.5 ms, 9973 x 48 rays of the 48^3 box in FP64
-// 277 -> 31 ms.
+// 1168 ms, with one copy 893; 806 ms now with the tree of full blocks, the ring
+// queue and one beam away from the faces).  All rays of the 128^3 box 102 ms
+// before -> 63.7, of the 262144-particle halo 44.1 -> 28.8.
 // Three blocks of 8 warps per SM (80 registers a thread).  Plain columns of many
 // rays: two blocks of 14 (72 registers; one M4 table for 14 warps leaves the
-// shared memory for 28 warps).  128^3 box: 28 warps 64.4 ms, 24 warps 67.8, 20
+// shared memory for 28 warps).  128^3 box: 28 warps 63.7 ms, 24 warps 67.8, 20
 // warps (96 registers) 72.0, 16 warps (128, no spills) 76.8, 32 warps (64) 66.1;
-// 262144-particle halo 30.2 -> 29.2 ms; but the 16^3 lattice's 3072 packets 0.33
+// 262144-particle halo 30.2 -> 28.8 ms; but the 16^3 lattice's 3072 packets 0.33
 // -> 0.36 ms, unevenly spread in blocks of 14.  The other FP32 modes need more
 // shared memory per warp (list-keeping 128^3 solve 101.9 ms, with 26 warps
 // 103.6; transpose of the 65536-particle halo 6.3 ms with 16 to 24 warps).
 // FP64: bound by the FP64 pipe (84 % busy before the queues of full and partial
-// chords, at 17 of 32 lanes), two blocks; 16^3 lattice solve 18.3 -> 11.4 ms,
-// 24^3 box 10.7 -> 5.2 ms, 8000-particle halo 13.1 -> 8.8 ms, 9973 x 48 rays of
-// the 48^3 box (G_t) 25.3 -> 18.7 ms with queues and table logarithms.
+// chords, at 17 of 32 lanes), two blocks; with queues and table logarithms the
+// 16^3 lattice solve 18.3 -> 11.0 ms (82 ms with every lane testing every staged
+// sphere), 24^3 box 10.7 -> 5.0 ms, 8000-particle halo 13.1 -> 8.4 ms, 9973 x 48
+// rays of the 48^3 box (G_t) 25.3 -> 18.7 ms (277).
 template <typename Real, int KERNEL, int XMODE, bool NF>
 __global__ void __launch_bounds__(32 * TraceLayout<Real, KERNEL, XMODE, NF>::kWarps, TraceLayout<Real, KERNEL, XMODE, NF>::kBlocks)
 k_trace(TraceParams P)
