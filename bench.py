@@ -75,15 +75,13 @@ def workload_name(key: str, w) -> str:
 #   k_trace: bytes per ray-sphere hit;  k_spmv: bytes per stored segment
 MEASURED_TRAFFIC = {
     # the 256^3 box's own traversal (one-pass capture), which also stores the
-    # segment lists: 34.2e9 + 180.7e9 DRAM bytes for 1.762e10 hits (captured
-    # at source hash 7f3194b2267f46f1, which differs from this key's source
-    # in one duplicated comment only)
-    "k_trace": {"510ddac9de652e18": 12.20},
-    # k_spmv8 on the 65536-particle halo (one-pass capture): 2.273e9 + 3.8e6
-    # DRAM bytes for 3.23e8 padded segments, captured at source hash
-    # 87756054aa5bee94; the files have since gained the chunk kernels and
-    # trailing argument fields, the body of k_spmv8 is unchanged
-    "k_spmv": {"92fdf220e9a3969d": 7.04},
+    # segment lists: 39.3e9 + 190.9e9 DRAM bytes for 1.762e10 hits
+    "k_trace": {"db7bf1c15441437a": 13.07},
+    # k_spmv8 by the bytes a stored segment takes.  65536-particle halo, one-pass
+    # captures: 6-byte segments 1.949e9 + 4.9e6 DRAM bytes for 3.23e8 padded
+    # segments; 7-byte segments 2.273e9 + 3.8e6, taken before the 6-byte form
+    # (the kernel's loop over 7-byte rows is unchanged since)
+    "k_spmv": {"d10a1d41f9b7eacc": {6: 6.05, 7: 7.04}},
 }
 KERNEL_SOURCES = {"k_trace": ("trace.cu", "common.cuh"), "k_spmv": ("linalg.cu", "linalg.cuh")}
 
@@ -336,11 +334,12 @@ def roofline_spmv(stats, hbm, peak_kind, n=1 << 24):
     moved = sum(st["spmv_bytes"] for st in stats)          # 6 or 7 per segment + columns + x
     st0 = stats[-1]
     extra = launches * (st0["n_active"] * 12 * 4 + st0["n_active"] * 4)
-    seg = max(moved - extra, 0) / (7.0 if n > 65536 else 6.0)
+    seg_bytes = 7 if n > 65536 else 6
+    seg = max(moved - extra, 0) / seg_bytes
     per_bytes = (seg * 8 + extra) / max(launches, 1)
     per_s = spmv_s / max(launches, 1)
     achieved = per_bytes / per_s / 1e9 if per_s > 0 else None
-    t = MEASURED_TRAFFIC["k_spmv"].get(source_hash("k_spmv"))
+    t = MEASURED_TRAFFIC["k_spmv"].get(source_hash("k_spmv"), {}).get(seg_bytes)
     return {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
             "frac": achieved / hbm if achieved else None, "traffic": (t * seg / max(launches, 1)) if t else None,
             "kernel": "k_spmv8 (FP32 stored segments)", "peak_kind": peak_kind, "alg_bytes_per_launch": per_bytes,
