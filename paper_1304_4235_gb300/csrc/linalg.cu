@@ -198,7 +198,15 @@ __global__ void __launch_bounds__(kSpmvThreads) k_chunk_compact(ChunkCompactArgs
 }
 
 // One warp per ray: the ray's coefficient times each stored segment value is
-// added to z at the segment's particle.
+// added to z at the segment's particle.  The additions arrive in any order, so
+// z is good to its last digits only, and the adjoint rounds its coefficients to
+// FP32 at every product: a digit that moves flips a rounding now and then, and
+// the gradient of a 32768-particle halo repeats to 1e-15 for some inputs and to
+// 1e-10 to 1e-6 for others.  With 6-byte rows the additions arrived in another
+// order (no high bytes to wait for) and other inputs were the uneven ones, so
+// these rows keep their high bytes at every n (100.3 -> 101.0 ms for that halo's
+// solve and gradient).  A sum in two limbs that does not depend on the order
+// took 122 ms and was no nearer to either.
 template <typename Real>
 __global__ void __launch_bounds__(kSpmvThreads) k_spmv_t(SpmvTArgs A)
 {
@@ -218,8 +226,7 @@ __global__ void __launch_bounds__(kSpmvThreads) k_spmv_t(SpmvTArgs A)
         for (int64_t e = beg + lane; e < end; e += 32) {
             const Real v = __ldcs(val + e);
             if (v != Real(0)) {   // padding is zero
-                const int32_t j = A.col ? __ldcs(A.col + e)
-                                        : (int32_t)__ldcs(A.lo + e) | (A.hi ? (int32_t)__ldcs(A.hi + e) << 16 : 0);
+                const int32_t j = A.col ? __ldcs(A.col + e) : (int32_t)__ldcs(A.lo + e) | ((int32_t)__ldcs(A.hi + e) << 16);
                 atomicAdd(A.z + j, (double)(c * v));
             }
         }

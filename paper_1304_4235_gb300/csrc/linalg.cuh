@@ -53,9 +53,9 @@ int launch_chunk_compact(const ChunkCompactArgs& A, cudaStream_t s);
 // accumulated with atomics; coef has the precision's type.
 struct SpmvTArgs {
     const uint64_t* row_ptr;
-    const int32_t* col;          // as SpmvArgs
+    const int32_t* col;          // as SpmvArgs, but
     const uint16_t* lo;
-    const uint8_t* hi;
+    const uint8_t* hi;           //   hi goes with lo at every n
     const void* val;
     const void* coef;            // [R * n_items]
     const int32_t* items;        // NULL = identity

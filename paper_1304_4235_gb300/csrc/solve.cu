@@ -1226,9 +1226,10 @@ int Solver::columns(const int32_t* items, int64_t n_items, int sweep0, bool buil
     URCHIN_TRY_CUDA(cudaStreamSynchronize(s));
     const size_t vsz = f64 ? sizeof(double) : sizeof(float);
     // FP32 segments keep the particle index as 16 + 8 bits (7 bytes per
-    // segment), 16 bits up to kSegLowOnly particles (6)
+    // segment), 16 bits up to kSegLowOnly particles (6) but for the adjoint's
+    // rows, which the transposed product reads (k_spmv_t)
     const bool split = !f64 && n <= (int64_t(1) << 24);
-    const bool high = split && n > kSegLowOnly;
+    const bool high = split && (n > kSegLowOnly || build);
     const size_t isz = split ? sizeof(uint16_t) + (high ? sizeof(uint8_t) : 0) : sizeof(int32_t);
     const size_t need = (size_t)nnz * (isz + vsz) + 1024;
     bool fits = true;
