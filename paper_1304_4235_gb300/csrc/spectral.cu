@@ -70,6 +70,15 @@ __global__ void k_equilibrium(const double* __restrict__ gamma, const float* __r
     }
 }
 
+// the double loop for one ray; ws(b) = w_b s_b, smin the smallest s_b
+template <typename Ws>
+__device__ __forceinline__ double rate_bar(double c, double t, const double* ss, Ws ws, int F, double smin)
+{
+    double S = 0.0;
+    for (int b = 0; b < F; ++b) S += ws(b) * exp(-(ss[b] - smin) * t);
+    return c != 0.0 && S > 0.0 ? -copysign(exp(log(fabs(c)) - smin * t + log(S)), c) : 0.0;
+}
+
 // Reverse mode of Eq. gamma_shld, in double.  With c_o = gamma_bar_o / R:
 //   tau_bar_ok = -c_o sum_b w_b s_b exp(-s_b tau_ok)
 //              = -sign(c_o) exp(ln|c_o| - s_min tau_ok + ln sum_b w_b s_b exp(-(s_b - s_min) tau_ok)),
@@ -96,12 +105,7 @@ __global__ void k_gamma_vjp_tau(const double* __restrict__ tau, int64_t n_rays, 
     const double smin = smin_s;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x) {
         const double c = gbar[r / R] / (double)R;
-        const double t = tau[r];
-        double S = 0.0;
-        for (int b = 0; b < F; ++b) S += ws[b] * exp(-(ss[b] - smin) * t);
-        double v = 0.0;
-        if (c != 0.0 && S > 0.0) v = -copysign(exp(log(fabs(c)) - smin * t + log(S)), c);
-        tau_bar[r] = v;
+        tau_bar[r] = rate_bar(c, tau[r], ss, [&](int b) { return ws[b]; }, F, smin);
     }
 }
 
@@ -114,42 +118,79 @@ __global__ void k_gamma_vjp_tau(const double* __restrict__ tau, int64_t n_rays, 
 // products are float pairs and the sum is compensated, so that S is good to
 // about 1e-9 and the FP32 result is the rounded one, as with double sums
 // (measured against 64 bits over 786432 rays: 2.5e-8 either way).  s_min is
-// taken over the bins with a weight.  Columns outside [0, 1e30) keep the
-// double loop.  65536 rows of 12 rays, 200 bins: 5.4 -> 0.23 ms.
+// taken over the bins with a weight.  65536 rows of 12 rays, 200 bins: 5.4 ->
+// 0.23 ms.
+// The pairs have the range of float, so the double loop stays for spectra whose
+// w_b s_b span more than 2^80 (a thermal spectrum's hard bins, which carry all
+// of a deeply shielded ray's rate; within 2^80 of the largest, S and every term
+// that counts in it are far above the smallest float, and the terms dropped
+// beyond 2^-140 are below 2^-60 of S) or lie at the ends of double, and for
+// columns outside [0, 1e30).
 constexpr int kExpTab = 64;
+constexpr double kPairSpan = 0x1p80;
+
 __global__ void __launch_bounds__(256) k_gamma_vjp_tau32(const float* __restrict__ tau, int64_t n_rays, int R,
                                                          const double* __restrict__ sv, const double* __restrict__ wv,
                                                          int F, const double* __restrict__ gbar, float* tau_bar)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4* cf = reinterpret_cast<float4*>(smem_raw);            // [F] exponent coefficient and weight, each a float pair
+    double* ss = reinterpret_cast<double*>(smem_raw);            // the double loop: [F] s_b and [F] w_b s_b
+    double* ws = ss + F;
     __shared__ float2 tab[kExpTab];
-    __shared__ double red[8], smin_s, scale_s;
-    double m = INFINITY, big = 0.0;
-    for (int b = threadIdx.x; b < F; b += blockDim.x) {
-        const double ws = wv[b] * sv[b];
-        if (ws != 0.0) m = fmin(m, sv[b]);
-        big = fmax(big, fabs(ws));
+    __shared__ double red[8][4], par[4];
+    {
+        // smallest s_b, of all bins and of those with a weight; largest and smallest weight
+        double ma = INFINITY, m = INFINITY, big = 0.0, lo = INFINITY;
+        for (int b = threadIdx.x; b < F; b += blockDim.x) {
+            const double q = wv[b] * sv[b];
+            ma = fmin(ma, sv[b]);
+            big = fmax(big, fabs(q));
+            if (q != 0.0) {
+                m = fmin(m, sv[b]);
+                lo = fmin(lo, fabs(q));
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            ma = fmin(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+            m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
+            big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        }
+        double* r = red[threadIdx.x >> 5];
+        if ((threadIdx.x & 31) == 0) {
+            r[0] = ma;
+            r[1] = m;
+            r[2] = big;
+            r[3] = lo;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int i = 1; i < 8; ++i) {
+                ma = fmin(ma, red[i][0]);
+                m = fmin(m, red[i][1]);
+                big = fmax(big, red[i][2]);
+                lo = fmin(lo, red[i][3]);
+            }
+            par[0] = ma;
+            par[1] = m < INFINITY ? m : 0.0;
+            par[2] = big;
+            par[3] = lo;
+        }
+        __syncthreads();
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
-        big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    const double sall = par[0], smin = par[1], scale = par[2];
+    if (scale > 0.0 && !(scale < 1e290 && scale > 1e-290 && par[3] * kPairSpan >= scale)) {
+        for (int b = threadIdx.x; b < F; b += blockDim.x) {
+            ss[b] = sv[b];
+            ws[b] = wv[b] * sv[b];
+        }
+        __syncthreads();
+        for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x)
+            tau_bar[r] = (float)rate_bar(gbar[r / R] / (double)R, (double)tau[r], ss, [&](int b) { return ws[b]; }, F, sall);
+        return;
     }
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < 8; ++i) m = fmin(m, red[i]);
-        smin_s = m < INFINITY ? m : 0.0;
-    }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = big;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < 8; ++i) big = fmax(big, red[i]);
-        scale_s = big;
-    }
-    __syncthreads();
-    const double smin = smin_s, scale = scale_s, iscale = scale > 0.0 ? 1.0 / scale : 0.0;
+    const double iscale = scale > 0.0 ? 1.0 / scale : 0.0;
     for (int b = threadIdx.x; b < F; b += blockDim.x) {
         const double ws = wv[b] * sv[b] * iscale, c = ws != 0.0 ? (sv[b] - smin) * 1.4426950408889634 : 0.0;
         cf[b] = make_float4((float)c, (float)(c - (double)(float)c), (float)ws, (float)(ws - (double)(float)ws));
@@ -193,15 +234,12 @@ __global__ void __launch_bounds__(256) k_gamma_vjp_tau32(const float* __restrict
             const double Sd = (double)S + (double)C;
             if (c != 0.0 && Sd > 0.0) {
                 // -c exp(-s_min tau) S without leaving the range of double: 2^-(s_min tau log2 e) in two factors
-                const double x = e0 * (double)t, n = rint(x);
-                const double f = (c * scale) * Sd * exp2(n - x);
-                out = (float)-(n < 4000.0 ? scalbn(f, -(int)n) : 0.0);
+                const double x = e0 * (double)t, n = rint(x), cs = c * scale;
+                if (fabs(cs) < 1e290 && fabs(cs) > 1e-290) out = (float)-(n < 4000.0 ? scalbn(cs * Sd * exp2(n - x), -(int)n) : 0.0);
+                else out = (float)-copysign(exp(log(fabs(c)) + log(scale) - smin * (double)t + log(Sd)), c);
             }
         } else {
-            const double td = (double)t;
-            double S = 0.0;
-            for (int b = 0; b < F; ++b) S += wv[b] * sv[b] * exp(-(sv[b] - smin) * td);
-            if (c != 0.0 && S > 0.0) out = (float)-copysign(exp(log(fabs(c)) - smin * td + log(S)), c);
+            out = (float)rate_bar(c, (double)t, sv, [&](int b) { return wv[b] * sv[b]; }, F, sall);
         }
         tau_bar[r] = out;
     }

@@ -32,3 +32,33 @@ def test_adjoint_rows_keep_the_high_bytes():
         # one product over every row: its segments, a column per ray and x
         assert st["n_active"] == w.n and st["nnz"] > 0
         assert st["spmv_bytes"] == st["nnz"] * per + w.n * 12 * 4 + w.n * 4
+
+
+@pytest.mark.parametrize("decades", [20, 30, 60, 250])
+def test_rate_transpose_fp32_of_wide_spectra(decades):
+    # weights over many decades, the hard bins the faint ones: behind deep
+    # columns those carry all of the rate, and the FP32 form stays the rounded
+    # double one (to 7e-8, as over ordinary spectra)
+    rng = np.random.default_rng(decades)
+    F, n, R = 40, 800, 12
+    E = np.exp(np.linspace(0.0, np.log(10.0), F))
+    s = E ** -3
+    wts = 1e-12 * 10.0 ** (-decades * (E - 1) / 9)
+    tau = (10.0 ** rng.uniform(-3, 4.0, (n, R))).astype(np.float32)
+    tau[0, :3] = [0.0, 1e30, np.inf]
+    # cotangents that bring the result into the range of float
+    gb = np.where(rng.random(n) < 0.5, -1.0, 1.0) * 10.0 ** rng.uniform(0, decades + 12, n)
+    a, _ = U.urchin_gamma_vjp(_dev(tau, np.float32), _dev(s), _dev(wts), _dev(gb), want_w=False)
+    b, _ = U.urchin_gamma_vjp(_dev(tau), _dev(s), _dev(wts), _dev(gb), want_w=False)
+    a, b = a.cpu().numpy().astype(np.float64), b.cpu().numpy()
+    with np.errstate(over="ignore"):
+        over = ~np.isfinite(b.astype(np.float32))
+    ok = (np.abs(b) > 1.2e-38) & ~over
+    assert ok.mean() > 0.2
+    assert (np.abs(a[ok] - b[ok]) <= 7e-8 * np.abs(b[ok])).all()
+    assert np.array_equal(np.isinf(a), over)
+    # two bins: the faint one alone is left behind a column of 2000
+    t = np.full((1, 1), 2000.0)
+    g, _ = U.urchin_gamma_vjp(_dev(t, np.float32), _dev([1.0, 0.02]), _dev([1e-12, 1e-60]), _dev([1e50]), want_w=False)
+    want = -1e50 * 1e-60 * 0.02 * np.exp(-40.0)
+    assert abs(float(g[0, 0]) - want) <= 1e-6 * abs(want)
