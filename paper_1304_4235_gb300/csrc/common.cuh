@@ -78,6 +78,12 @@ struct Layout {
 
 int grid_for(const void* kernel, int block, size_t smem, int* grid_out);
 
+// Raise the kernel's limit of dynamic shared memory where a launch of `bytes`
+// needs it: the default of 48 KB holds the kernel's static arrays too, at most
+// kStaticShared.
+constexpr size_t kStaticShared = 8 * 1024;
+int allow_shared(const void* kernel, size_t bytes);
+
 // The calling device's work-array pool (created on first use, keeps freed
 // memory reserved), and the bytes it holds reserved but unused.
 int library_pool(cudaMemPool_t* out);

@@ -642,8 +642,7 @@ int launch_sweep(const SweepArgs& A, cudaStream_t s)
         FoldSplit sp = fold_split(A.n_items, A.R, sms, d);
         const size_t sm = (d ? FoldTable<double>::kBytes : FoldTable<float>::kBytes) * (size_t)((A.F + 1) & ~1) + sp.lk_bytes;
         const void* fp = d ? (const void*)k_sweep_pp<double> : (const void*)k_sweep_pp<float>;
-        if (sm > 48 * 1024)
-            URCHIN_TRY_CUDA(cudaFuncSetAttribute(fp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        URCHIN_TRY(allow_shared(fp, sm));
         int g = 0;
         URCHIN_TRY(grid_for(fp, kFoldThreads, sm, &g));
         const int64_t need = (A.n_items + sp.rows - 1) / sp.rows;
@@ -664,8 +663,7 @@ int launch_sweep(const SweepArgs& A, cudaStream_t s)
         {(const void*)k_sweep<double, kSweepPlain>, (const void*)k_sweep<double, kSweepNearFar>,
          (const void*)k_sweep<double, kSweepHelium>}};
     const void* fn = fns[f64 ? 1 : 0][var];
-    if (smem > 48 * 1024)
-        URCHIN_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    URCHIN_TRY(allow_shared(fn, smem));
     int rows_per_block = kSweepThreads / A.R;
     int64_t need = (A.n_items + rows_per_block - 1) / rows_per_block;
     int grid = 0;
@@ -1953,8 +1951,7 @@ int Solver::adjoint(const uint8_t* state_orig, const double* xbar_orig, int cold
         // e2, wn and (FP32) the tail e2t of fold_prepare
         const size_t smem = (f64 ? 2 * sizeof(double) : 3 * sizeof(float)) * (size_t)P.spectrum.F;
         const void* fw = f64 ? (const void*)k_adj_wcoef<double> : (const void*)k_adj_wcoef<float>;
-        if (smem > 48 * 1024)
-            URCHIN_TRY_CUDA(cudaFuncSetAttribute(fw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        URCHIN_TRY(allow_shared(fw, smem));
         if (f64)
             k_adj_wcoef<double><<<ga, 256, smem, s>>>(list, na, P.R, static_cast<const double*>(tau), P.spectrum.s,
                                                       P.spectrum.w, P.spectrum.F, nu, E, x, nH, aA, aB, gc, latch,

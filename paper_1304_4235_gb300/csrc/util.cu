@@ -132,6 +132,13 @@ int grid_for(const void* kernel, int block, size_t smem, int* grid_out)
     return URCHIN_OK;
 }
 
+int allow_shared(const void* kernel, size_t bytes)
+{
+    if (bytes + kStaticShared > 48 * 1024)
+        URCHIN_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return URCHIN_OK;
+}
+
 // ---------------------------------------------------------------------------
 // Exclusive scan: tiles of kScanTile values per block, recursive on tile sums.
 // ---------------------------------------------------------------------------

@@ -1,4 +1,8 @@
 """Calls at the ends of their ranges and beside one another."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -62,3 +66,50 @@ def test_rate_transpose_fp32_of_wide_spectra(decades):
     g, _ = U.urchin_gamma_vjp(_dev(t, np.float32), _dev([1.0, 0.02]), _dev([1e-12, 1e-60]), _dev([1e50]), want_w=False)
     want = -1e50 * 1e-60 * 0.02 * np.exp(-40.0)
     assert abs(float(g[0, 0]) - want) <= 1e-6 * abs(want)
+
+
+def test_bins_that_fill_the_default_shared_memory():
+    # dynamic sizes within a block's static ones of 48 KB, in a process whose
+    # earlier calls have not raised the limit (24 B per bin in the fold, with
+    # the log rates of a block's rows, and 16 B in the rate transpose)
+    code = """
+import numpy as np, torch
+import workloads as W
+from gpu_helpers import build, small_halo
+from paper_1304_4235_gb300 import urchin as U
+def spec(F):
+    e, J = W.powerlaw_spectrum(F, 13.6, 54.4)
+    return [torch.from_numpy(a).cuda() for a in U.urchin_spectrum_weights(e, J, 1e-12)]
+g = torch.Generator(device="cuda").manual_seed(1)
+tau = lambda n, R: 10.0 ** (6 * torch.rand(n, R, generator=g, device="cuda") - 4)
+for n, R, F in ((130000, 12, 2048), (65536, 12, 1536), (40000, 48, 1024), (9000, 192, 1024)):
+    s, w = spec(F)
+    t = tau(n, R)
+    a = U.urchin_gamma(t, s, w)[0]
+    b = torch.exp(-t[:64, :, None].double() * s) @ w
+    assert float((a[:64] / b.mean(1) - 1).abs().max()) < 1e-5
+for F in (3040, 3072):
+    s, w = spec(F)
+    t = tau(300, 12)
+    one = torch.ones(300, dtype=torch.float64, device="cuda")
+    a = U.urchin_gamma_vjp(t, s, w, one, want_w=True)
+    b = U.urchin_gamma_vjp(t.double(), s, w, one, want_w=True)
+    assert float((a[0] / b[0] - 1).abs().max()) < 1e-6 and float((a[1] / b[1] - 1).abs().max()) < 1e-6
+for n, F in ((65536, 1536), (4096, 4093)):
+    w = small_halo(n=n, seed=2)
+    bvh, d = build(w, torch)
+    s, wt = spec(F)
+    state = torch.empty(n, dtype=torch.uint8, device="cuda")
+    x, _ = U.urchin_solve(bvh, U.urchin_healpix_dirs(1), w.l_ray, s, wt, d["nH"], d["T"], tol=1e-300, max_iter=1,
+                          state=state, raise_not_converged=False)
+    assert bool(torch.isfinite(x).all())
+    if n < 10000:
+        wb, _ = U.urchin_solve_vjp(bvh, U.urchin_healpix_dirs(1), w.l_ray, s, wt, d["nH"], d["T"], x, state,
+                                   torch.ones_like(x), max_iter=1, raise_not_converged=False)
+        assert bool(torch.isfinite(wb).all())
+print("done")
+"""
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(here), here]))
+    r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "done" in r.stdout, r.stderr[-2000:]
