@@ -640,9 +640,10 @@ int launch_sweep(const SweepArgs& A, cudaStream_t s)
         URCHIN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const bool d = A.precision == URCHIN_F64;
         FoldSplit sp = fold_split(A.n_items, A.R, sms, d);
-        const size_t sm = (d ? FoldTable<double>::kBytes : FoldTable<float>::kBytes) * (size_t)((A.F + 1) & ~1) + sp.lk_bytes;
+        const size_t per_bin = d ? FoldTable<double>::kBytes : FoldTable<float>::kBytes;
+        const size_t sm = per_bin * (size_t)((A.F + 1) & ~1) + sp.lk_bytes;
         const void* fp = d ? (const void*)k_sweep_pp<double> : (const void*)k_sweep_pp<float>;
-        URCHIN_TRY(allow_shared(fp, sm));
+        URCHIN_TRY(allow_shared(fp, per_bin * URCHIN_MAX_BINS + kFoldLogs));
         int g = 0;
         URCHIN_TRY(grid_for(fp, kFoldThreads, sm, &g));
         const int64_t need = (A.n_items + sp.rows - 1) / sp.rows;
@@ -654,8 +655,8 @@ int launch_sweep(const SweepArgs& A, cudaStream_t s)
     const bool f64 = A.precision == URCHIN_F64;
     // two per-ray log-rate arrays in double, then e2, wn, s, (FP32) e2t, (helium) s1, s2 and
     // their three FP32 tails
-    const size_t smem =
-        2 * sizeof(double) * kSweepThreads + ((f64 ? 3 : 4) + (A.he ? (f64 ? 2 : 5) : 0)) * (size_t)A.F * rsz;
+    const size_t logs = 2 * sizeof(double) * kSweepThreads, per_bin = ((f64 ? 3 : 4) + (A.he ? (f64 ? 2 : 5) : 0)) * rsz;
+    const size_t smem = logs + per_bin * (size_t)A.F;
     const int var = A.he ? kSweepHelium : (A.near_far ? kSweepNearFar : kSweepPlain);
     const void* fns[2][3] = {
         {(const void*)k_sweep<float, kSweepPlain>, (const void*)k_sweep<float, kSweepNearFar>,
@@ -663,7 +664,7 @@ int launch_sweep(const SweepArgs& A, cudaStream_t s)
         {(const void*)k_sweep<double, kSweepPlain>, (const void*)k_sweep<double, kSweepNearFar>,
          (const void*)k_sweep<double, kSweepHelium>}};
     const void* fn = fns[f64 ? 1 : 0][var];
-    URCHIN_TRY(allow_shared(fn, smem));
+    URCHIN_TRY(allow_shared(fn, logs + per_bin * URCHIN_MAX_BINS));
     int rows_per_block = kSweepThreads / A.R;
     int64_t need = (A.n_items + rows_per_block - 1) / rows_per_block;
     int grid = 0;
@@ -1949,9 +1950,9 @@ int Solver::adjoint(const uint8_t* state_orig, const double* xbar_orig, int cold
         stats.converged = gres.rel_residual <= P.tol ? 1 : 0;
         // active particles: w_bar_b += sum_a phi_a rho_ab
         // e2, wn and (FP32) the tail e2t of fold_prepare
-        const size_t smem = (f64 ? 2 * sizeof(double) : 3 * sizeof(float)) * (size_t)P.spectrum.F;
+        const size_t per_bin = f64 ? 2 * sizeof(double) : 3 * sizeof(float), smem = per_bin * (size_t)P.spectrum.F;
         const void* fw = f64 ? (const void*)k_adj_wcoef<double> : (const void*)k_adj_wcoef<float>;
-        URCHIN_TRY(allow_shared(fw, smem));
+        URCHIN_TRY(allow_shared(fw, per_bin * URCHIN_MAX_BINS));
         if (f64)
             k_adj_wcoef<double><<<ga, 256, smem, s>>>(list, na, P.R, static_cast<const double*>(tau), P.spectrum.s,
                                                       P.spectrum.w, P.spectrum.F, nu, E, x, nH, aA, aB, gc, latch,

@@ -46,7 +46,7 @@ int launch_gamma_t(const GammaJob& J, cudaStream_t s)
     const FoldSplit sp = fold_split(J.n_rows, J.R, sms, sizeof(Real) == 8);
     const size_t smem = FoldTable<Real>::kBytes * (size_t)((J.F + 1) & ~1) + sp.lk_bytes;
     auto fn = k_gamma<Real>;
-    URCHIN_TRY(allow_shared((const void*)fn, smem));
+    URCHIN_TRY(allow_shared((const void*)fn, FoldTable<Real>::kBytes * URCHIN_MAX_BINS + kFoldLogs));
     const int64_t need = (J.n_rows + sp.rows - 1) / sp.rows;
     int grid = 0;
     URCHIN_TRY(grid_for((const void*)fn, kFoldThreads, smem, &grid));
@@ -583,7 +583,7 @@ int gamma_vjp_t(const Real* tau, int64_t n_orig, int R, const urchin_spectrum* s
         void (*fn)(const Real*, int64_t, int, const double*, const double*, int, const double*, Real*);
         if constexpr (kF32) fn = k_gamma_vjp_tau32;
         else fn = k_gamma_vjp_tau;
-        URCHIN_TRY(allow_shared((const void*)fn, smem));
+        URCHIN_TRY(allow_shared((const void*)fn, 16 * (size_t)URCHIN_MAX_BINS));
         int grid = 0;
         URCHIN_TRY(grid_for((const void*)fn, 256, smem, &grid));
         grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (n_rays + 255) / 256));
@@ -628,10 +628,13 @@ int launch_wbar(const void* tau, int precision, int64_t n_rays, const double* lc
 {
     if (n_rays <= 0) return URCHIN_OK;
     const bool f64 = precision == URCHIN_F64;
-    const size_t smem = f64 ? sizeof(double) * (2 * (size_t)F + 3 * kWTile)
-                            : sizeof(double) * ((size_t)F + kWTile) + sizeof(float) * (2 * (size_t)F + 2 * kWTile);
+    auto bytes = [f64](size_t bins) {
+        return f64 ? sizeof(double) * (2 * bins + 3 * kWTile)
+                   : sizeof(double) * (bins + kWTile) + sizeof(float) * (2 * bins + 2 * kWTile);
+    };
+    const size_t smem = bytes((size_t)F);
     const void* fn = f64 ? (const void*)k_wbar_tiles<double> : (const void*)k_wbar_tiles_f32;
-    URCHIN_TRY(allow_shared(fn, smem));
+    URCHIN_TRY(allow_shared(fn, bytes(URCHIN_MAX_BINS)));
     const int64_t tiles = (n_rays + kWTile - 1) / kWTile;
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 608));
     Scratch part;
@@ -789,7 +792,7 @@ extern "C" int urchin_gamma_nearfar(const void* tau_far, const void* tau_near, i
     const size_t smem = sizeof(double) * 2 * (size_t)sp->F;
     const bool f64 = precision == URCHIN_F64;
     const void* fn = f64 ? (const void*)k_gamma_nearfar<double> : (const void*)k_gamma_nearfar<float>;
-    URCHIN_TRY(allow_shared(fn, smem));
+    URCHIN_TRY(allow_shared(fn, sizeof(double) * 2 * URCHIN_MAX_BINS));
     const int rows = kNearFarThreads / R;
     int grid = 0;
     URCHIN_TRY(grid_for(fn, kNearFarThreads, smem, &grid));
@@ -827,13 +830,13 @@ extern "C" int urchin_gamma_he(const void* tau, const void* tau_he1, const void*
     cudaStream_t s = (cudaStream_t)stream;
     const size_t smem = sizeof(double) * 4 * (size_t)sp->F;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_orig + 127) / 128, 4096));
+    URCHIN_TRY(allow_shared(precision == URCHIN_F64 ? (const void*)k_gamma_he<double> : (const void*)k_gamma_he<float>,
+                            sizeof(double) * 4 * URCHIN_MAX_BINS));
     if (precision == URCHIN_F64) {
-        URCHIN_TRY(allow_shared((const void*)k_gamma_he<double>, smem));
         k_gamma_he<double><<<grid, 128, smem, s>>>(static_cast<const double*>(tau), static_cast<const double*>(tau_he1),
                                                    static_cast<const double*>(tau_he2), n_orig, R, sp->s, sp->s_he1,
                                                    sp->s_he2, sp->w, sp->F, gamma_out, tau_eff_out);
     } else {
-        URCHIN_TRY(allow_shared((const void*)k_gamma_he<float>, smem));
         k_gamma_he<float><<<grid, 128, smem, s>>>(static_cast<const float*>(tau), static_cast<const float*>(tau_he1),
                                                   static_cast<const float*>(tau_he2), n_orig, R, sp->s, sp->s_he1,
                                                   sp->s_he2, sp->w, sp->F, gamma_out, tau_eff_out);

@@ -243,6 +243,7 @@ struct FoldSplit {
     size_t lk_bytes;              // shared memory for the log rates (G > 1)
 };
 constexpr int kFoldThreads = 256;
+constexpr size_t kFoldLogs = 24 * 1024;   // largest lk_bytes
 
 // Threads wanted per SM: 768 (FP64 1536).  ms with 256 / 768 / 1536 / 3072:
 // 50003 rows of 12 rays and 100 bins 0.130 / 0.113 / 0.119 / 0.148, solve of a
@@ -253,7 +254,7 @@ inline FoldSplit fold_split(int64_t n_rows, int R, int sms, bool f64)
     FoldSplit f;
     const int64_t want = (int64_t)sms * (f64 ? 1536 : 768);
     int64_t g = std::min<int64_t>(R, (want + n_rows - 1) / std::max<int64_t>(n_rows, 1));
-    // the log rates of a block's rows within 24 KB
+    // the log rates of a block's rows within kFoldLogs
     if (g > 1) g = std::min<int64_t>(R, std::max<int64_t>(g, (R + 11) / 12));
     f.per = (int)(R / g);
     if (g > 1 && f.per > 1) f.per &= ~1;           // rays are folded two at a time

@@ -132,10 +132,10 @@ int grid_for(const void* kernel, int block, size_t smem, int* grid_out)
     return URCHIN_OK;
 }
 
-int allow_shared(const void* kernel, size_t bytes)
+int allow_shared(const void* kernel, size_t most)
 {
-    if (bytes + kStaticShared > 48 * 1024)
-        URCHIN_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    if (most + kStaticShared > 48 * 1024)
+        URCHIN_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     return URCHIN_OK;
 }
 

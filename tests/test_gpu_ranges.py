@@ -2,6 +2,7 @@
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -113,3 +114,74 @@ print("done")
     env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(here), here]))
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "done" in r.stdout, r.stderr[-2000:]
+
+
+def test_threads_with_different_sizes():
+    # calls of one kernel with different amounts of shared memory from six threads
+    # at once: none is refused, and each gives what it gives alone
+    w = small_halo(n=600, seed=8)
+    bvh, _ = build(w, torch)
+    x = _dev(np.exp(np.random.default_rng(1).uniform(np.log(1e-4), 0.0, w.n)))
+    tau = torch.rand(64, 12, device="cuda") * 10
+
+    def columns(nside):
+        return lambda: U.urchin_trace_columns(bvh, x, U.urchin_healpix_dirs(nside), w.l_ray)
+
+    def rate(F):
+        e, J = W.powerlaw_spectrum(F, 13.6, 54.4)
+        s, wt = (_dev(a) for a in U.urchin_spectrum_weights(e, J, 1e-12))
+        return lambda: U.urchin_gamma(tau, s, wt)[0]
+
+    for fa, fb, times in ((columns(1), columns(4), 300), (rate(2100), rate(4096), 3000)):
+        want, bad = [fa(), fb()], []
+
+        def work(f, ref):
+            try:
+                for _ in range(times):
+                    if not torch.equal(f(), ref):
+                        bad.append("differs")
+            except Exception as e:      # noqa: BLE001
+                bad.append(repr(e))
+
+        th = [threading.Thread(target=work, args=a) for a in 3 * list(zip((fa, fb), want))]
+        for t in th:
+            t.start()
+        for t in th:
+            t.join()
+        assert not bad, bad[:3]
+
+
+@pytest.mark.parametrize("precision", [U.F32, U.F64])
+def test_192_directions_in_every_form(precision):
+    w = small_halo(n=1500, seed=9)
+    bvh, d = build(w, torch)
+    x = _dev(np.exp(np.random.default_rng(2).uniform(np.log(1e-4), 0.0, w.n)))
+    dirs = U.urchin_healpix_dirs(4)
+    pick = np.arange(0, 192, 17)
+    kw = dict(precision=precision)
+    # a ray does not depend on the other directions
+    full = U.urchin_trace_columns(bvh, x, dirs, w.l_ray, **kw)
+    part = U.urchin_trace_columns(bvh, x, dirs[pick], w.l_ray, **kw)
+    assert torch.equal(full[:, _dev(pick, np.int64)], part)
+    nf, np_ = (U.urchin_trace_columns_nearfar(bvh, x, q, w.l_ray, **kw) for q in (dirs, dirs[pick]))
+    # (near columns to 2 ulp in FP32: their few full chords are added between the
+    # partial ones as the packet's queue fills)
+    assert torch.equal(nf[0][:, _dev(pick, np.int64)], np_[0])
+    near = nf[1][:, _dev(pick, np.int64)]
+    assert float(((near - np_[1]).abs() / np_[1]).max()) <= (2.4e-7 if precision == U.F32 else 0.0)
+    # the transpose is linear in the rays: the two halves of the directions add
+    # up (FP64 sums in any order of values rounded alike)
+    tb = torch.rand(w.n, 192, device="cuda", dtype=torch.float64)
+    tb = tb.float() if precision == U.F32 else tb
+    xb = U.urchin_trace_columns_vjp(bvh, dirs, w.l_ray, tb, **kw)
+    parts = sum(U.urchin_trace_columns_vjp(bvh, dirs[a:a + 96], w.l_ray, tb[:, a:a + 96].contiguous(), **kw)
+                for a in (0, 96))
+    assert float(((xb - parts).abs() / parts.clamp_min(1e-300)).max()) < 1e-12
+    # lists kept while tracing (FP32), counted and filled, and no lists: sweep 0
+    # has the same columns
+    (s, wts), _ = spectra(w, torch)
+    for near_far in (False, True):
+        xs = [U.urchin_solve(bvh, dirs, w.l_ray, s, wts, d["nH"], d["T"], tol=1e-300, max_iter=1, segments=g,
+                             near_far=near_far, raise_not_converged=False, **kw)[0]
+              for g in (U.SEG_RECOMPUTE, U.SEG_AUTO, U.SEG_STORE)]
+        assert torch.equal(xs[0], xs[1]) and torch.equal(xs[0], xs[2])
