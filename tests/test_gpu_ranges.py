@@ -185,3 +185,24 @@ def test_192_directions_in_every_form(precision):
                              near_far=near_far, raise_not_converged=False, **kw)[0]
               for g in (U.SEG_RECOMPUTE, U.SEG_AUTO, U.SEG_STORE)]
         assert torch.equal(xs[0], xs[1]) and torch.equal(xs[0], xs[2])
+
+
+@pytest.mark.parametrize("precision", [U.F32, U.F64])
+def test_rays_longer_than_the_particle_set(precision):
+    # isolated particles: beyond the far side of the set there is nothing, so
+    # longer rays have the same columns (bit for bit: the same chords) and are
+    # filtered against no more spheres
+    w = small_halo(n=6000, seed=12)
+    bvh, d = build(w, torch)
+    x = _dev(np.exp(np.random.default_rng(3).uniform(np.log(1e-4), 0.0, w.n)))
+    (s, wts), _ = spectra(w, torch)
+    dirs = U.urchin_healpix_dirs(1)
+    ref, tests = None, None
+    for l in (1e3, 1e6, 1e9, 1e20, 1e30, 1e300):
+        tau = U.urchin_trace_columns(bvh, x, dirs, l, precision=precision)
+        _, st = U.urchin_solve(bvh, dirs, l, s, wts, d["nH"], d["T"], tol=1e-300, max_iter=1, profile=True,
+                               precision=precision, raise_not_converged=False)
+        if ref is None:
+            ref, tests = tau, st["sphere_tests"]
+        assert torch.equal(tau, ref)
+        assert st["sphere_tests"] <= 1.01 * tests
