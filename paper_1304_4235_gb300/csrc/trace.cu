@@ -534,6 +534,7 @@ struct Staged {
     float2 g[kF32 ? 32 : 1];      // 1/h and h^2
     float2 w23[k3 ? 32 : 1];      // the other tracers' weights
     int j[32];                    // Morton slot
+    int img_lo[3], img_n[2], img_batches;     // image_range, and the images' number / 32
     unsigned hit[kPairs / 32 + 1], full[kPairs / 32 + 1], any[kPairs / 32 + 1];   // bit per pair; any: near ones too
     uint16_t pair[kPairs];        // sphere << 5 | lane
 };
@@ -1317,6 +1318,28 @@ __device__ __forceinline__ void packet_image(const TraceParams& P, const unsigne
     __syncwarp();
 }
 
+// The images a of one axis, lo <= a < lo + n, whose particles (bounds [rl, rh]
+// + a L) a beam over [c - h, c + h] may reach; m covers the roundings of the
+// shifted bounds and origins.
+__device__ __forceinline__ void image_range(float c, float h, float rl, float rh, float L, float m, int nimg, int& lo,
+                                            int& n)
+{
+    m += 2e-6f * (fabsf(c) + h);
+    lo = max(-nimg, (int)ceilf((c - h - m - rh) / L));
+    n = max(0, min(nimg, (int)floorf((c + h + m - rl) / L)) - lo + 1);
+}
+
+// Shift of image i of a beam, in ascending order of (x, y, z).
+__device__ __forceinline__ int3 image_shift(int64_t i, const int* lo, int ny, int nz)
+{
+    if (i <= 0x7fffffff) {
+        const unsigned u = (unsigned)i, q = u / (unsigned)nz, x = q / (unsigned)ny;
+        return make_int3(lo[0] + (int)x, lo[1] + (int)(q - x * (unsigned)ny), lo[2] + (int)(u - q * (unsigned)nz));
+    }
+    const int64_t q = i / nz, x = q / ny;
+    return make_int3(lo[0] + (int)x, lo[1] + (int)(q - x * ny), lo[2] + (int)(i - q * nz));
+}
+
 // A packet's origins usually fit in a few smoothing lengths, but some packets
 // straddle a gap of the origins' order (a jump of the Morton curve, a sparse
 // sample of origins), and one beam around all of them would sweep much of the
@@ -1335,8 +1358,6 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
     const int lane = threadIdx.x & 31;
     const float Lf = P.l_beam;
     const int nimg = P.periodic ? P.nimg : 0;
-    const int side = 2 * nimg + 1;
-    const int images = side * side * side;
     constexpr bool kQueue = MODE != MODE_COUNT;
     float3 pt = make_float3(0.f, 0.f, 0.f);
     unsigned left = __ballot_sync(0xffffffffu, live);
@@ -1354,31 +1375,37 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
         const unsigned lv = __ballot_sync(0xffffffffu, in);
         left &= ~lv;
         // the images of the box that the unshifted beam may reach, 32 at a
-        // time, then one after the other in the order of their indices; away
-        // from the faces that is the box itself (image `home`), with the same
-        // beam
-        const int home = images / 2;
+        // time, then one after the other in ascending order; away from the faces
+        // that is the box itself, with the same beam
         bool have_beam = false;
-        for (int i0 = 0; i0 < (drain ? 1 : images); i0 += 32) {
+        for (int b = 0;; ++b) {
             unsigned im = 1u;
-            if (images > 1 && !drain) {
+            if (nimg > 0 && !drain) {
                 pt = make_beam<Real>(beam, lv, in, Real(o.x), Real(o.y), Real(o.z), (float)dx, (float)dy, (float)dz, Lf);
-                // the shifted faces and the shifted origins are each rounded
                 const float Lb = (float)P.Lbox, m1 = 2e-6f * (Lb + fabsf(P.root_lo[0]) + fabsf(P.root_hi[0]) + fabsf(P.root_lo[1]) +
                                                               fabsf(P.root_hi[1]) + fabsf(P.root_lo[2]) + fabsf(P.root_hi[2]));
                 const float4 bc = beam->c, bo = beam->o;
-                if (bc.x + bo.x < P.root_lo[0] + Lb - m1 && bc.x - bo.x > P.root_hi[0] - Lb + m1 &&
-                    bc.y + bo.y < P.root_lo[1] + Lb - m1 && bc.y - bo.y > P.root_hi[1] - Lb + m1 &&
-                    bc.z + bo.z < P.root_lo[2] + Lb - m1 && bc.z - bo.z > P.root_hi[2] - Lb + m1) {
-                    i0 = home & ~31;
-                    im = 1u << (home & 31);
-                    have_beam = true;
-                } else {
-                    const int i = i0 + lane;
+                int lo[3], nx, ny, nz;
+                image_range(bc.x, bo.x, P.root_lo[0], P.root_hi[0], Lb, m1, nimg, lo[0], nx);
+                image_range(bc.y, bo.y, P.root_lo[1], P.root_hi[1], Lb, m1, nimg, lo[1], ny);
+                image_range(bc.z, bo.z, P.root_lo[2], P.root_hi[2], Lb, m1, nimg, lo[2], nz);
+                const int64_t images = (int64_t)nx * ny * nz;
+                if (lane == 0) {
+                    S.img_lo[0] = lo[0];
+                    S.img_lo[1] = lo[1];
+                    S.img_lo[2] = lo[2];
+                    S.img_n[0] = ny;
+                    S.img_n[1] = nz;
+                    S.img_batches = (int)min((images + 31) >> 5, (int64_t)0x7fffffff);
+                }
+                __syncwarp();
+                have_beam = images == 1 && lo[0] == 0 && lo[1] == 0 && lo[2] == 0;
+                if (!have_beam) {
+                    const int64_t i = (int64_t)b * 32 + lane;
                     bool pass = false;
                     if (i < images) {
-                        const float ax = (float)(i / (side * side) - nimg) * Lb, ay = (float)((i / side) % side - nimg) * Lb,
-                                    az = (float)(i % side - nimg) * Lb;
+                        const int3 a = image_shift(i, lo, ny, nz);
+                        const float ax = (float)a.x * Lb, ay = (float)a.y * Lb, az = (float)a.z * Lb;
                         const float m = 1e-6f * (fabsf(ax) + fabsf(ay) + fabsf(az) + Lb);
                         pass = beam_box(*beam,
                                         make_float4(P.root_lo[0] + ax - m, P.root_lo[1] + ay - m, P.root_lo[2] + az - m, 0.f),
@@ -1388,25 +1415,25 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
                 }
             }
             for (; im; im &= im - 1u) {
-                const int i = i0 + __ffs(im) - 1;
-                const int ax = i / (side * side) - nimg, ay = (i / side) % side - nimg, az = i % side - nimg;
+                int3 a = make_int3(0, 0, 0);
+                if (nimg > 0 && !drain) a = image_shift((int64_t)b * 32 + __ffs(im) - 1, S.img_lo, S.img_n[0], S.img_n[1]);
                 // images of the particles at r_j + a L are reached by shifting the
                 // origin to r_i - a L
-                const Real sx = Real(o.x) - Real(ax) * Real(P.Lbox);
-                const Real sy = Real(o.y) - Real(ay) * Real(P.Lbox);
-                const Real sz = Real(o.z) - Real(az) * Real(P.Lbox);
+                const Real sx = Real(o.x) - Real(a.x) * Real(P.Lbox);
+                const Real sy = Real(o.y) - Real(a.y) * Real(P.Lbox);
+                const Real sz = Real(o.z) - Real(a.z) * Real(P.Lbox);
                 S.org[lane] = Origin<Real>{sx, sy, sz, sk.coef};
                 if (NF) {
-                    S.near_o[lane][0] = (double)o.x - (double)ax * P.Lbox;
-                    S.near_o[lane][1] = (double)o.y - (double)ay * P.Lbox;
-                    S.near_o[lane][2] = (double)o.z - (double)az * P.Lbox;
+                    S.near_o[lane][0] = (double)o.x - (double)a.x * P.Lbox;
+                    S.near_o[lane][1] = (double)o.y - (double)a.y * P.Lbox;
+                    S.near_o[lane][2] = (double)o.z - (double)a.z * P.Lbox;
                 }
                 if (!drain && !have_beam)
                     pt = make_beam<Real>(beam, lv, in, sx, sy, sz, (float)dx, (float)dy, (float)dz, Lf);
                 packet_image<Real, KERNEL, XMODE, NF>(P, tab, *beam, S, pq, qn, stash, pt, Lf, dx, dy, dz, in,
                                                      drain, sk, err, nvisit);
             }
-            if (have_beam) break;
+            if (nimg == 0 || drain || b + 1 >= S.img_batches) break;
         }
     }
 }

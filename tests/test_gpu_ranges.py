@@ -206,3 +206,18 @@ def test_rays_longer_than_the_particle_set(precision):
             ref, tests = tau, st["sphere_tests"]
         assert torch.equal(tau, ref)
         assert st["sphere_tests"] <= 1.01 * tests
+
+
+def test_rays_over_many_periodic_images():
+    # along an axis a shift by a multiple of the box is a symmetry: 700 boxes are
+    # seven times 100 (1401 images a side, more than 2^31 in all)
+    w = W.lattice_box(n_side=6, seed=4)
+    bvh, _ = build(w, torch)
+    x = _dev(np.full(w.n, 0.5))
+    for a in range(3):
+        d = np.zeros((1, 3))
+        d[0, a] = 1.0 if a < 2 else -1.0
+        one, many = (U.urchin_trace_columns(bvh, x, d, k * w.box, origins=_dev([0, 40, 215], np.int32),
+                                            precision=U.F64) for k in (100, 700))
+        assert float(one.min()) > 0.0
+        assert float((many / one / 7.0 - 1.0).abs().max()) < 1e-9
