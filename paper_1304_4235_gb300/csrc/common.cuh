@@ -110,6 +110,9 @@ int scan_counts_u64(const uint32_t* in, uint64_t* out, int64_t n, void* tmp, uin
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of key,
 // for `segs` arrays of n pairs that lie one after the other (each sorted by
 // itself; segs * n below 2^32).
+// Tiles of 4096 pairs once they fill the GPU (kRadixLarge pairs), of 1024 below
+// (more blocks): work space per pair is larger just below kRadixLarge.
+constexpr int64_t kRadixLarge = int64_t(1) << 21;
 size_t radix_tmp_bytes(int64_t n, int64_t segs = 1);
 int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, void* tmp, cudaStream_t s, int64_t segs = 1);
 
@@ -236,7 +239,7 @@ int launch_trace(const TraceJob& job, cudaStream_t s);
 // geometric mean of h, clamped to [1, 64].  Several directions are sorted in
 // one set of launches, up to kRayOrderBatch keys.  Short lists keep item
 // order (kRayOrderMinItems, kRayOrderMinSample).  order needs R * n_items int32; tmp needs
-// ray_order_tmp_bytes(n_items, R).
+// ray_order_tmp_bytes(n_items, R), which does for any shorter list as well.
 constexpr int64_t kRayOrderMinItems = 16384;
 // A caller's list of origins is a sample of the particles (or in any order),
 // so its neighbours lie apart and the order pays much earlier: 3000 of 64^3

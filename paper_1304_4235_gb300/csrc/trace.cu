@@ -1884,7 +1884,12 @@ int64_t order_batch(int64_t n_items, int R)
 
 }  // namespace
 
-size_t ray_order_tmp_bytes(int64_t n_items, int R) { return order_bytes(n_items, order_batch(n_items, R)); }
+// One direction of a list just below kRadixLarge can need more than all of a
+// longer one.
+size_t ray_order_tmp_bytes(int64_t n_items, int R)
+{
+    return std::max(order_bytes(n_items, order_batch(n_items, R)), order_bytes(std::min(n_items, kRadixLarge - 1), 1));
+}
 
 double ray_order_elongation(const urchin_bvh* b, double l_ray)
 {

@@ -279,9 +279,6 @@ int scan_counts_u64(const uint32_t* in, uint64_t* out, int64_t n, void* tmp, uin
 constexpr int kRadixThreads = 256;
 constexpr int kRadixDigits = 256;
 constexpr int kRadixItemsSmall = 4, kRadixItemsLarge = 16;
-// tiles of 4096 pairs once they fill the GPU, of 1024 below (more blocks)
-constexpr int64_t kRadixLarge = int64_t(1) << 21;
-
 static int radix_items(int64_t n, int64_t segs) { return n * segs >= kRadixLarge ? kRadixItemsLarge : kRadixItemsSmall; }
 
 template <int ITEMS>

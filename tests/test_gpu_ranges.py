@@ -221,3 +221,20 @@ def test_rays_over_many_periodic_images():
                                             precision=U.F64) for k in (100, 700))
         assert float(one.min()) > 0.0
         assert float((many / one / 7.0 - 1.0).abs().max()) < 1e-9
+
+
+def test_ray_order_of_a_list_shorter_than_the_particles():
+    # the sort of fewer than 2^21 keys takes smaller tiles, and so more work
+    # space per key: a list just below that of 2^21 particles, one direction
+    n = 1 << 21
+    g = torch.Generator(device="cuda").manual_seed(7)
+    p = torch.rand(3, n, generator=g, device="cuda") * 1000.0
+    h = torch.full((n,), 6.0, device="cuda")
+    bvh = U.urchin_build_bvh(p[0].contiguous(), p[1].contiguous(), p[2].contiguous(), h,
+                             torch.full((n,), 1e60, dtype=torch.float64, device="cuda"), False, 0.0, 3.0857e21)
+    one = torch.ones(n, dtype=torch.float64, device="cuda")
+    state = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    state[::2048] = 2                                    # 1024 frozen particles
+    wb, st = U.urchin_solve_vjp(bvh, np.array([[0.0, 0.6, 0.8]]), 10.0, one[:1].clone(), one[:1] * 1e-12, one * 1e-4,
+                                one * 1e4, one * 1e-3, state, one, max_iter=2, raise_not_converged=False)
+    assert st["n_active"] == n - 1024 and bool(torch.isfinite(wb).all())
