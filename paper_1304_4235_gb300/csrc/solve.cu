@@ -833,7 +833,6 @@ int Solver::timed_trace(TraceJob& job)
         job.out_2 = static_cast<float*>(tau_he1);
         job.out_3 = static_cast<float*>(tau_he2);
         he_w1 = he_w2 = nullptr;
-        stats.traversals += 2;                    // columns of two more tracers, as traversals of their own would count
     }
     cudaEvent_t stop;
     URCHIN_TRY(begin_timed(0, &stop));

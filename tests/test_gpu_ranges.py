@@ -238,3 +238,19 @@ def test_ray_order_of_a_list_shorter_than_the_particles():
     wb, st = U.urchin_solve_vjp(bvh, np.array([[0.0, 0.6, 0.8]]), 10.0, one[:1].clone(), one[:1] * 1e-12, one * 1e-4,
                                 one * 1e4, one * 1e-3, state, one, max_iter=2, raise_not_converged=False)
     assert st["n_active"] == n - 1024 and bool(torch.isfinite(wb).all())
+
+
+def test_traversals_are_those_made():
+    # helium columns traced along with the hydrogen columns are one traversal
+    w = W.lattice_box(n_side=8, seed=3)
+    bvh, d = build(w, torch)
+    edges = np.exp(np.linspace(np.log(13.6), np.log(136.0), 31))
+    mid = np.sqrt(edges[:-1] * edges[1:])
+    s, wts = U.urchin_spectrum_weights(edges, (mid / 13.6) ** -1.5, w.gamma_thin)
+    f1, f2 = W.helium_fractions(w, 9)
+    for g, traces in ((U.SEG_AUTO, 1), (U.SEG_RECOMPUTE, 1), (U.SEG_STORE, 4)):
+        _, st = U.urchin_solve(bvh, U.urchin_healpix_dirs(1), w.l_ray, _dev(s), _dev(wts), d["nH"], d["T"], tol=1e-300,
+                               max_iter=1, segments=g, s_he1=_dev(W.hei_cross_section_standin(edges)),
+                               s_he2=_dev(U.urchin_cross_section_ratio(edges, U.XSEC_HEII)), he1=_dev(f1),
+                               he2=_dev(f2), raise_not_converged=False)
+        assert st["trace_launches"] == traces and st["traversals"] == traces
