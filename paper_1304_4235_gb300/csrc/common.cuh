@@ -78,14 +78,14 @@ struct Layout {
 
 int grid_for(const void* kernel, int block, size_t smem, int* grid_out);
 
-// Raise the kernel's limit of dynamic shared memory to `most` bytes where the
-// default does not do: 48 KB, which hold the kernel's static arrays too, at most
-// kStaticShared.  The limit belongs to the kernel and not to the launch, so
-// `most` is the size of the kernel's largest launch, whatever the call: callers
-// on several threads then set the same value, and none lowers it between
-// another's setting and launch.
+// Raise the kernel's limit of dynamic shared memory to `most` bytes where a
+// launch of `bytes` needs more than the default: 48 KB, which hold the kernel's
+// static arrays too, at most kStaticShared.  The limit belongs to the kernel and
+// not to the launch, so `most` is the size of the kernel's largest launch,
+// whatever the call: callers on several threads then set the same value, and
+// none lowers it between another's setting and launch.
 constexpr size_t kStaticShared = 8 * 1024;
-int allow_shared(const void* kernel, size_t most);
+int allow_shared(const void* kernel, size_t bytes, size_t most);
 
 // The calling device's work-array pool (created on first use, keeps freed
 // memory reserved), and the bytes it holds reserved but unused.

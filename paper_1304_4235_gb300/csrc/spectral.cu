@@ -18,8 +18,53 @@ namespace urchin {
 
 namespace {
 
+constexpr int kGammaThreads = 256;
+
+// Threads (local, k) fold ray k of row `local` (fold_ray: the exponent of
+// every bin formed without rounding error); the per-row log-sum-exp runs with
+// one thread per row packed into the first lanes.
 template <typename Real>
-__global__ void __launch_bounds__(kFoldThreads) k_gamma(GammaJob J, FoldSplit sp)
+__global__ void __launch_bounds__(kGammaThreads) k_gamma(GammaJob J)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr bool kF32 = sizeof(Real) == 4;
+    double* lk = reinterpret_cast<double*>(smem_raw);
+    Real* e2 = reinterpret_cast<Real*>(lk + kGammaThreads);
+    Real* wn = e2 + J.F;
+    Real* e2t = kF32 ? wn + J.F : nullptr;
+    __shared__ double sh[2];
+    fold_prepare<Real>(J.s, J.w, J.F, e2, e2t, wn, nullptr, sh);
+    const int rows_per_block = kGammaThreads / J.R;
+    const int local = threadIdx.x / J.R;
+    const int k = threadIdx.x % J.R;
+    const double gthin = sh[0];
+    const double smin = sh[1];
+    for (int64_t row0 = (int64_t)blockIdx.x * rows_per_block; row0 < J.n_rows;
+         row0 += (int64_t)gridDim.x * rows_per_block) {
+        const int64_t row = row0 + local;
+        if (local < rows_per_block && row < J.n_rows) {
+            const Real tau = static_cast<const Real*>(J.tau)[row * J.row_stride + (int64_t)k * J.k_stride];
+            Real S, S2;
+            fold_ray<false>(tau, e2, e2t, wn, nullptr, J.F, S, S2);
+            lk[local * J.R + k] = ray_lnrate(smin, tau, S);
+        }
+        __syncthreads();
+        const int p = threadIdx.x;
+        const int64_t prow = row0 + p;
+        if (p < rows_per_block && prow < J.n_rows) {
+            RayMean<Real> lse;
+            for (int r = 0; r < J.R; ++r) lse.add(lk[p * J.R + r]);
+            const double lmean = lse.mean(J.R);     // ln(Gamma / Gamma_thin)
+            J.gamma_out[prow] = gthin * exp(lmean);
+            if (J.tau_eff_out) J.tau_eff_out[prow] = (float)(-lmean);
+        }
+        __syncthreads();
+    }
+}
+
+// The same with fewer threads than rays (fold_rows): the same bits.
+template <typename Real>
+__global__ void __launch_bounds__(kFoldThreads) k_gamma_rows(GammaJob J, FoldSplit sp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FoldTable<Real> T(smem_raw, J.F);
@@ -37,21 +82,44 @@ __global__ void __launch_bounds__(kFoldThreads) k_gamma(GammaJob J, FoldSplit sp
         });
 }
 
+// FP32: a thread for several rays where the rays still give 768 threads per SM
+// two each, and the spectrum's table (24 B per bin) leaves an SM its blocks.
+// 12 rays, ms with a thread per ray / per several: 60000 rows, 50 / 400 / 1000
+// bins 0.050 / 0.179 / 0.403 against 0.043 / 0.169 / 0.386, 400003 rows 0.243 /
+// 1.03 / 2.40 against 0.167 / 0.96 / 2.33; 192 rays, 8000 rows, 50 / 400 bins
+// 0.438 / 0.567 against 0.122 / 0.354.  Fewer rays: 2000 rows of 12 rays, 400 /
+// 1000 bins 0.0252 / 0.0426 against 0.0363 / 0.0705 with two rays per thread;
+// more bins: 2000 rows of 192 rays, 2000 bins 0.507 against 0.578.  FP64, whose
+// pipe leaves nothing to fold together: only where a row's log-sum-exp outweighs
+// its bins and the rows are many (192 rays, 8000 rows, 20 bins 3.19 against
+// 1.90 ms; 48 rays, 10000 rows, 200 bins 4.38 against 4.90).
+constexpr int kRowsMaxBins = 1400;
+
 template <typename Real>
 int launch_gamma_t(const GammaJob& J, cudaStream_t s)
 {
     int dev = 0, sms = 0;
     URCHIN_TRY_CUDA(cudaGetDevice(&dev));
     URCHIN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const FoldSplit sp = fold_split(J.n_rows, J.R, sms, sizeof(Real) == 8);
-    const size_t smem = FoldTable<Real>::kBytes * (size_t)((J.F + 1) & ~1) + sp.lk_bytes;
-    auto fn = k_gamma<Real>;
-    URCHIN_TRY(allow_shared((const void*)fn, FoldTable<Real>::kBytes * URCHIN_MAX_BINS + kFoldLogs));
-    const int64_t need = (J.n_rows + sp.rows - 1) / sp.rows;
+    constexpr bool kF32 = sizeof(Real) == 4;
+    const int64_t rays = J.n_rows * J.R;
+    const bool several = kF32 ? rays >= 2 * 768 * (int64_t)sms && J.F <= kRowsMaxBins
+                              : rays >= 6000 * (int64_t)sms && J.F < J.R;
+    const FoldSplit sp = several ? fold_split(J.n_rows, J.R, 1536 * (int64_t)sms, kF32 ? 2 : 1) : FoldSplit{};
+    const void* fn = several ? (const void*)k_gamma_rows<Real> : (const void*)k_gamma<Real>;
+    auto bytes = [several](int F, size_t logs) {     // the table and the rays' log rates
+        if (several) return FoldTable<Real>::kBytes * (size_t)((F + 1) & ~1) + logs;
+        return sizeof(double) * kGammaThreads + (kF32 ? 3 : 2) * (size_t)F * sizeof(Real);
+    };
+    const size_t smem = bytes(J.F, sp.lk_bytes);
+    URCHIN_TRY(allow_shared(fn, smem, bytes(URCHIN_MAX_BINS, kFoldLogs)));
+    const int rows = several ? sp.rows : kGammaThreads / J.R;
+    const int64_t need = (J.n_rows + rows - 1) / rows;
     int grid = 0;
-    URCHIN_TRY(grid_for((const void*)fn, kFoldThreads, smem, &grid));
+    URCHIN_TRY(grid_for(fn, kGammaThreads, smem, &grid));
     if (need < grid) grid = (int)std::max<int64_t>(need, 1);
-    fn<<<grid, kFoldThreads, smem, s>>>(J, sp);
+    if (several) k_gamma_rows<Real><<<grid, kFoldThreads, smem, s>>>(J, sp);
+    else k_gamma<Real><<<grid, kGammaThreads, smem, s>>>(J);
     URCHIN_TRY(launched());
     return URCHIN_OK;
 }
@@ -583,7 +651,7 @@ int gamma_vjp_t(const Real* tau, int64_t n_orig, int R, const urchin_spectrum* s
         void (*fn)(const Real*, int64_t, int, const double*, const double*, int, const double*, Real*);
         if constexpr (kF32) fn = k_gamma_vjp_tau32;
         else fn = k_gamma_vjp_tau;
-        URCHIN_TRY(allow_shared((const void*)fn, 16 * (size_t)URCHIN_MAX_BINS));
+        URCHIN_TRY(allow_shared((const void*)fn, smem, 16 * (size_t)URCHIN_MAX_BINS));
         int grid = 0;
         URCHIN_TRY(grid_for((const void*)fn, 256, smem, &grid));
         grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (n_rays + 255) / 256));
@@ -634,7 +702,7 @@ int launch_wbar(const void* tau, int precision, int64_t n_rays, const double* lc
     };
     const size_t smem = bytes((size_t)F);
     const void* fn = f64 ? (const void*)k_wbar_tiles<double> : (const void*)k_wbar_tiles_f32;
-    URCHIN_TRY(allow_shared(fn, bytes(URCHIN_MAX_BINS)));
+    URCHIN_TRY(allow_shared(fn, smem, bytes(URCHIN_MAX_BINS)));
     const int64_t tiles = (n_rays + kWTile - 1) / kWTile;
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 608));
     Scratch part;
@@ -792,7 +860,7 @@ extern "C" int urchin_gamma_nearfar(const void* tau_far, const void* tau_near, i
     const size_t smem = sizeof(double) * 2 * (size_t)sp->F;
     const bool f64 = precision == URCHIN_F64;
     const void* fn = f64 ? (const void*)k_gamma_nearfar<double> : (const void*)k_gamma_nearfar<float>;
-    URCHIN_TRY(allow_shared(fn, sizeof(double) * 2 * URCHIN_MAX_BINS));
+    URCHIN_TRY(allow_shared(fn, smem, sizeof(double) * 2 * URCHIN_MAX_BINS));
     const int rows = kNearFarThreads / R;
     int grid = 0;
     URCHIN_TRY(grid_for(fn, kNearFarThreads, smem, &grid));
@@ -831,7 +899,7 @@ extern "C" int urchin_gamma_he(const void* tau, const void* tau_he1, const void*
     const size_t smem = sizeof(double) * 4 * (size_t)sp->F;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_orig + 127) / 128, 4096));
     URCHIN_TRY(allow_shared(precision == URCHIN_F64 ? (const void*)k_gamma_he<double> : (const void*)k_gamma_he<float>,
-                            sizeof(double) * 4 * URCHIN_MAX_BINS));
+                            smem, sizeof(double) * 4 * URCHIN_MAX_BINS));
     if (precision == URCHIN_F64) {
         k_gamma_he<double><<<grid, 128, smem, s>>>(static_cast<const double*>(tau), static_cast<const double*>(tau_he1),
                                                    static_cast<const double*>(tau_he2), n_orig, R, sp->s, sp->s_he1,

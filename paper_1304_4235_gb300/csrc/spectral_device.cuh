@@ -233,9 +233,9 @@ struct RayMean {
 // SM.  The rays are combined in their order either way, so the result does
 // not depend on G.  Bound by the FP32 pipe and issue (FP64: its pipe): packed
 // operations take 10 issue slots per ray and bin instead of 15.  12 rays, 100
-// bins, FP32 / ms: 400003 rows with the equilibrium 0.58 -> 0.50; 200 bins, a
-// sweep of 32768 particles 0.077 -> 0.054; FP64, a sweep of 4096 particles and
-// 50 bins 0.93 -> 0.18 (16 blocks before).
+// bins, FP32 / ms: rates of 400003 rows 0.346 -> 0.277; 200 bins, a sweep of
+// 32768 particles 0.077 -> 0.054; FP64, a sweep of 4096 particles and 50 bins
+// 0.93 -> 0.18 (16 blocks before).
 struct FoldSplit {
     int G;                        // threads per row
     int per;                      // rays per thread
@@ -245,18 +245,14 @@ struct FoldSplit {
 constexpr int kFoldThreads = 256;
 constexpr size_t kFoldLogs = 24 * 1024;   // largest lk_bytes
 
-// Threads wanted per SM: 768 (FP64 1536).  ms with 256 / 768 / 1536 / 3072:
-// 50003 rows of 12 rays and 100 bins 0.130 / 0.113 / 0.119 / 0.148, solve of a
-// 65536-particle halo 195.3 / 192.9 / 194.7 / 203.6; FP64, 60003 rows 3.84 /
-// 3.82 / 3.26 / 3.25.
-inline FoldSplit fold_split(int64_t n_rows, int R, int sms, bool f64)
+// As many threads as `want` where the rows have the rays, at least min_per rays each.
+inline FoldSplit fold_split(int64_t n_rows, int R, int64_t want, int min_per = 1)
 {
     FoldSplit f;
-    const int64_t want = (int64_t)sms * (f64 ? 1536 : 768);
     int64_t g = std::min<int64_t>(R, (want + n_rows - 1) / std::max<int64_t>(n_rows, 1));
     // the log rates of a block's rows within kFoldLogs
     if (g > 1) g = std::min<int64_t>(R, std::max<int64_t>(g, (R + 11) / 12));
-    f.per = (int)(R / g);
+    f.per = std::max((int)(R / g), std::min(R, min_per));
     if (g > 1 && f.per > 1) f.per &= ~1;           // rays are folded two at a time
     f.G = (R + f.per - 1) / f.per;
     f.rows = kFoldThreads / f.G;

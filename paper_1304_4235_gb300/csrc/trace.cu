@@ -1618,7 +1618,7 @@ int launch_one(const TraceParams& P, cudaStream_t s)
     const void* fn = (const void*)k_trace<Real, KERNEL, MODE, NF>;
     using Lay = TraceLayout<Real, KERNEL, MODE, NF>;
     const size_t smem = Lay::bytes(P.R);
-    URCHIN_TRY(allow_shared(fn, Lay::bytes(URCHIN_MAX_RAYS)));
+    URCHIN_TRY(allow_shared(fn, smem, Lay::bytes(URCHIN_MAX_RAYS)));
     int grid = 0;
     URCHIN_TRY(grid_for(fn, 32 * Lay::kWarps, smem, &grid));
     const int64_t tasks = P.n_chunks * P.R;

@@ -132,9 +132,9 @@ int grid_for(const void* kernel, int block, size_t smem, int* grid_out)
     return URCHIN_OK;
 }
 
-int allow_shared(const void* kernel, size_t most)
+int allow_shared(const void* kernel, size_t bytes, size_t most)
 {
-    if (most + kStaticShared > 48 * 1024)
+    if (bytes + kStaticShared > 48 * 1024)
         URCHIN_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     return URCHIN_OK;
 }

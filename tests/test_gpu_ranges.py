@@ -254,3 +254,20 @@ def test_traversals_are_those_made():
                                s_he2=_dev(U.urchin_cross_section_ratio(edges, U.XSEC_HEII)), he1=_dev(f1),
                                he2=_dev(f2), raise_not_converged=False)
         assert st["trace_launches"] == traces and st["traversals"] == traces
+
+
+@pytest.mark.parametrize("dtype,R,F", [(np.float32, 12, 1400), (np.float32, 12, 1401), (np.float32, 5, 3),
+                                       (np.float64, 48, 47), (np.float64, 48, 48)])
+def test_rates_by_rays_and_by_rows(dtype, R, F):
+    # many rows are folded with several rays to a thread (FP32 up to 1400 bins,
+    # FP64 with fewer bins than rays), few by a thread per ray: the same bits
+    n = 960000 // R
+    g = torch.Generator(device="cuda").manual_seed(F)
+    tau = 10.0 ** (9 * torch.rand(n, R, generator=g, device="cuda", dtype=torch.float64) - 5)
+    tau = tau.to(torch.from_numpy(np.zeros(1, dtype)).dtype)
+    e, J = W.powerlaw_spectrum(F, 13.6, 54.4)
+    s, wts = (_dev(a) for a in U.urchin_spectrum_weights(e, J, 1e-12))
+    many = U.urchin_gamma(tau, s, wts)
+    for a in (0, n // 2):
+        few = U.urchin_gamma(tau[a:a + 100].contiguous(), s, wts)
+        assert torch.equal(few[0], many[0][a:a + 100]) and torch.equal(few[1], many[1][a:a + 100])
