@@ -433,16 +433,27 @@ __global__ void k_wbar_tiles_f32(const float* __restrict__ tau, int64_t n_rays, 
 }
 
 // coefficient of Eq. gamma_shld's reverse mode, the same for the rays of a
-// row: c = gamma_bar_o / R
-__global__ void k_gamma_coef(int64_t n_rows, int R, const double* __restrict__ gbar, double* lc, double* sg)
+// row: c = gamma_bar_o / R.  A block takes `rows` rows (at most its threads) at
+// a time: a thread per row for the logarithms, then all of them write (a thread
+// that wrote its row's rays took 500 rows of 192 rays from 0.091 to 0.129 ms).
+__global__ void __launch_bounds__(256) k_gamma_coef(int64_t n_rows, int R, int rows, const double* __restrict__ gbar,
+                                                    double* lc, double* sg)
 {
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n_rows; o += (int64_t)gridDim.x * blockDim.x) {
-        const double c = gbar[o] / (double)R;
-        const double l = c != 0.0 ? log(fabs(c)) : -INFINITY, g = c < 0.0 ? -1.0 : 1.0;
-        for (int k = 0; k < R; ++k) {
-            lc[o * R + k] = l;
-            sg[o * R + k] = g;
+    __shared__ double l[256], g[256];
+    for (int64_t o0 = (int64_t)blockIdx.x * rows; o0 < n_rows; o0 += (int64_t)gridDim.x * rows) {
+        const int m = (int)(n_rows - o0 < rows ? n_rows - o0 : rows);
+        if ((int)threadIdx.x < m) {
+            const double c = gbar[o0 + threadIdx.x] / (double)R;
+            l[threadIdx.x] = c != 0.0 ? log(fabs(c)) : -INFINITY;
+            g[threadIdx.x] = c < 0.0 ? -1.0 : 1.0;
         }
+        __syncthreads();
+        for (int i = threadIdx.x; i < m * R; i += blockDim.x) {
+            const int q = i / R;
+            lc[o0 * R + i] = l[q];
+            sg[o0 * R + i] = g[q];
+        }
+        __syncthreads();
     }
 }
 
@@ -663,8 +674,10 @@ int gamma_vjp_t(const Real* tau, int64_t n_orig, int R, const urchin_spectrum* s
         URCHIN_TRY(cf.alloc(2 * sizeof(double) * (size_t)n_rays + 256, s));
         double* lc = cf.at<double>(0);
         double* sg = lc + n_rays;
-        const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_orig + 255) / 256, 4096));
-        k_gamma_coef<<<g, 256, 0, s>>>(n_orig, R, gbar, lc, sg);
+        // blocks for every SM while the rows last
+        const int rows = (int)std::max<int64_t>(1, std::min<int64_t>(256, n_orig / 1024));
+        const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_orig + rows - 1) / rows, 4096));
+        k_gamma_coef<<<g, 256, 0, s>>>(n_orig, R, rows, gbar, lc, sg);
         URCHIN_TRY(launched());
         URCHIN_TRY(launch_wbar(tau, sizeof(Real) == 8 ? URCHIN_F64 : URCHIN_F32, n_rays, lc, sg, sp->s, F, w_bar, s));
         cf.release();

@@ -271,3 +271,18 @@ def test_rates_by_rays_and_by_rows(dtype, R, F):
     for a in (0, n // 2):
         few = U.urchin_gamma(tau[a:a + 100].contiguous(), s, wts)
         assert torch.equal(few[0], many[0][a:a + 100]) and torch.equal(few[1], many[1][a:a + 100])
+
+
+@pytest.mark.parametrize("n,R", [(1, 12), (1023, 48), (2049, 5), (1500, 192), (270001, 3)])
+def test_spectrum_gradient_of_the_rate(n, R):
+    # the coefficients' blocks take one row up to 256 rows; w_bar in FP64 is the
+    # sum of its terms to their rounding (1e-16 each, about 1e6 of them)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    tau = 10.0 ** (6 * torch.rand(n, R, generator=g, device="cuda", dtype=torch.float64) - 5)
+    gb = torch.randn(n, generator=g, device="cuda", dtype=torch.float64)
+    gb[::7] = 0.0
+    s, wts = _dev([1.0, 0.3, 0.02]), _dev([1e-12, 3e-13, 1e-13])
+    _, wb = U.urchin_gamma_vjp(tau, s, wts, gb, want_tau=False)
+    for b in range(3):
+        e = torch.exp(-float(s[b]) * tau) * (gb / R)[:, None]
+        assert abs(float(wb[b] - e.sum())) <= 1e-12 * float(e.abs().sum())
