@@ -1440,7 +1440,11 @@ __device__ __forceinline__ void ray_column(const TraceParams& P, const unsigned 
 
 // k_trace's shared memory: per warp the work space, the beam, the block of
 // chunks (MODE_CHUNK) and the queue of partial chords (FP64: of hits) in modes
-// that evaluate chords; the M4 table (FP64: of logarithms); the directions (double[3 R]).
+// that evaluate chords; the M4 table (FP64: of logarithms).  The same for any
+// number of directions (192 of them, 4608 B a block, left two blocks of three on
+// an SM): a packet reads its own from global memory.
+constexpr size_t kSmShared = 228 * 1024;      // an SM's shared memory, of which a block takes
+constexpr size_t kBlockShared = 1024;         // this much beside its own
 template <typename Real, int KERNEL, int XMODE, bool NF>
 struct TraceLayout {
     static constexpr int MODE = XMODE & 7;
@@ -1459,8 +1463,8 @@ struct TraceLayout {
     static constexpr size_t kTab = up(kStashAt + kWarps * 2 * sizeof(unsigned long long));
     static constexpr size_t kQueueAt =
         up(kTab + (!kTable ? 0 : kF32 ? sizeof(float2) * (kKTab + 1) : sizeof(double2) * kLogTab));
-    static constexpr size_t kDirs = up(kQueueAt + (kQueue ? sizeof(Queue) * kWarps : 0));
-    static size_t bytes(int R) { return kDirs + sizeof(double) * 3 * (size_t)R; }
+    static constexpr size_t kBytes = up(kQueueAt + (kQueue ? sizeof(Queue) * kWarps : 0));
+    static_assert(kBlocks * (kBytes + kBlockShared) <= kSmShared, "shared memory for the blocks of an SM");
 };
 static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, false>) % 16 == 0, "shared layout");
 
@@ -1504,7 +1508,6 @@ k_trace(TraceParams P)
     unsigned long long* stash = reinterpret_cast<unsigned long long*>(smem + Lay::kStashAt) + 2 * wid;
     unsigned char* s_tab = smem + Lay::kTab;
     typename Lay::Queue* pq = reinterpret_cast<typename Lay::Queue*>(smem + Lay::kQueueAt) + wid;
-    double* s_dirs = reinterpret_cast<double*>(smem + Lay::kDirs);
     if (kQueue) {
         pq->own[threadIdx.x & 31] = 0u;
         if (NF) pq->own[(threadIdx.x & 31) + kPQNear] = 0u;
@@ -1514,7 +1517,6 @@ k_trace(TraceParams P)
         stash[0] = 0ull;
         stash[1] = 0ull;
     }
-    for (int t = threadIdx.x; t < 3 * P.R; t += blockDim.x) s_dirs[t] = P.dirs[t];
     if (Lay::kTable && Lay::kF32)
         for (int t = threadIdx.x; t <= kKTab; t += blockDim.x) reinterpret_cast<float2*>(s_tab)[t] = P.ktab[t];
     if (Lay::kTable && !Lay::kF32) log_table(reinterpret_cast<double2*>(s_tab));
@@ -1539,7 +1541,8 @@ k_trace(TraceParams P)
         const int64_t item = !live ? 0 : (P.order ? (int64_t)P.order[(int64_t)k * P.n_items + slot] : slot);
         const int32_t org = live ? (P.items ? P.items[item] : (int32_t)item) : 0;
         float4 o = __ldg(P.xyzh + org);
-        Real dx = Real(s_dirs[3 * k]), dy = Real(s_dirs[3 * k + 1]), dz = Real(s_dirs[3 * k + 2]);
+        const double* dir = P.dirs + 3 * k;
+        Real dx = Real(__ldg(dir)), dy = Real(__ldg(dir + 1)), dz = Real(__ldg(dir + 2));
         unsigned nvisit = 0;
         Sink<Real> sk{};
         // stored-segment rows are indexed by direction and Morton slot (rows
@@ -1617,8 +1620,8 @@ int launch_one(const TraceParams& P, cudaStream_t s)
 {
     const void* fn = (const void*)k_trace<Real, KERNEL, MODE, NF>;
     using Lay = TraceLayout<Real, KERNEL, MODE, NF>;
-    const size_t smem = Lay::bytes(P.R);
-    URCHIN_TRY(allow_shared(fn, smem, Lay::bytes(URCHIN_MAX_RAYS)));
+    const size_t smem = Lay::kBytes;
+    URCHIN_TRY(allow_shared(fn, smem, smem));
     int grid = 0;
     URCHIN_TRY(grid_for(fn, 32 * Lay::kWarps, smem, &grid));
     const int64_t tasks = P.n_chunks * P.R;
