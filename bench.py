@@ -326,9 +326,10 @@ def timed(stream, fn):
 def roofline_spmv(stats, hbm, peak_kind, n=1 << 24):
     """k_spmv8 (stored-segment columns) against the HBM roofline: 8
     algorithmic bytes per segment (a 4-byte particle index and a 4-byte
-    value; the kernel moves 7, the index split in 16 + 8 bits, or 6 up to
-    65536 particles n), plus each ray's 4-byte column and the 4-byte x gather
-    per particle, over the launch's mean duration."""
+    value), or, up to 65536 particles n, 6 (a 2-byte index), plus each ray's
+    4-byte column and the 4-byte x gather per particle, over the launch's mean
+    duration.  row_gbs and row_frac count the bytes that the rows take instead:
+    7 per segment (the index split in 16 + 8 bits), or 6."""
     launches = sum(st["spmv_launches"] for st in stats)
     spmv_s = sum(st["spmv_s"] for st in stats)
     moved = sum(st["spmv_bytes"] for st in stats)          # 6 or 7 per segment + columns + x
@@ -336,14 +337,16 @@ def roofline_spmv(stats, hbm, peak_kind, n=1 << 24):
     extra = launches * (st0["n_active"] * 12 * 4 + st0["n_active"] * 4)
     seg_bytes = 7 if n > 65536 else 6
     seg = max(moved - extra, 0) / seg_bytes
-    per_bytes = (seg * 8 + extra) / max(launches, 1)
+    per_bytes = (seg * (8 if n > 65536 else 6) + extra) / max(launches, 1)
     per_s = spmv_s / max(launches, 1)
+    row_gbs = moved / max(launches, 1) / per_s / 1e9 if per_s > 0 else None
     achieved = per_bytes / per_s / 1e9 if per_s > 0 else None
     t = MEASURED_TRAFFIC["k_spmv"].get(source_hash("k_spmv"), {}).get(seg_bytes)
     return {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
             "frac": achieved / hbm if achieved else None, "traffic": (t * seg / max(launches, 1)) if t else None,
             "kernel": "k_spmv8 (FP32 stored segments)", "peak_kind": peak_kind, "alg_bytes_per_launch": per_bytes,
-            "launch_ms": per_s * 1e3, "segments_per_launch": seg / max(launches, 1)}
+            "launch_ms": per_s * 1e3, "segments_per_launch": seg / max(launches, 1),
+            "row_gbs": row_gbs, "row_frac": row_gbs / hbm if row_gbs else None}
 
 
 def roofline(stats, trace_launches_total, hbm, peak_kind, rays_per_sweep):

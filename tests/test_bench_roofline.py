@@ -70,3 +70,18 @@ def test_product_bytes_per_segment():
     per = (seg * 8 + extra) / launches
     assert r["alg_bytes_per_launch"] == pytest.approx(per)
     assert r["achieved"] == pytest.approx(per / 0.001 / 1e9)
+
+
+def test_product_bytes_of_6_byte_rows():
+    # up to 65536 particles a segment is 6 bytes, in the rows and at the least;
+    # above, the rows take 7
+    n_act, launches, seg = 1000, 3, 5.0e6
+    extra = launches * (n_act * 12 * 4 + n_act * 4)
+    for n, per_row, per_alg in ((65536, 6, 6), (65537, 7, 8)):
+        st = [{"spmv_launches": launches, "spmv_s": 0.003, "spmv_bytes": seg * per_row + extra, "n_active": n_act}]
+        r = bench.roofline_spmv(st, 6800.0, "fallback", n)
+        assert r["segments_per_launch"] == pytest.approx(seg / launches)
+        assert r["alg_bytes_per_launch"] == pytest.approx((seg * per_alg + extra) / launches)
+        assert r["achieved"] == pytest.approx((seg * per_alg + extra) / 0.003 / 1e9)
+        assert r["row_gbs"] == pytest.approx((seg * per_row + extra) / 0.003 / 1e9)
+        assert r["row_frac"] == pytest.approx(r["row_gbs"] / 6800.0)
