@@ -875,9 +875,10 @@ int Solver::order_for(const int32_t* items, int64_t n_items, const int32_t** out
 
 // The ray order of the active list, derived from sweep 0's order of all
 // particles instead of sorted afresh: ray_order sorts stably by a key of the
-// origin alone, and the list holds the active particles in ascending Morton
-// slot, so the full order restricted to the list is exactly the order a sort
-// of the list would give (2 R radix passes over the list saved per solve).
+// origin alone, so the full order restricted to the list is the order that a
+// sort of the list gives but for equal keys (here by slot, there by the list's
+// Morton order), which decide only what rays share a packet; the list's sort
+// (four passes of all directions) is saved.
 int Solver::derive_list_order(const int32_t* full)
 {
     const int64_t na = n_act;

@@ -164,7 +164,7 @@ template <> struct RealOps<double> {
 // results per clock and SM), so a chord takes as few FP64 operations as it can:
 // one ln b and one join for both ends, the two pieces' polynomials as one with
 // selected coefficients, and logarithms from a table (after Tang, 1990):
-// x = 2^e m, c about 1 / m from the top 7 bits of m, r = m c - 1 exactly,
+// x = 2^e m, c about 1 / m from the top 7 bits of m, r = m c - 1 rounded once,
 // ln x = e ln 2 - ln c + log1p(r), |r| < 0.004, the series to r^7; absolute
 // error about 1e-16, 11 operations where log() takes some 27.
 constexpr int kLogTab = 128;
