@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 import workloads as W
-from gpu_helpers import build, small_halo, spectra
+from gpu_helpers import build, lnrate_sensitivity, small_halo, spectra
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -286,3 +286,33 @@ def test_spectrum_gradient_of_the_rate(n, R):
     for b in range(3):
         e = torch.exp(-float(s[b]) * tau) * (gb / R)[:, None]
         assert abs(float(wb[b] - e.sum())) <= 1e-12 * float(e.abs().sum())
+
+
+@pytest.mark.parametrize("n,per", [(65536, 6), (65537, 7), (80000, 7)])
+def test_products_of_6_and_7_byte_rows(n, per):
+    # one sweep over rows (written by the filling traversal, and copied from the
+    # chunks before the fourth sweep) against the same sweep with traced columns.
+    # These differ by their order of summation, 2e-6, which moves a rate by D times
+    # that (D = sum tau |d ln Gamma / d tau|), and x by no more; the fold rounds its
+    # sums to 1e-6.  At 80000 particles 14464 indices need their high byte; without
+    # it they would be those of particles on the other side of the halo.
+    w = small_halo(n=n, seed=29)
+    bvh, d = build(w, torch)
+    (s, wts), (so, wo) = spectra(w, torch)
+    dirs = U.urchin_healpix_dirs(1)
+
+    def solve(seg, sweeps, x=None, **kw):
+        return U.urchin_solve(bvh, dirs, w.l_ray, s, wts, d["nH"], d["T"], x, tol=1e-300, max_iter=sweeps, segments=seg,
+                              tau_skip=0.0, case_rule=U.CASE_A, raise_not_converged=False, **kw)
+
+    pick = W.random_origins(n, 2500, 31)
+    for seg, before in ((U.SEG_STORE, 1), (U.SEG_AUTO, 4)):
+        x0, _ = solve(seg, before)
+        x1, st = solve(seg, before + 1, profile=True)
+        assert st["segments_stored"]
+        if seg == U.SEG_STORE:
+            assert st["n_active"] == n and st["spmv_bytes"] == st["nnz"] * per + n * 12 * 4 + n * 4
+        tau = U.urchin_trace_columns(bvh, x0, dirs, w.l_ray, origins=_dev(pick, np.int32)).cpu().numpy()
+        want, _ = solve(U.SEG_RECOMPUTE, 1, x0.clone(), warm_start=True)
+        dx = ((x1 - want).abs() / want).cpu().numpy()[pick]
+        assert (dx <= 2e-6 * lnrate_sensitivity(tau, so, wo) + 2e-6).all()
