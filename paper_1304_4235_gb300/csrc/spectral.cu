@@ -82,8 +82,12 @@ __global__ void __launch_bounds__(kFoldThreads) k_gamma_rows(GammaJob J, FoldSpl
         });
 }
 
-// FP32: a thread for several rays where the rays still give 768 threads per SM
-// two each, and the spectrum's table (24 B per bin) leaves an SM its blocks.
+// FP32: a thread for several rays where the rays still give 850 threads per SM
+// two each (at 768 the last wave is nearly empty: 240000 rays, 1400 bins 0.231
+// against 0.244 ms), and the spectrum's table (24 B per bin) leaves an SM its
+// blocks.  An odd number of rays leaves one that is folded alone, which only many
+// rows make up for (3 rays, 400000, 1000 bins 0.252 against 0.270, but 1200000,
+// 100 bins faster by 7 %); with one or two rays there is nothing to gain.
 // 12 rays, ms with a thread per ray / per several: 60000 rows, 50 / 400 / 1000
 // bins 0.050 / 0.179 / 0.403 against 0.043 / 0.169 / 0.386, 400003 rows 0.243 /
 // 1.03 / 2.40 against 0.167 / 0.96 / 2.33; 192 rays, 8000 rows, 50 / 400 bins
@@ -103,7 +107,8 @@ int launch_gamma_t(const GammaJob& J, cudaStream_t s)
     URCHIN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     constexpr bool kF32 = sizeof(Real) == 4;
     const int64_t rays = J.n_rows * J.R;
-    const bool several = kF32 ? rays >= 2 * 768 * (int64_t)sms && J.F <= kRowsMaxBins
+    const bool odd = (J.R & 1) && J.R < 16;
+    const bool several = kF32 ? J.R > 2 && rays >= (odd ? 6000 : 1700) * (int64_t)sms && J.F <= kRowsMaxBins
                               : rays >= 6000 * (int64_t)sms && J.F < J.R;
     const FoldSplit sp = several ? fold_split(J.n_rows, J.R, 1536 * (int64_t)sms, kF32 ? 2 : 1) : FoldSplit{};
     const void* fn = several ? (const void*)k_gamma_rows<Real> : (const void*)k_gamma<Real>;

@@ -321,6 +321,28 @@ __device__ __forceinline__ void fold_pair(const FoldTable<float>& T, int F, bool
     S1 = S.y;
 }
 
+// The same for one ray (the last of an odd number).
+__device__ __forceinline__ float fold_one(const FoldTable<float>& T, int F, bool skip, float t)
+{
+    t = t < 1e30f ? t : (t == t ? 1e30f : t);
+    float S = 0.f, nc = 0.f;
+    int j = 0;
+    if (skip)
+        while (j < F && __all_sync(0xffffffffu, t == t && T.a2[j].x * t <= -152.f)) ++j;
+    for (; j < F; ++j) {
+        const float4 q = T.a2[j];
+        const float np = __fmul_rn(q.x, t);
+        const float err = fmaf(q.z, t, fmaf(q.x, -t, np));
+        const float v0 = __fmul_rn(T.z2[j].x, exp2f(np));
+        const float v = fmaf(v0, __fmul_rn(err, -0.6931471805599453f), v0);
+        const float y = __fadd_rn(v, nc);
+        const float u = __fadd_rn(S, y);
+        nc = __fsub_rn(y, __fsub_rn(u, S));
+        S = u;
+    }
+    return S;
+}
+
 __device__ __forceinline__ void fold_pair(const FoldTable<double>& T, int F, bool, bool two, double t0, double t1,
                                           double& S0, double& S1)
 {
@@ -348,7 +370,12 @@ __device__ __forceinline__ void fold_rows(const FoldSplit sp, int64_t n_rows, in
             const Real t0 = in0 ? tau(row, k0) : Real(1e30);
             const Real t1 = in1 ? tau(row, k1) : t0;
             Real S0 = Real(0), S1 = Real(0);
-            if (sizeof(Real) == 4 || in0) fold_pair(T, F, skip, in1, t0, t1, S0, S1);
+            if constexpr (sizeof(Real) == 4) {
+                if (__any_sync(0xffffffffu, in1)) fold_pair(T, F, skip, in1, t0, t1, S0, S1);
+                else S0 = fold_one(T, F, skip, t0);
+            } else if (in0) {
+                fold_pair(T, F, skip, in1, t0, t1, S0, S1);
+            }
             if (sp.G == 1) {
                 if (in0) lse.add(ray_lnrate(smin, t0, S0));
                 if (in1) lse.add(ray_lnrate(smin, t1, S1));

@@ -316,3 +316,22 @@ def test_products_of_6_and_7_byte_rows(n, per):
         want, _ = solve(U.SEG_RECOMPUTE, 1, x0.clone(), warm_start=True)
         dx = ((x1 - want).abs() / want).cpu().numpy()[pick]
         assert (dx <= 2e-6 * lnrate_sensitivity(tau, so, wo) + 2e-6).all()
+
+
+@pytest.mark.parametrize("R,F", [(3, 100), (7, 20), (15, 33)])
+def test_rates_of_odd_ray_counts(R, F):
+    # the last ray of an odd number is folded by itself: the same bits as a thread
+    # per ray gives, also where bins underflow and for columns out of range
+    n = 1000000 // R + 1
+    g = torch.Generator(device="cuda").manual_seed(R)
+    tau = 10.0 ** (9 * torch.rand(n, R, generator=g, device="cuda") - 4)
+    tau[1] = float("nan")
+    tau[2, R - 1] = float("inf")
+    tau[3] = 0.0
+    e, J = W.powerlaw_spectrum(F, 13.6, 54.4)
+    s, wts = (_dev(a) for a in U.urchin_spectrum_weights(e, J, 1e-12))
+    many = U.urchin_gamma(tau, s, wts)
+    for a in (0, n // 2, n - 100):
+        few = U.urchin_gamma(tau[a:a + 100].contiguous(), s, wts)
+        for p, q in zip(few, many):
+            assert torch.equal(p.nan_to_num(-1.0), q[a:a + 100].nan_to_num(-1.0))
