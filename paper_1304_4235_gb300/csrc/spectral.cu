@@ -493,11 +493,18 @@ __global__ void k_equilibrium_vjp(const double* __restrict__ gamma, const float*
 
 // Near/far rate per origin (Eqs. gammafar, gammashldk, gammashld), in double:
 // ln(Gamma_far,k / Gamma_thin) by the factored fold and the slab solution, one
-// thread per ray, then a log-sum-exp over the rays in their order by one
-// thread per origin.  (One thread per origin for all of it left most of the
-// GPU idle.  50021 halo particles, 12 rays, numerical slab, with the spectrum
-// table below: columns and rate 7.23 -> 6.79 ms.)
+// thread per ray, then a log-sum-exp over the rays: the row's largest by one
+// thread, the exponentials by the rays' threads, their sum in order by one
+// thread.  Bound by the FP64 pipe (numerical slab in FP32: by its evaluations).
+// (One thread per origin for all of it left most of the GPU idle, and one for the
+// log-sum-exp, an exponential after the other, made 48 rays slower than that:
+// numerical slab, ms, 50021 rows, 12 rays x 100 bins 0.79 -> 0.59, 48 x 20 2.09
+// -> 2.57 with it, 1.88 without.)  Up to 4 rays, blocks of 64 threads, so that
+// few origins reach more SMs (700 rows of one ray, analytic slab 0.27 -> 0.15 ms;
+// one thread per origin 0.16); beyond, blocks of 64 leave more threads without a
+// ray (300000 rows, 12 rays 3.39 against 2.55 ms with 256).
 constexpr int kNearFarThreads = 256;
+constexpr int kNearFarFew = 64;
 template <typename Real>
 __global__ void __launch_bounds__(kNearFarThreads)
 k_gamma_nearfar(const Real* __restrict__ tf, const Real* __restrict__ tn, int64_t n_orig, int R,
@@ -526,7 +533,7 @@ k_gamma_nearfar(const Real* __restrict__ tf, const Real* __restrict__ tn, int64_
         ws[b] = wv[b] / gthin;
     }
     __syncthreads();
-    const int rows = kNearFarThreads / R, local = threadIdx.x / R, k = threadIdx.x - local * R;
+    const int rows = (int)blockDim.x / R, local = threadIdx.x / R, k = threadIdx.x - local * R;
     // the ray's share (1/R) of the radiation lights its slab; rates add over rays
     const double lnR = log((double)R);
     for (int64_t row0 = (int64_t)blockIdx.x * rows; row0 < n_orig; row0 += (int64_t)gridDim.x * rows) {
@@ -554,19 +561,25 @@ k_gamma_nearfar(const Real* __restrict__ tf, const Real* __restrict__ tn, int64_
             lk[local * R + k] = l;
         }
         __syncthreads();
+        // (al holds the row's largest from here on)
         if (threadIdx.x < rows && mine < n_orig) {
-            double m = -INFINITY, acc = 0.0;
+            double m = -INFINITY;
             for (int q = 0; q < R; ++q) {
                 const double l = lk[threadIdx.x * R + q];
-                if (!(l > -INFINITY)) continue;
-                if (l > m) {
-                    acc = acc * exp(m - l) + 1.0;
-                    m = l;
-                } else {
-                    acc += exp(l - m);
-                }
+                if (l > m) m = l;
             }
-            const double lr = m + log(acc / (double)R);
+            al[threadIdx.x] = m;
+        }
+        __syncthreads();
+        if (local < rows && o < n_orig) {
+            const double l = lk[local * R + k];
+            lk[local * R + k] = l > -INFINITY ? exp(l - al[local]) : 0.0;
+        }
+        __syncthreads();
+        if (threadIdx.x < rows && mine < n_orig) {
+            double acc = 0.0;
+            for (int q = 0; q < R; ++q) acc += lk[threadIdx.x * R + q];
+            const double lr = al[threadIdx.x] + log(acc / (double)R);
             gamma_out[mine] = gthin * exp(lr);
             if (tau_eff_out) tau_eff_out[mine] = (float)(-lr);
         }
@@ -879,16 +892,16 @@ extern "C" int urchin_gamma_nearfar(const void* tau_far, const void* tau_near, i
     const bool f64 = precision == URCHIN_F64;
     const void* fn = f64 ? (const void*)k_gamma_nearfar<double> : (const void*)k_gamma_nearfar<float>;
     URCHIN_TRY(allow_shared(fn, smem, sizeof(double) * 2 * URCHIN_MAX_BINS));
-    const int rows = kNearFarThreads / R;
+    const int threads = R <= 4 ? kNearFarFew : kNearFarThreads, rows = threads / R;
     int grid = 0;
-    URCHIN_TRY(grid_for(fn, kNearFarThreads, smem, &grid));
+    URCHIN_TRY(grid_for(fn, threads, smem, &grid));
     grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (n_orig + rows - 1) / rows));
     if (f64)
-        k_gamma_nearfar<double><<<grid, kNearFarThreads, smem, s>>>(
+        k_gamma_nearfar<double><<<grid, threads, smem, s>>>(
             static_cast<const double*>(tau_far), static_cast<const double*>(tau_near), n_orig, R, sp->s, sp->w, sp->F, nH,
             T, caseB, poly, gamma_out, tau_eff_out);
     else
-        k_gamma_nearfar<float><<<grid, kNearFarThreads, smem, s>>>(
+        k_gamma_nearfar<float><<<grid, threads, smem, s>>>(
             static_cast<const float*>(tau_far), static_cast<const float*>(tau_near), n_orig, R, sp->s, sp->w, sp->F, nH, T,
             caseB, poly, gamma_out, tau_eff_out);
     URCHIN_TRY(launched());

@@ -335,3 +335,31 @@ def test_rates_of_odd_ray_counts(R, F):
         few = U.urchin_gamma(tau[a:a + 100].contiguous(), s, wts)
         for p, q in zip(few, many):
             assert torch.equal(p.nan_to_num(-1.0), q[a:a + 100].nan_to_num(-1.0))
+
+
+@pytest.mark.parametrize("slab", [U.SLAB_THRESHOLD, U.SLAB_SPECTRUM])
+@pytest.mark.parametrize("R", [1, 2, 3, 48, 192])
+def test_near_far_rate_is_the_mean_of_its_rays(R, slab):
+    # a row whose rays all equal ray k has that ray's rate, and rows add up to the
+    # mean of those (a sum of R doubles: R roundings, and some in each exponential);
+    # a row does not depend on the others
+    n = 1300 if R <= 3 else 20
+    g = torch.Generator(device="cuda").manual_seed(R)
+    tf = 10.0 ** (5 * torch.rand(n, R, generator=g, device="cuda", dtype=torch.float64) - 4)
+    tn = 10.0 ** (5 * torch.rand(n, R, generator=g, device="cuda", dtype=torch.float64) - 4)
+    tf[1, R // 2] = tf[2] = float("inf") if slab == U.SLAB_SPECTRUM else 1e5
+    nH = torch.full((n,), 1e-2, dtype=torch.float64, device="cuda")
+    e, J = W.powerlaw_spectrum(30, 13.6, 54.4)
+    s, wts = (_dev(a) for a in U.urchin_spectrum_weights(e, J, 1e-12))
+
+    def rate(a, b):
+        m = a.shape[0]
+        return U.urchin_gamma_nearfar(a.contiguous(), b.contiguous(), s, wts, nH[:m], nH[:m] * 1e6, slab=slab)
+
+    gam, te = rate(tf, tn)
+    want = sum(rate(tf[:, k:k + 1].expand(n, R), tn[:, k:k + 1].expand(n, R))[0] for k in range(R)) / R
+    ok = want > 0
+    assert float(gam[~ok].abs().sum()) == 0.0
+    assert float(((gam - want).abs()[ok] / want[ok]).max()) < 1e-13 + 3e-16 * R
+    part = rate(tf[:7], tn[:7])
+    assert torch.equal(part[0], gam[:7]) and torch.equal(part[1], te[:7])
