@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kSpmvThreads) k_chunk_compact(ChunkCompactArgs
 // z is good to its last digits only, and the adjoint rounds its coefficients to
 // FP32 at every product: a digit that moves flips a rounding now and then, and
 // the gradient of a 32768-particle halo repeats to 1e-15 for some inputs and to
-// 1e-10 to 1e-6 for others.  With 6-byte rows the additions arrived in another
+// 1e-10 to 2e-5 for others.  With 6-byte rows the additions arrived in another
 // order (no high bytes to wait for) and other inputs were the uneven ones, so
 // these rows keep their high bytes at every n (100.3 -> 101.0 ms for that halo's
 // solve and gradient).  A sum in two limbs that does not depend on the order

@@ -501,7 +501,7 @@ __device__ __forceinline__ bool beam_box(const Beam& B, float4 lo, float4 hi)
 // A warp's work space: a block of up to 32 spheres that the beam may reach and
 // the list of (ray, sphere) pairs that the lanes' masks give for it, at most
 // kPairs at a time (4 spheres never give more than 128).  The sizes keep three
-// blocks of 8 warps on an SM.
+// blocks of 8 warps on an SM (TraceLayout asserts it).
 template <typename Real>
 struct alignas(4 * sizeof(Real)) Origin {
     Real x, y, z;                 // a lane's (image-shifted) origin
@@ -1468,11 +1468,11 @@ struct TraceLayout {
 };
 static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, false>) % 16 == 0, "shared layout");
 
-// Bound by instruction issue (75 % of the slots for plain columns, 71 % with the
+// Bound by instruction issue (80 % of the slots for plain columns, 73 % with the
 // lists; 1/5 of the stalls waiting for shared memory, DRAM idle but for the
-// lists): 28 warp instructions per crossed sphere on the log-normal box with 32
-// origins per beam, 34 with the lists, against 45 and 46 when every lane tested
-// every staged sphere exactly, and 14 on the halo's long rays (21).  The pair
+// lists): 29 warp instructions per crossed sphere on the 96^3 log-normal box with
+// 32 origins per beam, 36 with the lists, against 45 and 46 (128^3) when every lane
+// tested every staged sphere exactly, and 14 on a halo's long rays (21).  The pair
 // list keeps the exact test and the chords at 30 of 32 lanes (16 to 21 when
 // every lane took its own next candidate).  The traversal's loop has to fit
 // the instruction cache: with two copies of the partial chords' code in it the
@@ -1488,8 +1488,9 @@ static_assert(alignof(Staged<double, 2, true>) <= 32 && sizeof(Staged<float, 4, 
 // -> 0.36 ms, unevenly spread in blocks of 14.  The other FP32 modes need more
 // shared memory per warp (list-keeping 128^3 solve 101.9 ms, with 26 warps
 // 103.6; transpose of the 65536-particle halo 6.3 ms with 16 to 24 warps).
-// FP64: bound by the FP64 pipe (84 % busy before the queues of full and partial
-// chords, at 17 of 32 lanes), two blocks; with queues and table logarithms the
+// FP64: bound by the FP64 pipe (85 % busy on the 16^3 lattice, 84 % on a 32^3 box
+// with G_t, at 22 and 26 of 32 lanes; 17 before the queues of full and partial
+// chords), two blocks; with queues and table logarithms the
 // 16^3 lattice solve 18.3 -> 11.0 ms (82 ms with every lane testing every staged
 // sphere), 24^3 box 10.7 -> 5.0 ms, 8000-particle halo 13.1 -> 8.4 ms, 9973 x 48
 // rays of the 48^3 box (G_t) 25.3 -> 18.7 ms (277).
