@@ -81,8 +81,9 @@ typedef struct CUstream_st* urchin_stream_t;
 #define URCHIN_SEG_AUTO         2     /* store when the lists fit in memory     */
 /* A stored segment is the FP32 value and the particle's slot in the tree's
  * order split into 16 + 8 bits (7 bytes, or 6 without the high byte up to n =
- * 65536; n <= 2^24), or FP64 value and int32 index (12 bytes); each ray's list
- * is padded with zero entries to a multiple of 8.
+ * 65536, urchin_solve_vjp's rows excepted; n <= 2^24), or FP64 value and int32
+ * index (12 bytes); each ray's list is padded with zero entries to a multiple
+ * of 8.
  * URCHIN_SEG_AUTO in FP32 (no near/far split, blocks <= 1) keeps the lists
  * of the first sweep's traversal itself, in linked chunks of 32 (index,
  * value) pairs of 8 bytes sized from a sampled estimate, so that a solve of
